@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -139,12 +140,106 @@ void fold_bias(int32_t bias, int8_t w[kBiasRows]) {
   }
 }
 
+// Constants of the one-instruction requantisation (FloatRq, level_device.cuh) of a channel whose clip is
+// 0..top: rne((acc + beta) m - C) = floor((acc M0 + 2^(30+s)) / 2^(31+s)) for every acc on either side of
+// every threshold of the clipped result, and hence (both sides are non-decreasing) for every acc. The
+// multiply-add is exact before its one rounding, so this is arithmetic on integers: m = q 2^-e with a
+// 24-bit q. m alone (beta = C = 0) does for most channels; for the rest a shift beta of the bias and an
+// integer C move the line by beta m - C, any fraction of a unit.
+struct FloatChannel {
+  float m = 0.f;
+  int32_t beta = 0, C = 0;
+};
+bool float_requant(int32_t m0, int32_t s, int top, int64_t beta_room, FloatChannel* out) {
+  if (s < 1) return false;
+  std::vector<int64_t> T(top + 1);               // T[k]: smallest acc with result >= k
+  for (int k = 1; k <= top; ++k) {
+    const __int128 num = (__int128)(2 * k - 1) << (30 + s);
+    T[k] = (int64_t)((num + m0 - 1) / m0);
+  }
+  if (T[top] + beta_room >= (1 << 23)) return false;
+  const double slope = std::ldexp((double)m0, -(31 + s));
+  int e = 0;
+  std::frexp(slope, &e);                         // slope = f 2^e, f in [1/2, 1)
+  const int sh = 24 - e;                         // m = q 2^-sh, q in [2^23, 2^24)
+  if (sh > 60) return false;
+  const int64_t q0 = (int64_t)std::ldexp(slope, sh);
+  // offsets (units of 2^-sh) for which all thresholds are met with multiplier q: lo < offset < hi
+  auto window = [&](int64_t q, __int128* lo, __int128* hi) {
+    bool first = true;
+    for (int k = 1; k <= top; ++k) {
+      const __int128 edge = (__int128)(2 * k - 1) << (sh - 1);               // k - 1/2
+      const __int128 a = edge - (__int128)q * T[k], b = edge - (__int128)q * (T[k] - 1);
+      if (first || a > *lo) *lo = a;
+      if (first || b < *hi) *hi = b;
+      first = false;
+    }
+    return *lo < *hi;
+  };
+  __int128 lo = 0, hi = 0;
+  for (int64_t dq = 0; dq <= 8; ++dq)
+    for (int sign = 0; sign < (dq ? 2 : 1); ++sign) {
+      const int64_t q = sign ? q0 - dq : q0 + dq;
+      if (q < (1 << 23) || q >= (1 << 24) || !window(q, &lo, &hi) || lo >= 0 || hi <= 0) continue;
+      *out = FloatChannel{(float)std::ldexp((double)q, -sh), 0, 0};
+      return true;
+    }
+  for (int64_t dq = 0; dq <= 8; ++dq)
+    for (int sign = 0; sign < (dq ? 2 : 1); ++sign) {
+      const int64_t q = sign ? q0 - dq : q0 + dq;
+      if (q < (1 << 23) || q >= (1 << 24) || !window(q, &lo, &hi)) continue;
+      for (int32_t C = 1; C < 4096; ++C) {
+        const __int128 t = ((__int128)C << sh) + lo;                          // beta q - C 2^sh > lo
+        const int64_t beta = (int64_t)(t / q) + (t >= 0 ? 1 : 0);
+        if (beta > beta_room) break;
+        const __int128 off = (__int128)beta * q - ((__int128)C << sh);
+        if (off > lo && off < hi) {
+          *out = FloatChannel{(float)std::ldexp((double)q, -sh), (int32_t)beta, C};
+          return true;
+        }
+      }
+    }
+  return false;
+}
+
+// Order in which a hidden layer's channels are packed (a permutation of the rows of its weight matrix and
+// of the columns of the next one), and the constants of the floating-point flavour where it applies.
+struct HiddenOrder {
+  std::vector<int> ch;              // packed position -> channel
+  bool is_float = false;
+  std::vector<FloatChannel> fc;     // by channel
+  int nf = 0;                       // packed columns below nf need no addend
+};
+HiddenOrder order_hidden(const iodf_layer_desc& L, const Blobs& B, Act a, int n_pad) {
+  HiddenOrder o;
+  const int n = (int)L.c_out;
+  o.ch.resize(n);
+  for (int i = 0; i < n; ++i) o.ch[i] = i;
+  o.nf = n_pad;
+  const int32_t* bias = B.r + L.requant_off;
+  const int32_t* m0 = bias + n;
+  const int32_t* s = m0 + n;
+  if (a.lo != 0 || a.hi != 127) return o;
+  o.fc.resize(n);
+  for (int i = 0; i < n; ++i) {
+    const int64_t room = kFoldMaxBias - std::llabs((long long)bias[i]);
+    if (s[i] != s[0] || room < 0 || !float_requant(m0[i], s[i], a.hi, room, &o.fc[i])) return o;
+  }
+  o.is_float = true;
+  std::stable_partition(o.ch.begin(), o.ch.end(), [&](int i) { return o.fc[i].C == 0; });
+  int plain = 0;
+  while (plain < n && o.fc[o.ch[plain]].C == 0) ++plain;
+  if (plain < n) o.nf = plain / 16 * 16;
+  return o;
+}
+
 // Fills the constant tables of a hidden layer and picks its requantisation flavour:
+//   4: the floating-point form of 3 (FloatRq): table of float multipliers (mb[i])
 //   3: one shift s >= 1 for the whole layer and every bias foldable: table of multipliers (mb[i])
 //   2: one shift s >= 1: table of {m0, bias} pairs (mb[2i], mb[2i+1])
 //   1 / 0: per-channel shifts (HiddenRq table)
-void put_hidden_rq(HiddenRq* dst, int32_t* mb, const iodf_layer_desc& L, const Blobs& B, int n_pad, int* mode,
-                   int* uniform_s) {
+void put_hidden_rq(HiddenRq* dst, int32_t* mb, const iodf_layer_desc& L, const Blobs& B, const HiddenOrder& ord, int n_pad,
+                   int* mode, int* uniform_s) {
   const int32_t* bias = B.r + L.requant_off;
   const int32_t* m0 = bias + L.c_out;
   const int32_t* s = m0 + L.c_out;
@@ -176,6 +271,13 @@ void put_hidden_rq(HiddenRq* dst, int32_t* mb, const iodf_layer_desc& L, const B
   *uniform_s = uniform ? s[0] : 0;
   if (*mode == 3)
     for (int i = 0; i < n_pad; ++i) mb[i] = i < (int)L.c_out ? m0[i] : (1 << 30);
+  if (ord.is_float) {
+    *mode = 4;
+    for (int i = 0; i < n_pad; ++i) {
+      const float m = i < (int)L.c_out ? ord.fc[ord.ch[i]].m : 1.0f;
+      std::memcpy(&mb[i], &m, 4);
+    }
+  }
 }
 
 void put_out_rq(OutRq* dst, const iodf_layer_desc& L, const Blobs& B) {
@@ -234,16 +336,32 @@ PackedBlock pack_coupling(const iodf_coupling_desc& cp, const Blobs& B, int ca, 
   // requantisation tables: both flavours are built, only the one the layer's mode reads is kept
   std::vector<HiddenRq> h1(d.n1), h2(d.n2);
   std::vector<int32_t> u1(2 * d.n1), u2(2 * d.n2);
-  put_hidden_rq(h1.data(), u1.data(), L1, B, d.n1, &M.mode1, &M.us1);
-  put_hidden_rq(h2.data(), u2.data(), L2, B, d.n2, &M.mode2, &M.us2);
+  const HiddenOrder o1 = order_hidden(L1, B, a1, d.n1), o2 = order_hidden(L2, B, a2, d.n2);
+  put_hidden_rq(h1.data(), u1.data(), L1, B, o1, d.n1, &M.mode1, &M.us1);
+  put_hidden_rq(h2.data(), u2.data(), L2, B, o2, d.n2, &M.mode2, &M.us2);
+  M.nf1 = o1.nf; M.nf2 = o2.nf;
+  // addends -C (in units of the subnormal accumulator, 2^-149) of the columns from nf - 8 on
+  auto addends = [](const HiddenOrder& o, int n) {
+    std::vector<int32_t> t;
+    if (!o.is_float || o.nf >= n) return t;
+    t.assign(up((uint32_t)(n - o.nf + 8), 4), 0);
+    for (int i = o.nf; i < (int)o.ch.size(); ++i)
+      if (o.fc[o.ch[i]].C) t[i - o.nf + 8] = (int32_t)(0x80000000u | (uint32_t)o.fc[o.ch[i]].C);
+    return t;
+  };
+  const std::vector<int32_t> c1 = addends(o1, d.n1), c2 = addends(o2, d.n2);
   uint32_t off = sizeof(CouplingMeta);
   M.off_colA = (int)off; off += up(4 * ca, 16);
   M.off_colB = (int)off; off += up(4 * cb, 16);
   M.off_out = (int)off;  off += (uint32_t)sizeof(OutRq) * cb;
-  auto table_bytes = [](int mode, int n) { return mode == 3 ? 4u * n : mode == 2 ? 8u * n : (uint32_t)sizeof(HiddenRq) * n; };
+  auto table_bytes = [](int mode, int n) { return mode >= 3 ? 4u * n : mode == 2 ? 8u * n : (uint32_t)sizeof(HiddenRq) * n; };
   M.off_h1 = M.off_u1 = (int)off; off += table_bytes(M.mode1, d.n1);
   M.off_h2 = M.off_u2 = (int)off; off += table_bytes(M.mode2, d.n2);
+  M.off_c1 = (int)off; off += 4u * (uint32_t)c1.size();
+  M.off_c2 = (int)off; off += 4u * (uint32_t)c2.size();
   pb.meta.assign(off, 0);
+  if (!c1.empty()) std::memcpy(pb.meta.data() + M.off_c1, c1.data(), 4 * c1.size());
+  if (!c2.empty()) std::memcpy(pb.meta.data() + M.off_c2, c2.data(), 4 * c2.size());
   std::memcpy(pb.meta.data() + M.off_colA, colA, 4 * ca);
   std::memcpy(pb.meta.data() + M.off_colB, colB, 4 * cb);
   put_out_rq(reinterpret_cast<OutRq*>(pb.meta.data() + M.off_out), L3, B);
@@ -260,12 +378,12 @@ PackedBlock pack_coupling(const iodf_coupling_desc& cp, const Blobs& B, int ca, 
   for (int n = 0; n < k1; ++n)
     for (int tap = 0; tap < 9; ++tap)
       for (int c = 0; c < ca; ++c)
-        pb.w[0][wpos(d.n1, n, tap * cpad + c)] = (uint8_t)w1[((size_t)n * 9 + tap) * ca + c];
-  if (M.mode1 == 3) {            // bias rows right after the nine taps
+        pb.w[0][wpos(d.n1, n, tap * cpad + c)] = (uint8_t)w1[((size_t)o1.ch[n] * 9 + tap) * ca + c];
+  if (M.mode1 >= 3) {            // bias rows right after the nine taps
     const int32_t* b1 = B.r + L1.requant_off;
     for (int n = 0; n < k1; ++n) {
       int8_t bw[kBiasRows];
-      fold_bias(b1[n], bw);
+      fold_bias(b1[o1.ch[n]] + (o1.is_float ? o1.fc[o1.ch[n]].beta : 0), bw);
       for (int j = 0; j < kBiasRows; ++j) pb.w[0][wpos(d.n1, n, 9 * cpad + j)] = (uint8_t)bw[j];
     }
   }
@@ -273,12 +391,12 @@ PackedBlock pack_coupling(const iodf_coupling_desc& cp, const Blobs& B, int ca, 
   pb.w[1].assign((size_t)d.n2 * d.kd2, 0);
   const int8_t* w2 = B.w + L2.weight_off;
   for (int n = 0; n < k2; ++n)
-    for (int k = 0; k < k1; ++k) pb.w[1][wpos(d.n2, n, k)] = (uint8_t)w2[(size_t)n * k1 + k];
-  if (M.mode2 == 3) {            // bias rows right after the (padded) hidden channels
+    for (int k = 0; k < k1; ++k) pb.w[1][wpos(d.n2, n, k)] = (uint8_t)w2[(size_t)o2.ch[n] * k1 + o1.ch[k]];
+  if (M.mode2 >= 3) {            // bias rows right after the (padded) hidden channels
     const int32_t* b2 = B.r + L2.requant_off;
     for (int n = 0; n < k2; ++n) {
       int8_t bw[kBiasRows];
-      fold_bias(b2[n], bw);
+      fold_bias(b2[o2.ch[n]] + (o2.is_float ? o2.fc[o2.ch[n]].beta : 0), bw);
       for (int j = 0; j < kBiasRows; ++j) pb.w[1][wpos(d.n2, n, d.n1 + j)] = (uint8_t)bw[j];
     }
   }
@@ -288,7 +406,7 @@ PackedBlock pack_coupling(const iodf_coupling_desc& cp, const Blobs& B, int ca, 
   for (int c = 0; c < cb; ++c)
     for (int tap = 0; tap < 9; ++tap)
       for (int k = 0; k < k2; ++k)
-        pb.w[2][wpos(d.n3, tap * cbp + c, k)] = (uint8_t)w3[((size_t)c * 9 + tap) * k2 + k];
+        pb.w[2][wpos(d.n3, tap * cbp + c, k)] = (uint8_t)w3[((size_t)c * 9 + tap) * k2 + o2.ch[k]];
   return pb;
 }
 
@@ -334,7 +452,7 @@ constexpr int kPipeMinTiles = IODF_PIPE_MIN_TILES;
 
 // What that kernel needs to know about a level.
 struct PipeDims {
-  bool eligible = false;           // every coupling in the folded flavour with the 0..127 clip
+  bool eligible = false;           // every coupling in the floating-point requantisation flavour
   uint32_t a1_bytes = 16;          // im2col operand of a tile (couplings and prior head)
   uint32_t n_hidden = 0;           // widest accumulator of the first two GEMMs (and of the prior head)
   uint32_t n_taps = 0;             // accumulator of the third GEMM: nine taps x padded C/2
@@ -776,7 +894,7 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
       a_bytes = std::max<uint32_t>(a_bytes, kTileM * std::max(d.kd1, std::max(d.kd2, d.kd3)));
       n_max = std::max<uint32_t>(n_max, std::max(d.n1, std::max(d.n2, d.n3)));
       const CouplingMeta* cm = reinterpret_cast<const CouplingMeta*>(blocks.back().meta.data());
-      if (cm->mode1 != 3 || cm->mode2 != 3 || a1.lo != 0 || a1.hi != 127 || a2r.lo != 0 || a2r.hi != 127) pd.eligible = false;
+      if (cm->mode1 != 4 || cm->mode2 != 4) pd.eligible = false;
       pd.n_hidden = std::max<uint32_t>(pd.n_hidden, (uint32_t)std::max(d.n1, d.n2));
       pd.a1_bytes = std::max<uint32_t>(pd.a1_bytes, (uint32_t)kTileM * d.kd1);
       pd.n_taps = std::max<uint32_t>(pd.n_taps, (uint32_t)d.n3);

@@ -64,14 +64,17 @@ struct CouplingMeta {
   int32_t n3;                    // 9*cbp padded to 16 (per-tap partial outputs of the last conv)
   int32_t lo1, hi1, lo2, hi2;    // effective activation clips (ReLU folded in)
   int32_t mode1, mode2;          // requantisation flavour of the two hidden layers:
+                                 //   4: as 3 with the 0..127 clip, in floating point (FloatRq; float m table)
                                  //   3: one shift s >= 1 and the bias folded into the GEMM (m0 table)
                                  //   2: one shift s >= 1 for the whole layer ({m0, bias} table)
                                  //   1: per-channel shifts, all >= 1 (HiddenRq table, high-word path)
                                  //   0: any shift (HiddenRq table, full 64-bit shift)
-  int32_t us1, us2;              // the uniform shift (modes 2 and 3)
+  int32_t us1, us2;              // the uniform shift (modes 2, 3 and 4)
   int32_t off_colA, off_colB, off_out, off_h1, off_h2;   // byte offsets from the meta start
-  int32_t off_u1, off_u2;        // {m0, bias} tables (int2 per channel; mode 3: int32 m0 per channel)
-  int32_t pad[9];
+  int32_t off_u1, off_u2;        // {m0, bias} tables (int2 per channel; mode 3: int32 m0, mode 4: float m)
+  int32_t off_c1, off_c2;        // mode 4: float addends of the columns from nf on (the table starts at column nf - 8)
+  int32_t nf1, nf2;
+  int32_t pad[5];
 };
 static_assert(sizeof(CouplingMeta) == 128, "meta header is 128 bytes");
 
@@ -117,11 +120,10 @@ struct LevelPlan {
   int32_t streamed;              // 1: weights are streamed per tile in 32-byte K-slices through a ring of
                                  //    kRingDepth slots at s_w[0] (hidden widths above 256, one tile in flight)
   uint32_t ring_slot_bytes;
-  int32_t lean;                  // 1: every hidden layer in the folded requantisation flavour with the 0..127 clip,
+  int32_t lean;                  // 1: every hidden layer in the floating-point requantisation flavour (mode 4),
                                  //    weights not streamed: the general kernel's small variant runs the level
   int32_t pipe;                  // 1: the level runs in the kernel that splits a tile's work by role (several
-                                 //    tiles per CTA, two tile slots, resident weights, folded requantisation with
-                                 //    the 0..127 clip)
+                                 //    tiles per CTA, two tile slots, resident weights, mode 4 requantisation)
   int32_t r_col[3];              // that kernel's tensor-memory columns: slot s has its hidden-layer accumulators
                                  //    at s * r_col[0] and its per-tap partials at r_col[1] + s * r_col[2]
                                  //    (r_col[1] = 0: the partials share the slot's main columns)

@@ -168,6 +168,7 @@ __device__ __forceinline__ void build_im2col(const Ctx& cx, uint8_t* __restrict_
 }
 
 // Requantisation flavours of a hidden layer (chosen per layer when the model is packed):
+//   kModeFloat    as kModeFolded with ReLU and the clip to 0..127: one floating-point multiply-add (FloatRq)
 //   kModeFolded   the same shift s >= 1 for every channel and the bias already in the accumulator
 //                 (bias rows of the GEMM): constant m0 per channel, y = hi32(acc * m0 + 2^(30+s)) >> (s-1)
 //   kModeUniform  every channel has the same shift s >= 1: constants {m0, bias} per channel,
@@ -175,7 +176,7 @@ __device__ __forceinline__ void build_im2col(const Ctx& cx, uint8_t* __restrict_
 //   kModeFast     per-channel shifts, all s >= 1: y = hi32(acc * m0 + c64) >> (s-1)
 //   kModeExact    any s: y = (acc * m0 + c64) >> (31 + s) in 64 bits
 // All are exact: for s >= 1, floor(x / 2^(31+s)) = floor(floor(x / 2^32) / 2^(s-1)).
-constexpr int kModeFolded = 3, kModeUniform = 2, kModeFast = 1, kModeExact = 0;
+constexpr int kModeFloat = 4, kModeFolded = 3, kModeUniform = 2, kModeFast = 1, kModeExact = 0;
 
 // Clip flavours: kClipS8Relu is the common ReLU + clip to [0, 127]: the saturating 32->8 bit pack
 // clips to [-128, 127] and the negative bytes are then cleared; kClipU8Relu is ReLU + clip to
@@ -249,13 +250,52 @@ struct Requant {
   }
 };
 
+// The folded flavour with the 0..127 clip as ONE multiply-add per activation. The accumulator's bits are
+// read as a float: a non-negative int32 below 2^23 is the subnormal number a * 2^-149, so
+//     fma.rn.sat(a * 2^-149, m, -C * 2^-149)  =  rne(a m - C) * 2^-149
+// is a subnormal whose bits are the integer rne(a m - C) again: multiply, rescale, round and ReLU at once.
+// (A negative accumulator's bits are a NaN or a negative number, which .sat turns into 0; one of 2^23
+// and more only makes the result larger, and the pack's saturation clips it to 127.) Exactness is a
+// property of the constants: the host picks m (and for the few channels that need it a shift of the
+// bias and C) so that all 127 thresholds of y = floor((a M0 + 2^(30+s)) / 2^(31+s)) are hit to the unit,
+// and checks every one of them in integer arithmetic (float_requant in iodf_api.cu). Channels that need C
+// are packed last, from column nf on. Measured per SM from 16 warps: 34 activations per clock against
+// 16 for the integer form (high multiply-add, shift, pack, sign mask).
+struct FloatRq {
+  const float* __restrict__ m;         // multiplier per column
+  const float* __restrict__ c;         // addend of columns nf - 8, nf - 7, ...
+  int nf;
+  static __device__ __forceinline__ int one(uint32_t acc, float m, float c) {
+    float y;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(__uint_as_float(acc)), "f"(m), "f"(c));
+    return __float_as_int(y);
+  }
+  template <bool kC>
+  __device__ __forceinline__ uint32_t quad_t(const uint32_t* r, int ch0) const {
+    const float4 f = *reinterpret_cast<const float4*>(m + ch0);
+    float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (kC) d = *reinterpret_cast<const float4*>(c + (ch0 - nf + 8));
+    return pack4_sat(one(r[0], f.x, d.x), one(r[1], f.y, d.y), one(r[2], f.z, d.z), one(r[3], f.w, d.w));
+  }
+  __device__ __forceinline__ uint32_t quad(const uint32_t* r, int ch0) const {
+    return ch0 < nf ? quad_t<false>(r, ch0) : quad_t<true>(r, ch0);
+  }
+  __device__ __forceinline__ uint4 chunk(const uint32_t* r, int ch0) const {
+    if (ch0 + 16 <= nf)
+      return make_uint4(quad_t<false>(r, ch0), quad_t<false>(r + 4, ch0 + 4), quad_t<false>(r + 8, ch0 + 8),
+                        quad_t<false>(r + 12, ch0 + 12));
+    return make_uint4(quad_t<true>(r, ch0), quad_t<true>(r + 4, ch0 + 4), quad_t<true>(r + 8, ch0 + 8),
+                      quad_t<true>(r + 12, ch0 + 12));
+  }
+};
+
 // TMEM accumulator -> requantised int8 activations in the next GEMM's A layout. n is a multiple
 // of 16; kd (the next GEMM's K) is n rounded up to 32, the extra chunk being zero. The unit of work
 // is one 16-column chunk (= one 16-byte piece of the A row), dealt round-robin to the column
 // splits so that they differ by at most one chunk; a warp takes its chunks two at a time.
-template <int kMode, int kClip>
-__device__ __forceinline__ void epilogue_hidden_t(const Ctx& cx, int n, int kd, const Requant<kMode, kClip> q,
-                                                  uint32_t pad_lo, uint32_t pad_hi, uint8_t* __restrict__ sOut) {
+template <class Rq>
+__device__ __forceinline__ void epilogue_hidden_t(const Ctx& cx, int n, int kd, const Rq q, uint32_t pad_lo, uint32_t pad_hi,
+                                                  uint8_t* __restrict__ sOut) {
   const int nch = n >> 4;
   // A chunk goes to this thread's row in every replica of the tile (one replica: the row itself).
   uint8_t* out = sOut + cx.row * 16;
@@ -293,14 +333,15 @@ __device__ __forceinline__ void epilogue_hidden_t(const Ctx& cx, int n, int kd, 
 
 // mode: layer flavour (see above); us: the layer's uniform shift (kModeFolded, kModeUniform).
 __device__ __forceinline__ void epilogue_hidden(const Ctx& cx, int mode, int us, int n, int kd, const HiddenRq* rq,
-                                                const int2* mb, int lo, int hi, uint32_t pad_lo, uint32_t pad_hi,
+                                                const int2* mb, const FloatRq& fq, int lo, int hi, uint32_t pad_lo, uint32_t pad_hi,
                                                 uint8_t* sOut) {
   const bool s8relu = lo == 0 && hi == 127, u8relu = lo == 0 && hi == 255;
-  if (mode >= kModeUniform) {
+  if (mode == kModeFloat) {
+    epilogue_hidden_t(cx, n, kd, fq, pad_lo, pad_hi, sOut);
+  } else if (mode >= kModeUniform) {
     const long long rnd64 = 1ll << (30 + us);
     if (mode == kModeFolded) {
-      if (s8relu) epilogue_hidden_t(cx, n, kd, Requant<kModeFolded, kClipS8Relu>{rq, mb, lo, hi, us - 1, rnd64}, pad_lo, pad_hi, sOut);
-      else if (u8relu) epilogue_hidden_t(cx, n, kd, Requant<kModeFolded, kClipU8Relu>{rq, mb, lo, hi, us - 1, rnd64}, pad_lo, pad_hi, sOut);
+      if (u8relu) epilogue_hidden_t(cx, n, kd, Requant<kModeFolded, kClipU8Relu>{rq, mb, lo, hi, us - 1, rnd64}, pad_lo, pad_hi, sOut);
       else epilogue_hidden_t(cx, n, kd, Requant<kModeFolded, kClipAny>{rq, mb, lo, hi, us - 1, rnd64}, pad_lo, pad_hi, sOut);
     } else {
       if (s8relu) epilogue_hidden_t(cx, n, kd, Requant<kModeUniform, kClipS8Relu>{rq, mb, lo, hi, us - 1, rnd64}, pad_lo, pad_hi, sOut);

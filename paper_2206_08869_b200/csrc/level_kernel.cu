@@ -406,6 +406,8 @@ __device__ __forceinline__ void run_workers(Ctx& cx, const LevelPlan& P, const L
       const HiddenRq* h2 = reinterpret_cast<const HiddenRq*>(mb + M.off_h2);
       const int2* u1 = reinterpret_cast<const int2*>(mb + M.off_u1);
       const int2* u2 = reinterpret_cast<const int2*>(mb + M.off_u2);
+      const FloatRq q1{reinterpret_cast<const float*>(mb + M.off_u1), reinterpret_cast<const float*>(mb + M.off_c1), M.nf1};
+      const FloatRq q2{reinterpret_cast<const float*>(mb + M.off_u2), reinterpret_cast<const float*>(mb + M.off_c2), M.nf2};
       for (int t0 = 0; t0 < ntv; t0 += nslots) {
         const int nt = min(nslots, ntv - t0);
         for (int sl = 0; sl < nt; ++sl) {                     // conv 3x3: input -> hidden 1
@@ -417,16 +419,15 @@ __device__ __forceinline__ void run_workers(Ctx& cx, const LevelPlan& P, const L
         for (int sl = 0; sl < nt; ++sl) {                     // requant, conv 1x1
           wait_d(sl);
           use_slot(sl);
-          if (kLean) epilogue_hidden_t(cx, M.n1, M.kd2, Requant<kModeFolded, kClipS8Relu>{h1, u1, 0, 127, M.us1 - 1, 1ll << (30 + M.us1)},
-                                       kBiasColumnsLo, kBiasColumnsHi, sA);
-          else epilogue_hidden(cx, M.mode1, M.us1, M.n1, M.kd2, h1, u1, M.lo1, M.hi1, kBiasColumnsLo, kBiasColumnsHi, sA);
+          if (kLean) epilogue_hidden_t(cx, M.n1, M.kd2, q1, kBiasColumnsLo, kBiasColumnsHi, sA);
+          else epilogue_hidden(cx, M.mode1, M.us1, M.n1, M.kd2, h1, u1, q1, M.lo1, M.hi1, kBiasColumnsLo, kBiasColumnsHi, sA);
           arrive_a(sl);
         }
         for (int sl = 0; sl < nt; ++sl) {                     // requant, conv 3x3 as per-tap partials
           wait_d(sl);
           use_slot(sl);
-          if (kLean) epilogue_hidden_t(cx, M.n2, M.kd3, Requant<kModeFolded, kClipS8Relu>{h2, u2, 0, 127, M.us2 - 1, 1ll << (30 + M.us2)}, 0u, 0u, sA);
-          else epilogue_hidden(cx, M.mode2, M.us2, M.n2, M.kd3, h2, u2, M.lo2, M.hi2, 0u, 0u, sA);
+          if (kLean) epilogue_hidden_t(cx, M.n2, M.kd3, q2, 0u, 0u, sA);
+          else epilogue_hidden(cx, M.mode2, M.us2, M.n2, M.kd3, h2, u2, q2, M.lo2, M.hi2, 0u, 0u, sA);
           arrive_a(sl);
         }
         for (int sl = 0; sl < nt; ++sl) {                     // shifted sum into the accumulator

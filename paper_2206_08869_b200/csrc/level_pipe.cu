@@ -89,14 +89,11 @@ struct SlotCount {
 };
 
 // Columns [c0, c0 + m) of a tile's accumulator (this thread's row) -> requantised bytes of the next
-// operand's row: y = clip(hi32(acc * m0 + 2^(30+s)) >> (s-1), 0, 127), the bias being part of the
-// accumulator (folded flavour). c0 and m are multiples of 8. A tensor-memory load takes a few hundred
+// operand's row (FloatRq: the bias is part of the accumulator). c0 and m are multiples of 8. A tensor-memory load takes a few hundred
 // clocks from issue to use and tcgen05.wait::ld waits for every load in flight, so the loop is
 // pipelined by hand: the load of piece k+1 is issued right after the wait for piece k and travels
 // while piece k is requantised; only the first load of a phase is exposed.
-__device__ __forceinline__ void epilogue_lean(uint32_t taddr, int c0, int m, const int32_t* __restrict__ m0tab, int sh,
-                                              long long rnd64, uint8_t* __restrict__ out_row) {
-  const Requant<kModeFolded, kClipS8Relu> q{nullptr, reinterpret_cast<const int2*>(m0tab), 0, 127, sh, rnd64};
+__device__ __forceinline__ void epilogue_lean(uint32_t taddr, int c0, int m, const FloatRq q, uint8_t* __restrict__ out_row) {
   const bool aligned = (c0 & 15) == 0;
   auto store16 = [&](int col, const uint4 v) {
     uint8_t* d = out_row + (size_t)(col >> 4) * (kTileM * 16);
@@ -404,9 +401,9 @@ __device__ __forceinline__ void pipe_workers(const Pipe& pp, const LevelPlan& P,
         }
 #pragma unroll 1
         for (int layer = 0; layer < 2; ++layer) {
-          const int n = layer ? Mp->n2 : Mp->n1, kd = layer ? Mp->kd3 : Mp->kd2, us = layer ? Mp->us2 : Mp->us1;
-          const int32_t* m0tab = reinterpret_cast<const int32_t*>(mb + (layer ? Mp->off_u2 : Mp->off_u1));
-          const long long rnd64 = 1ll << (30 + us);
+          const int n = layer ? Mp->n2 : Mp->n1, kd = layer ? Mp->kd3 : Mp->kd2;
+          const FloatRq q{reinterpret_cast<const float*>(mb + (layer ? Mp->off_u2 : Mp->off_u1)),
+                          reinterpret_cast<const float*>(mb + (layer ? Mp->off_c2 : Mp->off_c1)), layer ? Mp->nf2 : Mp->nf1};
           // this warp's share of the columns: a quarter of the 8-column units
           const int units = n >> 3;
           const int c0 = ((units * cs) >> 2) << 3, c1 = ((units * (cs + 1)) >> 2) << 3;
@@ -421,7 +418,7 @@ __device__ __forceinline__ void pipe_workers(const Pipe& pp, const LevelPlan& P,
             for (int j = (n >> 4) + cs; j < (kd >> 4); j += 4)
               *reinterpret_cast<uint4*>(out_row + (size_t)j * (kTileM * 16)) =
                   (layer == 0 && j == (n >> 4)) ? make_uint4(kBiasColumnsLo, kBiasColumnsHi, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
-            epilogue_lean(main_cols(sl), c0, c1 - c0, m0tab, us - 1, rnd64, out_row);
+            epilogue_lean(main_cols(sl), c0, c1 - c0, q, out_row);
             pipe_arrive(pp, layer ? &ctl->a3_full[sl] : &ctl->a2_full[sl], true);
           }
         }
