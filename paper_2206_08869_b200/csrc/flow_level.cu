@@ -1,0 +1,798 @@
+// One flow level of three-conv couplings (the arithmetic of level_kernel.cu) in a kernel built to be
+// short: a coupling is a chain of a dozen phases that every warp runs once or a few times, so what a
+// phase costs is latency (hand-overs, tensor-memory loads, MMA round trips) and instruction fetch. The
+// general kernel's 209 KB of code does not fit the instruction caches: its phases took 1 000 - 2 000
+// clocks each for fewer than a hundred instructions per warp. This one is a few KB per phase loop.
+//
+//   * No im2col. The requantised network input sits in shared memory as a zero-bordered frame of
+//     16-byte records, and the first conv's operand descriptors point straight into it: a tile is an
+//     8-column block of the image, so its 8-row core-matrix groups are image rows, one frame row apart
+//     (the descriptor's stride offset), and a tap is a start address. Two 16-byte chunks make a K step;
+//     the leading offset is whatever lies between them (the next tap, or the record's next plane).
+//     Up to six input channels: a record holds its own pixel and the right neighbour (eight bytes each), so
+//     that a row of three taps is one K step. 4 x 4 levels build the operand by hand: whoever
+//     requantises a word writes it to the (up to) nine places that need it.
+//   * Bias columns are bytes of the records that no channel uses.
+//   * Hidden epilogues read 16 rows x 32 columns per unit: four threads share a row, a thread meets the same
+//     eight columns in two rows, which halves the loads of constants; the order of the channels within the
+//     next GEMM's K is free, so a thread's eight results are eight adjacent operand bytes.
+//   * The per-tap partial products of the last conv are added to a pixel-major accumulator (odd
+//     stride) with one shared-memory reduction each.
+//   * CTAs of several tiles have two in flight (slots), each with eight of the sixteen workers and an MMA
+//     warp of its own, so that one slot's hand-overs and MMAs run under the other's requantisation; CTAs of
+//     one tile put all sixteen workers on it. One lane of another warp streams weights and meta blocks.
+#include "flow_level.h"
+#include "level_device.cuh"
+
+namespace iodf {
+
+namespace {
+
+struct __align__(16) FlowCtl {
+  uint64_t xa_ready;      // workers -> MMA warp, loader: network input of the step written   (count kFlowWarps)
+  uint64_t a_ready[2];    // slot's workers -> its MMA warp: the next hidden operand is written
+  uint64_t dm_ready[2];   // tensor core -> workers: first / second GEMM of the slot's tile complete
+  uint64_t d3_ready[2];   // tensor core -> workers: per-tap partials of the slot's tile complete
+  uint64_t w_full[3], w_empty[3];   // weight slots: copy landed / last MMAs (of each tile slot) that read it complete
+  uint64_t meta_full[2];
+  uint32_t tmem_base;
+  uint32_t abort;
+  int4 tile[kFlowMaxTiles];         // {image, first row, first column, 16-byte units from the frame's start to that position}
+};
+
+struct Flow {
+  uint8_t* smem;
+  FlowCtl* ctl;
+  uint32_t* status;
+  uint32_t tmem;
+  int tid, warp, lane;
+  int nimg, pvalid, tiles;      // images, pixels and tiles of this CTA
+  int slots;                    // tile slots in use: 1 or 2
+  int sl, cs, ncs;              // worker: its slot, its share of a lane quarter's work (cs of ncs warps)
+};
+
+// One test, then suspended (spinning warps take issue slots and shared-memory bandwidth from the others).
+// Out of line: a dozen inlined copies cost more in instruction fetch than the call does.
+__device__ __noinline__ void flow_wait_at(uint32_t bar, uint32_t parity, FlowCtl* ctl, uint32_t* status) {
+  if (ptx::mbar_test_wait(bar, parity)) return;
+  for (uint32_t it = 0; it < kSpinLimit; ++it) {
+    if (ptx::mbar_try_wait(bar, parity)) return;
+    if (*reinterpret_cast<volatile uint32_t*>(&ctl->abort)) return;      // bounded: see ptx::bounded_wait
+  }
+  *reinterpret_cast<volatile uint32_t*>(&ctl->abort) = 1;
+  atomicExch(status, 1u);
+}
+__device__ __forceinline__ void flow_wait(const Flow& f, uint64_t* bar, uint32_t parity) {
+  const uint32_t b = ptx::smem_u32(bar);
+  if (ptx::mbar_test_wait(b, parity) || ptx::mbar_try_wait(b, parity)) return;
+  flow_wait_at(b, parity, f.ctl, f.status);
+}
+__device__ __forceinline__ void flow_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ptx::smem_u32(bar)) : "memory");
+}
+// this warp's shared-memory writes (towards the tensor core) and tensor-memory reads are done
+__device__ __forceinline__ void flow_hand_over(const Flow& f, uint64_t* bar) {
+  ptx::tc_fence_before();
+  ptx::fence_async_smem();
+  __syncwarp();
+  if (f.lane == 0) flow_arrive(bar);
+}
+__device__ __forceinline__ void worker_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kFlowWorkers) : "memory"); }
+
+// ---- weight and meta loader (one lane) -----------------------------------------------------------------
+__device__ void flow_loader(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st) {
+  FlowCtl* ctl = f.ctl;
+  uint32_t nl[3] = {0u, 0u, 0u};
+  auto copy = [&](uint32_t off, uint32_t bytes, uint32_t dst, uint64_t* bar) {
+    const uint32_t b = ptx::smem_u32(bar);
+    ptx::mbar_expect_tx(b, bytes);
+    ptx::bulk_g2s(ptx::smem_u32(f.smem + dst), a.blob + off, bytes, b);
+  };
+  auto meta = [&](int step) {
+    if (step >= st.nsteps) return;
+    const BlockRef& br = step_ref(*a.plan, st, step);
+    copy(br.meta_off, br.meta_bytes, P.s_meta[step & 1], &ctl->meta_full[step & 1]);
+  };
+  auto load = [&](int step, int g) {
+    if (step >= st.nsteps || (g > 0 && st.is_prior(step))) return;
+    const int s = (P.alias && g == 2) ? 0 : g;
+    const BlockRef& br = step_ref(*a.plan, st, step);
+    const uint32_t off = br.w_off[g], bytes = br.w_bytes[g];
+    if (nl[s] > 0) flow_wait(f, &ctl->w_empty[s], (nl[s] - 1u) & 1u);
+    ++nl[s];
+    copy(off, bytes, P.s_w[s], &ctl->w_full[s]);
+  };
+  meta(0);
+  load(0, 0);
+  load(0, 1);
+  if (!P.alias) load(0, 2);
+  meta(1);
+#pragma unroll 1
+  for (int i = 0; i < st.nsteps; ++i) {
+    if (P.alias) {          // in the order in which the slots become free
+      load(i, 2);
+      load(i + 1, 1);
+      load(i + 1, 0);
+    } else {
+      load(i + 1, 0);
+      load(i + 1, 1);
+      load(i + 1, 2);
+    }
+    // meta slot of step i: its last reader is the pixel pass of step i + 1
+    if (i + 2 < st.nsteps) {
+      flow_wait(f, &ctl->xa_ready, (uint32_t)(i + 1) & 1u);
+      meta(i + 2);
+    }
+  }
+}
+
+// ---- MMA warp --------------------------------------------------------------------------------------------
+// D (+)= A B^T over ks steps of 32 K bytes; n above 256 in two parts. The whole warp runs the loop on uniform
+// values, `lead` issues.
+__device__ __forceinline__ void flow_gemm(bool lead, uint32_t d, uint32_t al, uint32_t a_step, uint32_t bl, int n, int ks,
+                                          uint32_t idesc_m) {
+  const uint32_t hi = ptx::kUmmaDescHi, b_step = 2u * (uint32_t)n;
+  const int na = n > 256 ? 256 : n;
+  const uint32_t idesc = idesc_m | ((uint32_t)(na >> 3) << 17), idesc2 = idesc_m | ((uint32_t)((n - na) >> 3) << 17);
+#pragma unroll 1
+  for (int k = 0; k < ks; ++k) {
+    if (lead) ptx::umma_i8_hl(d, al, hi, bl, hi, idesc, k > 0 ? 1u : 0u);
+    if (n > 256 && lead) ptx::umma_i8_hl(d + 256u, al, hi, bl + 256u, hi, idesc2, k > 0 ? 1u : 0u);
+    al += a_step;
+    bl += b_step;
+  }
+}
+
+// MMA warp of tile slot `sl`: tiles sl, sl + 2, ...
+__device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int sl) {
+  if (sl >= f.slots) return;
+  FlowCtl* ctl = f.ctl;
+  uint8_t* smem = f.smem;
+  const bool lead = ptx::elect_one();
+  const uint32_t idesc_m = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.m >> 4) << 24);     // s8 x s8 -> s32
+  const uint32_t xa16 = ptx::smem_u32(smem + P.s_xa) >> 4;
+  const uint32_t a1_hi = (uint32_t)P.sbo16 | (1u << 14);
+  const uint32_t pitch16 = (uint32_t)P.pitch >> 4;
+  const uint32_t a_lo = ((ptx::smem_u32(smem + P.s_a[sl]) >> 4) & 0x3FFFu) | (pitch16 << 16);
+  const uint32_t dm = f.tmem + (uint32_t)(sl * P.d_col), d3 = f.tmem + (uint32_t)(P.d3_col + sl * P.d3_step);
+  const int s3 = P.alias ? 0 : 2;
+  auto commit = [&](uint64_t* bar) { if (lead) ptx::umma_commit(ptx::smem_u32(bar)); };
+  uint32_t used[3] = {0u, 0u, 0u}, apar = 0u;
+  auto wait_w = [&](int s) { flow_wait(f, &ctl->w_full[s], used[s] & 1u); };
+  auto wait_a = [&]() {
+    flow_wait(f, &ctl->a_ready[sl], apar);
+    apar ^= 1u;
+    ptx::tc_fence_after();
+  };
+#pragma unroll 1
+  for (int i = 0; i < st.nsteps; ++i) {
+    const bool prior = st.is_prior(i);
+    flow_wait(f, &ctl->meta_full[i & 1], (uint32_t)(i >> 1) & 1u);
+    const FlowMeta* M = reinterpret_cast<const FlowMeta*>(smem + P.s_meta[i & 1]);
+    // (through a shuffle: tells the compiler that the values are the same in all lanes, so that the operands of
+    // the MMAs are computed in uniform registers)
+    auto uniform = [](int x) { return __shfl_sync(0xFFFFFFFFu, x, 0); };
+    const int n1 = prior ? P.n_prior : uniform(M->n1), n2 = uniform(M->n2), n3 = uniform(M->n3);
+    const int ks2 = uniform(M->ks2), ks3 = uniform(M->ks3);
+    wait_w(0);
+    ++used[0];
+    const uint32_t b1 = ((ptx::smem_u32(smem + P.s_w[0]) >> 4) & 0x3FFFu) | ((uint32_t)n1 << 16);
+    const uint32_t b2 = ((ptx::smem_u32(smem + P.s_w[1]) >> 4) & 0x3FFFu) | ((uint32_t)n2 << 16);
+    const uint32_t b3 = ((ptx::smem_u32(smem + P.s_w[s3]) >> 4) & 0x3FFFu) | ((uint32_t)n3 << 16);
+    const uint32_t idesc1 = idesc_m | ((uint32_t)(n1 >> 3) << 17);
+    // first conv of a tile: steps from the table {start offset, leading offset}
+    auto first_conv = [&](int t, uint32_t d) {
+      const uint32_t base = xa16 + (uint32_t)uniform(ctl->tile[t].w);
+      uint32_t bl = b1;
+#pragma unroll 1
+      for (int s = 0; s < P.ks1; ++s) {
+        const uint32_t al = base + (uint32_t)P.step[s];
+        if (lead) ptx::umma_i8_hl(d, al, a1_hi, bl, ptx::kUmmaDescHi, idesc1, s > 0 ? 1u : 0u);
+        bl += 2u * (uint32_t)n1;
+      }
+    };
+    flow_wait(f, &ctl->xa_ready, (uint32_t)i & 1u);
+    ptx::tc_fence_after();
+    if (prior) {
+#pragma unroll 1
+      for (int t = sl; t < f.tiles; t += 2) first_conv(t, f.tmem + (uint32_t)(t * P.n_prior));
+      commit(&ctl->dm_ready[sl]);
+      commit(&ctl->w_empty[0]);
+      continue;
+    }
+#pragma unroll 1
+    for (int t = sl; t < f.tiles; t += 2) {
+      // the slot's accumulator has been drained: its last tile's third GEMM was issued after that
+      const bool last = t + 2 >= f.tiles;
+      first_conv(t, dm);
+      commit(&ctl->dm_ready[sl]);
+      if (last) commit(&ctl->w_empty[0]);
+      if (t == sl) wait_w(1);
+      wait_a();
+      flow_gemm(lead, dm, a_lo, 2u * pitch16, b2, n2, ks2, idesc_m);
+      commit(&ctl->dm_ready[sl]);
+      if (last) commit(&ctl->w_empty[1]);
+      if (t == sl) wait_w(s3);
+      wait_a();
+      flow_gemm(lead, d3, a_lo, 2u * pitch16, b3, n3, ks3, idesc_m);
+      commit(&ctl->d3_ready[sl]);
+      if (last) commit(&ctl->w_empty[s3]);
+    }
+    ++used[1];
+    ++used[s3];
+  }
+}
+
+// ---- workers ---------------------------------------------------------------------------------------------
+// Integer form (rare: blocks with a channel that has no floating-point constants)
+__device__ __forceinline__ uint32_t flow_integer_one(uint32_t acc, float m, int us) {
+  const long long p = (long long)(int)acc * (long long)__float_as_int(m) + (1ll << (30 + us));
+  return (uint32_t)max(0, (int)(p >> 32) >> (us - 1));
+}
+
+// Hidden epilogue of one tile: n accumulator columns at `taddr` (this warp's lane quarter) -> bytes of
+// the next GEMM's operand, ks 32-column blocks, dealt to the quarter's warps; rows in halves of 16. A
+// thread meets the same eight columns in all its rows, so their constants are loaded once per block. From
+// block n / 32 on the operand holds constants (cw) beyond the columns.
+template <int kHalves>
+__device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, uint32_t taddr, const FlowMeta* __restrict__ M, int layer,
+                                            uint8_t* __restrict__ sA, uint64_t* ready, uint32_t parity) {
+  // everything that does not depend on the accumulator comes before the wait for it
+  const int n = layer ? M->n2 : M->n1, ks = layer ? M->ks3 : M->ks2, nfi = layer ? M->nfi2 : M->nfi1;
+  const int nfb = layer ? M->nfb2 : M->nfb1;
+  const int q = f.lane & 3, nfull = n >> 5, plain = min(min(nfb, nfi), nfull);
+  const uint8_t* mb = reinterpret_cast<const uint8_t*>(M);
+  const float4* ft = reinterpret_cast<const float4*>(mb + (layer ? M->off_f2 : M->off_f1)) + q * 2;
+  const float4* ct = reinterpret_cast<const float4*>(mb + (layer ? M->off_c2 : M->off_c1)) + q * 2 - nfb * 8;
+  const uint32_t cw = layer ? 0u : kBiasColumnsLo;
+  uint8_t* out = sA + (q >> 1) * P.pitch + ((f.warp & 3) * (16 * kHalves) + (f.lane >> 2)) * 16 + (q & 1) * 8;
+  flow_wait(f, ready, parity);
+  ptx::tc_fence_after();
+#pragma unroll 1
+  for (int b = f.cs; b < ks; b += f.ncs) {
+    uint32_t r[kHalves][16];
+#pragma unroll
+    for (int h = 0; h < kHalves; ++h) ptx::tmem_ld_16x32(taddr + ((uint32_t)h << 20) + (uint32_t)(b << 5), r[h]);
+    const float4 m0 = ft[b * 8], m1 = ft[b * 8 + 1];
+    float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
+    const float m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+    const bool tail = b >= nfull, none = tail && !(n & 16);
+    uint8_t* o = out + (size_t)(2 * b) * P.pitch;
+    ptx::tmem_ld_wait16(r[0]);
+#pragma unroll
+    for (int h = 1; h < kHalves; ++h) ptx::tmem_ld_wait16_nosync(r[h]);
+    if (b < plain) {
+#pragma unroll
+      for (int h = 0; h < kHalves; ++h) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) r[h][k] = (uint32_t)FloatRq::one(r[h][k], m[2 * (k >> 2) + (k & 1)], 0.f);
+#pragma unroll
+        for (int e = 0; e < 4; e += 2)
+          *reinterpret_cast<uint2*>(o + h * 256 + e * 64) =
+              make_uint2(pack4_sat((int)r[h][e], (int)r[h][e + 1], (int)r[h][e + 4], (int)r[h][e + 5]),
+                         pack4_sat((int)r[h][e + 8], (int)r[h][e + 9], (int)r[h][e + 12], (int)r[h][e + 13]));
+      }
+      continue;
+    }
+    if (b >= nfb) {
+      c0 = ct[b * 8];
+      c1 = ct[b * 8 + 1];
+    }
+    const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+    if (b >= nfi) {
+      const int us = layer ? M->us2 : M->us1;
+#pragma unroll
+      for (int h = 0; h < kHalves; ++h)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) r[h][k] = flow_integer_one(r[h][k], m[2 * (k >> 2) + (k & 1)], us);
+    } else {
+#pragma unroll
+      for (int h = 0; h < kHalves; ++h)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) r[h][k] = (uint32_t)FloatRq::one(r[h][k], m[2 * (k >> 2) + (k & 1)], c[2 * (k >> 2) + (k & 1)]);
+    }
+#pragma unroll
+    for (int h = 0; h < kHalves; ++h)
+#pragma unroll
+      for (int e = 0; e < 4; e += 2) {
+        const uint32_t w0 = pack4_sat((int)r[h][e], (int)r[h][e + 1], (int)r[h][e + 4], (int)r[h][e + 5]);
+        const uint32_t w1 = pack4_sat((int)r[h][e + 8], (int)r[h][e + 9], (int)r[h][e + 12], (int)r[h][e + 13]);
+        *reinterpret_cast<uint2*>(o + h * 256 + e * 64) = make_uint2(none ? cw : w0, tail ? cw : w1);
+      }
+  }
+}
+
+// rq with the shift folded to the high word; the host admits only shifts s >= 1 to this kernel
+__device__ __forceinline__ int32_t rq_hi(int32_t a, const OutRq o) {
+  const long long c64 = (long long)(((unsigned long long)o.c_hi << 32) | (unsigned long long)o.c_lo);
+  return (int32_t)(((long long)a * (long long)o.m0 + c64) >> 32) >> (o.s - 1);
+}
+
+// Per-tap partials of tile t -> accumulator. A lane quarter is kR rows of the tile's eight columns, and a
+// thread holds a column: the three vertical taps of one horizontal tap v meet in its registers, so unit
+// (granule of 8 channels, v) costs kR + 2 reductions per channel instead of 3 kR. Products whose output
+// pixel is outside the image are dropped (zero padding).
+template <int kR>
+__device__ __forceinline__ void flow_sum(const Flow& f, const FlowPlan& P, int t, uint32_t taddr, int32_t* __restrict__ acc,
+                                         uint64_t* ready, uint32_t parity) {
+  const int ng = (P.cb + 7) >> 3;
+  const int4 tp = f.ctl->tile[t];
+  const int i0 = tp.y + (f.warp & 3) * kR, j0 = tp.z + (f.lane >> 2) + 1, ch0 = 2 * (f.lane & 3);
+  const uint32_t row = (uint32_t)P.w * 4u, next_ch = (uint32_t)P.acc_stride * 4u, du = (uint32_t)(3 * ng) << 3;
+  // output row i0 - 1, the column right of the thread's (v = 0), the thread's channels of granule 0
+  const uint32_t dst0 = ptx::smem_u32(acc + ch0 * P.acc_stride + tp.x * P.px + (i0 - 1) * P.w + j0);
+  const bool top = i0 > 0, bottom = i0 + kR < P.h;
+  int g = 0, v = f.ncs == 2 ? (f.cs ^ (t >> 1)) & 1 : f.cs;       // (two warps: which of them has the odd unit alternates)
+  flow_wait(f, ready, parity);
+  ptx::tc_fence_after();
+#pragma unroll 1
+  for (;; v += f.ncs) {
+    while (v >= 3) { v -= 3; ++g; }
+    if (g >= ng) break;
+    uint32_t r[3][kR / 2][4];
+    const uint32_t col = taddr + (uint32_t)((v * ng + g) << 3);
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+#pragma unroll
+      for (int h = 0; h < kR / 2; ++h) ptx::tmem_ld_16x8(col + ((uint32_t)h << 20) + (uint32_t)u * du, r[u][h]);
+    uint32_t dst = dst0 + (uint32_t)(g * 8) * next_ch - (uint32_t)(4 * v);
+    const bool ok = (uint32_t)(j0 - v) < (uint32_t)P.w && g * 8 + ch0 < P.cb;
+    const bool first = ok && top, last = ok && bottom;
+    ptx::tmem_ld_wait4(r[0][0]);
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+#pragma unroll
+      for (int h = 0; h < kR / 2; ++h) ptx::tmem_ld_wait4_nosync(r[u][h]);
+#pragma unroll
+    for (int o = -1; o <= kR; ++o) {
+      int sum[2] = {0, 0};
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        const int i = o + u - 1;
+        if (i < 0 || i >= kR) continue;
+        sum[0] += (int)r[u][i >> 1][2 * (i & 1)];
+        sum[1] += (int)r[u][i >> 1][2 * (i & 1) + 1];
+      }
+      ptx::red_add2_s32(dst, next_ch, sum[0], sum[1], o < 0 ? first : (o == kR ? last : ok));
+      dst += row;
+    }
+  }
+}
+
+// 4 x 4 levels: a lane quarter is a whole image, so the nine taps meet by shuffles and the translation is
+// applied on the spot, without an accumulator. Lane T holds pixels T / 4 and T / 4 + 8: rows 0, 2 in the lower
+// half-warp, 1, 3 in the upper one.
+template <bool kInv>
+__device__ __forceinline__ void flow_sum_4x4(const Flow& f, const FlowPlan& P, int t, uint32_t taddr, const uint8_t* mb,
+                                             int32_t* __restrict__ v, uint64_t* ready, uint32_t parity) {
+  const int ng = (P.cb + 7) >> 3, lane = f.lane, j = (lane >> 2) & 3;
+  const FlowMeta* M = reinterpret_cast<const FlowMeta*>(mb);
+  const int32_t* colB = reinterpret_cast<const int32_t*>(mb + M->off_colB);
+  const OutRq* orq = reinterpret_cast<const OutRq*>(mb + M->off_out);
+  const bool odd = lane >= 16;
+  flow_wait(f, ready, parity);
+  ptx::tc_fence_after();
+#pragma unroll 1
+  for (int g = f.cs; g < ng; g += f.ncs) {
+    int lo[2] = {0, 0}, hi[2] = {0, 0};
+    uint32_t ra[3][3][4];
+#pragma unroll
+    for (int tv = 0; tv < 3; ++tv)
+#pragma unroll
+      for (int u = 0; u < 3; ++u) ptx::tmem_ld_16x8(taddr + (uint32_t)(((3 * u + tv) * ng + g) << 3), ra[tv][u]);
+    ptx::tmem_ld_wait4(ra[0][0]);
+#pragma unroll
+    for (int tv = 0; tv < 3; ++tv) {
+#pragma unroll
+      for (int u = 0; u < 3; ++u) ptx::tmem_ld_wait4_nosync(ra[tv][u]);
+      const uint32_t (&r)[3][4] = ra[tv];
+      const bool ok = (uint32_t)(j + tv - 1) < 4u;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int a0 = __shfl_xor_sync(0xFFFFFFFFu, (int)r[0][e], 16), a2 = __shfl_xor_sync(0xFFFFFFFFu, (int)r[0][e + 2], 16);
+        const int b0 = __shfl_xor_sync(0xFFFFFFFFu, (int)r[2][e], 16), b2 = __shfl_xor_sync(0xFFFFFFFFu, (int)r[2][e + 2], 16);
+        const int s0 = (int)r[1][e] + (odd ? a0 + b2 : b0), s2 = (int)r[1][e + 2] + (odd ? a2 : a0 + b2);
+        const int t0 = __shfl_sync(0xFFFFFFFFu, s0, lane + 4 * (tv - 1)), t2 = __shfl_sync(0xFFFFFFFFu, s2, lane + 4 * (tv - 1));
+        lo[e] += ok ? t0 : 0;
+        hi[e] += ok ? t2 : 0;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int ch = g * 8 + 2 * (lane & 3) + e;
+      if (ch < P.cb) {
+        const OutRq o = orq[ch];
+        int32_t* vp = v + colB[ch] * P.pg + (4 * t + (f.warp & 3)) * 16 + (lane >> 2);
+        const uint32_t y0 = (uint32_t)rq_hi(lo[e], o), y8 = (uint32_t)rq_hi(hi[e], o);
+        vp[0] = (int32_t)(kInv ? (uint32_t)vp[0] - y0 : (uint32_t)vp[0] + y0);
+        vp[8] = (int32_t)(kInv ? (uint32_t)vp[8] - y8 : (uint32_t)vp[8] + y8);
+      }
+    }
+  }
+}
+
+// Prior head: accumulators of all tiles -> mu and clipped log-scale index in global memory. Unit = (tile, 8 columns).
+__device__ void flow_prior(const Flow& f, const FlowPlan& P, const LevelArgs& a, const PriorMeta* M, int img0) {
+  const int wq = f.warp & 3, hs = P.m >> 7;
+  const OutRq* orq = reinterpret_cast<const OutRq*>(reinterpret_cast<const uint8_t*>(M) + M->off_out);
+  const int ng = (2 * P.cb + 7) >> 3;
+  const int lane_row = (wq << (4 + hs)) + (f.lane & (hs ? 31 : 15));
+  int t = f.sl, g = f.cs;
+#pragma unroll 1
+  for (; ; g += f.ncs) {
+    while (g >= ng) { g -= ng; t += f.slots; }
+    if (t >= f.tiles) break;
+    uint32_t r[8];
+    ptx::tmem_ld8(f.tmem + (uint32_t)(t * P.n_prior + g * 8) + ((uint32_t)(wq * 32) << 16), r);
+    const int4 tp = f.ctl->tile[t];
+    int img = tp.x, at = (tp.y + (lane_row >> 3)) * P.w + tp.z + (lane_row & 7);
+    if (P.im2col) { img += lane_row >> 4; at = lane_row & 15; }
+    int32_t* mu = a.prior + (size_t)(img0 + img) * (size_t)(2 * P.d_fact) + P.prior_off + at;
+    ptx::tmem_ld_wait8(r);
+    if (!(hs || f.lane < 16) || img >= f.nimg) continue;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int col = g * 8 + e;
+      if (col < 2 * P.cb) {
+        const int32_t y = rq_hi((int32_t)r[e], orq[col]);
+        if (col < P.cb) mu[(size_t)col * P.px] = y;
+        else mu[P.d_fact + (size_t)(col - P.cb) * P.px] = clampi(y, M->ls_lo, M->ls_hi);
+      }
+    }
+  }
+}
+
+// Work split of the pixel pass: thread -> (pair of neighbouring pixels, part) with `parts` threads per
+// pair. With one part a thread has all channels of its pixels and needs no barrier between the two halves of the pass.
+struct PixelMap {
+  int p, j, parts;              // first pixel (-1: none), part
+  int32_t* v;                   // the pair in plane 0 of the flow variable
+  int32_t* acc;                 // and of the accumulator
+  uint8_t* rec;                 // its first pixel's record (4 x 4 levels: operand row)
+  uint32_t taps;                // 4 x 4 levels: bit t (16 + t): the first (second) pixel's value is read by tap t of a pixel
+};
+
+template <bool kInv>
+__device__ __forceinline__ void flow_translate(const FlowPlan& P, const PixelMap& pm, const uint8_t* mb) {
+  const FlowMeta* M = reinterpret_cast<const FlowMeta*>(mb);
+  const int32_t* colB = reinterpret_cast<const int32_t*>(mb + M->off_colB);
+  const OutRq* orq = reinterpret_cast<const OutRq*>(mb + M->off_out);
+#pragma unroll 1
+  for (int c = pm.j; c < P.cb; c += pm.parts) {
+    int2* ap = reinterpret_cast<int2*>(pm.acc + c * P.acc_stride);
+    uint2* vp = reinterpret_cast<uint2*>(pm.v + colB[c] * P.pg);
+    const OutRq o = orq[c];
+    const int2 s = *ap;
+    uint2 x = *vp;
+    *ap = make_int2(0, 0);
+    const uint32_t t0 = (uint32_t)rq_hi(s.x, o), t1 = (uint32_t)rq_hi(s.y, o);
+    x.x = kInv ? x.x - t0 : x.x + t0;
+    x.y = kInv ? x.y - t1 : x.y + t1;
+    *vp = x;
+  }
+}
+
+// network input: words of four requantised channels (then the constants 1, 127, 127, ...) into the frame
+__device__ __forceinline__ void flow_requant(const FlowPlan& P, const PixelMap& pm, const int32_t* cols, int32_t m0, int32_t s) {
+  const int nw = (P.ca + 3) >> 2;
+  const long long rnd = 1ll << (30 + s);
+#pragma unroll 1
+  for (int wd = pm.j; wd < nw; wd += pm.parts) {
+    const int4 c4 = *reinterpret_cast<const int4*>(cols + wd * 4);       // (entries beyond ca: any column)
+    const int col[4] = {c4.x, c4.y, c4.z, c4.w};
+    int y[2][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int2 x = *reinterpret_cast<const int2*>(pm.v + col[e] * P.pg);
+      y[0][e] = (int32_t)(((long long)x.x * (long long)m0 + rnd) >> 32) >> (s - 1);
+      y[1][e] = (int32_t)(((long long)x.y * (long long)m0 + rnd) >> 32) >> (s - 1);
+    }
+    // the clip to -128..127 is the pack's saturation
+    uint32_t w0 = pack4_sat(y[0][0], y[0][1], y[0][2], y[0][3]), w1 = pack4_sat(y[1][0], y[1][1], y[1][2], y[1][3]);
+    const int over = wd * 4 + 4 - P.ca;          // bytes of the word that hold no channel (two, C being a multiple of four)
+    if (over > 0) {
+      w0 = (w0 & 0xFFFFu) | 0x7F010000u;
+      w1 = (w1 & 0xFFFFu) | 0x7F010000u;
+    }
+    if (!P.im2col) {
+      uint32_t* rec = reinterpret_cast<uint32_t*>(pm.rec + (wd >> 2) * P.plane16 * 16 + (wd & 3) * 4);
+      rec[0] = w0;
+      rec[4] = w1;
+      if (P.paired) {                            // second half of the left neighbour's record
+        rec[-2] = w0;
+        rec[2] = w1;
+      }
+    } else {
+      // word (tap, wd) of the rows of the pixels that read this one: row - 4 (u - 1) - (v - 1)
+      int k = wd;
+#pragma unroll
+      for (int t = 0; t < 9; ++t, k += P.ca >> 2) {
+        uint8_t* d = pm.rec + (k >> 2) * P.plane16 * 16 + (k & 3) * 4 - ((t / 3 - 1) * 4 + (t % 3 - 1)) * 16;
+        if (pm.taps >> t & 1u) *reinterpret_cast<uint32_t*>(d) = w0;
+        if (pm.taps >> (16 + t) & 1u) *reinterpret_cast<uint32_t*>(d + 16) = w1;
+      }
+    }
+  }
+}
+
+template <bool kInv>
+__device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st, int img0) {
+  FlowCtl* ctl = f.ctl;
+  uint8_t* smem = f.smem;
+  int32_t* v = reinterpret_cast<int32_t*>(smem + P.s_v);
+  int32_t* acc = reinterpret_cast<int32_t*>(smem + P.s_acc);
+  const uint32_t lane_field = (uint32_t)((f.warp & 3) * 32) << 16;
+  // (4 x 4 levels: a lane quarter is an image; quarters without one only take part in the hand-overs)
+  PixelMap pm;
+  const int pairs = P.pg >> 1;
+  pm.parts = kFlowWorkers / pairs;
+  pm.j = f.tid / pairs;
+  pm.p = 2 * (f.tid - pm.j * pairs);
+  if (pm.j >= pm.parts || pm.p >= f.pvalid) pm.j = 1 << 20;      // no work
+  {
+    const int img = fdiv(pm.p, P.mul_px), px = pm.p - img * P.px, r = fdiv(px, P.mul_w), c = px - r * P.w;
+    pm.v = v + pm.p;
+    pm.acc = acc + pm.p;
+    pm.rec = smem + P.s_xa + 16 * (P.im2col ? img * 16 + px : img * P.frame + (r + 1) * P.wp + c + 1);
+    pm.taps = 0;
+    for (int t = 0; t < 9; ++t) {
+      const int oi = r - (t / 3 - 1), oj = c - (t % 3 - 1);
+      if ((uint32_t)oi < (uint32_t)P.h && (uint32_t)oj < (uint32_t)P.w) pm.taps |= 1u << t;
+      if ((uint32_t)oi < (uint32_t)P.h && (uint32_t)(oj + 1) < (uint32_t)P.w) pm.taps |= 1u << (16 + t);
+    }
+  }
+  const uint32_t dm = f.tmem + (uint32_t)(f.sl * P.d_col) + lane_field, d3 = f.tmem + (uint32_t)(P.d3_col + f.sl * P.d3_step) + lane_field;
+  uint8_t* sA = smem + P.s_a[f.sl];
+  uint32_t dpar = 0u, tpar = 0u;
+  const uint8_t* prev = nullptr;                // coupling whose translation is still to be applied
+#pragma unroll 1
+  for (int i = 0; i <= st.nsteps; ++i) {
+    if (prev && !P.im2col) {
+      flow_translate<kInv>(P, pm, prev);
+      if (pm.parts > 1) worker_barrier();       // the network input may read channels that were just updated
+    }
+    if (i == st.nsteps) break;
+    flow_wait(f, &ctl->meta_full[i & 1], (uint32_t)(i >> 1) & 1u);
+    const uint8_t* mb = smem + P.s_meta[i & 1];
+    const bool prior = st.is_prior(i);
+    const FlowMeta* M = reinterpret_cast<const FlowMeta*>(mb);
+    // (the first two words of both kinds of meta block)
+    flow_requant(P, pm, prior ? a.plan->col_out : reinterpret_cast<const int32_t*>(mb + M->off_colA), M->in_m0, M->in_s);
+    flow_hand_over(f, &ctl->xa_ready);
+    prev = prior ? nullptr : mb;
+    if (prior) {
+      flow_wait(f, &ctl->dm_ready[f.sl], dpar);
+      dpar ^= 1u;
+      ptx::tc_fence_after();
+      flow_prior(f, P, a, reinterpret_cast<const PriorMeta*>(mb), img0);
+    } else {
+#pragma unroll 1
+      for (int t = f.sl; t < f.tiles; t += f.slots) {
+        const bool quarter = !P.im2col || 4 * t + (f.warp & 3) < f.nimg;
+#pragma unroll 1
+        for (int layer = 0; layer < 2; ++layer) {
+          if (P.m == 128) flow_hidden<2>(f, P, dm, M, layer, sA, &ctl->dm_ready[f.sl], dpar);
+          else if (quarter) flow_hidden<1>(f, P, dm, M, layer, sA, &ctl->dm_ready[f.sl], dpar);
+          else flow_wait(f, &ctl->dm_ready[f.sl], dpar);      // (never a phase ahead in its arrivals)
+          dpar ^= 1u;
+          flow_hand_over(f, &ctl->a_ready[f.sl]);
+        }
+        if (P.im2col) {
+          if (quarter) flow_sum_4x4<kInv>(f, P, t, d3, mb, v, &ctl->d3_ready[f.sl], tpar);
+        } else if (P.m == 128) {
+          flow_sum<4>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
+        } else {
+          flow_sum<2>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
+        }
+        tpar ^= 1u;
+      }
+    }
+    ptx::tc_fence_before();
+    worker_barrier();                           // every product has been added
+  }
+}
+
+// ---- a level's input and output index maps (four neighbouring elements per thread and step) ----------------
+__device__ __forceinline__ size_t patch_index(const FlowPlan& P, const LevelArgs& a, int b, int ci, int y, int x) {
+  const int by = fdiv(b, a.mul_patches_x), bx = b - by * a.patches_x;
+  return ((size_t)ci * a.img_h + (size_t)(by * 2 * P.h + y)) * a.img_w + (size_t)(bx * 2 * P.w + x);
+}
+
+// pre-squeeze element e (a multiple of four, image-major over the CTA's images) -> address in the level's
+// input / output array and the flow variable's two planes (dx = 0 at d0, dx = 1 at d0 + pg)
+__device__ __forceinline__ void squeeze_map(const FlowPlan& P, const LevelArgs& a, int img0, int e, size_t* at, int* d0) {
+  const int per_img = P.c * P.px, w2 = 2 * P.w;
+  const int g = fdiv(e, P.mul_per_img), r = e - g * per_img;
+  const int ci = fdiv(r, P.mul_4px), r2 = r - ci * 4 * P.px;
+  const int y = fdiv(r2, P.mul_w2), x = r2 - y * w2;
+  *at = (P.is_first && a.img_w > 0) ? patch_index(P, a, img0 + g, ci, y, x) : (size_t)(img0 + g) * per_img + r;
+  *d0 = (ci * 4 + (y & 1) * 2) * P.pg + g * P.px + (y >> 1) * P.w + (x >> 1);
+}
+
+// logical element e (a multiple of four) of the level's channels -> its place in z, in the kept channels
+// (stride `keep_stride` per image) and in the flow variable
+template <typename Fn>
+__device__ __forceinline__ void split_map(const FlowPlan& P, const LevelArgs& a, const int32_t* col_out, int img0, int e,
+                                          int32_t* keep, size_t keep_stride, Fn fn) {
+  const int per_img = P.c * P.px;
+  const int g = fdiv(e, P.mul_per_img), r = e - g * per_img;
+  const int k = fdiv(r, P.mul_px), q = r - k * P.px;
+  const size_t b = (size_t)(img0 + g);
+  int32_t* dst = k >= P.keep_c ? a.z + b * P.d + P.z_off + (size_t)(k - P.keep_c) * P.px + q
+                               : keep + b * keep_stride + (size_t)k * P.px + q;
+  fn(k, dst, col_out[k] * P.pg + g * P.px + q);
+}
+
+template <bool kInv>
+__device__ __forceinline__ void flow_load(const Flow& f, const FlowPlan& P, const LevelArgs& a, int img0, int32_t* v) {
+  const int n = f.nimg * P.c * P.px;
+  if (!kInv) {
+#pragma unroll 1
+    for (int e = 4 * f.tid; e < n; e += 4 * kFlowWorkers) {
+      size_t at; int d0;
+      squeeze_map(P, a, img0, e, &at, &d0);
+      int4 q;
+      if (P.is_first) {
+        const uint32_t b4 = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint8_t*>(a.in) + at);
+        q = make_int4((int)(b4 & 0xFFu), (int)((b4 >> 8) & 0xFFu), (int)((b4 >> 16) & 0xFFu), (int)(b4 >> 24));
+      } else {
+        q = *reinterpret_cast<const int4*>(reinterpret_cast<const int32_t*>(a.in) + at);
+      }
+      *reinterpret_cast<int2*>(v + d0) = make_int2(q.x, q.z);
+      *reinterpret_cast<int2*>(v + d0 + P.pg) = make_int2(q.y, q.w);
+    }
+  } else {
+    int32_t* keep = const_cast<int32_t*>(reinterpret_cast<const int32_t*>(a.in));
+#pragma unroll 1
+    for (int e = 4 * f.tid; e < n; e += 4 * kFlowWorkers)
+      split_map(P, a, a.plan->col_out, img0, e, keep, (size_t)a.in_stride, [&](int k, const int32_t* src, int d) {
+        // (prior head only: z's block is not read)
+        if (a.phase != 1 || k < P.keep_c) *reinterpret_cast<int4*>(v + d) = *reinterpret_cast<const int4*>(src);
+      });
+  }
+}
+
+template <bool kInv>
+__device__ __forceinline__ void flow_store(const Flow& f, const FlowPlan& P, const LevelArgs& a, int img0, const int32_t* v) {
+  const int n = f.nimg * P.c * P.px;
+  if (!kInv) {
+    int32_t* keep = P.is_last ? a.z + P.z_final_off : reinterpret_cast<int32_t*>(a.out);
+    const size_t keep_stride = P.is_last ? (size_t)P.d : (size_t)P.keep_c * P.px;
+#pragma unroll 1
+    for (int e = 4 * f.tid; e < n; e += 4 * kFlowWorkers)
+      split_map(P, a, a.plan->col_out, img0, e, keep, keep_stride,
+                [&](int, int32_t* dst, int d) { *reinterpret_cast<int4*>(dst) = *reinterpret_cast<const int4*>(v + d); });
+  } else if (a.phase != 1) {
+    uint32_t bad = 0;
+#pragma unroll 1
+    for (int e = 4 * f.tid; e < n; e += 4 * kFlowWorkers) {
+      size_t at; int d0;
+      squeeze_map(P, a, img0, e, &at, &d0);
+      const int2 x0 = *reinterpret_cast<const int2*>(v + d0), x1 = *reinterpret_cast<const int2*>(v + d0 + P.pg);
+      if (P.is_first) {
+        *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(a.out) + at) = pack4(x0.x, x1.x, x0.y, x1.y);
+        bad += (uint32_t)((uint32_t)x0.x > 255u) + (uint32_t)((uint32_t)x1.x > 255u) + (uint32_t)((uint32_t)x0.y > 255u) +
+               (uint32_t)((uint32_t)x1.y > 255u);
+      } else {
+        *reinterpret_cast<int4*>(reinterpret_cast<int32_t*>(a.out) + at) = make_int4(x0.x, x1.x, x0.y, x1.y);
+      }
+    }
+    if (P.is_first && a.oor != nullptr) {
+      bad = __reduce_add_sync(0xFFFFFFFFu, bad);
+      if (f.lane == 0 && bad) atomicAdd(a.oor, bad);
+    }
+  }
+}
+
+template <bool kInv>
+__global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const LevelArgs a, const __grid_constant__ FlowPlan P) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  __shared__ FlowCtl ctl;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
+
+  ptx::grid_launch_dependents();         // the next kernel in the stream may start its prologue
+  const int img0 = blockIdx.x * P.group, nimg = min(P.group, a.batch - img0);
+  const int tiles = P.im2col ? (nimg + 3) >> 2 : nimg * P.tiles_img, slots = min(2, tiles);
+  if (tid == 0) {
+    ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), (uint32_t)kFlowWarps);
+    for (int s = 0; s < 2; ++s) {
+      ptx::mbar_init(ptx::smem_u32(&ctl.a_ready[s]), (uint32_t)(kFlowWarps / slots));
+      ptx::mbar_init(ptx::smem_u32(&ctl.dm_ready[s]), 1);
+      ptx::mbar_init(ptx::smem_u32(&ctl.d3_ready[s]), 1);
+      ptx::mbar_init(ptx::smem_u32(&ctl.meta_full[s]), 1);
+    }
+    for (int s = 0; s < 3; ++s) {
+      ptx::mbar_init(ptx::smem_u32(&ctl.w_full[s]), 1);
+      ptx::mbar_init(ptx::smem_u32(&ctl.w_empty[s]), (uint32_t)slots);
+    }
+    ptx::mbar_init_fence();
+    ctl.abort = 0;
+  }
+  if (warp == 0) ptx::tmem_alloc(ptx::smem_u32(&ctl.tmem_base), (uint32_t)P.tmem_cols);
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+
+  Flow f;
+  f.smem = smem; f.ctl = &ctl; f.status = a.status; f.tmem = ctl.tmem_base;
+  f.tid = tid; f.warp = warp; f.lane = lane;
+  f.nimg = nimg; f.pvalid = nimg * P.px; f.tiles = tiles; f.slots = slots;
+  f.ncs = kFlowWarps / 4 / slots;
+  f.sl = slots == 2 && warp >= kFlowWarps / 2 ? 1 : 0;
+  f.cs = (warp - f.sl * (kFlowWarps / 2)) >> 2;
+  Steps st;
+  st.n_couplings = (kInv && a.phase == 1) ? 0 : P.n_couplings;
+  st.do_prior = P.has_prior && a.prior != nullptr && !(kInv && a.phase == 2);
+  st.nsteps = st.n_couplings + (st.do_prior ? 1 : 0);
+  st.inverse = kInv;
+
+  if (warp == kFlowWarps + 2) {
+    if (lane == 0) flow_loader(f, P, a, st);        // packed blocks: written once, at model creation
+  } else if (warp >= kFlowWarps) {
+    flow_mma(f, P, st, warp - kFlowWarps);
+  } else {
+    // frame of the network input: zero channels, and the constants that multiply the bias rows in the
+    // bytes that no channel uses (at 4 x 4 levels: after the nine taps)
+    const int lim = P.im2col ? 9 * P.ca : P.ca, unit = P.paired ? 8 : P.plane16 * 16;
+    for (uint32_t o = 16 * tid; o < P.s_xa_end - P.s_xa; o += 16 * kFlowWorkers) {
+      const int first = P.paired ? 0 : (int)(o / (uint32_t)unit) * 16;       // first byte of the 16-byte plane in a record
+      uint32_t wd[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        wd[k] = 0;
+        for (int e = 0; e < 4; ++e) {
+          const int byte = first + ((P.paired ? k & 1 : k) << 2) + e;
+          wd[k] |= (byte < lim ? 0u : (byte == lim ? 1u : 127u)) << (8 * e);
+        }
+      }
+      *reinterpret_cast<uint4*>(smem + P.s_xa + o) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+    }
+    if (tid < f.tiles) {
+      int4 tp = make_int4(4 * tid, 0, 0, 64 * tid);                          // (im2col: first of four images)
+      if (!P.im2col) {
+        tp.x = tid / P.tiles_img;
+        const int tt = tid - tp.x * P.tiles_img;
+        tp.y = tt / P.tiles_x * (P.m >> 3);
+        tp.z = tt % P.tiles_x * 8;
+        tp.w = tp.x * P.frame + (tp.y + 1) * P.wp + tp.z + 1;
+      }
+      ctl.tile[tid] = tp;
+    }
+    for (int o = tid; o < (P.im2col ? 0 : P.cb * P.acc_stride); o += kFlowWorkers) reinterpret_cast<int32_t*>(smem + P.s_acc)[o] = 0;
+    int32_t* v = reinterpret_cast<int32_t*>(smem + P.s_v);
+    ptx::grid_dependency_wait();         // from here on: what the previous kernel in the stream wrote
+    flow_load<kInv>(f, P, a, img0, v);
+    worker_barrier();
+    flow_workers<kInv>(f, P, a, st, img0);
+    worker_barrier();
+    flow_store<kInv>(f, P, a, img0, v);
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) ptx::tmem_dealloc(ctl.tmem_base, (uint32_t)P.tmem_cols);
+}
+
+}  // namespace
+
+cudaError_t launch_flow_level(const LevelArgs& args, const FlowPlan& plan, bool inverse, int grid, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)kFlowThreads);
+  cfg.dynamicSmemBytes = plan.s_total;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return inverse ? cudaLaunchKernelEx(&cfg, flow_level_kernel<true>, args, plan)
+                 : cudaLaunchKernelEx(&cfg, flow_level_kernel<false>, args, plan);
+}
+
+cudaError_t configure_flow_kernels(uint32_t max_smem_bytes) {
+  cudaError_t e = cudaFuncSetAttribute(flow_level_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem_bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(flow_level_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem_bytes);
+}
+
+}  // namespace iodf

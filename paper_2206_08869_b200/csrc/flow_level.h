@@ -1,0 +1,69 @@
+// Flow levels of three-conv couplings whose geometry and requantisation fit the compact kernel
+// (flow_level.cu): the launch-time plan, the packed meta blocks and the launch interface.
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "iodf_dev.h"
+#include "level_kernel.h"
+
+namespace iodf {
+
+constexpr int kFlowWarps = 16;                       // requantising warps, four per TMEM lane quarter
+constexpr int kFlowWorkers = kFlowWarps * 32;
+constexpr int kFlowThreads = kFlowWorkers + 3 * 32;  // + an MMA-issuing warp per tile slot and the weight-loading warp
+constexpr int kFlowMaxTiles = 32;                    // of a CTA
+constexpr int kFlowMaxSteps = 18;                    // K steps of the first conv
+
+// Everything about a level that the kernel needs and that is the same for all its couplings; passed
+// by value (constant bank), so that no index computation waits for a global load.
+struct FlowPlan {
+  int32_t c, h, w, px, ca, cb;
+  int32_t n_couplings, has_prior, is_first, is_last, keep_c;
+  int32_t group;                 // images per CTA
+  int32_t pg;                    // pixels of the CTA (group * px): plane stride of the flow variable
+  // GEMM tiles. A tile is an 8-column block of an image, 16 (m = 128) or 8 (m = 64) rows high, or, at
+  // 4 x 4 levels (im2col), up to four whole images of 16 pixels each (m = 64)
+  int32_t m, im2col;
+  int32_t tiles;                 // of the CTA
+  int32_t tiles_img, tiles_x;    // of an image; 8-column blocks per row
+  int32_t rec;                   // bytes of a position's record in the network-input frame
+  int32_t paired;                // records are [pixel j | pixel j + 1], eight bytes each
+  int32_t wp, frame;             // frame of an image: (h + 2) rows of wp = w + 2 positions
+  int32_t plane16;               // 16-byte units between the 16-byte planes of a record
+  int32_t sbo16;                 // 16-byte units between 8-row groups of the first conv's operand
+  int32_t ks1;                   // its K steps; step s: offset of the first 16-byte chunk from the tile's first position
+  uint32_t step[kFlowMaxSteps];  // (mod 2^32) + distance of the second chunk << 16, in 16-byte units
+  int32_t pitch;                 // bytes between 16-byte K chunks of the hidden operands
+  int32_t acc_stride;            // words per channel plane of the translation accumulator (pg + 4: no bank conflicts)
+  int32_t alias;                 // 1: the third matrix travels through the first one's slot
+  int32_t d_col, d3_col, d3_step;// TMEM columns: slot s has its accumulators at s * d_col, its per-tap partials at
+                                 // d3_col + s * d3_step
+  int32_t n_prior;               // columns of the prior head (padded to 16)
+  int32_t tmem_cols;
+  uint32_t s_v, s_xa, s_xa_end, s_acc, s_a[2], s_meta[2], s_w[3], s_total;
+  uint32_t mul_per_img, mul_4px, mul_w2, mul_px, mul_w;
+  int64_t z_off, prior_off, z_final_off, d, d_fact;
+};
+static_assert(sizeof(FlowPlan) < 1024, "travels as a kernel parameter");
+
+// Meta part of a coupling's packed block. Followed by colA[ca], colB[cb] (physical columns of the flow
+// variable), OutRq[cb], and per hidden layer the FloatRq multipliers of its 32-column blocks, thread
+// order (block, lane & 3, 8 columns), and addends of the blocks from nfb on, in the same order.
+struct FlowMeta {
+  int32_t in_m0, in_s;
+  int32_t n1, n2, n3;            // MMA N of the three GEMMs
+  int32_t ks2, ks3;              // K steps of the second and third GEMM = 32-column blocks of their operands
+  int32_t nfb1, nfb2;            // blocks below need no addend
+  int32_t nfi1, nfi2;            // blocks from here on hold a channel that has no floating-point constants: integer
+                                 // form, the multiplier table holds M0
+  int32_t us1, us2;              // the layers' shifts (integer form)
+  int32_t off_colA, off_colB, off_out, off_f1, off_f2, off_c1, off_c2;
+  int32_t pad[12];
+};
+static_assert(sizeof(FlowMeta) == 128, "meta header is 128 bytes");
+
+cudaError_t configure_flow_kernels(uint32_t max_smem_bytes);
+cudaError_t launch_flow_level(const LevelArgs& args, const FlowPlan& plan, bool inverse, int grid, cudaStream_t stream);
+
+}  // namespace iodf

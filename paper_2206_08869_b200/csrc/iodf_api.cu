@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdlib>
@@ -13,6 +14,7 @@
 
 #include "../../include/iodf.h"
 #include "iodf_dev.h"
+#include "flow_level.h"
 #include "rans_kernel.h"
 #include "res_level.h"
 #include "level_kernel.h"
@@ -29,6 +31,8 @@ inline uint32_t up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 
 struct HostLevel {
   LevelPlan plan;
+  FlowPlan flow;                     // levels that run in the compact kernel (use_flow)
+  bool use_flow = false;
   std::vector<uint8_t> blob;
   int grid_group = 1;
   int32_t ls_lo = 0, ls_hi = 0;      // clip of the prior head's log-scale index (levels with a head)
@@ -149,6 +153,7 @@ void fold_bias(int32_t bias, int8_t w[kBiasRows]) {
 struct FloatChannel {
   float m = 0.f;
   int32_t beta = 0, C = 0;
+  bool none = false;                 // no such constants (about one channel in 2 000, at large shifts)
 };
 bool float_requant(int32_t m0, int32_t s, int top, int64_t beta_room, FloatChannel* out) {
   if (s < 1) return false;
@@ -205,8 +210,10 @@ bool float_requant(int32_t m0, int32_t s, int top, int64_t beta_room, FloatChann
 // Order in which a hidden layer's channels are packed (a permutation of the rows of its weight matrix and
 // of the columns of the next one), and the constants of the floating-point flavour where it applies.
 struct HiddenOrder {
-  std::vector<int> ch;              // packed position -> channel
-  bool is_float = false;
+  std::vector<int> ch;              // packed position -> channel: plain multipliers, then those with an addend, then `none`
+  bool folded = false;              // clip 0..127, one shift s >= 1, every bias foldable
+  bool is_float = false;            // and every channel has floating-point constants
+  int shift = 0;
   std::vector<FloatChannel> fc;     // by channel
   int nf = 0;                       // packed columns below nf need no addend
 };
@@ -223,10 +230,20 @@ HiddenOrder order_hidden(const iodf_layer_desc& L, const Blobs& B, Act a, int n_
   o.fc.resize(n);
   for (int i = 0; i < n; ++i) {
     const int64_t room = kFoldMaxBias - std::llabs((long long)bias[i]);
-    if (s[i] != s[0] || room < 0 || !float_requant(m0[i], s[i], a.hi, room, &o.fc[i])) return o;
+    if (s[i] != s[0] || s[i] < 1 || room < 0) return o;
   }
-  o.is_float = true;
-  std::stable_partition(o.ch.begin(), o.ch.end(), [&](int i) { return o.fc[i].C == 0; });
+  o.folded = o.is_float = true;
+  o.shift = s[0];
+  for (int i = 0; i < n; ++i)
+    if (!float_requant(m0[i], s[i], a.hi, kFoldMaxBias - std::llabs((long long)bias[i]), &o.fc[i])) {
+      o.fc[i] = FloatChannel{};
+      o.fc[i].none = true;
+      o.is_float = false;
+    }
+  std::stable_sort(o.ch.begin(), o.ch.end(), [&](int i, int j) {
+    auto rank = [&](int k) { return o.fc[k].none ? 2 : (o.fc[k].C ? 1 : 0); };
+    return rank(i) < rank(j);
+  });
   int plain = 0;
   while (plain < n && o.fc[o.ch[plain]].C == 0) ++plain;
   if (plain < n) o.nf = plain / 16 * 16;
@@ -247,16 +264,17 @@ void put_hidden_rq(HiddenRq* dst, int32_t* mb, const iodf_layer_desc& L, const B
   for (int i = 0; i < n_pad; ++i) {
     HiddenRq h;
     if (i < (int)L.c_out) {
-      const long long c64 = (long long)bias[i] * (long long)m0[i] + (1ll << (30 + s[i]));
-      h.m0 = m0[i];
-      h.sh = s[i] - 1;
+      const int ch = ord.ch[i];
+      const long long c64 = (long long)bias[ch] * (long long)m0[ch] + (1ll << (30 + s[ch]));
+      h.m0 = m0[ch];
+      h.sh = s[ch] - 1;
       h.c_lo = (uint32_t)((unsigned long long)c64 & 0xFFFFFFFFull);
       h.c_hi = (uint32_t)((unsigned long long)c64 >> 32);
-      if (s[i] < 1) fast = false;
-      if (s[i] != s[0] || s[i] < 1) uniform = false;
-      if (std::llabs((long long)bias[i]) > kFoldMaxBias) foldable = false;
-      mb[2 * i] = m0[i];
-      mb[2 * i + 1] = bias[i];
+      if (s[ch] < 1) fast = false;
+      if (s[ch] != s[0] || s[ch] < 1) uniform = false;
+      if (std::llabs((long long)bias[ch]) > kFoldMaxBias) foldable = false;
+      mb[2 * i] = m0[ch];
+      mb[2 * i + 1] = bias[ch];
     } else {  // padding channel: acc = 0 -> 0 (its weights in the next layer are zero anyway)
       h.m0 = 1 << 30;
       h.sh = 0;
@@ -270,7 +288,7 @@ void put_hidden_rq(HiddenRq* dst, int32_t* mb, const iodf_layer_desc& L, const B
   *mode = uniform ? (foldable ? 3 : 2) : (fast ? 1 : 0);
   *uniform_s = uniform ? s[0] : 0;
   if (*mode == 3)
-    for (int i = 0; i < n_pad; ++i) mb[i] = i < (int)L.c_out ? m0[i] : (1 << 30);
+    for (int i = 0; i < n_pad; ++i) mb[i] = i < (int)L.c_out ? m0[ord.ch[i]] : (1 << 30);
   if (ord.is_float) {
     *mode = 4;
     for (int i = 0; i < n_pad; ++i) {
@@ -317,7 +335,7 @@ void append_block(std::vector<uint8_t>& blob, const PackedBlock& pb, BlockRef* r
 struct Dims { int n1, n2, n3, kd1, kd2, kd3; };
 
 PackedBlock pack_coupling(const iodf_coupling_desc& cp, const Blobs& B, int ca, int cb, const int* colA,
-                          const int* colB, Act a1, Act a2, Dims* dims) {
+                          const int* colB, Act a1, Act a2, const HiddenOrder& o1, const HiddenOrder& o2, Dims* dims) {
   const iodf_layer_desc& L1 = cp.layers[0];
   const iodf_layer_desc& L2 = cp.layers[1];
   const iodf_layer_desc& L3 = cp.layers[2];
@@ -336,7 +354,6 @@ PackedBlock pack_coupling(const iodf_coupling_desc& cp, const Blobs& B, int ca, 
   // requantisation tables: both flavours are built, only the one the layer's mode reads is kept
   std::vector<HiddenRq> h1(d.n1), h2(d.n2);
   std::vector<int32_t> u1(2 * d.n1), u2(2 * d.n2);
-  const HiddenOrder o1 = order_hidden(L1, B, a1, d.n1), o2 = order_hidden(L2, B, a2, d.n2);
   put_hidden_rq(h1.data(), u1.data(), L1, B, o1, d.n1, &M.mode1, &M.us1);
   put_hidden_rq(h2.data(), u2.data(), L2, B, o2, d.n2, &M.mode2, &M.us2);
   M.nf1 = o1.nf; M.nf2 = o2.nf;
@@ -441,6 +458,181 @@ uint32_t pow2_cols(uint32_t need) {
   return c;
 }
 
+// ---- levels of the compact kernel (flow_level.cu) -------------------------------------------------------
+// What byte k of the first conv's operand row is: a channel of a tap, or a constant.
+struct KByte { int tap = -1, ch = 0; int kind = 0; };     // kind 0: nothing, 1: channel, 2: the constant 1, 3: 127
+
+// The parts of the plan that do not depend on the group; false if the kernel cannot run the level's shape.
+bool flow_geometry(FlowPlan& F, std::vector<KByte>& kmap) {
+  F.im2col = 0; F.paired = 0;
+  if (F.w % 8 == 0 && F.h % 8 == 0) {
+    F.m = F.h % 16 == 0 ? 128 : 64;
+    F.tiles_x = F.w / 8;
+    F.tiles_img = F.tiles_x * (F.h / (F.m / 8));
+    F.wp = F.w + 2;
+    F.frame = F.wp * (F.h + 2);
+    F.sbo16 = F.wp;
+    F.paired = F.ca <= 6;
+    F.rec = F.paired ? 16 : (int)up((uint32_t)F.ca + 2, 16);
+  } else if (F.w == 4 && F.h == 4 && F.ca % 4 == 0) {
+    F.im2col = 1;
+    F.m = 64; F.tiles_x = 0; F.tiles_img = 0; F.wp = 0; F.frame = 16; F.sbo16 = 8;
+    F.rec = (int)up(9u * F.ca + kBiasRows, 32);
+  } else {
+    return false;
+  }
+  // bytes of a step's two chunks
+  kmap.clear();
+  auto channel = [&](int tap, int ch) { KByte k; k.tap = tap; k.ch = ch; k.kind = 1; return k; };
+  auto constant = [&](int c, int lim) { KByte k; k.kind = c == lim ? 2 : 3; return k; };
+  if (F.paired) {
+    F.ks1 = 3;
+    for (int u = 0; u < 3; ++u)
+      for (int b = 0; b < 32; ++b) {
+        const int v = b >> 3, c = b & 7;
+        kmap.push_back(v == 3 ? KByte() : (c < F.ca ? channel(3 * u + v, c) : constant(c, F.ca)));
+      }
+  } else if (F.im2col) {
+    F.ks1 = F.rec / 32;
+    for (int k = 0; k < F.rec; ++k)
+      kmap.push_back(k < 9 * F.ca ? channel(k / F.ca, k % F.ca) : (k < 9 * F.ca + kBiasRows ? constant(k, 9 * F.ca) : KByte()));
+  } else {
+    const int planes = F.rec / 16, chunks = 9 * planes;
+    F.ks1 = (chunks + 1) / 2;
+    for (int ck = 0; ck < 2 * F.ks1; ++ck)
+      for (int b = 0; b < 16; ++b) {
+        const int c = (ck / 9) * 16 + b;
+        kmap.push_back(ck >= chunks ? KByte() : (c < F.ca ? channel(ck % 9, c) : constant(c, F.ca)));
+      }
+  }
+  return F.ks1 <= kFlowMaxSteps;
+}
+
+// K position of hidden channel position n (packed order) in the operand a hidden epilogue writes: within a block of
+// 32 columns, thread q of a row holds columns 8 i + 2 q + e at byte 8 q + 2 i + e.
+inline int flow_kpos(int n) {
+  const int b = n & ~31, c = n & 31;
+  return b + 8 * ((c >> 1) & 3) + 2 * (c >> 3) + (c & 1);
+}
+
+void flow_first_matrix(std::vector<uint8_t>& out, int n_pad, const std::vector<KByte>& kmap, const int8_t* w, int ca, int rows,
+                       const int* order, const int32_t* bias) {
+  out.assign((size_t)n_pad * kmap.size(), 0);
+  for (int n = 0; n < rows; ++n) {
+    const int ch = order ? order[n] : n;
+    int8_t bw[kBiasRows] = {0};
+    if (bias) fold_bias(bias[n], bw);
+    int ones = 0, used = 1;
+    for (size_t k = 0; k < kmap.size(); ++k) {
+      int8_t val = 0;
+      if (kmap[k].kind == 1) val = w[((size_t)ch * 9 + kmap[k].tap) * ca + kmap[k].ch];
+      else if (kmap[k].kind == 2 && ones == 0) { val = bw[0]; ones = 1; }
+      else if (kmap[k].kind == 3 && used < kBiasRows) val = bw[used++];
+      out[wpos(n_pad, n, (int)k)] = (uint8_t)val;
+    }
+  }
+}
+
+struct FlowDims { int n1, n2, n3, ks2, ks3; };
+
+PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, const FlowPlan& F, const std::vector<KByte>& kmap,
+                               const HiddenOrder& o1, const HiddenOrder& o2, const int* colA, const int* colB, FlowDims* dims) {
+  const iodf_layer_desc& L1 = cp.layers[0];
+  const iodf_layer_desc& L2 = cp.layers[1];
+  const iodf_layer_desc& L3 = cp.layers[2];
+  const int k1 = (int)L1.c_out, k2 = (int)L2.c_out, ca = F.ca, cb = F.cb, cbp = (int)up((uint32_t)cb, 8);
+  FlowMeta M{};
+  M.in_m0 = cp.in_m0; M.in_s = cp.in_s;
+  M.n1 = (int)up(k1, 16); M.n2 = (int)up(k2, 16); M.n3 = (int)up(9 * cbp, 16);
+  M.ks2 = (int)up((uint32_t)M.n1 + kBiasRows, 32) / 32; M.ks3 = (int)up((uint32_t)M.n2, 32) / 32;
+  *dims = FlowDims{M.n1, M.n2, M.n3, M.ks2, M.ks3};
+  PackedBlock pb;
+  uint32_t off = sizeof(FlowMeta);
+  auto take = [&](uint32_t bytes) { const uint32_t o = off; off += up(bytes, 16); return (int)o; };
+  M.off_colA = take(16 * ((ca + 3) / 4));
+  M.off_colB = take(4 * cb);
+  M.off_out = take((uint32_t)sizeof(OutRq) * cb);
+  M.off_f1 = take(128 * M.ks2); M.off_f2 = take(128 * M.ks3);
+  auto first_block = [](const HiddenOrder& o, int blocks, bool integer) {
+    int b = blocks;
+    for (int i = (int)o.ch.size() - 1; i >= 0 && (o.fc[o.ch[i]].none || (!integer && o.fc[o.ch[i]].C)); --i) b = i / 32;
+    return b;
+  };
+  M.nfb1 = first_block(o1, M.ks2, false); M.nfb2 = first_block(o2, M.ks3, false);
+  M.nfi1 = first_block(o1, M.ks2, true); M.nfi2 = first_block(o2, M.ks3, true);
+  M.us1 = o1.shift; M.us2 = o2.shift;
+  M.off_c1 = take(128 * (M.ks2 - M.nfb1)); M.off_c2 = take(128 * (M.ks3 - M.nfb2));
+  pb.meta.assign(off, 0);
+  std::memcpy(pb.meta.data() + M.off_colA, colA, 4 * ca);
+  std::memcpy(pb.meta.data() + M.off_colB, colB, 4 * cb);
+  put_out_rq(reinterpret_cast<OutRq*>(pb.meta.data() + M.off_out), L3, B);
+  auto tables = [&](const HiddenOrder& o, const iodf_layer_desc& L, int off_f, int off_c, int nfb, int nfi) {
+    float* ft = reinterpret_cast<float*>(pb.meta.data() + off_f);
+    int32_t* ct = reinterpret_cast<int32_t*>(pb.meta.data() + off_c);
+    for (int i = 0; i < (int)o.ch.size(); ++i) {
+      const FloatChannel& fc = o.fc[o.ch[i]];
+      if (i >= 32 * nfi) {           // integer blocks: M0 itself
+        std::memcpy(&ft[flow_kpos(i)], B.r + L.requant_off + L.c_out + o.ch[i], 4);
+        continue;
+      }
+      ft[flow_kpos(i)] = fc.m;
+      if (fc.C) ct[flow_kpos(i) - 32 * nfb] = (int32_t)(0x80000000u | (uint32_t)fc.C);     // -C * 2^-149
+    }
+  };
+  tables(o1, L1, M.off_f1, M.off_c1, M.nfb1, M.nfi1);
+  tables(o2, L2, M.off_f2, M.off_c2, M.nfb2, M.nfi2);
+  std::memcpy(pb.meta.data(), &M, sizeof(M));
+
+  const int32_t* b1 = B.r + L1.requant_off;
+  const int32_t* b2 = B.r + L2.requant_off;
+  std::vector<int32_t> bias1(k1), bias2(k2);
+  for (int n = 0; n < k1; ++n) bias1[n] = b1[o1.ch[n]] + (n < 32 * M.nfi1 ? o1.fc[o1.ch[n]].beta : 0);
+  for (int n = 0; n < k2; ++n) bias2[n] = b2[o2.ch[n]] + (n < 32 * M.nfi2 ? o2.fc[o2.ch[n]].beta : 0);
+  flow_first_matrix(pb.w[0], M.n1, kmap, B.w + L1.weight_off, ca, k1, o1.ch.data(), bias1.data());
+  // 1x1 conv: hidden channels at their operand positions, the bias rows where the epilogue writes the constants
+  // (1, 127, 127, 127), the last four bytes of every group of eight in the block behind the columns
+  pb.w[1].assign((size_t)M.n2 * 32 * M.ks2, 0);
+  const int8_t* w2 = B.w + L2.weight_off;
+  const int cblock = (M.n1 >> 5) * 32;
+  for (int n = 0; n < k2; ++n) {
+    for (int k = 0; k < k1; ++k) pb.w[1][wpos(M.n2, n, flow_kpos(k))] = (uint8_t)w2[(size_t)o2.ch[n] * k1 + o1.ch[k]];
+    int8_t bw[kBiasRows];
+    fold_bias(bias2[n], bw);
+    int used = 1;
+    for (int q = 0; q < 4; ++q)
+      for (int e = 0; e < 4; ++e) {
+        int8_t val = 0;
+        if (e == 0) val = q == 0 ? bw[0] : 0;
+        else if (used < kBiasRows) val = bw[used++];
+        pb.w[1][wpos(M.n2, n, cblock + 8 * q + 4 + e)] = (uint8_t)val;
+      }
+  }
+  // last conv: one row per (tap, out channel)
+  pb.w[2].assign((size_t)M.n3 * 32 * M.ks3, 0);
+  const int8_t* w3 = B.w + L3.weight_off;
+  for (int c = 0; c < cb; ++c)
+    for (int tap = 0; tap < 9; ++tap)
+      for (int k = 0; k < k2; ++k)
+        pb.w[2][wpos(M.n3, tap * cbp + c, flow_kpos(k))] = (uint8_t)w3[((size_t)c * 9 + tap) * k2 + o2.ch[k]];
+  return pb;
+}
+
+PackedBlock pack_flow_prior(const iodf_level_desc& lv, const Blobs& B, const FlowPlan& F, const std::vector<KByte>& kmap) {
+  const iodf_layer_desc& L = lv.prior_layer;
+  PackedBlock pb;
+  PriorMeta M{};
+  M.in_m0 = lv.prior_in_m0; M.in_s = lv.prior_in_s;
+  M.n = F.n_prior;
+  M.kd = (int)kmap.size();
+  M.ls_lo = lv.ls_lo; M.ls_hi = lv.ls_hi;
+  M.off_out = (int)sizeof(PriorMeta);
+  pb.meta.assign(sizeof(PriorMeta) + sizeof(OutRq) * 2 * F.cb, 0);
+  put_out_rq(reinterpret_cast<OutRq*>(pb.meta.data() + M.off_out), L, B);
+  std::memcpy(pb.meta.data(), &M, sizeof(M));
+  flow_first_matrix(pb.w[0], M.n, kmap, B.w + L.weight_off, F.ca, 2 * F.cb, nullptr, nullptr);
+  return pb;
+}
+
 // Levels of at least this many tiles per CTA run in the kernel that splits a tile's work by role
 // (level_pipe.cu) when they are eligible for it. Measured on the ImageNet64-shaped flow: 5 % faster
 // than the general kernel at eight tiles per image, 5 % slower at two (nothing follows the one
@@ -528,6 +720,82 @@ bool plan_smem(LevelPlan& P, uint32_t a_bytes, uint32_t meta_bytes, const uint32
       if (off <= limit) return true;
     }
     if (group == 1) break;
+  }
+  return false;
+}
+
+// Group, tensor-memory columns and shared-memory layout of a level in the compact kernel. false: it does not fit.
+struct FlowNeeds { uint32_t n_hidden = 32, n_taps = 16, kb = 1, meta = 16, w[3] = {16, 16, 16}; };
+bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, uint32_t max_batch, int num_sms, bool throughput) {
+  int group = F.px >= kTileM ? 1 : kTileM / F.px;
+  if (F.im2col) group = std::min(group, 4);            // an image per lane quarter
+  group = std::max(1, std::min<int>(group, (int)max_batch));
+  // the latency plan keeps groups small while the CTAs of a full batch would not fill the SMs
+  while (!throughput && group > 1 && ((int)max_batch + group - 1) / group < num_sms) group /= 2;
+  for (; group >= 1; group /= 2) {
+    F.group = group;
+    F.pg = group * F.px;
+    F.tiles = F.im2col ? (group + 3) / 4 : group * F.tiles_img;
+    const uint32_t nh = up(nd.n_hidden, 16), nh32 = up(nd.n_hidden, 32);
+    if (nd.n_hidden > 256 || nd.n_taps > 512 || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
+      continue;
+    if (F.tiles == 1) {
+      F.d_col = 0; F.d3_col = 0; F.d3_step = 0;
+      F.tmem_cols = (int)pow2_cols(std::max(std::max(nh32, nd.n_taps), (uint32_t)F.n_prior));
+    } else {
+      // several tiles: two slots; with more than two tiles the per-tap partials need columns of their own, because
+      // a slot's next tile starts before its shifted sum
+      const bool apart = 2 * nh + 2 * nd.n_taps <= 512u && nh + nh32 <= 512u;
+      if (!apart && (F.tiles > 2 || std::max(nh32, nd.n_taps) > 256u)) continue;
+      F.d_col = apart ? (int)nh : 256;
+      F.d3_col = apart ? 2 * (int)nh : 0;
+      F.d3_step = apart ? (int)nd.n_taps : 256;
+      F.tmem_cols = 512;
+    }
+    F.pitch = F.m * 16 + 64;
+    F.acc_stride = F.pg + 4;
+    for (int alias = 0; alias < 2; ++alias) {
+      if (alias && F.tiles > 2) continue;
+      uint32_t off = 0;
+      auto take = [&](uint32_t bytes) { const uint32_t o = off; off = up(off + bytes, kAlign); return o; };
+      F.alias = alias;
+      F.s_v = take((uint32_t)F.c * F.pg * 4);
+      if (F.im2col) {
+        F.plane16 = 16 * group;
+        F.s_xa = take((uint32_t)(F.rec / 16) * F.plane16 * 16 + 64 * 16);       // a tile's 64 rows read past a short last plane
+      } else {
+        F.plane16 = group * F.frame;
+        F.s_xa = take((uint32_t)(F.rec / 16) * F.plane16 * 16);
+      }
+      F.s_xa_end = off;
+      F.s_acc = F.im2col ? 0 : take((uint32_t)F.cb * F.acc_stride * 4);
+      const uint32_t a_bytes = 2u * nd.kb * F.pitch;
+      F.s_a[0] = take(a_bytes);
+      F.s_a[1] = F.tiles > 1 ? take(a_bytes) : F.s_a[0];
+      F.s_meta[0] = take(nd.meta);
+      F.s_meta[1] = take(nd.meta);
+      F.s_w[0] = take(alias ? std::max(nd.w[0], nd.w[2]) : nd.w[0]);
+      F.s_w[1] = take(nd.w[1]);
+      F.s_w[2] = alias ? F.s_w[0] : take(nd.w[2]);
+      F.s_total = off;
+      if (off > limit) continue;
+      // operand chunks of the first conv's K steps, now that the planes' distance is known
+      for (int st = 0; st < F.ks1; ++st) {
+        auto chunk = [&](int ck) -> int {
+          if (F.im2col) return ck * F.plane16;
+          const int tap = ck % 9;
+          return (tap / 3 - 1) * F.wp + (tap % 3 - 1) + (ck / 9) * F.plane16;
+        };
+        if (F.paired) {
+          F.step[st] = (uint32_t)((st - 1) * F.wp - 1) + (2u << 16);
+          continue;
+        }
+        const int chunks = F.im2col ? F.rec / 16 : 9 * (F.rec / 16);
+        const int lbo = 2 * st + 1 < chunks ? chunk(2 * st + 1) - chunk(2 * st) : 1;       // (the last may be half used)
+        F.step[st] = (uint32_t)chunk(2 * st) + ((uint32_t)lbo << 16);
+      }
+      return true;
+    }
   }
   return false;
 }
@@ -729,6 +997,52 @@ int pack_residual_level(const iodf_level_desc& lv, const Blobs& B, LevelPlan& P,
   return IODF_OK;
 }
 
+// Packs a level for the compact kernel, if that can run it.
+bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, const std::vector<std::vector<int>>& cols,
+                     const std::vector<std::array<HiddenOrder, 2>>& orders, uint32_t smem_limit, uint32_t max_batch,
+                     int num_sms, bool throughput) {
+  LevelPlan& P = hl.plan;
+  FlowPlan& F = hl.flow;
+  std::memset(&F, 0, sizeof(F));
+  F.c = P.c; F.h = P.h; F.w = P.w; F.px = P.px; F.ca = P.ca; F.cb = P.cb;
+  F.n_couplings = P.n_couplings; F.has_prior = P.has_prior; F.is_first = P.is_first; F.is_last = P.is_last; F.keep_c = P.keep_c;
+  F.mul_per_img = P.mul_per_img; F.mul_4px = P.mul_4px; F.mul_w2 = P.mul_w2; F.mul_px = P.mul_px; F.mul_w = P.mul_w;
+  F.z_off = (int64_t)P.z_off; F.prior_off = (int64_t)P.prior_off; F.z_final_off = (int64_t)P.z_final_off;
+  F.d = (int64_t)P.d; F.d_fact = (int64_t)P.d_fact;
+  F.n_prior = lv.has_prior ? (int)up(2 * (uint32_t)F.cb, 16) : 16;
+  std::vector<KByte> kmap;
+  if (!flow_geometry(F, kmap)) return false;
+  // the kernel's 64-bit requantisations keep the high word: shifts s >= 1
+  auto shifts_ok = [&](const iodf_layer_desc& L) {
+    const int32_t* sh = B.r + L.requant_off + 2 * (size_t)L.c_out;
+    return std::all_of(sh, sh + L.c_out, [](int32_t x) { return x >= 1; });
+  };
+  for (uint32_t ki = 0; ki < lv.n_couplings; ++ki)
+    if (lv.couplings[ki].in_s < 1 || !shifts_ok(lv.couplings[ki].layers[2])) return false;
+  if (lv.has_prior && (lv.prior_in_s < 1 || !shifts_ok(lv.prior_layer))) return false;
+  FlowNeeds nd;
+  std::vector<PackedBlock> blocks;
+  for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) {
+    FlowDims d;
+    blocks.push_back(pack_flow_coupling(lv.couplings[ki], B, F, kmap, orders[ki][0], orders[ki][1], cols[ki].data(),
+                                        cols[ki].data() + F.ca, &d));
+    nd.n_hidden = std::max<uint32_t>(nd.n_hidden, (uint32_t)std::max(d.n1, d.n2));
+    nd.n_taps = std::max<uint32_t>(nd.n_taps, (uint32_t)d.n3);
+    nd.kb = std::max<uint32_t>(nd.kb, (uint32_t)std::max(d.ks2, d.ks3));
+  }
+  PackedBlock prior;
+  if (lv.has_prior) prior = pack_flow_prior(lv, B, F, kmap);
+  hl.blob.clear();
+  auto add = [&](const PackedBlock& pb, BlockRef* ref) {
+    append_block(hl.blob, pb, ref);
+    nd.meta = std::max(nd.meta, ref->meta_bytes);
+    for (int g = 0; g < 3; ++g) nd.w[g] = std::max(nd.w[g], ref->w_bytes[g]);
+  };
+  for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) add(blocks[ki], &P.coupling[ki]);
+  if (lv.has_prior) add(prior, &P.prior);
+  return plan_flow(F, nd, smem_limit, max_batch, num_sms, throughput);
+}
+
 int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_model* m) {
   if (desc->abi_version != IODF_ABI_VERSION) return IODF_EVERSION;
   if (!desc->levels || desc->n_levels < 1 || desc->n_levels > IODF_MAX_LEVELS || desc->max_batch < 1 ||
@@ -876,6 +1190,34 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
       if (lv.split) c = (uint32_t)ca;
       continue;
     }
+    std::vector<std::vector<int>> cols;          // physical columns of every coupling's logical channels
+    std::vector<std::array<HiddenOrder, 2>> orders;
+    bool all_folded = lv.n_couplings > 0;
+    for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) {
+      const iodf_coupling_desc& cp = lv.couplings[ki];
+      std::vector<int> nxt(c);
+      for (uint32_t k = 0; k < c; ++k) nxt[k] = pi[cp.perm[k]];
+      pi.swap(nxt);
+      cols.push_back(pi);
+      Act a1, a2;
+      hidden_range(cp.layers[0], &a1);
+      hidden_range(cp.layers[1], &a2);
+      orders.push_back({order_hidden(cp.layers[0], B, a1, (int)up(cp.layers[0].c_out, 16)),
+                        order_hidden(cp.layers[1], B, a2, (int)up(cp.layers[1].c_out, 16))});
+      all_folded = all_folded && orders.back()[0].folded && orders.back()[1].folded;
+    }
+    for (int k = 0; k < (int)c; ++k) P.col_out[k] = pi[k];
+    // the index maps divide numbers below group * c * px by at most c * px with a 32-bit magic multiplier
+    auto index_maps_fit = [&](int group) { return (uint64_t)group * c * h * w * ((uint64_t)c * h * w) < (1ull << 32); };
+    if (all_folded && plan_flow_level(lv, B, hl, cols, orders, (uint32_t)smem_limit, desc->max_batch, num_sms,
+                                     desc->plan == IODF_PLAN_THROUGHPUT) &&
+        index_maps_fit(hl.flow.group)) {
+      hl.use_flow = true;
+      P.group = hl.flow.group; P.s_total = hl.flow.s_total;
+      if (lv.split) c = (uint32_t)ca;
+      continue;
+    }
+    hl.blob.clear();
     uint32_t a_bytes = 16, meta = 16, wmax[3] = {16, 16, 16};
     uint32_t n_max = 32;
     PipeDims pd;
@@ -883,14 +1225,11 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
     std::vector<PackedBlock> blocks;
     for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) {
       const iodf_coupling_desc& cp = lv.couplings[ki];
-      std::vector<int> nxt(c);
-      for (uint32_t k = 0; k < c; ++k) nxt[k] = pi[cp.perm[k]];
-      pi.swap(nxt);
       Act a1, a2r;
       hidden_range(cp.layers[0], &a1);
       hidden_range(cp.layers[1], &a2r);
       Dims d;
-      blocks.push_back(pack_coupling(cp, B, ca, cb, pi.data(), pi.data() + ca, a1, a2r, &d));
+      blocks.push_back(pack_coupling(cp, B, ca, cb, cols[ki].data(), cols[ki].data() + ca, a1, a2r, orders[ki][0], orders[ki][1], &d));
       a_bytes = std::max<uint32_t>(a_bytes, kTileM * std::max(d.kd1, std::max(d.kd2, d.kd3)));
       n_max = std::max<uint32_t>(n_max, std::max(d.n1, std::max(d.n2, d.n3)));
       const CouplingMeta* cm = reinterpret_cast<const CouplingMeta*>(blocks.back().meta.data());
@@ -899,7 +1238,6 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
       pd.a1_bytes = std::max<uint32_t>(pd.a1_bytes, (uint32_t)kTileM * d.kd1);
       pd.n_taps = std::max<uint32_t>(pd.n_taps, (uint32_t)d.n3);
     }
-    for (int k = 0; k < (int)c; ++k) P.col_out[k] = pi[k];
     PackedBlock prior_block;
     if (lv.has_prior) {
       int n, kd;
@@ -939,8 +1277,7 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
     if (!plan_smem(P, a_bytes, meta, wmax, n_max, (uint32_t)smem_limit, desc->max_batch, num_sms, pd,
                    desc->plan == IODF_PLAN_THROUGHPUT))
       return IODF_EUNSUPPORTED;
-    // the index maps divide numbers below group * c * px by at most c * px with a 32-bit magic multiplier
-    if ((uint64_t)P.group * c * h * w * ((uint64_t)c * h * w) >= (1ull << 32)) return IODF_EUNSUPPORTED;
+    if (!index_maps_fit(P.group)) return IODF_EUNSUPPORTED;
     max_smem = std::max(max_smem, P.s_total);
     if (lv.split) c = (uint32_t)ca;
   }
@@ -952,6 +1289,7 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
   CU(m, configure_level_kernels((uint32_t)smem_limit));
   CU(m, configure_res_kernels((uint32_t)smem_limit));
   CU(m, configure_pipe_kernels((uint32_t)smem_limit));
+  CU(m, configure_flow_kernels((uint32_t)smem_limit));
   const size_t L = desc->n_levels;
   m->d_plan.assign(L, nullptr); m->d_blob.assign(L, nullptr); m->d_keep.assign(L, nullptr);
   for (size_t li = 0; li < L; ++li) {
@@ -987,8 +1325,10 @@ void set_patch_grid(LevelArgs& a, const PatchGrid& g) {
 }
 
 // The kernel that runs a level: residual couplings, the stage pipeline, or the general kernel.
-cudaError_t launch_any_level(const LevelPlan& P, const LevelArgs& a, bool inverse, int B, cudaStream_t st) {
+cudaError_t launch_any_level(const HostLevel& hl, const LevelArgs& a, bool inverse, int B, cudaStream_t st) {
+  const LevelPlan& P = hl.plan;
   const int grid = (B + P.group - 1) / P.group;
+  if (hl.use_flow) return launch_flow_level(a, hl.flow, inverse, grid, st);
   if (P.residual) return launch_res_level(a, inverse, grid, P.res_bands, P.s_total, st);
   if (P.pipe) return launch_level_pipe(a, inverse, grid, P.s_total, st);
   return launch_level(a, inverse, P.lean != 0, grid, P.s_total, st);
@@ -1012,7 +1352,7 @@ int run_forward(iodf_model* m, const uint8_t* x, int B, int32_t* z, int32_t* pri
     a.status = m->d_status;
     a.batch = B;
     if (li == 0) set_patch_grid(a, grid);
-    CU(m, launch_any_level(P, a, false, B, st));
+    CU(m, launch_any_level(m->levels[li], a, false, B, st));
     if (timed) CU(m, cudaEventRecord(m->ev[li + 1], st));
   }
   return IODF_OK;
@@ -1036,7 +1376,7 @@ int launch_inverse_level(iodf_model* m, int li, int phase, const int32_t* z, int
   a.batch = B;
   a.phase = phase;
   if (li == 0) set_patch_grid(a, grid);
-  CU(m, launch_any_level(P, a, true, B, st));
+  CU(m, launch_any_level(m->levels[li], a, true, B, st));
   return IODF_OK;
 }
 
@@ -1158,7 +1498,7 @@ int iodf_forward_static(iodf_model* m, const uint8_t* x_u8, int B, int32_t* z, i
     a.oor = nullptr;
     a.status = m->d_status;
     a.batch = B;
-    CU(m, launch_any_level(P, a, false, B, st));
+    CU(m, launch_any_level(m->levels[li], a, false, B, st));
   }
   return IODF_OK;
 }
@@ -1589,6 +1929,7 @@ int iodf_int8_mma_peak(iodf_model* m, uint32_t mma_groups, void* cuda_stream, un
 const char* iodf_level_kernel_name(const iodf_model* m, int level) {
   if (!m || level < 0 || level >= (int)m->levels.size()) return "";
   const LevelPlan& P = m->levels[level].plan;
+  if (m->levels[level].use_flow) return "flow_level_kernel";
   return P.residual ? "res_level_kernel" : (P.pipe ? "level_pipe_kernel" : "level_kernel");
 }
 

@@ -135,7 +135,7 @@ struct LevelPlan {
   uint32_t recip_gpa, recip_gpb; // floor(g / (cpad/8)) = (g * recip_gpa) >> 16 for g < 4096; same for cbp/8
   // global layout
   uint64_t z_off, prior_off, z_final_off, d, d_fact;
-  int32_t col_out[kMaxC];        // physical column of logical channel k after the last coupling
+  alignas(16) int32_t col_out[kMaxC];   // physical column of logical channel k after the last coupling
   // im2col granule g of the first conv's K (8 bytes): {byte offset of its source relative to the
   // pixel's xa record, validity selector: tap 0..8 = bit of the row's gather mask, kGranBias, kGranPad}
   int32_t n_gran;

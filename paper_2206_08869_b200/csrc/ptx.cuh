@@ -88,6 +88,18 @@ __device__ __forceinline__ void red_add_s32(uint32_t saddr, int val, bool pred) 
       : "memory");
 }
 
+// Two predicated fire-and-forget adds (channels `stride` bytes apart).
+__device__ __forceinline__ void red_add2_s32(uint32_t saddr, uint32_t stride, int v0, int v1, bool pred) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .u32 a;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "add.u32 a, %0, %1;\n\t"
+      "@p red.shared.add.s32 [%0], %2;\n\t"
+      "@p red.shared.add.s32 [a], %3;\n\t}" ::"r"(saddr),
+      "r"(stride), "r"(v0), "r"(v1), "r"((uint32_t)pred)
+      : "memory");
+}
+
 // Fire-and-forget add at a compile-time byte offset from saddr (the offset rides in the instruction).
 template <int kOff>
 __device__ __forceinline__ void red_add_s32_at(uint32_t saddr, int val) {
@@ -166,6 +178,9 @@ __device__ __forceinline__ void tmem_ld_wait32(uint32_t (&r)[32]) {
                  "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
                  "+r"(r[29]), "+r"(r[30]), "+r"(r[31]));
 }
+__device__ __forceinline__ void tmem_ld_wait4_nosync(uint32_t (&r)[4]) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]));
+}
 // No instruction: only tells the compiler that r is valid from here on (the wait that covered its
 // load has been executed already, for another register set).
 __device__ __forceinline__ void tmem_ld_wait16_nosync(uint32_t (&r)[16]) {
@@ -209,6 +224,22 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
+}
+
+// 16 lanes (0..15 or 16..31 of the warp's quarter, by the address) x 32 columns: r[4 i + e] and
+// r[4 i + 2 + e] of lane T are column 8 i + 2 (T & 3) + e of lanes T / 4 and T / 4 + 8.
+__device__ __forceinline__ void tmem_ld_16x32(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+// the same for 8 columns (i = 0)
+__device__ __forceinline__ void tmem_ld_16x8(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
 }
 
 // ---- tcgen05.mma, 8-bit integer operands, int32 accumulator in TMEM ---------------------------
@@ -267,6 +298,26 @@ __device__ __forceinline__ void umma_i8_acc(uint32_t d_tmem, uint64_t adesc, uin
       "setp.eq.b32 p, 0, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc)
+      : "memory");
+}
+// One lane of a converged warp, the same one every time. Code behind it is warp-uniform for the compiler
+// (operands of tcgen05.mma stay in uniform registers): measured 40 clocks per MMA issued against 52 and a
+// round trip of 373 against 447 clocks behind a `lane == 0` branch.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// Operand descriptors given by both words (operands whose row-group stride is not 128 bytes).
+__device__ __forceinline__ void umma_i8_hl(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                           uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %2};\n\t"
+      "mov.b64 db, {%3, %4};\n\t"
+      "setp.ne.b32 p, %6, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %5, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // Arrive on the mbarrier once every tcgen05.mma issued so far by this thread has completed.
