@@ -16,6 +16,7 @@
 #include "iodf_dev.h"
 #include "flow_level.h"
 #include "rans_kernel.h"
+#include "res_flow.h"
 #include "res_level.h"
 #include "level_kernel.h"
 #include "level_pipe.h"
@@ -33,6 +34,8 @@ struct HostLevel {
   LevelPlan plan;
   FlowPlan flow;                     // levels that run in the compact kernel (use_flow)
   bool use_flow = false;
+  RfPlan rf;                         // residual levels that run in the overlapped kernel (use_rf)
+  bool use_rf = false;
   std::vector<uint8_t> blob;
   int grid_group = 1;
   int32_t ls_lo = 0, ls_hi = 0;      // clip of the prior head's log-scale index (levels with a head)
@@ -724,6 +727,232 @@ bool plan_smem(LevelPlan& P, uint32_t a_bytes, uint32_t meta_bytes, const uint32
   return false;
 }
 
+// ---- residual levels of the overlapped kernel (res_flow.cu) ---------------------------------------------
+// bias = w[0] + c (w[1] + ... + w[15]), |w| <= 127 (the constant operand row is 1, c, ..., c)
+bool fold_bias_row(int64_t bias, int c, int8_t w[16]) {
+  int64_t q = bias >= 0 ? (bias + c / 2) / c : -((-bias + c / 2) / c);
+  w[0] = (int8_t)(bias - c * q);
+  for (int j = 1; j < 16; ++j) {
+    const int64_t t = std::max<int64_t>(-127, std::min<int64_t>(127, q));
+    w[j] = (int8_t)t;
+    q -= t;
+  }
+  return q == 0;
+}
+
+// float m with rne(x m) = floor((x m0 + 2^(30+s)) / 2^(31+s)) for every x in 0..255
+bool shortcut_multiplier(int32_t m0, int32_t s, float* out) {
+  float m = (float)std::ldexp((double)m0, -(31 + s));
+  for (int k = 0; k < 4; ++k) m = std::nextafterf(m, 0.f);
+  for (int k = 0; k < 64; ++k, m = std::nextafterf(m, 2.f)) {
+    bool ok = true;
+    for (int x = 0; x < 256 && ok; ++x) {
+      const double p = (double)x * (double)m;                       // exact: 8 + 24 bits
+      ok = (int64_t)std::nearbyint(p) == (((int64_t)x * m0 + (1ll << (30 + s))) >> (31 + s));
+    }
+    if (ok) { *out = m; return true; }
+  }
+  return false;
+}
+
+bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, const std::vector<std::vector<int>>& cols,
+                         uint32_t smem_limit, uint32_t max_batch, int num_sms, bool throughput) {
+  const LevelPlan& P = hl.plan;
+  RfPlan& R = hl.rf;
+  std::memset(&R, 0, sizeof(R));
+  R.c = P.c; R.h = P.h; R.w = P.w; R.px = P.px; R.ca = P.ca; R.cb = P.cb;
+  R.n_couplings = P.n_couplings; R.has_prior = P.has_prior; R.is_first = P.is_first; R.is_last = P.is_last; R.keep_c = P.keep_c;
+  R.z_off = (int64_t)P.z_off; R.prior_off = (int64_t)P.prior_off; R.z_final_off = (int64_t)P.z_final_off;
+  R.d = (int64_t)P.d; R.d_fact = (int64_t)P.d_fact;
+  R.group = 1;
+  if (R.w % 16 == 0 && R.h % 16 == 0) {
+    R.bh = R.bw = 16; R.m = 128;
+    R.tiles = R.bw / 8;
+  } else if (R.w == 8 && R.h == 8) {
+    R.bw = R.bh = 8; R.m = 64; R.tiles = 1;
+  } else if (R.w == 4 && R.h == 4) {
+    R.bw = R.bh = 4; R.tiles = 1; R.small = 1;
+    // three images fill a 128-row tile; the latency plan takes them together only where SMs run out
+    R.group = std::min<int>(3, throughput ? (int)max_batch : ((int)max_batch + num_sms - 1) / num_sms);
+    R.m = R.group > 1 ? 128 : 64;
+  } else {
+    return false;
+  }
+  R.nbx = R.w / R.bw; R.nby = R.h / R.bh;
+  if (R.nbx * R.nby > 8 || R.ca > kResMaxWidth) return false;
+  R.wp = R.bw + 2;
+  R.plane16 = R.small ? (R.m / 8 + 2) * R.wp + 8 : (R.bh + 2) * R.wp;
+  R.pg = R.group * R.bw * R.bh;
+  R.xa_chunks = (int)up((uint32_t)R.ca, 32) / 32;
+  const uint32_t nc = lv.n_couplings;
+  R.convs_per_coupling = (int)lv.couplings[0].n_layers;
+  for (uint32_t ki = 0; ki < nc; ++ki)
+    if ((int)lv.couplings[ki].n_layers != R.convs_per_coupling) return false;
+
+  std::vector<uint8_t>& blob = hl.blob;
+  blob.clear();
+  auto place = [&](size_t bytes) { blob.resize(up((uint32_t)blob.size(), kAlign), 0); const uint32_t o = (uint32_t)blob.size(); blob.resize(o + bytes, 0); return o; };
+  const uint32_t n_convs = nc * (uint32_t)R.convs_per_coupling + (lv.has_prior ? 1u : 0u);
+  R.conv_off = place(sizeof(RfConv) * n_convs);
+  std::vector<RfConv> convs;
+  int chunks[3] = {R.xa_chunks, 1, R.xa_chunks};
+  uint32_t meta_max = 0;
+  int n_max = 16;
+
+  // One conv. rows: packed output position -> filter of L (-1: none). korder: packed input position -> input
+  // channel (empty: natural order, the network input). fc: floating-point constants by filter (hidden convs).
+  auto add_conv = [&](const iodf_layer_desc& L, RfMeta M, const std::vector<int>& rows, const std::vector<int>& korder,
+                      const std::vector<FloatChannel>* fc, const int32_t* c_cols, int n_cols) -> bool {
+    const int32_t* bias = B.r + L.requant_off;
+    const int32_t* m0 = bias + L.c_out;
+    const int32_t* s = m0 + L.c_out;
+    const bool table = M.kind == kRfHidden || M.kind == kRfBranch;
+    M.n = (int)rows.size(); M.n_pad = (int)up((uint32_t)M.n, 16); M.nb = (int)up((uint32_t)M.n, 32) / 32;
+    M.nk = (int)up(L.c_in, 32) / 32;
+    if (M.n_pad > 128 || M.nb > kRfChunks || M.nk > kRfChunks) return false;
+    if (table) {
+      M.us = s[0];
+      for (uint32_t i = 0; i < L.c_out; ++i)
+        if (s[i] != s[0] || s[i] < 1) return false;
+      chunks[M.dst] = std::max(chunks[M.dst], M.nb);
+    }
+    chunks[M.src] = std::max(chunks[M.src], M.nk);
+    // meta block
+    std::vector<uint8_t> meta(sizeof(RfMeta), 0);
+    M.nfi = M.nb;
+    if (table) {
+      meta.resize(sizeof(RfMeta) + (M.kind == kRfHidden ? 2 : 1) * kRfChunks * 128, 0);
+      int32_t* mt = reinterpret_cast<int32_t*>(meta.data() + sizeof(RfMeta));
+      int32_t* ct = mt + kRfChunks * 32;
+      if (fc)
+        for (int i = M.n - 1; i >= 0 && (*fc)[rows[i]].none; --i) M.nfi = i / 32;
+      for (int i = 0; i < M.nb * 32; ++i) {
+        const int k = flow_kpos(i), j = i < M.n ? rows[i] : -1;
+        if (!fc || i >= 32 * M.nfi) {
+          mt[k] = j >= 0 ? m0[j] : (1 << 30);
+        } else if (j >= 0) {
+          std::memcpy(&mt[k], &(*fc)[j].m, 4);
+          if ((*fc)[j].C) ct[k] = (int32_t)(0x80000000u | (uint32_t)(*fc)[j].C);
+        }
+      }
+    } else {
+      meta.resize(sizeof(RfMeta) + sizeof(OutRq) * (size_t)M.n, 0);
+      put_out_rq(reinterpret_cast<OutRq*>(meta.data() + sizeof(RfMeta)), L, B);
+    }
+    if (n_cols) {
+      M.cols_off = (uint32_t)meta.size();
+      meta.resize(meta.size() + up(4u * (uint32_t)n_cols, 16), 0);
+      std::memcpy(meta.data() + M.cols_off, c_cols, 4 * (size_t)n_cols);
+    }
+    std::memcpy(meta.data(), &M, sizeof(M));
+    meta_max = std::max(meta_max, (uint32_t)meta.size());
+    n_max = std::max(n_max, M.n_pad);
+    // weights: [kc][u]{bias rows first}[v][2][n_pad][16]
+    RfConv c{};
+    c.n_pad = M.n_pad; c.nk = M.nk;
+    c.meta_bytes = (uint32_t)meta.size();
+    c.meta_off = place(meta.size());
+    std::memcpy(blob.data() + c.meta_off, meta.data(), meta.size());
+    const size_t step = 32 * (size_t)M.n_pad;
+    c.w_off = place(step * (9 * (size_t)M.nk + 1));
+    uint8_t* out = blob.data() + c.w_off;
+    const int cst = M.a_unsigned ? 255 : 127;
+    if (table)
+      for (int i = 0; i < M.n; ++i) {
+        if (rows[i] < 0) continue;
+        int8_t w[16];
+        const int64_t beta = fc && i < 32 * M.nfi ? (*fc)[rows[i]].beta : 0;
+        if (!fold_bias_row((int64_t)bias[rows[i]] + beta, cst, w)) return false;
+        std::memcpy(out + (size_t)i * 16, w, 16);
+      }
+    out += step;
+    const int8_t* w = B.w + L.weight_off;
+    for (int kc = 0; kc < M.nk; ++kc)
+      for (int tap = 0; tap < 9; ++tap, out += step)
+        for (int i = 0; i < M.n; ++i) {
+          if (rows[i] < 0) continue;
+          for (int k = 0; k < 32; ++k) {
+            const int at = kc * 32 + k;                                        // packed input position
+            const int kk = korder.empty() ? k : flow_kpos(at) - kc * 32;       // its byte
+            if (at >= (int)L.c_in) continue;
+            const int ch = korder.empty() ? at : korder[at];
+            out[(size_t)(kk >> 4) * M.n_pad * 16 + (size_t)i * 16 + (kk & 15)] = (uint8_t)w[((size_t)rows[i] * 9 + tap) * L.c_in + ch];
+          }
+        }
+    convs.push_back(c);
+    return true;
+  };
+  // constants of a hidden conv and the order of its outputs (channels without constants last)
+  auto hidden = [&](const iodf_layer_desc& L, int cst, std::vector<FloatChannel>& fc, std::vector<int>& order) {
+    const int32_t* bias = B.r + L.requant_off;
+    const int32_t* m0 = bias + L.c_out;
+    const int32_t* s = m0 + L.c_out;
+    fc.assign(L.c_out, FloatChannel{});
+    order.resize(L.c_out);
+    for (uint32_t i = 0; i < L.c_out; ++i) {
+      order[i] = (int)i;
+      const int64_t room = 127ll * cst * 15 - std::llabs((long long)bias[i]);
+      if (room < 0 || !float_requant(m0[i], s[i], 255, room, &fc[i])) {
+        fc[i] = FloatChannel{};
+        fc[i].none = true;
+      }
+    }
+    std::stable_partition(order.begin(), order.end(), [&](int i) { return !fc[i].none; });
+  };
+  auto natural = [](int n) { std::vector<int> v(n); for (int i = 0; i < n; ++i) v[i] = i; return v; };
+
+  for (uint32_t ki = 0; ki < nc; ++ki) {
+    const iodf_coupling_desc& cp = lv.couplings[ki];
+    std::vector<int32_t> colA(cols[ki].begin(), cols[ki].begin() + R.ca), colB(cols[ki].begin() + R.ca, cols[ki].begin() + R.ca + R.cb);
+    std::vector<FloatChannel> fc;
+    std::vector<int> xorder, korder;
+    hidden(cp.layers[0], 127, fc, xorder);
+    RfMeta M{};
+    M.kind = kRfHidden; M.src = 0; M.dst = 1; M.input = 1; M.in_m0 = cp.in_m0; M.in_s = cp.in_s;
+    if (!add_conv(cp.layers[0], M, xorder, {}, &fc, colA.data(), R.ca)) return false;
+    for (uint32_t b = 0; b < cp.n_blocks; ++b) {
+      const iodf_layer_desc& la = cp.layers[1 + 2 * b];
+      const iodf_layer_desc& lb = cp.layers[2 + 2 * b];
+      hidden(la, 255, fc, korder);
+      M = RfMeta{};
+      M.kind = kRfHidden; M.src = 1; M.dst = 2; M.a_unsigned = 1;
+      if (!add_conv(la, M, korder, xorder, &fc, nullptr, 0)) return false;
+      M = RfMeta{};
+      M.kind = kRfBranch; M.src = 2; M.dst = 1; M.a_unsigned = 1;
+      if (!shortcut_multiplier(cp.blocks[b].short_m0, cp.blocks[b].short_s, &M.short_m)) return false;
+      std::vector<int> filter_of(xorder.size(), -1), rows(xorder.size());
+      for (uint32_t j = 0; j < cp.blocks[b].n_idx; ++j) filter_of[cp.blocks[b].idx[j]] = (int)j;
+      for (size_t i = 0; i < xorder.size(); ++i) rows[i] = filter_of[xorder[i]];
+      if (!add_conv(lb, M, rows, korder, nullptr, nullptr, 0)) return false;
+    }
+    M = RfMeta{};
+    M.kind = kRfOut; M.src = 1; M.a_unsigned = 1;
+    if (!add_conv(cp.layers[cp.n_layers - 1], M, natural(R.cb), xorder, nullptr, colB.data(), R.cb)) return false;
+  }
+  if (lv.has_prior) {
+    RfMeta M{};
+    M.kind = kRfPrior; M.src = 2; M.input = 1; M.in_m0 = lv.prior_in_m0; M.in_s = lv.prior_in_s; M.ls_lo = lv.ls_lo; M.ls_hi = lv.ls_hi;
+    std::vector<int32_t> colA(P.col_out, P.col_out + R.ca);
+    if (!add_conv(lv.prior_layer, M, natural(2 * R.cb), {}, nullptr, colA.data(), R.ca)) return false;
+  }
+  std::memcpy(blob.data() + R.conv_off, convs.data(), sizeof(RfConv) * convs.size());
+
+  uint32_t off = 0;
+  auto take = [&](uint32_t bytes) { const uint32_t o = off; off = up(off + bytes, kAlign); return o; };
+  R.s_v = take((uint32_t)R.c * R.pg * 4);
+  for (int b = 0; b < 3; ++b) R.s_buf[b] = take((uint32_t)(2 * chunks[b]) * R.plane16 * 16);
+  take(256);                                       // (an 8-row group of a 4 x 4 image reads a few positions past the last plane)
+  R.s_buf_end = off;
+  R.s_const = take(2 * 2304);
+  for (int i = 0; i < 3; ++i) R.s_meta[i] = take(meta_max);
+  R.slot_bytes = 4u * 32u * (uint32_t)n_max;
+  R.s_ring = off;
+  if (off + 3 * R.slot_bytes > smem_limit) return false;
+  R.n_slots = std::min<int>(kRfMaxSlots, (int)((smem_limit - off) / R.slot_bytes));
+  R.s_total = off + (uint32_t)R.n_slots * R.slot_bytes;
+  return true;
+}
+
 // Group, tensor-memory columns and shared-memory layout of a level in the compact kernel. false: it does not fit.
 struct FlowNeeds { uint32_t n_hidden = 32, n_taps = 16, kb = 1, meta = 16, w[3] = {16, 16, 16}; };
 bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, uint32_t max_batch, int num_sms, bool throughput) {
@@ -1183,6 +1412,13 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
         cols.push_back(pi);
       }
       for (int k = 0; k < (int)c; ++k) P.col_out[k] = pi[k];
+      if (plan_res_flow_level(lv, B, hl, cols, (uint32_t)smem_limit, desc->max_batch, num_sms, desc->plan == IODF_PLAN_THROUGHPUT)) {
+        hl.use_rf = true;
+        P.residual = 1; P.group = hl.rf.group; P.s_total = hl.rf.s_total;
+        if (lv.split) c = (uint32_t)ca;
+        continue;
+      }
+      hl.blob.clear();
       int rc = pack_residual_level(lv, B, P, hl.blob, cols, (uint32_t)smem_limit, desc->max_batch,
                                    desc->plan == IODF_PLAN_THROUGHPUT);
       if (rc) return rc;
@@ -1290,6 +1526,7 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
   CU(m, configure_res_kernels((uint32_t)smem_limit));
   CU(m, configure_pipe_kernels((uint32_t)smem_limit));
   CU(m, configure_flow_kernels((uint32_t)smem_limit));
+  CU(m, configure_res_flow_kernels((uint32_t)smem_limit));
   const size_t L = desc->n_levels;
   m->d_plan.assign(L, nullptr); m->d_blob.assign(L, nullptr); m->d_keep.assign(L, nullptr);
   for (size_t li = 0; li < L; ++li) {
@@ -1329,6 +1566,7 @@ cudaError_t launch_any_level(const HostLevel& hl, const LevelArgs& a, bool inver
   const LevelPlan& P = hl.plan;
   const int grid = (B + P.group - 1) / P.group;
   if (hl.use_flow) return launch_flow_level(a, hl.flow, inverse, grid, st);
+  if (hl.use_rf) return launch_res_flow(a, hl.rf, inverse, grid * hl.rf.nbx * hl.rf.nby, st);
   if (P.residual) return launch_res_level(a, inverse, grid, P.res_bands, P.s_total, st);
   if (P.pipe) return launch_level_pipe(a, inverse, grid, P.s_total, st);
   return launch_level(a, inverse, P.lean != 0, grid, P.s_total, st);
@@ -1930,6 +2168,7 @@ const char* iodf_level_kernel_name(const iodf_model* m, int level) {
   if (!m || level < 0 || level >= (int)m->levels.size()) return "";
   const LevelPlan& P = m->levels[level].plan;
   if (m->levels[level].use_flow) return "flow_level_kernel";
+  if (m->levels[level].use_rf) return "res_flow_kernel";
   return P.residual ? "res_level_kernel" : (P.pipe ? "level_pipe_kernel" : "level_kernel");
 }
 
