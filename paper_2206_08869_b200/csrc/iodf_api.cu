@@ -945,9 +945,9 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
   R.s_buf_end = off;
   R.s_const = take(2 * 2304);
   for (int i = 0; i < 3; ++i) R.s_meta[i] = take(meta_max);
-  R.slot_bytes = 4u * 32u * (uint32_t)n_max;
+  R.slot_bytes = 10u * 32u * (uint32_t)n_max;
   R.s_ring = off;
-  if (off + 3 * R.slot_bytes > smem_limit) return false;
+  if (off + 2 * R.slot_bytes > smem_limit) return false;
   R.n_slots = std::min<int>(kRfMaxSlots, (int)((smem_limit - off) / R.slot_bytes));
   R.s_total = off + (uint32_t)R.n_slots * R.slot_bytes;
   return true;

@@ -19,8 +19,8 @@
 //   * Larger images are cut into 16-row blocks of 16 or 8 columns, one CTA of a cluster each. Edge
 //     positions are stored into the neighbours' frames, and their chunk barriers take the neighbours'
 //     arrivals: no cluster barrier between convs. 16 x 16 images use two CTAs while that fits the machine.
-//   * One warp issues the MMAs, one lane of another streams weights (groups of three taps of a chunk)
-//     and the convs' meta blocks.
+//   * One warp issues the MMAs (a chunk's nine taps per wait: waits and commits cost its lane 150 clocks
+//     each, an MMA 40), one lane of another streams weights and the convs' meta blocks.
 #include "res_flow.h"
 #include "level_device.cuh"
 
@@ -88,7 +88,18 @@ __device__ __forceinline__ void rf_hand_over(const Rf& f, uint64_t* bar) {
     __syncwarp();
     if (f.lane < f.nn)
       asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rf_peer(ptx::smem_u32(bar), f.nb_rank)) : "memory");
-    if (f.lane == 31) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rf_peer(ptx::smem_u32(bar), (uint32_t)f.rank)) : "memory");
+    if (f.lane == 31) rf_arrive_local(bar);
+  }
+}
+// arrival of a warp that has written nothing
+__device__ __forceinline__ void rf_arrive(const Rf& f, uint64_t* bar) {
+  __syncwarp();
+  if (f.nn == 0) {
+    if (f.lane == 0) rf_arrive_local(bar);
+  } else {
+    if (f.lane < f.nn)
+      asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rf_peer(ptx::smem_u32(bar), f.nb_rank)) : "memory");
+    if (f.lane == 31) rf_arrive_local(bar);
   }
 }
 // the MMA warp's wait for such a hand-over: acquires at cluster scope when neighbours write here
@@ -151,8 +162,8 @@ __device__ void rf_loader(const Rf& f, const RfPlan& P, const LevelArgs& a, cons
     }
     const uint8_t* src = a.blob + c.w_off;
 #pragma unroll 1
-    for (int g = 0; g < 3 * c.nk; ++g) {
-      const uint32_t bytes = (uint32_t)(g == 0 ? 4 : 3) * 32u * (uint32_t)c.n_pad;
+    for (int g = 0; g < c.nk; ++g) {
+      const uint32_t bytes = (uint32_t)(g == 0 ? 10 : 9) * 32u * (uint32_t)c.n_pad;
       if (round > 0) rf_wait(f, &ctl->w_empty[slot], (round - 1u) & 1u);
       const uint32_t b = ptx::smem_u32(&ctl->w_full[slot]);
       ptx::mbar_expect_tx(b, bytes);
@@ -167,7 +178,6 @@ __device__ void rf_loader(const Rf& f, const RfPlan& P, const LevelArgs& a, cons
 __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq) {
   RfCtl* ctl = f.ctl;
   uint8_t* smem = f.smem;
-  const bool lead = ptx::elect_one();
   auto uniform = [](int x) { return __shfl_sync(0xFFFFFFFFu, x, 0); };
   // (in a cluster a shared-memory address also carries the CTA's rank above the descriptor's 14 bits)
   auto addr16 = [&](uint32_t s) { return (ptx::smem_u32(smem + s) >> 4) & 0x3FFFu; };
@@ -188,37 +198,51 @@ __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq) {
     uint32_t a_chunk = addr16(P.s_buf[src]) + (uint32_t)P.wp + 1u + (plane << 16);
 #pragma unroll 1
     for (int kc = 0; kc < nk; ++kc) {
+      rf_wait(f, &ctl->w_full[slot], round & 1u);
       if (input) {
         if (kc == 0) { rf_wait_operand(f, &ctl->xa_ready, xa_par); xa_par ^= 1u; }
       } else {
         rf_wait_operand(f, &ctl->chunk_ready[kc], (ready >> kc) & 1u);
         ready ^= 1u << kc;
       }
-#pragma unroll 1
-      for (int u = 0; u < 3; ++u) {
-        rf_wait(f, &ctl->w_full[slot], round & 1u);
-        uint32_t bl = addr16(P.s_ring + slot * P.slot_bytes) | b_lbo;
-        if (kc == 0 && u == 0) {          // bias rows: the operand is the same constant row everywhere
-          const uint32_t al = addr16(P.s_const + (uns ? 0u : 2304u)) | (8u << 16);
-          for (int t = 0; t < P.tiles; ++t)
-            if (lead) ptx::umma_i8_hl(d0 + (uint32_t)(t * 128), al, ptx::kUmmaDescHi, bl, ptx::kUmmaDescHi, idesc, 0u);
+      uint32_t bl = addr16(P.s_ring + slot * P.slot_bytes) | b_lbo;
+      const uint32_t a_bias = addr16(P.s_const + (uns ? 0u : 2304u)) | (8u << 16);
+      if (ptx::elect_one()) {
+        if (kc == 0) {                    // bias rows: the operand is the same constant row everywhere
+          ptx::umma_i8_hl(d0, a_bias, ptx::kUmmaDescHi, bl, ptx::kUmmaDescHi, idesc, 0u);
+          if (P.tiles == 2) ptx::umma_i8_hl(d0 + 128u, a_bias, ptx::kUmmaDescHi, bl, ptx::kUmmaDescHi, idesc, 0u);
           bl += tap_step;
         }
-        uint32_t al = a_chunk + (uint32_t)((u - 1) * P.wp - 1);
+        uint32_t al = a_chunk - (uint32_t)P.wp - 1u;
+        if (P.tiles == 2) {
 #pragma unroll
-        for (int v = 0; v < 3; ++v) {
-          if (lead) ptx::umma_i8_hl(d0, al, a_hi, bl, ptx::kUmmaDescHi, idesc, 1u);
-          if (P.tiles == 2 && lead) ptx::umma_i8_hl(d0 + 128u, al + 8u, a_hi, bl, ptx::kUmmaDescHi, idesc, 1u);
-          al += 1u;
-          bl += tap_step;
+          for (int u = 0; u < 3; ++u) {
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+              ptx::umma_i8_hl(d0, al + (uint32_t)v, a_hi, bl, ptx::kUmmaDescHi, idesc, 1u);
+              ptx::umma_i8_hl(d0 + 128u, al + (uint32_t)(v + 8), a_hi, bl, ptx::kUmmaDescHi, idesc, 1u);
+              bl += tap_step;
+            }
+            al += (uint32_t)P.wp;
+          }
+        } else {
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+              ptx::umma_i8_hl(d0, al + (uint32_t)v, a_hi, bl, ptx::kUmmaDescHi, idesc, 1u);
+              bl += tap_step;
+            }
+            al += (uint32_t)P.wp;
+          }
         }
-        if (lead) ptx::umma_commit(ptx::smem_u32(&ctl->w_empty[slot]));
-        if (++slot == (uint32_t)P.n_slots) { slot = 0; ++round; }
+        ptx::umma_commit(ptx::smem_u32(&ctl->w_empty[slot]));
+        if (kc + 1 == nk) ptx::umma_commit(ptx::smem_u32(&ctl->d_ready[q & 1]));
       }
+      __syncwarp();
+      if (++slot == (uint32_t)P.n_slots) { slot = 0; ++round; }
       a_chunk += 2u * plane;
     }
-    if (lead) ptx::umma_commit(ptx::smem_u32(&ctl->d_ready[q & 1]));
-    __syncwarp();
   }
 }
 
@@ -425,8 +449,12 @@ __device__ void rf_workers(const Rf& f, const RfPlan& P, const LevelArgs& a, con
     if (kind == kRfHidden || kind == kRfBranch) {
 #pragma unroll 1
       for (int b = 0; b < nb; ++b) {
-        if ((b & (cstep - 1)) == c0) rf_unit(f, P, M, d, t, h, b);
-        rf_hand_over(f, &ctl->chunk_ready[b]);
+        if ((b & (cstep - 1)) == c0) {
+          rf_unit(f, P, M, d, t, h, b);
+          rf_hand_over(f, &ctl->chunk_ready[b]);
+        } else if (b == 0) {
+          rf_arrive(f, &ctl->chunk_ready[0]);       // (every warp arrives once per conv: nobody can miss a phase)
+        }
       }
     } else {
       rf_out<kInv>(f, P, a, M, d, v, b0);
@@ -524,7 +552,9 @@ __global__ void __launch_bounds__(kRfThreads, 1) res_flow_kernel(const LevelArgs
       }
   if (tid == 0) {
     const uint32_t arrivals = (uint32_t)(kRfWarps * (1 + f.nn));
-    for (int c = 0; c < kRfChunks; ++c) ptx::mbar_init(ptx::smem_u32(&ctl.chunk_ready[c]), arrivals);
+    // (chunk 0 takes every warp's arrival, the others those of the warps that work on them)
+    for (int c = 0; c < kRfChunks; ++c)
+      ptx::mbar_init(ptx::smem_u32(&ctl.chunk_ready[c]), c ? arrivals * (uint32_t)(P.tiles * (P.m >> 6)) / 4u : arrivals);
     ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), arrivals);
     for (int s = 0; s < 2; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.d_ready[s]), 1);
     for (int s = 0; s < 3; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.meta_full[s]), 1);

@@ -12,7 +12,7 @@ namespace iodf {
 constexpr int kRfWarps = 16;                        // requantising warps, four per TMEM lane quarter
 constexpr int kRfWorkers = kRfWarps * 32;
 constexpr int kRfThreads = kRfWorkers + 2 * 32;     // + the MMA-issuing warp and the weight-loading warp
-constexpr int kRfMaxSlots = 12;                     // weight ring
+constexpr int kRfMaxSlots = 4;                      // weight ring
 constexpr int kRfChunks = 4;                        // 32-channel chunks of the widest activation (128 channels)
 
 // What a conv's epilogue does (see res_flow.cu).
@@ -25,8 +25,8 @@ struct RfConv {
   int32_t pad[3];
 };
 static_assert(sizeof(RfConv) == 32, "32-byte records");
-// Its weights: for every chunk kc, for every tap row: three taps [2][n_pad][16 bytes]; the very first group
-// is preceded by the bias rows [2][n_pad][16] (they meet a constant operand row 1, c, c, ...).
+// Its weights: for every chunk kc nine taps [2][n_pad][16 bytes], preceded in the first chunk by the bias rows
+// [2][n_pad][16] (they meet a constant operand row 1, c, c, ...). A ring slot holds a chunk.
 
 // Head of a conv's meta block (shared memory), followed by kRfHidden / kRfBranch: float or int32 constants
 // [chunk][lane & 3][8] (multipliers), then kRfHidden: addends in the same order; kRfOut / kRfPrior: OutRq[n].
