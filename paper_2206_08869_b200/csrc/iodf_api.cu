@@ -767,6 +767,7 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
   R.group = 1;
   if (R.w % 16 == 0 && R.h % 16 == 0) {
     R.bh = R.bw = 16; R.m = 128;
+    if (getenv("RF8")) R.bw = 8;
     R.tiles = R.bw / 8;
   } else if (R.w == 8 && R.h == 8) {
     R.bw = R.bh = 8; R.m = 64; R.tiles = 1;

@@ -47,6 +47,7 @@ struct Rf {
   int rank, by, bx;                 // CTA of the cluster, its block
   int nn;                           // neighbours: lane k < nn of every warp owns one
   uint32_t nb_rank;                 // that neighbour's rank
+  bool edge;                        // worker's lane k: its warp's unit of a tile touches that neighbour's edge
 };
 
 __device__ __noinline__ void rf_wait_slow(uint32_t bar, uint32_t parity, RfCtl* ctl, uint32_t* status) {
@@ -76,31 +77,21 @@ __device__ __forceinline__ uint32_t rf_peer(uint32_t saddr, uint32_t rank) {
 __device__ __forceinline__ void rf_arrive_local(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ptx::smem_u32(bar)) : "memory");
 }
-// this warp's part of an activation (or nothing) is written: here and, for their edge positions, at the neighbours
-__device__ __forceinline__ void rf_hand_over(const Rf& f, uint64_t* bar) {
+// this warp's part of an activation is written: here and, for edge positions, at the neighbours. `remote`: this
+// lane's neighbour has been written to (a release at cluster scope costs a trip to the other SM, so that
+// warps without edge positions only arrive here).
+__device__ __forceinline__ void rf_hand_over(const Rf& f, uint64_t* bar, bool remote) {
   ptx::tc_fence_before();
-  if (f.nn == 0) {
-    ptx::fence_async_smem();
-    __syncwarp();
-    if (f.lane == 0) rf_arrive_local(bar);
-  } else {
+  if (f.nn && __any_sync(0xFFFFFFFFu, remote)) {
     asm volatile("fence.proxy.async;" ::: "memory");
     __syncwarp();
-    if (f.lane < f.nn)
+    if (remote)
       asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rf_peer(ptx::smem_u32(bar), f.nb_rank)) : "memory");
-    if (f.lane == 31) rf_arrive_local(bar);
-  }
-}
-// arrival of a warp that has written nothing
-__device__ __forceinline__ void rf_arrive(const Rf& f, uint64_t* bar) {
-  __syncwarp();
-  if (f.nn == 0) {
-    if (f.lane == 0) rf_arrive_local(bar);
   } else {
-    if (f.lane < f.nn)
-      asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rf_peer(ptx::smem_u32(bar), f.nb_rank)) : "memory");
-    if (f.lane == 31) rf_arrive_local(bar);
+    ptx::fence_async_smem();
+    __syncwarp();
   }
+  if (f.lane == 31) rf_arrive_local(bar);
 }
 // the MMA warp's wait for such a hand-over: acquires at cluster scope when neighbours write here
 __device__ __forceinline__ void rf_wait_operand(const Rf& f, uint64_t* bar, uint32_t parity) {
@@ -288,10 +279,11 @@ __device__ __forceinline__ void rf_store4(const Rf& f, const RfPlan& P, uint8_t*
 }
 
 // One unit: 16 rows (half `h` of this warp's lane quarter of tile `t`) x 32 columns (chunk b) of a hidden or branch conv.
-__device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMeta* __restrict__ M, uint32_t d, int t, int h, int b) {
+__device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMeta* __restrict__ M, uint32_t d, int t, int h, int b,
+                                        uint64_t* ready, uint32_t parity) {
   const int q = f.lane & 3, x = f.lane >> 2, hs = P.m >> 7;
+  // (what does not depend on the accumulator comes before the wait for it)
   uint32_t r[16];
-  ptx::tmem_ld_16x32(d + (uint32_t)(t * 128 + b * 32) + ((uint32_t)h << 20) + ((uint32_t)((f.warp & 3) * 32) << 16), r);
   const uint8_t* tab = reinterpret_cast<const uint8_t*>(M) + sizeof(RfMeta) + b * 128 + q * 32;
   const float4 m0 = *reinterpret_cast<const float4*>(tab), m1 = *reinterpret_cast<const float4*>(tab + 16);
   const float m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
@@ -305,6 +297,12 @@ __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMe
   }
   const uint32_t row = (uint32_t)P.wp * 16u;
   const int j = t * 8 + x;
+  auto accumulator = [&]() {
+    rf_wait(f, ready, parity);
+    ptx::tc_fence_after();
+    ptx::tmem_ld_16x32(d + (uint32_t)(t * 128 + b * 32) + ((uint32_t)h << 20) + ((uint32_t)((f.warp & 3) * 32) << 16), r);
+    ptx::tmem_ld_wait16(r);
+  };
   if (M->kind == kRfHidden) {
     float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
     if (b < M->nfi) {
@@ -312,8 +310,9 @@ __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMe
       c1 = *reinterpret_cast<const float4*>(tab + kRfChunks * 128 + 16);
     }
     const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-    ptx::tmem_ld_wait16(r);
-    if (b < M->nfi) {
+    const bool integer = b >= M->nfi;
+    accumulator();
+    if (!integer) {
 #pragma unroll
       for (int k = 0; k < 16; ++k) r[k] = (uint32_t)FloatRq::one(r[k], m[2 * (k >> 2) + (k & 1)], c[2 * (k >> 2) + (k & 1)]);
     } else {
@@ -330,7 +329,7 @@ __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMe
     const float ms = M->short_m;
     const long long rnd = 1ll << (30 + M->us);
     const int sh = M->us - 1;
-    ptx::tmem_ld_wait16(r);
+    accumulator();
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       const uint32_t word = (k & 8) ? ((k & 2) ? x1.y : x0.y) : ((k & 2) ? x1.x : x0.x);
@@ -440,23 +439,26 @@ __device__ void rf_workers(const Rf& f, const RfPlan& P, const LevelArgs& a, con
     if (++ms == 3) { ms = 0; mpar ^= 1u; }
     if (M->input) {
       rf_requant(f, P, M, v);
-      rf_hand_over(f, &ctl->xa_ready);
+      rf_hand_over(f, &ctl->xa_ready, f.lane < f.nn);
     }
     const uint32_t d = f.tmem + (uint32_t)((q & 1) * P.tiles * 128);
     const int nb = M->nb, kind = M->kind;
-    rf_wait(f, &ctl->d_ready[q & 1], (uint32_t)(q >> 1) & 1u);
-    ptx::tc_fence_after();
+    uint64_t* dr = &ctl->d_ready[q & 1];
+    const uint32_t dp = (uint32_t)(q >> 1) & 1u;
     if (kind == kRfHidden || kind == kRfBranch) {
+      if (c0 != 0) {                       // every warp arrives once per conv: nobody can miss a phase
+        rf_wait(f, dr, dp);
+        __syncwarp();
+        if (f.lane == 31) rf_arrive_local(&ctl->chunk_ready[0]);
+      }
 #pragma unroll 1
-      for (int b = 0; b < nb; ++b) {
-        if ((b & (cstep - 1)) == c0) {
-          rf_unit(f, P, M, d, t, h, b);
-          rf_hand_over(f, &ctl->chunk_ready[b]);
-        } else if (b == 0) {
-          rf_arrive(f, &ctl->chunk_ready[0]);       // (every warp arrives once per conv: nobody can miss a phase)
-        }
+      for (int b = c0; b < nb; b += cstep) {
+        rf_unit(f, P, M, d, t, h, b, dr, dp);
+        rf_hand_over(f, &ctl->chunk_ready[b], f.edge);
       }
     } else {
+      rf_wait(f, dr, dp);
+      ptx::tc_fence_after();
       rf_out<kInv>(f, P, a, M, d, v, b0);
       ptx::tc_fence_before();
       asm volatile("bar.sync 1, %0;" ::"n"(kRfWorkers) : "memory");      // the next network input reads what was updated
@@ -542,20 +544,31 @@ __global__ void __launch_bounds__(kRfThreads, 1) res_flow_kernel(const LevelArgs
   f.by = f.rank / P.nbx; f.bx = f.rank - f.by * P.nbx;
   const int b0 = (int)(blockIdx.x / nblk) * P.group;
   f.nimg = min(P.group, a.batch - b0);
+  // neighbours, and how many of their warps write edge positions here: a warp's unit is two rows of a tile's
+  // eight columns
   f.nn = 0;
   f.nb_rank = 0;
-  for (int dy = -1; dy <= 1; ++dy)
-    for (int dx = -1; dx <= 1; ++dx)
-      if ((dy || dx) && (uint32_t)(f.by + dy) < (uint32_t)P.nby && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx) {
-        if (f.nn == lane) f.nb_rank = (uint32_t)((f.by + dy) * P.nbx + f.bx + dx);
-        ++f.nn;
-      }
+  f.edge = false;
+  uint32_t edges = 0;
+  {
+    const int hs = P.m >> 7, per = P.tiles << hs, me = (warp >> 2) & (per - 1);
+    const int t = me >> hs, g = ((warp & 3) << (1 + hs)) + 2 * (me & hs);
+    for (int dy = -1; dy <= 1; ++dy)
+      for (int dx = -1; dx <= 1; ++dx)
+        if ((dy || dx) && (uint32_t)(f.by + dy) < (uint32_t)P.nby && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx) {
+          if (f.nn == lane) {
+            f.nb_rank = (uint32_t)((f.by + dy) * P.nbx + f.bx + dx);
+            f.edge = (dy == 0 || (dy < 0 ? g == 0 : g + 2 == P.bh)) && (dx == 0 || (dx < 0 ? t == 0 : t + 1 == P.tiles));
+          }
+          ++f.nn;
+          edges += (uint32_t)((dy ? 1 : P.bh / 2) * (dx ? 1 : P.tiles));
+        }
+  }
   if (tid == 0) {
-    const uint32_t arrivals = (uint32_t)(kRfWarps * (1 + f.nn));
-    // (chunk 0 takes every warp's arrival, the others those of the warps that work on them)
-    for (int c = 0; c < kRfChunks; ++c)
-      ptx::mbar_init(ptx::smem_u32(&ctl.chunk_ready[c]), c ? arrivals * (uint32_t)(P.tiles * (P.m >> 6)) / 4u : arrivals);
-    ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), arrivals);
+    // (chunk 0 takes every warp's arrival here, the others those of the warps that work on them)
+    const uint32_t part = (uint32_t)(4 * (P.tiles * (P.m >> 6)));
+    for (int c = 0; c < kRfChunks; ++c) ptx::mbar_init(ptx::smem_u32(&ctl.chunk_ready[c]), (c ? part : (uint32_t)kRfWarps) + edges);
+    ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), (uint32_t)(kRfWarps * (1 + f.nn)));
     for (int s = 0; s < 2; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.d_ready[s]), 1);
     for (int s = 0; s < 3; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.meta_full[s]), 1);
     for (int s = 0; s < kRfMaxSlots; ++s) {
