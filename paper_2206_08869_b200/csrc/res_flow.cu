@@ -16,9 +16,9 @@
 //   * Biases are a tenth operand row group: one more K step against a constant operand (1, c, ..., c).
 //     Hidden outputs are then one fma.rn.sat each (FloatRq), the branch of a block one high multiply-add
 //     and shift, its shortcut one multiply on the byte as a subnormal.
-//   * Larger images are cut into 16-row blocks of 16 or 8 columns, one CTA of a cluster each. Edge
-//     positions are stored into the neighbours' frames, and their chunk barriers take the neighbours'
-//     arrivals: no cluster barrier between convs. 16 x 16 images use two CTAs while that fits the machine.
+//   * Larger images are cut into 16 x 16 blocks, one CTA of a cluster each. Edge positions are also stored
+//     into the neighbours' frames, asynchronously: the neighbours' chunk barriers count the bytes, and there is no
+//     cluster barrier between convs.
 //   * One warp issues the MMAs (a chunk's nine taps per wait: waits and commits cost its lane 150 clocks
 //     each, an MMA 40), one lane of another streams weights and the convs' meta blocks.
 #include "res_flow.h"
@@ -29,7 +29,8 @@ namespace iodf {
 namespace {
 
 struct __align__(16) RfCtl {
-  uint64_t chunk_ready[kRfChunks];  // workers (and the neighbours' workers) -> MMA warp: 32 channels of a conv's output
+  uint64_t chunk_ready[2][kRfChunks];  // workers (and the neighbours' edge bytes) -> MMA warp: 32 channels of the output of
+                                       // an even / odd conv (a neighbour may be one conv ahead)
   uint64_t xa_ready;                // the same for the network input
   uint64_t d_ready[2];              // tensor core -> workers: conv's accumulators complete
   uint64_t w_full[kRfMaxSlots], w_empty[kRfMaxSlots];
@@ -45,9 +46,7 @@ struct Rf {
   int tid, warp, lane;
   int nimg;
   int rank, by, bx;                 // CTA of the cluster, its block
-  int nn;                           // neighbours: lane k < nn of every warp owns one
-  uint32_t nb_rank;                 // that neighbour's rank
-  bool edge;                        // worker's lane k: its warp's unit of a tile touches that neighbour's edge
+  uint32_t halo;                    // positions of this CTA's frame that neighbours write (0: no neighbours)
 };
 
 __device__ __noinline__ void rf_wait_slow(uint32_t bar, uint32_t parity, RfCtl* ctl, uint32_t* status) {
@@ -77,44 +76,30 @@ __device__ __forceinline__ uint32_t rf_peer(uint32_t saddr, uint32_t rank) {
 __device__ __forceinline__ void rf_arrive_local(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ptx::smem_u32(bar)) : "memory");
 }
-// this warp's part of an activation is written: here and, for edge positions, at the neighbours. `remote`: this
-// lane's neighbour has been written to (a release at cluster scope costs a trip to the other SM, so that
-// warps without edge positions only arrive here).
-__device__ __forceinline__ void rf_hand_over(const Rf& f, uint64_t* bar, bool remote) {
+// this warp's part of an activation is written; `bytes`: what the neighbours' asynchronous stores will add to the
+// phase (announced by one warp; others pass 0)
+__device__ __forceinline__ void rf_hand_over(const Rf& f, uint64_t* bar, uint32_t bytes) {
   ptx::tc_fence_before();
-  if (f.nn && __any_sync(0xFFFFFFFFu, remote)) {
-    asm volatile("fence.proxy.async;" ::: "memory");
-    __syncwarp();
-    if (remote)
-      asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(rf_peer(ptx::smem_u32(bar), f.nb_rank)) : "memory");
-  } else {
-    ptx::fence_async_smem();
-    __syncwarp();
+  ptx::fence_async_smem();
+  __syncwarp();
+  if (f.lane == 0) {
+    if (bytes) ptx::mbar_expect_tx(ptx::smem_u32(bar), bytes);
+    else rf_arrive_local(bar);
   }
-  if (f.lane == 31) rf_arrive_local(bar);
 }
-// the MMA warp's wait for such a hand-over: acquires at cluster scope when neighbours write here
+// store of an edge position into a neighbour's frame: its barrier counts the bytes when they have landed, so the
+// writer needs no fence and no arrival of its own (a release at cluster scope per chunk and warp stalled the
+// edge warps: 0.84 -> 0.69 ms for the 32 x 32 level of config R64)
+__device__ __forceinline__ void rf_store_async8(uint32_t addr, uint32_t bar, const uint2 v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void rf_store_async4(uint32_t addr, uint32_t bar, const uint32_t v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
+}
+// the MMA warp's wait for an operand; the neighbours' bytes came through the generic proxy
 __device__ __forceinline__ void rf_wait_operand(const Rf& f, uint64_t* bar, uint32_t parity) {
-  if (f.nn == 0) {
-    rf_wait(f, bar, parity);
-  } else {
-    const uint32_t b = ptx::smem_u32(bar);
-    for (uint32_t it = 0; it < kSpinLimit; ++it) {
-      uint32_t ok;
-      asm volatile(
-          "{\n\t.reg .pred p;\n\t"
-          "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-          "selp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(ok) : "r"(b), "r"(parity), "r"(100000u) : "memory");
-      if (ok) break;
-      if (*reinterpret_cast<volatile uint32_t*>(&f.ctl->abort)) break;
-      if (it + 1 == kSpinLimit) {
-        *reinterpret_cast<volatile uint32_t*>(&f.ctl->abort) = 1;
-        atomicExch(f.status, 1u);
-      }
-    }
-    asm volatile("fence.proxy.async;" ::: "memory");
-  }
+  rf_wait(f, bar, parity);
+  if (f.halo) asm volatile("fence.proxy.async;" ::: "memory");
   ptx::tc_fence_after();
 }
 
@@ -173,7 +158,7 @@ __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq) {
   // (in a cluster a shared-memory address also carries the CTA's rank above the descriptor's 14 bits)
   auto addr16 = [&](uint32_t s) { return (ptx::smem_u32(smem + s) >> 4) & 0x3FFFu; };
   const uint32_t a_hi = (uint32_t)P.wp | (1u << 14), plane = (uint32_t)P.plane16;
-  uint32_t slot = 0, round = 0, ready = 0, xa_par = 0;     // ready: bit c: parity of chunk barrier c
+  uint32_t slot = 0, round = 0, ready = 0, xa_par = 0;     // ready: bit 4 s + c: parity of chunk barrier [s][c]
   int ms = 0;
   uint32_t mpar = 0;
 #pragma unroll 1
@@ -193,8 +178,9 @@ __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq) {
       if (input) {
         if (kc == 0) { rf_wait_operand(f, &ctl->xa_ready, xa_par); xa_par ^= 1u; }
       } else {
-        rf_wait_operand(f, &ctl->chunk_ready[kc], (ready >> kc) & 1u);
-        ready ^= 1u << kc;
+        const int set = (q - 1) & 1;
+        rf_wait_operand(f, &ctl->chunk_ready[set][kc], (ready >> (4 * set + kc)) & 1u);
+        ready ^= 1u << (4 * set + kc);
       }
       uint32_t bl = addr16(P.s_ring + slot * P.slot_bytes) | b_lbo;
       const uint32_t a_bias = addr16(P.s_const + (uns ? 0u : 2304u)) | (8u << 16);
@@ -245,42 +231,29 @@ struct RfPos {             // a thread's two positions of a tile half (rows of t
 
 __device__ __forceinline__ uint32_t rf_pack_u8(int y0, int y1, int y2, int y3) { return pack4_sat_u8(y0, y1, y2, y3); }
 
-// 8 bytes of an activation at position pos of this CTA's frame (plane address `d` included), and in the
-// neighbours' frames where the pixel (i, j) of the block lies on an edge
-__device__ __forceinline__ void rf_store8(const Rf& f, const RfPlan& P, uint8_t* d, const uint2 v, int i, int j) {
-  *reinterpret_cast<uint2*>(d) = v;
-  if (f.nn) {
-    const uint32_t s = ptx::smem_u32(d);
+// 8 (4) bytes of an activation in this CTA's frame and, where the pixel (i, j) of the block lies on an edge, in
+// the neighbours' frames
+template <typename V>
+__device__ __forceinline__ void rf_store(const Rf& f, const RfPlan& P, uint8_t* d, const V v, int i, int j, uint64_t* bar) {
+  *reinterpret_cast<V*>(d) = v;
+  if (f.halo) {
     const int dy = i == 0 ? -1 : (i == P.bh - 1 ? 1 : 0), dx = j == 0 ? -1 : (j == P.bw - 1 ? 1 : 0);
     const bool ny = dy && (uint32_t)(f.by + dy) < (uint32_t)P.nby, nx = dx && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx;
-    const int sy = dy * P.bh * P.wp * 16, sx = dx * P.bw * 16, r = f.rank + dy * P.nbx;
-    auto put = [&](uint32_t at, int rank) {
-      asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(rf_peer(at, (uint32_t)rank)), "r"(v.x), "r"(v.y) : "memory");
+    const uint32_t s = ptx::smem_u32(d), b = ptx::smem_u32(bar);
+    auto put = [&](int oy, int ox) {
+      const uint32_t rank = (uint32_t)(f.rank + oy * P.nbx + ox), at = rf_peer(s - (uint32_t)((oy * P.bh * P.wp + ox * P.bw) * 16), rank);
+      if constexpr (sizeof(V) == 8) rf_store_async8(at, rf_peer(b, rank), v);
+      else rf_store_async4(at, rf_peer(b, rank), v);
     };
-    if (ny) put(s - (uint32_t)sy, r);
-    if (nx) put(s - (uint32_t)sx, f.rank + dx);
-    if (ny && nx) put(s - (uint32_t)(sy + sx), r + dx);
-  }
-}
-__device__ __forceinline__ void rf_store4(const Rf& f, const RfPlan& P, uint8_t* d, const uint32_t v, int i, int j) {
-  *reinterpret_cast<uint32_t*>(d) = v;
-  if (f.nn) {
-    const uint32_t s = ptx::smem_u32(d);
-    const int dy = i == 0 ? -1 : (i == P.bh - 1 ? 1 : 0), dx = j == 0 ? -1 : (j == P.bw - 1 ? 1 : 0);
-    const bool ny = dy && (uint32_t)(f.by + dy) < (uint32_t)P.nby, nx = dx && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx;
-    const int sy = dy * P.bh * P.wp * 16, sx = dx * P.bw * 16, r = f.rank + dy * P.nbx;
-    auto put = [&](uint32_t at, int rank) {
-      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(rf_peer(at, (uint32_t)rank)), "r"(v) : "memory");
-    };
-    if (ny) put(s - (uint32_t)sy, r);
-    if (nx) put(s - (uint32_t)sx, f.rank + dx);
-    if (ny && nx) put(s - (uint32_t)(sy + sx), r + dx);
+    if (ny) put(dy, 0);
+    if (nx) put(0, dx);
+    if (ny && nx) put(dy, dx);
   }
 }
 
 // One unit: 16 rows (half `h` of this warp's lane quarter of tile `t`) x 32 columns (chunk b) of a hidden or branch conv.
 __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMeta* __restrict__ M, uint32_t d, int t, int h, int b,
-                                        uint64_t* ready, uint32_t parity) {
+                                        uint64_t* ready, uint32_t parity, uint64_t* chunk) {
   const int q = f.lane & 3, x = f.lane >> 2, hs = P.m >> 7;
   // (what does not depend on the accumulator comes before the wait for it)
   uint32_t r[16];
@@ -343,8 +316,8 @@ __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMe
   // ReLU and clip to 0..255 are the pack's saturation
   const uint2 v0 = make_uint2(rf_pack_u8((int)r[0], (int)r[1], (int)r[4], (int)r[5]), rf_pack_u8((int)r[8], (int)r[9], (int)r[12], (int)r[13]));
   const uint2 v1 = make_uint2(rf_pack_u8((int)r[2], (int)r[3], (int)r[6], (int)r[7]), rf_pack_u8((int)r[10], (int)r[11], (int)r[14], (int)r[15]));
-  if (ok0) rf_store8(f, P, o, v0, g, j);
-  if (ok1) rf_store8(f, P, o + row, v1, g + 1, j);
+  if (ok0) rf_store(f, P, o, v0, g, j, chunk);
+  if (ok1) rf_store(f, P, o + row, v1, g + 1, j, chunk);
 }
 
 // thread's two pixels (of the CTA) for operand rows g, g + 1 of tile t; -1: none
@@ -417,7 +390,7 @@ __device__ __forceinline__ void rf_requant(const Rf& f, const RfPlan& P, const R
     }
     const int row = P.small ? (p >> 4) * 5 + ((p >> 2) & 3) : p / P.bw, j = P.small ? p & 3 : p - row * P.bw;
     uint8_t* d = f.smem + P.s_buf[M->src] + ((wd >> 2) * P.plane16 + (row + 1) * P.wp + 1 + j) * 16 + (wd & 3) * 4;
-    rf_store4(f, P, d, pack4_sat(y[0], y[1], y[2], y[3]), row, j);
+    rf_store(f, P, d, pack4_sat(y[0], y[1], y[2], y[3]), row, j, &f.ctl->xa_ready);
   }
 }
 
@@ -439,7 +412,7 @@ __device__ void rf_workers(const Rf& f, const RfPlan& P, const LevelArgs& a, con
     if (++ms == 3) { ms = 0; mpar ^= 1u; }
     if (M->input) {
       rf_requant(f, P, M, v);
-      rf_hand_over(f, &ctl->xa_ready, f.lane < f.nn);
+      rf_hand_over(f, &ctl->xa_ready, f.warp == 0 ? f.halo * 4u * (uint32_t)((P.ca + 3) >> 2) : 0u);
     }
     const uint32_t d = f.tmem + (uint32_t)((q & 1) * P.tiles * 128);
     const int nb = M->nb, kind = M->kind;
@@ -449,12 +422,13 @@ __device__ void rf_workers(const Rf& f, const RfPlan& P, const LevelArgs& a, con
       if (c0 != 0) {                       // every warp arrives once per conv: nobody can miss a phase
         rf_wait(f, dr, dp);
         __syncwarp();
-        if (f.lane == 31) rf_arrive_local(&ctl->chunk_ready[0]);
+        if (f.lane == 0) rf_arrive_local(&ctl->chunk_ready[q & 1][0]);
       }
 #pragma unroll 1
       for (int b = c0; b < nb; b += cstep) {
-        rf_unit(f, P, M, d, t, h, b, dr, dp);
-        rf_hand_over(f, &ctl->chunk_ready[b], f.edge);
+        uint64_t* cr = &ctl->chunk_ready[q & 1][b];
+        rf_unit(f, P, M, d, t, h, b, dr, dp, cr);
+        rf_hand_over(f, cr, me == 0 && (f.warp & 3) == 0 ? f.halo * 32u : 0u);
       }
     } else {
       rf_wait(f, dr, dp);
@@ -544,31 +518,16 @@ __global__ void __launch_bounds__(kRfThreads, 1) res_flow_kernel(const LevelArgs
   f.by = f.rank / P.nbx; f.bx = f.rank - f.by * P.nbx;
   const int b0 = (int)(blockIdx.x / nblk) * P.group;
   f.nimg = min(P.group, a.batch - b0);
-  // neighbours, and how many of their warps write edge positions here: a warp's unit is two rows of a tile's
-  // eight columns
-  f.nn = 0;
-  f.nb_rank = 0;
-  f.edge = false;
-  uint32_t edges = 0;
-  {
-    const int hs = P.m >> 7, per = P.tiles << hs, me = (warp >> 2) & (per - 1);
-    const int t = me >> hs, g = ((warp & 3) << (1 + hs)) + 2 * (me & hs);
-    for (int dy = -1; dy <= 1; ++dy)
-      for (int dx = -1; dx <= 1; ++dx)
-        if ((dy || dx) && (uint32_t)(f.by + dy) < (uint32_t)P.nby && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx) {
-          if (f.nn == lane) {
-            f.nb_rank = (uint32_t)((f.by + dy) * P.nbx + f.bx + dx);
-            f.edge = (dy == 0 || (dy < 0 ? g == 0 : g + 2 == P.bh)) && (dx == 0 || (dx < 0 ? t == 0 : t + 1 == P.tiles));
-          }
-          ++f.nn;
-          edges += (uint32_t)((dy ? 1 : P.bh / 2) * (dx ? 1 : P.tiles));
-        }
-  }
+  f.halo = 0;
+  for (int dy = -1; dy <= 1; ++dy)
+    for (int dx = -1; dx <= 1; ++dx)
+      if ((dy || dx) && (uint32_t)(f.by + dy) < (uint32_t)P.nby && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx)
+        f.halo += (uint32_t)((dy ? 1 : P.bh) * (dx ? 1 : P.bw));
   if (tid == 0) {
-    // (chunk 0 takes every warp's arrival here, the others those of the warps that work on them)
-    const uint32_t part = (uint32_t)(4 * (P.tiles * (P.m >> 6)));
-    for (int c = 0; c < kRfChunks; ++c) ptx::mbar_init(ptx::smem_u32(&ctl.chunk_ready[c]), (c ? part : (uint32_t)kRfWarps) + edges);
-    ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), (uint32_t)(kRfWarps * (1 + f.nn)));
+    // (chunk 0 takes every warp's arrival, the others those of the warps that work on them)
+    for (int c = 0; c < 2 * kRfChunks; ++c)
+      ptx::mbar_init(ptx::smem_u32(&ctl.chunk_ready[c >> 2][c & 3]), (c & 3) ? (uint32_t)(4 * (P.tiles * (P.m >> 6))) : (uint32_t)kRfWarps);
+    ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), (uint32_t)kRfWarps);
     for (int s = 0; s < 2; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.d_ready[s]), 1);
     for (int s = 0; s < 3; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.meta_full[s]), 1);
     for (int s = 0; s < kRfMaxSlots; ++s) {
@@ -636,6 +595,27 @@ cudaError_t launch_res_flow(const LevelArgs& args, const RfPlan& plan, bool inve
   cfg.attrs = attr;
   cfg.numAttrs = plan.nbx * plan.nby > 1 ? 2 : 1;
   return inverse ? cudaLaunchKernelEx(&cfg, res_flow_kernel<true>, args, plan) : cudaLaunchKernelEx(&cfg, res_flow_kernel<false>, args, plan);
+}
+
+int max_res_flow_clusters(int ctas, uint32_t smem_bytes) {
+  if (configure_res_flow_kernels(smem_bytes) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3((unsigned)kRfThreads);
+  cfg.dynamicSmemBytes = smem_bytes;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, res_flow_kernel<false>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
 }
 
 cudaError_t configure_res_flow_kernels(uint32_t max_smem_bytes) {

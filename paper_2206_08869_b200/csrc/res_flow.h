@@ -63,6 +63,8 @@ struct RfPlan {
 static_assert(sizeof(RfPlan) < 1024, "travels as a kernel parameter");
 
 cudaError_t configure_res_flow_kernels(uint32_t max_smem_bytes);
+// clusters of `ctas` CTAs that can be resident at once (0 if that cannot be determined)
+int max_res_flow_clusters(int ctas, uint32_t smem_bytes);
 cudaError_t launch_res_flow(const LevelArgs& args, const RfPlan& plan, bool inverse, int ctas, cudaStream_t stream);
 
 }  // namespace iodf
