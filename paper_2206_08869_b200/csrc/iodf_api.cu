@@ -69,6 +69,8 @@ struct iodf_codec {
   uint8_t* d_tables = nullptr;      // R then G
   uint32_t* d_errors = nullptr;
   uint32_t* d_sizes = nullptr;      // max_batch record sizes (packing scratch)
+  uint32_t* d_ranges = nullptr;     // symbol ranges of the decoder's first look-up
+  uint32_t* h_payload = nullptr;    // pinned: payload size of the batch that is being compressed
   // staging of the host-buffer entry points, allocated by their first call
   uint16_t* d_words = nullptr;
   uint32_t* d_counts = nullptr;
@@ -1928,6 +1930,40 @@ int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_cod
   a.R = reinterpret_cast<const uint32_t*>(c->d_tables);
   a.G = reinterpret_cast<const uint16_t*>(c->d_tables + rbytes);
   a.errors = c->d_errors;
+  // Decoder's first look-up: the symbols k whose range [Cum(k), Cum(k + 1)) meets slots 256 b .. 256 b + 255, as {first,
+  // count << 16}, for every scale index: at most 257 of the 4 097 (a symbol has at least one slot).
+  {
+    std::vector<uint32_t> ranges((size_t)desc->n_scales * 256);
+    std::vector<uint32_t> cum(2 * 2048 + 2);
+    for (uint32_t ls = 0; ls < desc->n_scales; ++ls) {
+      cum[0] = 0;
+      for (int k = 1; k <= 2 * 2048; ++k) {
+        int64_t u = ((int64_t)(2 * (k - 2048) - 1) * (int64_t)desc->inv_scale[ls]) >> 16;       // floor
+        u = std::max<int64_t>(-(int64_t)desc->umax, std::min<int64_t>((int64_t)desc->umax, u));
+        cum[k] = (uint32_t)k + desc->sigmoid_table[u + desc->umax];
+      }
+      cum[2 * 2048 + 1] = 1u << 16;
+      int k = 0;
+      for (uint32_t b = 0; b < 256; ++b) {
+        while (k < 2 * 2048 && cum[k + 1] <= 256 * b) ++k;
+        int e = k;
+        while (e < 2 * 2048 && cum[e + 1] <= 256 * b + 255) ++e;
+        ranges[(size_t)ls * 256 + b] = (uint32_t)k | ((uint32_t)(e - k + 1) << 16);
+      }
+    }
+    e = cudaGetDevice(&prev);
+    if (e == cudaSuccess) e = cudaSetDevice(c->device);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_ranges, 4 * ranges.size());
+    if (e == cudaSuccess) e = cudaMemcpy(c->d_ranges, ranges.data(), 4 * ranges.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaHostAlloc(&c->h_payload, sizeof(uint32_t), cudaHostAllocDefault);
+    cudaSetDevice(prev);
+    if (e != cudaSuccess) {
+      const int rc = e == cudaErrorMemoryAllocation ? IODF_ENOMEM : IODF_ECUDA;
+      iodf_codec_destroy(c);
+      return rc;
+    }
+    a.ranges = c->d_ranges;
+  }
   *out = c;
   return IODF_OK;
 }
@@ -1938,6 +1974,8 @@ void iodf_codec_destroy(iodf_codec* c) {
   if (c->d_tables) cudaFree(c->d_tables);
   if (c->d_errors) cudaFree(c->d_errors);
   if (c->d_sizes) cudaFree(c->d_sizes);
+  if (c->d_ranges) cudaFree(c->d_ranges);
+  if (c->h_payload) cudaFreeHost(c->h_payload);
   if (c->d_words) cudaFree(c->d_words);
   if (c->d_counts) cudaFree(c->d_counts);
   if (c->d_packed) cudaFree(c->d_packed);
@@ -2041,10 +2079,9 @@ int iodf_compress_host(iodf_model* m, iodf_codec* c, const uint8_t* x_u8_host, i
   CUC(c, launch_rans_encode(a, m->d_z, prior, c->d_words, c->d_counts, st));
   CUC(c, launch_rans_pack(a, c->d_words, c->d_counts, c->d_sizes, c->d_packed, st));
   // the payload size is only known now: read it, then copy exactly header + payload
-  uint32_t payload = 0;
-  CUC(c, cudaMemcpyAsync(&payload, c->d_packed + 4 * (size_t)B, sizeof(payload), cudaMemcpyDeviceToHost, st));
+  CUC(c, cudaMemcpyAsync(c->h_payload, c->d_packed + 4 * (size_t)B, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   CUC(c, cudaStreamSynchronize(st));
-  const size_t total = 4 * ((size_t)B + 1) + payload;
+  const size_t total = 4 * ((size_t)B + 1) + *c->h_payload;
   *out_bytes = total;
   if (total > out_capacity) return IODF_ELIMIT;
   CUC(c, cudaMemcpyAsync(out_host, c->d_packed, total, cudaMemcpyDeviceToHost, st));

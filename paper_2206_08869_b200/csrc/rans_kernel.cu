@@ -32,16 +32,27 @@ struct Tables {
   int umax, n_scales;
 };
 
-__device__ __forceinline__ uint32_t cum(const Tables& t, int ls, int k) {
+__device__ __forceinline__ uint32_t cum_of(const Tables& t, uint32_t R, int k) {
   if (k <= 0) return 0u;
   if (k >= 2 * kWin + 1) return kM;
   // floor(edge2 * R / 2^16) in 32-bit pieces: with R = Rh 2^16 + Rl it is edge2 * Rh + floor(edge2 * Rl /
   // 2^16) exactly (|edge2| < 2^13, Rl < 2^16, Rh < 2^15 for the scales a codec accepts)
   const int edge2 = 2 * (k - kWin) - 1;
-  const uint32_t R = t.R[ls];
   int u = edge2 * (int)(R >> 16) + ((edge2 * (int)(R & 0xFFFFu)) >> 16);      // arithmetic shift: floor
   u = max(-t.umax, min(t.umax, u));
   return (uint32_t)k + t.G[u + t.umax];
+}
+
+// x / F and x mod F for 0 < F <= 2^16 and x < F 2^16: the quotient is below 2^16, so that x times the float reciprocal of F
+// is off by less than one before truncation (three roundings of 2^-24 on a value below 2^16), and two
+// conditional corrections make it exact. A 32-bit division is several times as long, and it sits on the chain.
+__device__ __forceinline__ uint32_t divide(uint32_t x, uint32_t F, uint32_t* rem) {
+  uint32_t q = __float2uint_rz(__uint2float_rz(x) * __frcp_rn(__uint2float_rn(F)));
+  uint32_t r = x - q * F;
+  if ((int32_t)r < 0) { --q; r += F; }
+  if (r >= F) { ++q; r -= F; }
+  *rem = r;
+  return q;
 }
 
 __device__ __forceinline__ void load_tables(const RansArgs& a, uint16_t* sG, uint32_t* sR) {
@@ -86,22 +97,47 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_encode_kernel(const Ran
       out[pos++] = (uint16_t)(x & 0xFFFFu);
       x >>= 16;
     }
-    x = ((x / F) << 16) + (x % F) + C;
+    uint32_t r;
+    const uint32_t q = divide(x, F, &r);
+    x = (q << 16) + r + C;
   };
-  for (long i = n_el - 1; i >= 0; --i) {
+  // Elements and prior parameters of the next kAhead symbols are on their way while the current ones are coded:
+  // their addresses do not depend on the state, and a trip to memory is longer than several symbols.
+  constexpr int kAhead = 4;
+  int32_t zn[kAhead], mun[kAhead];
+  int lsn[kAhead];
+  auto fetch = [&](int s, long i) {
+    zn[s] = 0; mun[s] = 0; lsn[s] = a.final_ls;
+    if (i < 0) return;
     const long e = j + i * ns;
-    const int32_t zv = zb[e];
-    int32_t mu; int ls;
-    prior_of(a, blk, pb, e, &mu, &ls, &bad);
-    long long r = (long long)zv - (long long)mu;
-    r = r < -kWin ? -kWin : (r > kWin ? kWin : r);
-    const int k = (int)r + kWin;
-    if (k == 0 || k == 2 * kWin) {
-      push(1u, (uint32_t)zv & 0xFFFFu);
-      push(1u, ((uint32_t)zv >> 16) & 0xFFFFu);
+    zn[s] = zb[e];
+    if (blk.prior_off >= 0) {
+      mun[s] = pb[blk.prior_off + e];
+      lsn[s] = pb[a.d_fact + blk.prior_off + e];
     }
-    const uint32_t C = cum(t, ls, k), F = cum(t, ls, k + 1) - C;
-    push(F, C);
+  };
+#pragma unroll
+  for (int s = 0; s < kAhead; ++s) fetch(s, n_el - 1 - s);
+  for (long i0 = n_el - 1; i0 >= 0; i0 -= kAhead) {
+#pragma unroll
+    for (int s = 0; s < kAhead; ++s) {
+      const long i = i0 - s;
+      if (i < 0) break;
+      const int32_t zv = zn[s], mu = mun[s];
+      int ls = lsn[s];
+      fetch(s, i - kAhead);
+      if (ls < 0 || ls >= a.n_scales) { bad = 1u; ls = ls < 0 ? 0 : a.n_scales - 1; }
+      long long r = (long long)zv - (long long)mu;
+      r = r < -kWin ? -kWin : (r > kWin ? kWin : r);
+      const int k = (int)r + kWin;
+      if (k == 0 || k == 2 * kWin) {
+        push(1u, (uint32_t)zv & 0xFFFFu);
+        push(1u, ((uint32_t)zv >> 16) & 0xFFFFu);
+      }
+      const uint32_t R = t.R[ls];
+      const uint32_t C = cum_of(t, R, k), F = cum_of(t, R, k + 1) - C;
+      push(F, C);
+    }
   }
   out[pos++] = (uint16_t)(x & 0xFFFFu);
   out[pos++] = (uint16_t)(x >> 16);
@@ -112,9 +148,11 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_encode_kernel(const Ran
 // Decode: one WARP per stream. The state, the word pointer and every step are the same in all 32
 // lanes; what the lanes share out is everything that would otherwise be a dependent trip to memory
 // or a dependent search step on the stream's serial chain (state -> symbol -> state):
-//   * the symbol search: instead of 13 bisection steps, three rounds in which lane L tests one
-//     candidate k each (steps of 129, 5 and 1) and a ballot picks the largest k with Cum(k) <= slot;
-//     the last round's values also give C = Cum(k) and Cum(k + 1) by shuffle;
+//   * the symbol search: the slot's upper eight bits select, for the element's scale, the symbols that it can
+//     mean (a table made with the codec: first and count, usually a handful, 257 at most); lane L tests one
+//     candidate and a ballot picks the largest k with Cum(k) <= slot, after a round in steps of up to nine where there
+//     are more than 32. The last round's values also give C = Cum(k) and Cum(k + 1) by shuffle. (Three rounds
+//     over all 4 097 symbols before.)
 //   * the prior parameters: the (mu, scale index) of the next 32 elements are loaded by the 32 lanes
 //     in one go and handed out by shuffle, so no global-memory latency sits between two symbols;
 //   * the coded words: the lanes hold a window of the stream's next 32 words (the decoder reads the
@@ -163,24 +201,27 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const Ran
     int32_t mu_l = 0, zv_l = 0;
     int ls_l = a.final_ls;
     if (i0 + lane < n_el) prior_of(a, blk, pb, j + (i0 + lane) * ns, &mu_l, &ls_l, &bad);
+    const uint32_t R_l = t.R[ls_l];
     const int n_here = (int)min(32l, n_el - i0);
     for (int ii = 0; ii < n_here; ++ii) {
       const int32_t mu = __shfl_sync(0xFFFFFFFFu, mu_l, ii);
       const int ls = __shfl_sync(0xFFFFFFFFu, ls_l, ii);
+      const uint32_t R = __shfl_sync(0xFFFFFFFFu, R_l, ii);
       const uint32_t slot = x & 0xFFFFu;
-      // largest k in [0, 4096] with Cum(k) <= slot (Cum(0) = 0 <= slot always; Cum(k > 4096) = M > slot)
-      int k = 0;
-#pragma unroll
-      for (int round = 0; round < 2; ++round) {
-        const int step = round == 0 ? 129 : 5;
-        const unsigned ok = __ballot_sync(0xFFFFFFFFu, cum(t, ls, k + lane * step) <= slot);   // a prefix of the lanes (Cum is monotone)
+      // largest k with Cum(k) <= slot, among the symbols that the slot can mean
+      const uint32_t range = __ldg(a.ranges + (ls << 8) + (slot >> 8));
+      int k = (int)(range & 0xFFFFu);
+      const int count = (int)(range >> 16);
+      if (count > 32) {
+        const int step = (count + 31) >> 5;
+        const unsigned ok = __ballot_sync(0xFFFFFFFFu, cum_of(t, R, k + lane * step) <= slot);   // a prefix of the lanes (Cum is monotone)
         k += (31 - __clz((int)ok)) * step;
       }
-      const uint32_t cl = cum(t, ls, k + lane);
+      const uint32_t cl = cum_of(t, R, k + lane);
       const int sel = 31 - __clz((int)__ballot_sync(0xFFFFFFFFu, cl <= slot));
       k += sel;
       const uint32_t C = __shfl_sync(0xFFFFFFFFu, cl, sel);
-      const uint32_t Cn = sel < 31 ? __shfl_sync(0xFFFFFFFFu, cl, sel + 1) : cum(t, ls, k + 1);
+      const uint32_t Cn = sel < 31 ? __shfl_sync(0xFFFFFFFFu, cl, sel + 1) : cum_of(t, R, k + 1);
       const uint32_t F = Cn - C;
       x = F * (x >> 16) + slot - C;
       if (x < (1u << 16)) x = (x << 16) | next();
