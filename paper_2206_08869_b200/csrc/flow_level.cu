@@ -33,7 +33,7 @@ struct __align__(16) FlowCtl {
   uint64_t a_ready[2];    // slot's workers -> its MMA warp: the next hidden operand is written
   uint64_t dm_ready[2];   // tensor core -> workers: first / second GEMM of the slot's tile complete
   uint64_t d3_ready[2];   // tensor core -> workers: per-tap partials of the slot's tile complete
-  uint64_t w_full[3], w_empty[3];   // weight slots: copy landed / last MMAs (of each tile slot) that read it complete
+  uint64_t w_full[kFlowMaxRing], w_empty[kFlowMaxRing];   // weight slots: copy landed / last MMAs (of each tile slot) that read it complete
   uint64_t meta_full[2];
   uint32_t tmem_base;
   uint32_t abort;
@@ -123,6 +123,39 @@ __device__ void flow_loader(const Flow& f, const FlowPlan& P, const LevelArgs& a
       flow_wait(f, &ctl->xa_ready, (uint32_t)(i + 1) & 1u);
       meta(i + 2);
     }
+  }
+}
+
+// Streamed weights (P.ring): for every tile the K steps of its GEMMs, in order, through the ring
+__device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st) {
+  FlowCtl* ctl = f.ctl;
+  uint32_t slot = 0, round = 0;
+#pragma unroll 1
+  for (int i = 0; i < st.nsteps; ++i) {
+    const BlockRef& br = step_ref(*a.plan, st, i);
+    // meta slot of step i: its last reader was the pixel pass of step i - 1
+    if (i >= 2) flow_wait(f, &ctl->xa_ready, (uint32_t)(i - 1) & 1u);
+    {
+      const uint32_t b = ptx::smem_u32(&ctl->meta_full[i & 1]);
+      ptx::mbar_expect_tx(b, br.meta_bytes);
+      ptx::bulk_g2s(ptx::smem_u32(f.smem + P.s_meta[i & 1]), a.blob + br.meta_off, br.meta_bytes, b);
+    }
+    const int gemms = st.is_prior(i) ? 1 : 3;
+#pragma unroll 1
+    for (int t = 0; t < f.tiles; ++t)
+#pragma unroll 1
+      for (int g = 0; g < gemms; ++g) {
+        const uint32_t ks = br.k_slices[g], bytes = br.w_bytes[g] / ks;
+        const uint8_t* src = a.blob + br.w_off[g];
+#pragma unroll 1
+        for (uint32_t k = 0; k < ks; ++k, src += bytes) {
+          if (round > 0) flow_wait(f, &ctl->w_empty[slot], (round - 1u) & 1u);
+          const uint32_t b = ptx::smem_u32(&ctl->w_full[slot]);
+          ptx::mbar_expect_tx(b, bytes);
+          ptx::bulk_g2s(ptx::smem_u32(f.smem + P.s_w[0] + slot * P.ring_slot_bytes), src, bytes, b);
+          if (++slot == (uint32_t)P.ring) { slot = 0; ++round; }
+        }
+      }
   }
 }
 
@@ -223,6 +256,69 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
   }
 }
 
+// MMA warp of levels with streamed weights: one tile at a time, all accumulators from column 0 on
+__device__ void flow_mma_ring(const Flow& f, const FlowPlan& P, const Steps& st) {
+  FlowCtl* ctl = f.ctl;
+  uint8_t* smem = f.smem;
+  auto uniform = [](int x) { return __shfl_sync(0xFFFFFFFFu, x, 0); };
+  const uint32_t idesc_m = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.m >> 4) << 24);
+  const uint32_t xa16 = ptx::smem_u32(smem + P.s_xa) >> 4, hi = ptx::kUmmaDescHi;
+  const uint32_t a1_hi = (uint32_t)P.sbo16 | (1u << 14), pitch16 = (uint32_t)P.pitch >> 4;
+  const uint32_t a_lo = ((ptx::smem_u32(smem + P.s_a[0]) >> 4) & 0x3FFFu) | (pitch16 << 16);
+  uint32_t slot = 0, round = 0, apar = 0;
+  // one GEMM: K step s reads A at al(s); N above 256 in two parts
+  auto gemm = [&](uint32_t d, int n, int ks, auto al, uint32_t ahi, uint64_t* done) {
+    const int na = min(n, 256);
+    const uint32_t idesc = idesc_m | ((uint32_t)(na >> 3) << 17), idesc2 = idesc_m | ((uint32_t)((n - na) >> 3) << 17);
+#pragma unroll 1
+    for (int s = 0; s < ks; ++s) {
+      flow_wait(f, &ctl->w_full[slot], round & 1u);
+      ptx::tc_fence_after();
+      const uint32_t bl = ((ptx::smem_u32(smem + P.s_w[0] + slot * P.ring_slot_bytes) >> 4) & 0x3FFFu) | ((uint32_t)n << 16);
+      const uint32_t a = al(s);
+      if (ptx::elect_one()) {
+        ptx::umma_i8_hl(d, a, ahi, bl, hi, idesc, s > 0 ? 1u : 0u);
+        if (n > 256) ptx::umma_i8_hl(d + 256u, a, ahi, bl + 256u, hi, idesc2, s > 0 ? 1u : 0u);
+        ptx::umma_commit(ptx::smem_u32(&ctl->w_empty[slot]));
+        if (s + 1 == ks && done) ptx::umma_commit(ptx::smem_u32(done));
+      }
+      __syncwarp();
+      if (++slot == (uint32_t)P.ring) { slot = 0; ++round; }
+    }
+  };
+  auto wait_a = [&]() {
+    flow_wait(f, &ctl->a_ready[0], apar);
+    apar ^= 1u;
+    ptx::tc_fence_after();
+  };
+  auto hidden = [&](int s) { return a_lo + (uint32_t)s * 2u * pitch16; };
+#pragma unroll 1
+  for (int i = 0; i < st.nsteps; ++i) {
+    const bool prior = st.is_prior(i);
+    flow_wait(f, &ctl->meta_full[i & 1], (uint32_t)(i >> 1) & 1u);
+    const FlowMeta* M = reinterpret_cast<const FlowMeta*>(smem + P.s_meta[i & 1]);
+    const int n1 = prior ? P.n_prior : uniform(M->n1), n2 = uniform(M->n2), n3 = uniform(M->n3);
+    const int ks2 = uniform(M->ks2), ks3 = uniform(M->ks3);
+    flow_wait(f, &ctl->xa_ready, (uint32_t)i & 1u);
+    ptx::tc_fence_after();
+#pragma unroll 1
+    for (int t = 0; t < f.tiles; ++t) {
+      const uint32_t base = xa16 + (uint32_t)uniform(ctl->tile[t].w);
+      auto first = [&](int s) { return base + P.step[s]; };
+      if (prior) {
+        gemm(f.tmem + (uint32_t)(t * P.n_prior), n1, P.ks1, first, a1_hi, t + 1 == f.tiles ? &ctl->dm_ready[0] : nullptr);
+        continue;
+      }
+      if (t > 0) wait_a();                     // the last tile's partials have been summed
+      gemm(f.tmem, n1, P.ks1, first, a1_hi, &ctl->dm_ready[0]);
+      wait_a();
+      gemm(f.tmem, n2, ks2, hidden, hi, &ctl->dm_ready[0]);
+      wait_a();
+      gemm(f.tmem, n3, ks3, hidden, hi, &ctl->d3_ready[0]);
+    }
+  }
+}
+
 // ---- workers ---------------------------------------------------------------------------------------------
 // Integer form (rare: blocks with a channel that has no floating-point constants)
 __device__ __forceinline__ uint32_t flow_integer_one(uint32_t acc, float m, int us) {
@@ -240,7 +336,7 @@ __device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, ui
   // everything that does not depend on the accumulator comes before the wait for it
   const int n = layer ? M->n2 : M->n1, ks = layer ? M->ks3 : M->ks2, nfi = layer ? M->nfi2 : M->nfi1;
   const int nfb = layer ? M->nfb2 : M->nfb1;
-  const int q = f.lane & 3, nfull = n >> 5, plain = min(min(nfb, nfi), nfull);
+  const int q = f.lane & 3, nfull = n >> 5, last = (n - 1) >> 5, plain = min(min(nfb, nfi), nfull);
   const uint8_t* mb = reinterpret_cast<const uint8_t*>(M);
   const float4* ft = reinterpret_cast<const float4*>(mb + (layer ? M->off_f2 : M->off_f1)) + q * 2;
   const float4* ct = reinterpret_cast<const float4*>(mb + (layer ? M->off_c2 : M->off_c1)) + q * 2 - nfb * 8;
@@ -252,7 +348,7 @@ __device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, ui
   for (int b = f.cs; b < ks; b += f.ncs) {
     uint32_t r[kHalves][16];
 #pragma unroll
-    for (int h = 0; h < kHalves; ++h) ptx::tmem_ld_16x32(taddr + ((uint32_t)h << 20) + (uint32_t)(b << 5), r[h]);
+    for (int h = 0; h < kHalves; ++h) ptx::tmem_ld_16x32(taddr + ((uint32_t)h << 20) + (uint32_t)(min(b, last) << 5), r[h]);
     const float4 m0 = ft[b * 8], m1 = ft[b * 8 + 1];
     float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
     const float m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
@@ -585,6 +681,8 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
           flow_sum<2>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
         }
         tpar ^= 1u;
+        // (streamed weights: the next tile's first GEMM writes where the partials were)
+        if (P.ring && t + 1 < f.tiles) flow_hand_over(f, &ctl->a_ready[0]);
       }
     }
     ptx::tc_fence_before();
@@ -692,7 +790,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
 
   ptx::grid_launch_dependents();         // the next kernel in the stream may start its prologue
   const int img0 = blockIdx.x * P.group, nimg = min(P.group, a.batch - img0);
-  const int tiles = P.im2col ? (nimg + 3) >> 2 : nimg * P.tiles_img, slots = min(2, tiles);
+  const int tiles = P.im2col ? (nimg + 3) >> 2 : nimg * P.tiles_img, slots = P.ring ? 1 : min(2, tiles);
   if (tid == 0) {
     ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), (uint32_t)kFlowWarps);
     for (int s = 0; s < 2; ++s) {
@@ -701,7 +799,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
       ptx::mbar_init(ptx::smem_u32(&ctl.d3_ready[s]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl.meta_full[s]), 1);
     }
-    for (int s = 0; s < 3; ++s) {
+    for (int s = 0; s < kFlowMaxRing; ++s) {
       ptx::mbar_init(ptx::smem_u32(&ctl.w_full[s]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl.w_empty[s]), (uint32_t)slots);
     }
@@ -727,9 +825,14 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
   st.inverse = kInv;
 
   if (warp == kFlowWarps + 2) {
-    if (lane == 0) flow_loader(f, P, a, st);        // packed blocks: written once, at model creation
+    // packed blocks: written once, at model creation
+    if (lane == 0) {
+      if (P.ring) flow_loader_ring(f, P, a, st);
+      else flow_loader(f, P, a, st);
+    }
   } else if (warp >= kFlowWarps) {
-    flow_mma(f, P, st, warp - kFlowWarps);
+    if (!P.ring) flow_mma(f, P, st, warp - kFlowWarps);
+    else if (warp == kFlowWarps) flow_mma_ring(f, P, st);
   } else {
     // frame of the network input: zero channels, and the constants that multiply the bias rows in the
     // bytes that no channel uses (at 4 x 4 levels: after the nine taps)

@@ -12,6 +12,7 @@ namespace iodf {
 constexpr int kFlowWarps = 16;                       // requantising warps, four per TMEM lane quarter
 constexpr int kFlowWorkers = kFlowWarps * 32;
 constexpr int kFlowThreads = kFlowWorkers + 3 * 32;  // + an MMA-issuing warp per tile slot and the weight-loading warp
+constexpr int kFlowMaxRing = 12;                     // slots of the weight ring
 constexpr int kFlowMaxTiles = 32;                    // of a CTA
 constexpr int kFlowMaxSteps = 18;                    // K steps of the first conv
 
@@ -37,6 +38,8 @@ struct FlowPlan {
   int32_t pitch;                 // bytes between 16-byte K chunks of the hidden operands
   int32_t acc_stride;            // words per channel plane of the translation accumulator (pg + 4: no bank conflicts)
   int32_t alias;                 // 1: the third matrix travels through the first one's slot
+  int32_t ring;                  // > 0: hidden widths above 256: one tile in flight, weights streamed for every tile in K
+  uint32_t ring_slot_bytes;      // steps of 32 bytes through a ring of that many slots at s_w[0]
   int32_t d_col, d3_col, d3_step;// TMEM columns: slot s has its accumulators at s * d_col, its per-tap partials at
                                  // d3_col + s * d3_step
   int32_t n_prior;               // columns of the prior head (padded to 16)

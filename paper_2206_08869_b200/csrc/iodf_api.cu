@@ -619,6 +619,7 @@ PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, con
     for (int tap = 0; tap < 9; ++tap)
       for (int k = 0; k < k2; ++k)
         pb.w[2][wpos(M.n3, tap * cbp + c, flow_kpos(k))] = (uint8_t)w3[((size_t)c * 9 + tap) * k2 + o2.ch[k]];
+  pb.k_slices[0] = (uint32_t)kmap.size() / 32; pb.k_slices[1] = (uint32_t)M.ks2; pb.k_slices[2] = (uint32_t)M.ks3;
   return pb;
 }
 
@@ -635,6 +636,7 @@ PackedBlock pack_flow_prior(const iodf_level_desc& lv, const Blobs& B, const Flo
   put_out_rq(reinterpret_cast<OutRq*>(pb.meta.data() + M.off_out), L, B);
   std::memcpy(pb.meta.data(), &M, sizeof(M));
   flow_first_matrix(pb.w[0], M.n, kmap, B.w + L.weight_off, F.ca, 2 * F.cb, nullptr, nullptr);
+  pb.k_slices[0] = (uint32_t)kmap.size() / 32;
   return pb;
 }
 
@@ -968,15 +970,18 @@ bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, uint32_t max_ba
   group = std::max(1, std::min<int>(group, (int)max_batch));
   // the latency plan keeps groups small while the CTAs of a full batch would not fill the SMs
   while (!throughput && group > 1 && ((int)max_batch + group - 1) / group < num_sms) group /= 2;
+  const bool wide = nd.n_hidden > 256;
   for (; group >= 1; group /= 2) {
     F.group = group;
     F.pg = group * F.px;
     F.tiles = F.im2col ? (group + 3) / 4 : group * F.tiles_img;
     const uint32_t nh = up(nd.n_hidden, 16), nh32 = up(nd.n_hidden, 32);
-    if (nd.n_hidden > 256 || nd.n_taps > 512 || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
+    if (nd.n_hidden > 512 || nd.n_taps > 512 || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
       continue;
-    if (F.tiles == 1) {
-      F.d_col = 0; F.d3_col = 0; F.d3_step = 0;
+    F.d_col = 0; F.d3_col = 0; F.d3_step = 0;
+    if (wide) {
+      F.tmem_cols = 512;
+    } else if (F.tiles == 1) {
       F.tmem_cols = (int)pow2_cols(std::max(std::max(nh32, nd.n_taps), (uint32_t)F.n_prior));
     } else {
       // several tiles: two slots; with more than two tiles the per-tap partials need columns of their own, because
@@ -991,7 +996,7 @@ bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, uint32_t max_ba
     F.pitch = F.m * 16 + 64;
     F.acc_stride = F.pg + 4;
     for (int alias = 0; alias < 2; ++alias) {
-      if (alias && F.tiles > 2) continue;
+      if (alias && (F.tiles > 2 || wide)) continue;
       uint32_t off = 0;
       auto take = [&](uint32_t bytes) { const uint32_t o = off; off = up(off + bytes, kAlign); return o; };
       F.alias = alias;
@@ -1007,12 +1012,20 @@ bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, uint32_t max_ba
       F.s_acc = F.im2col ? 0 : take((uint32_t)F.cb * F.acc_stride * 4);
       const uint32_t a_bytes = 2u * nd.kb * F.pitch;
       F.s_a[0] = take(a_bytes);
-      F.s_a[1] = F.tiles > 1 ? take(a_bytes) : F.s_a[0];
+      F.s_a[1] = F.tiles > 1 && !wide ? take(a_bytes) : F.s_a[0];
       F.s_meta[0] = take(nd.meta);
       F.s_meta[1] = take(nd.meta);
-      F.s_w[0] = take(alias ? std::max(nd.w[0], nd.w[2]) : nd.w[0]);
-      F.s_w[1] = take(nd.w[1]);
-      F.s_w[2] = alias ? F.s_w[0] : take(nd.w[2]);
+      if (wide) {          // a ring of K steps in what is left: at least three, so that copies and MMAs overlap
+        F.ring_slot_bytes = up(32u * std::max(nd.n_hidden, std::max(nd.n_taps, (uint32_t)F.n_prior)), kAlign);
+        F.s_w[0] = F.s_w[1] = F.s_w[2] = off;
+        if (off + 3 * F.ring_slot_bytes > limit) continue;
+        F.ring = std::min<int>(kFlowMaxRing, (int)((limit - off) / F.ring_slot_bytes));
+        off += (uint32_t)F.ring * F.ring_slot_bytes;
+      } else {
+        F.s_w[0] = take(alias ? std::max(nd.w[0], nd.w[2]) : nd.w[0]);
+        F.s_w[1] = take(nd.w[1]);
+        F.s_w[2] = alias ? F.s_w[0] : take(nd.w[2]);
+      }
       F.s_total = off;
       if (off > limit) continue;
       // operand chunks of the first conv's K steps, now that the planes' distance is known
