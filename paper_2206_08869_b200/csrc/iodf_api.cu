@@ -19,7 +19,6 @@
 #include "res_flow.h"
 #include "res_level.h"
 #include "level_kernel.h"
-#include "level_pipe.h"
 #include "selftest.h"
 
 using namespace iodf;
@@ -640,33 +639,14 @@ PackedBlock pack_flow_prior(const iodf_level_desc& lv, const Blobs& B, const Flo
   return pb;
 }
 
-// Levels of at least this many tiles per CTA run in the kernel that splits a tile's work by role
-// (level_pipe.cu) when they are eligible for it. Measured on the ImageNet64-shaped flow: 5 % faster
-// than the general kernel at eight tiles per image, 5 % slower at two (nothing follows the one
-// pair of tiles that the role split could overlap with).
-#ifndef IODF_PIPE_MIN_TILES
-#define IODF_PIPE_MIN_TILES 4
-#endif
-constexpr int kPipeMinTiles = IODF_PIPE_MIN_TILES;
-
-// What that kernel needs to know about a level.
-struct PipeDims {
-  bool eligible = false;           // every coupling in the floating-point requantisation flavour
-  uint32_t a1_bytes = 16;          // im2col operand of a tile (couplings and prior head)
-  uint32_t n_hidden = 0;           // widest accumulator of the first two GEMMs (and of the prior head)
-  uint32_t n_taps = 0;             // accumulator of the third GEMM: nine taps x padded C/2
-};
-
 // Choose images per CTA, tiles in flight and the shared-memory layout. Returns false if nothing fits.
-//   pipe:   two tile slots, every weight matrix resident, the work of a tile split by role
-//           (level_pipe.cu; needs an eligible level of several tiles per CTA)
 //   mode 0: two tile slots, every weight matrix resident      (needs all N <= 256 and >= 2 tiles)
 //   mode 1: one tile slot, every weight matrix resident
 //   mode 2: one tile slot, W1 and W3 share a slot and are re-fetched per tile
 //   mode 3: one tile slot, weights streamed per tile in 32-byte K-slices through a small ring
 //           (the only mode for hidden widths above 256: a 512 x 512 matrix alone is 256 KB)
 bool plan_smem(LevelPlan& P, uint32_t a_bytes, uint32_t meta_bytes, const uint32_t wmax[3], uint32_t n_max,
-               uint32_t limit, uint32_t max_batch, int num_sms, const PipeDims& pd, bool throughput) {
+               uint32_t limit, uint32_t max_batch, int num_sms, bool lean, bool throughput) {
   int group = P.px >= kTileM ? 1 : kTileM / P.px;
   group = std::max(1, std::min<int>(group, (int)max_batch));
   // A level's time is set by the serial chain of its couplings inside one CTA, not by how many
@@ -677,14 +657,9 @@ bool plan_smem(LevelPlan& P, uint32_t a_bytes, uint32_t meta_bytes, const uint32
   while (!throughput && group > 1 && ((int)max_batch + group - 1) / group < num_sms) group /= 2;
   for (; group >= 1; group = (group > 1 ? group / 2 : 0)) {
     const int tiles = (group * P.px + kTileM - 1) / kTileM;
-    // the role-split kernel first with im2col buffers of its own (mode -2), then sharing the slot's buffer (-1)
-    for (int mode = -2; mode < 4; ++mode) {
-      const bool pipe = mode < 0;
-      // per-tap partials in columns of their own when two slots of both kinds fit the 512 columns
-      const bool r3_separate = 2u * pd.n_hidden + 2u * pd.n_taps <= 512u;
-      if (pipe && (!pd.eligible || tiles < kPipeMinTiles || std::max(pd.n_hidden, pd.n_taps) > (uint32_t)kSlotCols)) continue;
+    for (int mode = 0; mode < 4; ++mode) {
       if (mode == 0 && (tiles < 2 || n_max > (uint32_t)kSlotCols)) continue;
-      if (mode >= 0 && mode < 3 && n_max > 2u * kSlotCols) continue;
+      if (mode < 3 && n_max > 2u * kSlotCols) continue;
       if (mode == 3 && n_max <= (uint32_t)kSlotCols) continue;   // resident weights are faster when they fit
       if (mode == 3 && throughput && group > 1) continue;        // streamed weights cost more than the fuller tile saves
       const uint32_t pg = up((uint32_t)group * P.px, 32);
@@ -696,9 +671,7 @@ bool plan_smem(LevelPlan& P, uint32_t a_bytes, uint32_t meta_bytes, const uint32
       P.s_rowinfo = take((uint32_t)tiles * kTileM * 4);
       P.s_gran = take((uint32_t)P.n_gran * 8);
       P.s_a[0] = take(a_bytes);
-      P.s_a[1] = (pipe || mode == 0) ? take(a_bytes) : P.s_a[0];
-      P.s_a1[0] = mode == -2 ? take(pd.a1_bytes) : P.s_a[0];
-      P.s_a1[1] = mode == -2 ? take(pd.a1_bytes) : P.s_a[1];
+      P.s_a[1] = mode == 0 ? take(a_bytes) : P.s_a[0];
       P.s_meta[0] = take(meta_bytes);
       P.s_meta[1] = take(meta_bytes);
       P.ring_slot_bytes = up(32u * n_max, kAlign);
@@ -711,15 +684,11 @@ bool plan_smem(LevelPlan& P, uint32_t a_bytes, uint32_t meta_bytes, const uint32
         P.s_w[2] = mode == 2 ? P.s_w[0] : take(wmax[2]);
       }
       P.s_total = off;
-      P.pipe = pipe ? 1 : 0;
-      P.lean = (pd.eligible && mode != 3) ? 1 : 0;
-      P.r_col[0] = r3_separate ? (int)pd.n_hidden : kSlotCols;
-      P.r_col[1] = r3_separate ? 2 * (int)pd.n_hidden : 0;
-      P.r_col[2] = r3_separate ? (int)pd.n_taps : kSlotCols;
+      P.lean = (lean && mode != 3) ? 1 : 0;
       P.w13_alias = mode == 2;
       P.streamed = mode == 3;
       P.nslots = mode == 0 ? 2 : 1;
-      P.tmem_cols = (int)(pipe ? 512 : (mode == 0 ? 2 * kSlotCols : pow2_cols(n_max)));
+      P.tmem_cols = (int)(mode == 0 ? 2 * kSlotCols : pow2_cols(n_max));
       P.group = group;
       P.pg = (int)pg;
       P.tiles = tiles;
@@ -964,13 +933,13 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
 
 // Group, tensor-memory columns and shared-memory layout of a level in the compact kernel. false: it does not fit.
 struct FlowNeeds { uint32_t n_hidden = 32, n_taps = 16, kb = 1, meta = 16, w[3] = {16, 16, 16}; };
-bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, uint32_t max_batch, int num_sms, bool throughput) {
+// wide: weights streamed for every tile, one tile in flight.
+bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, uint32_t max_batch, int num_sms, bool throughput, bool wide) {
   int group = F.px >= kTileM ? 1 : kTileM / F.px;
   if (F.im2col) group = std::min(group, 4);            // an image per lane quarter
   group = std::max(1, std::min<int>(group, (int)max_batch));
   // the latency plan keeps groups small while the CTAs of a full batch would not fill the SMs
   while (!throughput && group > 1 && ((int)max_batch + group - 1) / group < num_sms) group /= 2;
-  const bool wide = nd.n_hidden > 256;
   for (; group >= 1; group /= 2) {
     F.group = group;
     F.pg = group * F.px;
@@ -1289,7 +1258,10 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   };
   for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) add(blocks[ki], &P.coupling[ki]);
   if (lv.has_prior) add(prior, &P.prior);
-  return plan_flow(F, nd, smem_limit, max_batch, num_sms, throughput);
+  // resident weights where they and the accumulators of two tiles fit; streaming them costs a copy of 16 - 64 KB per GEMM
+  // and tile, which one tile's chain of GEMMs does not hide
+  return (nd.n_hidden <= 256 && plan_flow(F, nd, smem_limit, max_batch, num_sms, throughput, false)) ||
+         plan_flow(F, nd, smem_limit, max_batch, num_sms, throughput, true);
 }
 
 int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_model* m) {
@@ -1476,8 +1448,7 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
     hl.blob.clear();
     uint32_t a_bytes = 16, meta = 16, wmax[3] = {16, 16, 16};
     uint32_t n_max = 32;
-    PipeDims pd;
-    pd.eligible = lv.n_couplings > 0;
+    bool lean = lv.n_couplings > 0;               // every hidden layer in the floating-point flavour
     std::vector<PackedBlock> blocks;
     for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) {
       const iodf_coupling_desc& cp = lv.couplings[ki];
@@ -1489,10 +1460,7 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
       a_bytes = std::max<uint32_t>(a_bytes, kTileM * std::max(d.kd1, std::max(d.kd2, d.kd3)));
       n_max = std::max<uint32_t>(n_max, std::max(d.n1, std::max(d.n2, d.n3)));
       const CouplingMeta* cm = reinterpret_cast<const CouplingMeta*>(blocks.back().meta.data());
-      if (cm->mode1 != 4 || cm->mode2 != 4) pd.eligible = false;
-      pd.n_hidden = std::max<uint32_t>(pd.n_hidden, (uint32_t)std::max(d.n1, d.n2));
-      pd.a1_bytes = std::max<uint32_t>(pd.a1_bytes, (uint32_t)kTileM * d.kd1);
-      pd.n_taps = std::max<uint32_t>(pd.n_taps, (uint32_t)d.n3);
+      if (cm->mode1 != 4 || cm->mode2 != 4) lean = false;
     }
     PackedBlock prior_block;
     if (lv.has_prior) {
@@ -1500,8 +1468,6 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
       prior_block = pack_prior(lv, B, ca, cb, &n, &kd);
       a_bytes = std::max<uint32_t>(a_bytes, kTileM * kd);
       n_max = std::max<uint32_t>(n_max, n);
-      pd.n_hidden = std::max<uint32_t>(pd.n_hidden, (uint32_t)n);
-      pd.a1_bytes = std::max<uint32_t>(pd.a1_bytes, (uint32_t)kTileM * kd);
     }
     if (n_max > 512) return IODF_EUNSUPPORTED;
     {   // im2col granule table of the level's first convs (couplings and prior head share it)
@@ -1530,7 +1496,7 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
       wmax[0] = std::max(wmax[0], P.prior.w_bytes[0]);
     }
     if (hl.blob.empty()) hl.blob.resize(kAlign, 0);
-    if (!plan_smem(P, a_bytes, meta, wmax, n_max, (uint32_t)smem_limit, desc->max_batch, num_sms, pd,
+    if (!plan_smem(P, a_bytes, meta, wmax, n_max, (uint32_t)smem_limit, desc->max_batch, num_sms, lean,
                    desc->plan == IODF_PLAN_THROUGHPUT))
       return IODF_EUNSUPPORTED;
     if (!index_maps_fit(P.group)) return IODF_EUNSUPPORTED;
@@ -1544,7 +1510,6 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
   (void)max_smem;
   CU(m, configure_level_kernels((uint32_t)smem_limit));
   CU(m, configure_res_kernels((uint32_t)smem_limit));
-  CU(m, configure_pipe_kernels((uint32_t)smem_limit));
   CU(m, configure_flow_kernels((uint32_t)smem_limit));
   CU(m, configure_res_flow_kernels((uint32_t)smem_limit));
   const size_t L = desc->n_levels;
@@ -1581,14 +1546,13 @@ void set_patch_grid(LevelArgs& a, const PatchGrid& g) {
   a.mul_patches_x = g.patches_x > 1 ? (uint32_t)(((1ull << 32) + g.patches_x - 1) / g.patches_x) : 0u;
 }
 
-// The kernel that runs a level: residual couplings, the stage pipeline, or the general kernel.
+// The kernel that runs a level: residual couplings or the general kernel.
 cudaError_t launch_any_level(const HostLevel& hl, const LevelArgs& a, bool inverse, int B, cudaStream_t st) {
   const LevelPlan& P = hl.plan;
   const int grid = (B + P.group - 1) / P.group;
   if (hl.use_flow) return launch_flow_level(a, hl.flow, inverse, grid, st);
   if (hl.use_rf) return launch_res_flow(a, hl.rf, inverse, grid * hl.rf.nbx * hl.rf.nby, st);
   if (P.residual) return launch_res_level(a, inverse, grid, P.res_bands, P.s_total, st);
-  if (P.pipe) return launch_level_pipe(a, inverse, grid, P.s_total, st);
   return launch_level(a, inverse, P.lean != 0, grid, P.s_total, st);
 }
 
@@ -2224,7 +2188,7 @@ const char* iodf_level_kernel_name(const iodf_model* m, int level) {
   const LevelPlan& P = m->levels[level].plan;
   if (m->levels[level].use_flow) return "flow_level_kernel";
   if (m->levels[level].use_rf) return "res_flow_kernel";
-  return P.residual ? "res_level_kernel" : (P.pipe ? "level_pipe_kernel" : "level_kernel");
+  return P.residual ? "res_level_kernel" : "level_kernel";
 }
 
 int iodf_level_images_per_cta(const iodf_model* m, int level) {

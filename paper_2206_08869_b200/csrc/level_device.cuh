@@ -1,6 +1,6 @@
-// Device code shared by the flow-level kernels (level_kernel.cu: every level shape; level_pipe.cu:
-// the stage-pipelined kernel for levels of several tiles): requantisation, im2col, the epilogues,
-// step bookkeeping, MMA issue and weight copies, and the index maps of a level's load and store.
+// Device code of the general level kernel (level_kernel.cu: every level shape): requantisation, im2col, the
+// epilogues, step bookkeeping, MMA issue and weight copies, and the index maps of a level's load and
+// store. flow_level.cu and res_flow.cu use its requantisation and step bookkeeping.
 #pragma once
 #include "iodf_dev.h"
 #include "level_kernel.h"
@@ -354,46 +354,6 @@ __device__ __forceinline__ void epilogue_hidden(const Ctx& cx, int mode, int us,
   }
 }
 
-// ---- im2col without the granule table ---------------------------------------------------------------
-// im2col of this thread's tile row by taps: split `cs` of `ncs` (a power of two) takes the taps t
-// with t % ncs == cs, one predicated load per 8-byte granule straight from the pixel-major network
-// input (the tap's bit of the row's gather mask says whether its source pixel is inside the image),
-// and one split also writes what follows the nine taps: the eight bias columns and zeros up to kd.
-// kCpad = bytes per pixel of the network input (C/2 rounded up to 8). The bytes are those of
-// build_im2col; only the way to them differs.
-template <int kCpad>
-__device__ __forceinline__ void build_im2col_taps(uint8_t* __restrict__ a_row, const int8_t* __restrict__ xa, int w,
-                                                   int kd, const RowPos rp, int cs, int ncs) {
-  constexpr int kG = kCpad / 8;          // granules per tap
-  const int8_t* base = xa + (size_t)rp.p * kCpad;
-  auto at = [&](int g) { return a_row + (size_t)(g >> 1) * (kTileM * 16) + (g & 1) * 8; };
-#pragma unroll
-  for (int t = 0; t < 9; ++t) {
-    if ((t & (ncs - 1)) != cs) continue;
-    const int8_t* src = base + (((t / 3) - 1) * w + (t % 3) - 1) * kCpad;
-    const bool ok = ((rp.gmask >> t) & 1u) != 0;
-    if (kG % 2 == 0) {                   // whole 16-byte chunks
-#pragma unroll
-      for (int gi = 0; gi < kG; gi += 2) {
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (ok) v = *reinterpret_cast<const uint4*>(src + gi * 8);
-        *reinterpret_cast<uint4*>(at(t * kG + gi)) = v;
-      }
-    } else {
-#pragma unroll
-      for (int gi = 0; gi < kG; ++gi) {
-        uint2 v = make_uint2(0u, 0u);
-        if (ok) v = *reinterpret_cast<const uint2*>(src + gi * 8);
-        *reinterpret_cast<uint2*>(at(t * kG + gi)) = v;
-      }
-    }
-  }
-  if (cs == (9 & (ncs - 1))) {
-    const int ng = kd >> 3;
-    if (9 * kG < ng) *reinterpret_cast<uint2*>(at(9 * kG)) = make_uint2(kBiasColumnsLo, kBiasColumnsHi);
-    for (int g = 9 * kG + 1; g < ng; ++g) *reinterpret_cast<uint2*>(at(g)) = make_uint2(0u, 0u);
-  }
-}
 
 // Per-tap partial products -> shifted sum into the translation accumulator.
 // Column granule (tap, gq) holds out channels gq*8 .. gq*8+8 of that tap. The partial product of

@@ -1,0 +1,71 @@
+"""The compact level kernels at the edges of their ranges: shapes of tiles, ragged groups, widths on either side
+of a dispatch, channels that need each form of requantisation, and the entropy coder's symbol look-up over
+every range of scales; against the CPU oracle, bit for bit."""
+import numpy as np
+import pytest
+
+import iodf_synth as S
+import oracle as O
+from test_gpu_parity import G, _check_both_ways, _t  # noqa: F401  (G: the fixture)
+from test_gpu_residual import _both_ways
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hw,splits,hidden,batch", [
+    (16, [True, True], 16, 5),           # the last level 4 x 4: four images and one
+    (16, [True, True], 31, 3),           # 8 x 8 tiles of 64 rows, six and twelve channels in
+    (32, [True, True, True], 33, 2),     # 16 x 16: two tiles
+    (48, [True], 16, 2),                 # 24 x 24: nine 64-row tiles
+    (32, [False, True], 256, 2),         # the widest that can be resident
+    (64, [True], 200, 1),                # eight tiles whose accumulators do not fit side by side: streamed
+    (64, [True, True], 257, 1),          # the narrowest streamed weights, eight tiles
+    (16, [True, True], 512, 6),          # the widest; 4 x 4 level with two ragged groups
+])
+@pytest.mark.parametrize("plan", [0, 1])
+def test_three_conv_levels(G, hw, splits, hidden, batch, plan):
+    model = S.make_model(0xF100 + hw + hidden, 3, hw, hw, splits, 3, hidden)
+    x = S.smooth_field_images(0xF200 + hw, batch, hw, hw, 2.0)
+    m, _ = _check_both_ways(G, model, x, plan=plan)
+    assert {G.iodf_level_kernel_name(m, k) for k in range(len(splits))} == {"flow_level_kernel"}
+
+
+@pytest.mark.parametrize("hw,splits,couplings,hidden,blocks,prune,batch,plan", [
+    (64, [True], 1, 128, 1, None, 1, 0),           # 32 x 32 in eight 8 x 16 blocks
+    (64, [True], 1, 128, 1, None, 1, 1),           # ... in four 16 x 16 ones
+    (32, [True], 2, 97, 2, (0.4, 0.7), 2, 0),      # 16 x 16: one block, four chunks with a ragged last one
+    (16, [True], 1, 32, 1, None, 3, 0),            # 8 x 8: one chunk
+    (8, [True], 1, 65, 2, None, 5, 1),             # 4 x 4: three images and two
+])
+def test_residual_levels(G, hw, splits, couplings, hidden, blocks, prune, batch, plan):
+    model = S.make_residual_model(0xF300 + hw + hidden, 3, hw, hw, splits, couplings, hidden, blocks, prune=prune)
+    x = S.smooth_field_images(0xF400 + hw, batch, hw, hw, 2.0)
+    m, _, _ = _both_ways(G, model, x, plan=plan)
+    assert {G.iodf_level_kernel_name(m, k) for k in range(len(splits))} == {"res_flow_kernel"}
+
+
+@pytest.mark.parametrize("ls", [0, 20, 40, 63])
+def test_symbol_look_up_at_every_kind_of_scale(G, ls):
+    """Residuals over the whole window at one scale: slots that mean one symbol and slots that mean hundreds."""
+    import torch
+    model = S.make_model(0xF500, 3, 32, 32, [True, False], 1, 16)
+    codec = S.logistic_codec(elems_per_stream=97)
+    B, d, d_fact = 3, 3 * 32 * 32, 6 * 256
+    rng = np.random.default_rng(ls)
+    prior = np.stack([rng.integers(-50, 50, (B, d_fact)), np.full((B, d_fact), ls)], axis=1).astype(np.int32)
+    z = rng.integers(-2200, 2201, (B, d)).astype(np.int32)
+    z[:, ::3] = rng.integers(-3, 4, z[:, ::3].shape)
+    w_ref, c_ref = O.rans_encode(codec, model, z, prior)
+    m = G.iodf_create(model, B)
+    cd = G.iodf_codec_create(m, codec)
+    words, counts = G.iodf_rans_encode(cd, _t(z), _t(prior))
+    cc = counts.cpu().numpy().view(np.uint32)
+    np.testing.assert_array_equal(cc, c_ref)
+    w = words.cpu().numpy().view(np.uint16)
+    valid = np.arange(w.shape[2])[None, None, :] < cc[:, :, None]
+    np.testing.assert_array_equal(np.where(valid, w, 0), np.where(valid, w_ref, 0))
+    out = torch.zeros((B, d), dtype=torch.int32, device="cuda")
+    for q in range(cd.n_blocks):
+        G.iodf_rans_decode_block(cd, q, words, counts, _t(prior), out)
+    G.iodf_codec_check(cd)
+    np.testing.assert_array_equal(out.cpu().numpy(), z)
