@@ -29,7 +29,10 @@ namespace iodf {
 namespace {
 
 struct __align__(16) FlowCtl {
-  uint64_t xa_ready;      // workers -> MMA warp, loader: network input of the step written   (count kFlowWarps)
+  uint64_t xa_ready[2];   // workers (and the neighbours' edge bytes) -> MMA warp, loader: network input of an even / odd
+                          // step written (count kFlowWarps; a neighbour may be one step ahead)
+  uint64_t acc_full;      // split images: the neighbours' products of a coupling have been added
+  uint64_t peers_done;    // split images: the neighbours have read the prior head's input
   uint64_t a_ready[2];    // slot's workers -> its MMA warp: the next hidden operand is written
   uint64_t dm_ready[2];   // tensor core -> workers: first / second GEMM of the slot's tile complete
   uint64_t d3_ready[2];   // tensor core -> workers: per-tap partials of the slot's tile complete
@@ -48,6 +51,8 @@ struct Flow {
   int tid, warp, lane;
   int nimg, pvalid, tiles;      // images, pixels and tiles of this CTA
   int slots;                    // tile slots in use: 1 or 2
+  int rank, by, bx;             // split images: this CTA's block
+  uint32_t halo;                // ... and the bytes of network input that its neighbours send each step
   int sl, cs, ncs;              // worker: its slot, its share of a lane quarter's work (cs of ncs warps)
 };
 
@@ -71,12 +76,42 @@ __device__ __forceinline__ void flow_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ptx::smem_u32(bar)) : "memory");
 }
 // this warp's shared-memory writes (towards the tensor core) and tensor-memory reads are done
-__device__ __forceinline__ void flow_hand_over(const Flow& f, uint64_t* bar) {
+// (bytes: what neighbours' asynchronous stores add to the phase, announced by one warp)
+__device__ __forceinline__ void flow_hand_over(const Flow& f, uint64_t* bar, uint32_t bytes = 0u) {
   ptx::tc_fence_before();
   ptx::fence_async_smem();
   __syncwarp();
-  if (f.lane == 0) flow_arrive(bar);
+  if (f.lane == 0) {
+    if (bytes) ptx::mbar_expect_tx(ptx::smem_u32(bar), bytes);
+    else flow_arrive(bar);
+  }
 }
+// the MMA warp's wait for the network input of step i; a neighbour's bytes came through the generic proxy
+__device__ __forceinline__ void flow_wait_input(const Flow& f, int i) {
+  flow_wait(f, &f.ctl->xa_ready[i & 1], (uint32_t)(i >> 1) & 1u);
+  if (f.halo) asm volatile("fence.proxy.async;" ::: "memory");
+}
+// ---- between the CTAs of a split image ----
+__device__ __forceinline__ uint32_t flow_peer(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// a word into / a sum onto a neighbour's shared memory; its barrier counts the four bytes when they are there
+__device__ __forceinline__ void flow_store_async(uint32_t addr, uint32_t bar, uint32_t v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void flow_red_async(uint32_t addr, uint32_t bar, int32_t v) {
+  asm volatile("red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.add.s32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void flow_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ bool flow_block_exists(const FlowPlan& P, const Flow& f, int dy, int dx) {
+  return (uint32_t)(f.by + dy) < (uint32_t)P.nby && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx;
+}
+
 __device__ __forceinline__ void worker_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kFlowWorkers) : "memory"); }
 
 // ---- weight and meta loader (one lane) -----------------------------------------------------------------
@@ -120,7 +155,7 @@ __device__ void flow_loader(const Flow& f, const FlowPlan& P, const LevelArgs& a
     }
     // meta slot of step i: its last reader is the pixel pass of step i + 1
     if (i + 2 < st.nsteps) {
-      flow_wait(f, &ctl->xa_ready, (uint32_t)(i + 1) & 1u);
+      flow_wait(f, &ctl->xa_ready[(i + 1) & 1], (uint32_t)((i + 1) >> 1) & 1u);
       meta(i + 2);
     }
   }
@@ -134,7 +169,7 @@ __device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelAr
   for (int i = 0; i < st.nsteps; ++i) {
     const BlockRef& br = step_ref(*a.plan, st, i);
     // meta slot of step i: its last reader was the pixel pass of step i - 1
-    if (i >= 2) flow_wait(f, &ctl->xa_ready, (uint32_t)(i - 1) & 1u);
+    if (i >= 2) flow_wait(f, &ctl->xa_ready[(i - 1) & 1], (uint32_t)((i - 1) >> 1) & 1u);
     {
       const uint32_t b = ptx::smem_u32(&ctl->meta_full[i & 1]);
       ptx::mbar_expect_tx(b, br.meta_bytes);
@@ -183,7 +218,8 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
   uint8_t* smem = f.smem;
   const bool lead = ptx::elect_one();
   const uint32_t idesc_m = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.m >> 4) << 24);     // s8 x s8 -> s32
-  const uint32_t xa16 = ptx::smem_u32(smem + P.s_xa) >> 4;
+  // (in a cluster a shared-memory address also carries the CTA's rank above the descriptor's 14 bits)
+  const uint32_t xa16 = (ptx::smem_u32(smem + P.s_xa) >> 4) & 0x3FFFu;
   const uint32_t a1_hi = (uint32_t)P.sbo16 | (1u << 14);
   const uint32_t pitch16 = (uint32_t)P.pitch >> 4;
   const uint32_t a_lo = ((ptx::smem_u32(smem + P.s_a[sl]) >> 4) & 0x3FFFu) | (pitch16 << 16);
@@ -224,7 +260,7 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
         bl += 2u * (uint32_t)n1;
       }
     };
-    flow_wait(f, &ctl->xa_ready, (uint32_t)i & 1u);
+    flow_wait_input(f, i);
     ptx::tc_fence_after();
     if (prior) {
 #pragma unroll 1
@@ -262,7 +298,7 @@ __device__ void flow_mma_ring(const Flow& f, const FlowPlan& P, const Steps& st)
   uint8_t* smem = f.smem;
   auto uniform = [](int x) { return __shfl_sync(0xFFFFFFFFu, x, 0); };
   const uint32_t idesc_m = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P.m >> 4) << 24);
-  const uint32_t xa16 = ptx::smem_u32(smem + P.s_xa) >> 4, hi = ptx::kUmmaDescHi;
+  const uint32_t xa16 = (ptx::smem_u32(smem + P.s_xa) >> 4) & 0x3FFFu, hi = ptx::kUmmaDescHi;
   const uint32_t a1_hi = (uint32_t)P.sbo16 | (1u << 14), pitch16 = (uint32_t)P.pitch >> 4;
   const uint32_t a_lo = ((ptx::smem_u32(smem + P.s_a[0]) >> 4) & 0x3FFFu) | (pitch16 << 16);
   uint32_t slot = 0, round = 0, apar = 0;
@@ -299,7 +335,7 @@ __device__ void flow_mma_ring(const Flow& f, const FlowPlan& P, const Steps& st)
     const FlowMeta* M = reinterpret_cast<const FlowMeta*>(smem + P.s_meta[i & 1]);
     const int n1 = prior ? P.n_prior : uniform(M->n1), n2 = uniform(M->n2), n3 = uniform(M->n3);
     const int ks2 = uniform(M->ks2), ks3 = uniform(M->ks3);
-    flow_wait(f, &ctl->xa_ready, (uint32_t)i & 1u);
+    flow_wait_input(f, i);
     ptx::tc_fence_after();
 #pragma unroll 1
     for (int t = 0; t < f.tiles; ++t) {
@@ -407,8 +443,8 @@ __device__ __forceinline__ int32_t rq_hi(int32_t a, const OutRq o) {
 // Per-tap partials of tile t -> accumulator. A lane quarter is kR rows of the tile's eight columns, and a
 // thread holds a column: the three vertical taps of one horizontal tap v meet in its registers, so unit
 // (granule of 8 channels, v) costs kR + 2 reductions per channel instead of 3 kR. Products whose output
-// pixel is outside the image are dropped (zero padding).
-template <int kR>
+// pixel is outside the image are dropped (zero padding), or added to the neighbour's accumulator where an image is split.
+template <int kR, bool kSplit>
 __device__ __forceinline__ void flow_sum(const Flow& f, const FlowPlan& P, int t, uint32_t taddr, int32_t* __restrict__ acc,
                                          uint64_t* ready, uint32_t parity) {
   const int ng = (P.cb + 7) >> 3;
@@ -434,6 +470,22 @@ __device__ __forceinline__ void flow_sum(const Flow& f, const FlowPlan& P, int t
     uint32_t dst = dst0 + (uint32_t)(g * 8) * next_ch - (uint32_t)(4 * v);
     const bool ok = (uint32_t)(j0 - v) < (uint32_t)P.w && g * 8 + ch0 < P.cb;
     const bool first = ok && top, last = ok && bottom;
+    // split images: where the row above, the quarter's own rows and the row below go if not to this CTA (-1: nowhere)
+    int away[3] = {-1, -1, -1};
+    uint32_t away_at[3] = {0, 0, 0};
+    bool any = false;
+    if constexpr (kSplit) {
+      const int dx = j0 < v ? -1 : (j0 - v >= P.w ? 1 : 0);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int dy = k == 0 && i0 == 0 ? -1 : (k == 2 && i0 + kR == P.h ? 1 : 0);
+        if ((dy || dx) && flow_block_exists(P, f, dy, dx) && g * 8 + ch0 < P.cb) {
+          away[k] = f.rank + dy * P.nbx + dx;
+          away_at[k] = (uint32_t)(dy * P.h * P.w + dx * P.w) * 4u;
+        }
+      }
+      any = __any_sync(0xFFFFFFFFu, away[0] >= 0 || away[1] >= 0 || away[2] >= 0);
+    }
     ptx::tmem_ld_wait4(r[0][0]);
 #pragma unroll
     for (int u = 0; u < 3; ++u)
@@ -450,6 +502,14 @@ __device__ __forceinline__ void flow_sum(const Flow& f, const FlowPlan& P, int t
         sum[1] += (int)r[u][i >> 1][2 * (i & 1) + 1];
       }
       ptx::red_add2_s32(dst, next_ch, sum[0], sum[1], o < 0 ? first : (o == kR ? last : ok));
+      if constexpr (kSplit) {
+        const int k = o < 0 ? 0 : (o == kR ? 2 : 1);
+        if (any && away[k] >= 0) {
+          const uint32_t at = flow_peer(dst - away_at[k], (uint32_t)away[k]), bar = flow_peer(ptx::smem_u32(&f.ctl->acc_full), (uint32_t)away[k]);
+          flow_red_async(at, bar, sum[0]);
+          flow_red_async(at + next_ch, bar, sum[1]);
+        }
+      }
       dst += row;
     }
   }
@@ -508,6 +568,7 @@ __device__ __forceinline__ void flow_sum_4x4(const Flow& f, const FlowPlan& P, i
 }
 
 // Prior head: accumulators of all tiles -> mu and clipped log-scale index in global memory. Unit = (tile, 8 columns).
+template <bool kSplit>
 __device__ void flow_prior(const Flow& f, const FlowPlan& P, const LevelArgs& a, const PriorMeta* M, int img0) {
   const int wq = f.warp & 3, hs = P.m >> 7;
   const OutRq* orq = reinterpret_cast<const OutRq*>(reinterpret_cast<const uint8_t*>(M) + M->off_out);
@@ -522,6 +583,8 @@ __device__ void flow_prior(const Flow& f, const FlowPlan& P, const LevelArgs& a,
     ptx::tmem_ld8(f.tmem + (uint32_t)(t * P.n_prior + g * 8) + ((uint32_t)(wq * 32) << 16), r);
     const int4 tp = f.ctl->tile[t];
     int img = tp.x, at = (tp.y + (lane_row >> 3)) * P.w + tp.z + (lane_row & 7);
+    if constexpr (kSplit) at = (f.by * P.h + tp.y + (lane_row >> 3)) * P.fw + f.bx * P.w + tp.z + (lane_row & 7);
+    const int plane = kSplit ? P.fpx : P.px;
     if (P.im2col) { img += lane_row >> 4; at = lane_row & 15; }
     int32_t* mu = a.prior + (size_t)(img0 + img) * (size_t)(2 * P.d_fact) + P.prior_off + at;
     ptx::tmem_ld_wait8(r);
@@ -531,8 +594,8 @@ __device__ void flow_prior(const Flow& f, const FlowPlan& P, const LevelArgs& a,
       const int col = g * 8 + e;
       if (col < 2 * P.cb) {
         const int32_t y = rq_hi((int32_t)r[e], orq[col]);
-        if (col < P.cb) mu[(size_t)col * P.px] = y;
-        else mu[P.d_fact + (size_t)(col - P.cb) * P.px] = clampi(y, M->ls_lo, M->ls_hi);
+        if (col < P.cb) mu[(size_t)col * plane] = y;
+        else mu[P.d_fact + (size_t)(col - P.cb) * plane] = clampi(y, M->ls_lo, M->ls_hi);
       }
     }
   }
@@ -545,6 +608,8 @@ struct PixelMap {
   int32_t* v;                   // the pair in plane 0 of the flow variable
   int32_t* acc;                 // and of the accumulator
   uint8_t* rec;                 // its first pixel's record (4 x 4 levels: operand row)
+  int dy, dx;                   // split images: the edge of the block that the pair is on (at most one of each: blocks are
+                                // eight rows and columns or more)
   uint32_t taps;                // 4 x 4 levels: bit t (16 + t): the first (second) pixel's value is read by tap t of a pixel
 };
 
@@ -569,7 +634,8 @@ __device__ __forceinline__ void flow_translate(const FlowPlan& P, const PixelMap
 }
 
 // network input: words of four requantised channels (then the constants 1, 127, 127, ...) into the frame
-__device__ __forceinline__ void flow_requant(const FlowPlan& P, const PixelMap& pm, const int32_t* cols, int32_t m0, int32_t s) {
+template <bool kSplit>
+__device__ __forceinline__ void flow_requant(const Flow& f, const FlowPlan& P, const PixelMap& pm, uint64_t* input, const int32_t* cols, int32_t m0, int32_t s) {
   const int nw = (P.ca + 3) >> 2;
   const long long rnd = 1ll << (30 + s);
 #pragma unroll 1
@@ -598,6 +664,25 @@ __device__ __forceinline__ void flow_requant(const FlowPlan& P, const PixelMap& 
         rec[-2] = w0;
         rec[2] = w1;
       }
+      if constexpr (kSplit) {                    // pixels on an edge of the block also go to the neighbours' frames
+        const uint32_t base = ptx::smem_u32(rec), bar = ptx::smem_u32(input);
+        auto put = [&](int dy, int dx, uint32_t at, uint32_t w) {
+          if (!flow_block_exists(P, f, dy, dx)) return;
+          const uint32_t rank = (uint32_t)(f.rank + dy * P.nbx + dx), b = flow_peer(bar, rank);
+          const uint32_t d = flow_peer(at - (uint32_t)((dy * P.h * P.wp + dx * P.w) * 16), rank);
+          flow_store_async(d, b, w);
+          if (P.paired && dx == 0) flow_store_async(d - 8u, b, w);
+        };
+        if (pm.dy) {
+          put(pm.dy, 0, base, w0);
+          put(pm.dy, 0, base + 16u, w1);
+        }
+        if (pm.dx) {                             // the left edge's first pixel or the right edge's second one
+          const uint32_t at = pm.dx < 0 ? base : base + 16u, w = pm.dx < 0 ? w0 : w1;
+          put(0, pm.dx, at, w);
+          if (pm.dy) put(pm.dy, pm.dx, at, w);
+        }
+      }
     } else {
       // word (tap, wd) of the rows of the pixels that read this one: row - 4 (u - 1) - (v - 1)
       int k = wd;
@@ -611,7 +696,7 @@ __device__ __forceinline__ void flow_requant(const FlowPlan& P, const PixelMap& 
   }
 }
 
-template <bool kInv>
+template <bool kInv, bool kSplit>
 __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st, int img0) {
   FlowCtl* ctl = f.ctl;
   uint8_t* smem = f.smem;
@@ -630,6 +715,8 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
     pm.v = v + pm.p;
     pm.acc = acc + pm.p;
     pm.rec = smem + P.s_xa + 16 * (P.im2col ? img * 16 + px : img * P.frame + (r + 1) * P.wp + c + 1);
+    pm.dy = r == 0 ? -1 : (r == P.h - 1 ? 1 : 0);
+    pm.dx = c == 0 ? -1 : (c == P.w - 2 ? 1 : 0);
     pm.taps = 0;
     for (int t = 0; t < 9; ++t) {
       const int oi = r - (t / 3 - 1), oj = c - (t % 3 - 1);
@@ -639,7 +726,7 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
   }
   const uint32_t dm = f.tmem + (uint32_t)(f.sl * P.d_col) + lane_field, d3 = f.tmem + (uint32_t)(P.d3_col + f.sl * P.d3_step) + lane_field;
   uint8_t* sA = smem + P.s_a[f.sl];
-  uint32_t dpar = 0u, tpar = 0u;
+  uint32_t dpar = 0u, tpar = 0u, npar = 0u;
   const uint8_t* prev = nullptr;                // coupling whose translation is still to be applied
 #pragma unroll 1
   for (int i = 0; i <= st.nsteps; ++i) {
@@ -653,14 +740,15 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
     const bool prior = st.is_prior(i);
     const FlowMeta* M = reinterpret_cast<const FlowMeta*>(mb);
     // (the first two words of both kinds of meta block)
-    flow_requant(P, pm, prior ? a.plan->col_out : reinterpret_cast<const int32_t*>(mb + M->off_colA), M->in_m0, M->in_s);
-    flow_hand_over(f, &ctl->xa_ready);
+    uint64_t* input = &ctl->xa_ready[i & 1];
+    flow_requant<kSplit>(f, P, pm, input, prior ? a.plan->col_out : reinterpret_cast<const int32_t*>(mb + M->off_colA), M->in_m0, M->in_s);
+    flow_hand_over(f, input, kSplit && f.warp == 0 ? f.halo : 0u);
     prev = prior ? nullptr : mb;
     if (prior) {
       flow_wait(f, &ctl->dm_ready[f.sl], dpar);
       dpar ^= 1u;
       ptx::tc_fence_after();
-      flow_prior(f, P, a, reinterpret_cast<const PriorMeta*>(mb), img0);
+      flow_prior<kSplit>(f, P, a, reinterpret_cast<const PriorMeta*>(mb), img0);
     } else {
 #pragma unroll 1
       for (int t = f.sl; t < f.tiles; t += f.slots) {
@@ -676,9 +764,9 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
         if (P.im2col) {
           if (quarter) flow_sum_4x4<kInv>(f, P, t, d3, mb, v, &ctl->d3_ready[f.sl], tpar);
         } else if (P.m == 128) {
-          flow_sum<4>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
+          flow_sum<4, kSplit>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
         } else {
-          flow_sum<2>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
+          flow_sum<2, kSplit>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
         }
         tpar ^= 1u;
         // (streamed weights: the next tile's first GEMM writes where the partials were)
@@ -686,49 +774,75 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
       }
     }
     ptx::tc_fence_before();
+    if (kSplit && !prior && f.tid == 0) ptx::mbar_expect_tx(ptx::smem_u32(&ctl->acc_full), (uint32_t)(P.reds[f.rank] * P.cb * 4));
     worker_barrier();                           // every product has been added
+    if constexpr (kSplit) {
+      if (!prior) {
+        flow_wait(f, &ctl->acc_full, npar);
+        npar ^= 1u;
+      } else if (i + 1 < st.nsteps) {
+        // The next step's edge pixels overwrite what the neighbours' prior heads read. (After a coupling their products
+        // say that they are past it.)
+        const int dy = f.lane / 3 - 1, dx = f.lane % 3 - 1;
+        if (f.warp == 0 && f.lane < 9 && (dy || dx) && flow_block_exists(P, f, dy, dx))
+          asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                           flow_peer(ptx::smem_u32(&ctl->peers_done), (uint32_t)(f.rank + dy * P.nbx + dx))) : "memory");
+        __syncwarp();
+        flow_wait(f, &ctl->peers_done, 0u);
+      }
+    }
   }
 }
 
 // ---- a level's input and output index maps (four neighbouring elements per thread and step) ----------------
 __device__ __forceinline__ size_t patch_index(const FlowPlan& P, const LevelArgs& a, int b, int ci, int y, int x) {
   const int by = fdiv(b, a.mul_patches_x), bx = b - by * a.patches_x;
-  return ((size_t)ci * a.img_h + (size_t)(by * 2 * P.h + y)) * a.img_w + (size_t)(bx * 2 * P.w + x);
+  return ((size_t)ci * a.img_h + (size_t)(by * 2 * P.fh + y)) * a.img_w + (size_t)(bx * 2 * P.fw + x);
 }
 
 // pre-squeeze element e (a multiple of four, image-major over the CTA's images) -> address in the level's
 // input / output array and the flow variable's two planes (dx = 0 at d0, dx = 1 at d0 + pg)
-__device__ __forceinline__ void squeeze_map(const FlowPlan& P, const LevelArgs& a, int img0, int e, size_t* at, int* d0) {
+template <bool kSplit>
+__device__ __forceinline__ void squeeze_map(const Flow& f, const FlowPlan& P, const LevelArgs& a, int img0, int e, size_t* at, int* d0) {
   const int per_img = P.c * P.px, w2 = 2 * P.w;
   const int g = fdiv(e, P.mul_per_img), r = e - g * per_img;
   const int ci = fdiv(r, P.mul_4px), r2 = r - ci * 4 * P.px;
   const int y = fdiv(r2, P.mul_w2), x = r2 - y * w2;
-  *at = (P.is_first && a.img_w > 0) ? patch_index(P, a, img0 + g, ci, y, x) : (size_t)(img0 + g) * per_img + r;
+  const int fy = kSplit ? f.by * 2 * P.h + y : y, fx = kSplit ? f.bx * w2 + x : x;
+  if (P.is_first && a.img_w > 0) *at = patch_index(P, a, img0 + g, ci, fy, fx);
+  else if (kSplit) *at = (size_t)img0 * P.c * P.fpx + (size_t)ci * 4 * P.fpx + (size_t)fy * 2 * P.fw + fx;
+  else *at = (size_t)(img0 + g) * per_img + r;
   *d0 = (ci * 4 + (y & 1) * 2) * P.pg + g * P.px + (y >> 1) * P.w + (x >> 1);
 }
 
 // logical element e (a multiple of four) of the level's channels -> its place in z, in the kept channels
 // (stride `keep_stride` per image) and in the flow variable
-template <typename Fn>
-__device__ __forceinline__ void split_map(const FlowPlan& P, const LevelArgs& a, const int32_t* col_out, int img0, int e,
+template <bool kSplit, typename Fn>
+__device__ __forceinline__ void split_map(const Flow& f, const FlowPlan& P, const LevelArgs& a, const int32_t* col_out, int img0, int e,
                                           int32_t* keep, size_t keep_stride, Fn fn) {
   const int per_img = P.c * P.px;
   const int g = fdiv(e, P.mul_per_img), r = e - g * per_img;
   const int k = fdiv(r, P.mul_px), q = r - k * P.px;
   const size_t b = (size_t)(img0 + g);
-  int32_t* dst = k >= P.keep_c ? a.z + b * P.d + P.z_off + (size_t)(k - P.keep_c) * P.px + q
-                               : keep + b * keep_stride + (size_t)k * P.px + q;
+  int at = q, plane = P.px;
+  if constexpr (kSplit) {
+    const int y = fdiv(q, P.mul_w), x = q - y * P.w;
+    at = (f.by * P.h + y) * P.fw + f.bx * P.w + x;
+    plane = P.fpx;
+  }
+  int32_t* dst = k >= P.keep_c ? a.z + b * P.d + P.z_off + (size_t)(k - P.keep_c) * plane + at
+                               : keep + b * keep_stride + (size_t)k * plane + at;
   fn(k, dst, col_out[k] * P.pg + g * P.px + q);
 }
 
-template <bool kInv>
+template <bool kInv, bool kSplit>
 __device__ __forceinline__ void flow_load(const Flow& f, const FlowPlan& P, const LevelArgs& a, int img0, int32_t* v) {
   const int n = f.nimg * P.c * P.px;
   if (!kInv) {
 #pragma unroll 1
     for (int e = 4 * f.tid; e < n; e += 4 * kFlowWorkers) {
       size_t at; int d0;
-      squeeze_map(P, a, img0, e, &at, &d0);
+      squeeze_map<kSplit>(f, P, a, img0, e, &at, &d0);
       int4 q;
       if (P.is_first) {
         const uint32_t b4 = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint8_t*>(a.in) + at);
@@ -743,29 +857,29 @@ __device__ __forceinline__ void flow_load(const Flow& f, const FlowPlan& P, cons
     int32_t* keep = const_cast<int32_t*>(reinterpret_cast<const int32_t*>(a.in));
 #pragma unroll 1
     for (int e = 4 * f.tid; e < n; e += 4 * kFlowWorkers)
-      split_map(P, a, a.plan->col_out, img0, e, keep, (size_t)a.in_stride, [&](int k, const int32_t* src, int d) {
+      split_map<kSplit>(f, P, a, a.plan->col_out, img0, e, keep, (size_t)a.in_stride, [&](int k, const int32_t* src, int d) {
         // (prior head only: z's block is not read)
         if (a.phase != 1 || k < P.keep_c) *reinterpret_cast<int4*>(v + d) = *reinterpret_cast<const int4*>(src);
       });
   }
 }
 
-template <bool kInv>
+template <bool kInv, bool kSplit>
 __device__ __forceinline__ void flow_store(const Flow& f, const FlowPlan& P, const LevelArgs& a, int img0, const int32_t* v) {
   const int n = f.nimg * P.c * P.px;
   if (!kInv) {
     int32_t* keep = P.is_last ? a.z + P.z_final_off : reinterpret_cast<int32_t*>(a.out);
-    const size_t keep_stride = P.is_last ? (size_t)P.d : (size_t)P.keep_c * P.px;
+    const size_t keep_stride = P.is_last ? (size_t)P.d : (size_t)P.keep_c * P.fpx;
 #pragma unroll 1
     for (int e = 4 * f.tid; e < n; e += 4 * kFlowWorkers)
-      split_map(P, a, a.plan->col_out, img0, e, keep, keep_stride,
+      split_map<kSplit>(f, P, a, a.plan->col_out, img0, e, keep, keep_stride,
                 [&](int, int32_t* dst, int d) { *reinterpret_cast<int4*>(dst) = *reinterpret_cast<const int4*>(v + d); });
   } else if (a.phase != 1) {
     uint32_t bad = 0;
 #pragma unroll 1
     for (int e = 4 * f.tid; e < n; e += 4 * kFlowWorkers) {
       size_t at; int d0;
-      squeeze_map(P, a, img0, e, &at, &d0);
+      squeeze_map<kSplit>(f, P, a, img0, e, &at, &d0);
       const int2 x0 = *reinterpret_cast<const int2*>(v + d0), x1 = *reinterpret_cast<const int2*>(v + d0 + P.pg);
       if (P.is_first) {
         *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(a.out) + at) = pack4(x0.x, x1.x, x0.y, x1.y);
@@ -782,18 +896,34 @@ __device__ __forceinline__ void flow_store(const Flow& f, const FlowPlan& P, con
   }
 }
 
-template <bool kInv>
+template <bool kInv, bool kSplit>
 __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const LevelArgs a, const __grid_constant__ FlowPlan P) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ FlowCtl ctl;
   const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
 
   ptx::grid_launch_dependents();         // the next kernel in the stream may start its prologue
-  const int img0 = blockIdx.x * P.group, nimg = min(P.group, a.batch - img0);
+  const int nblk = kSplit ? P.nbx * P.nby : 1;
+  const int img0 = (kSplit ? blockIdx.x / nblk : blockIdx.x) * P.group, nimg = min(P.group, a.batch - img0);
   const int tiles = P.im2col ? (nimg + 3) >> 2 : nimg * P.tiles_img, slots = P.ring ? 1 : min(2, tiles);
+  Flow f;
+  f.halo = 0;
+  f.rank = kSplit ? blockIdx.x % nblk : 0;
+  f.by = kSplit ? f.rank / P.nbx : 0;
+  f.bx = kSplit ? f.rank - f.by * P.nbx : 0;
+  int neighbours = 0;
+  if constexpr (kSplit)
+    for (int dy = -1; dy <= 1; ++dy)
+      for (int dx = -1; dx <= 1; ++dx)
+        if ((dy || dx) && flow_block_exists(P, f, dy, dx)) {
+          ++neighbours;
+          f.halo += (uint32_t)(dx == 0 ? P.w * P.halo_bytes[0] : (dy == 0 ? P.h * P.halo_bytes[1] : P.halo_bytes[2]));
+        }
   if (tid == 0) {
-    ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), (uint32_t)kFlowWarps);
+    ptx::mbar_init(ptx::smem_u32(&ctl.acc_full), 1);
+    ptx::mbar_init(ptx::smem_u32(&ctl.peers_done), (uint32_t)max(neighbours, 1));
     for (int s = 0; s < 2; ++s) {
+      ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready[s]), (uint32_t)kFlowWarps);
       ptx::mbar_init(ptx::smem_u32(&ctl.a_ready[s]), (uint32_t)(kFlowWarps / slots));
       ptx::mbar_init(ptx::smem_u32(&ctl.dm_ready[s]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl.d3_ready[s]), 1);
@@ -811,7 +941,6 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
   __syncthreads();
   ptx::tc_fence_after();
 
-  Flow f;
   f.smem = smem; f.ctl = &ctl; f.status = a.status; f.tmem = ctl.tmem_base;
   f.tid = tid; f.warp = warp; f.lane = lane;
   f.nimg = nimg; f.pvalid = nimg * P.px; f.tiles = tiles; f.slots = slots;
@@ -824,6 +953,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
   st.nsteps = st.n_couplings + (st.do_prior ? 1 : 0);
   st.inverse = kInv;
 
+  if (warp >= kFlowWarps && kSplit) flow_cluster_sync();        // (the workers below, after the frame)
   if (warp == kFlowWarps + 2) {
     // packed blocks: written once, at model creation
     if (lane == 0) {
@@ -863,39 +993,77 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
     }
     for (int o = tid; o < (P.im2col ? 0 : P.cb * P.acc_stride); o += kFlowWorkers) reinterpret_cast<int32_t*>(smem + P.s_acc)[o] = 0;
     int32_t* v = reinterpret_cast<int32_t*>(smem + P.s_v);
+    if constexpr (kSplit) flow_cluster_sync();     // frame, accumulator and barriers are ready for the neighbours
     ptx::grid_dependency_wait();         // from here on: what the previous kernel in the stream wrote
-    flow_load<kInv>(f, P, a, img0, v);
+    flow_load<kInv, kSplit>(f, P, a, img0, v);
     worker_barrier();
-    flow_workers<kInv>(f, P, a, st, img0);
+    flow_workers<kInv, kSplit>(f, P, a, st, img0);
     worker_barrier();
-    flow_store<kInv>(f, P, a, img0, v);
+    flow_store<kInv, kSplit>(f, P, a, img0, v);
   }
   ptx::tc_fence_before();
   __syncthreads();
+  if constexpr (kSplit) flow_cluster_sync();       // nothing is on its way to this CTA's memory any more
   if (warp == 0) ptx::tmem_dealloc(ctl.tmem_base, (uint32_t)P.tmem_cols);
 }
 
 }  // namespace
 
-cudaError_t launch_flow_level(const LevelArgs& args, const FlowPlan& plan, bool inverse, int grid, cudaStream_t stream) {
+namespace {
+template <bool kInv, bool kSplit>
+cudaError_t launch(const LevelArgs& args, const FlowPlan& plan, int grid, cudaStream_t stream) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)kFlowThreads);
   cfg.dynamicSmemBytes = plan.s_total;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)(plan.nbx * plan.nby);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = kSplit ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, flow_level_kernel<kInv, kSplit>, args, plan);
+}
+}  // namespace
+
+cudaError_t launch_flow_level(const LevelArgs& args, const FlowPlan& plan, bool inverse, int grid, cudaStream_t stream) {
+  if (plan.nbx * plan.nby > 1)
+    return inverse ? launch<true, true>(args, plan, grid, stream) : launch<false, true>(args, plan, grid, stream);
+  return inverse ? launch<true, false>(args, plan, grid, stream) : launch<false, false>(args, plan, grid, stream);
+}
+
+int max_flow_clusters(int ctas, uint32_t smem_bytes, uint32_t smem_limit) {
+  if (configure_flow_kernels(smem_limit) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3((unsigned)kFlowThreads);
+  cfg.dynamicSmemBytes = smem_bytes;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return inverse ? cudaLaunchKernelEx(&cfg, flow_level_kernel<true>, args, plan)
-                 : cudaLaunchKernelEx(&cfg, flow_level_kernel<false>, args, plan);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, flow_level_kernel<false, true>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
 }
 
 cudaError_t configure_flow_kernels(uint32_t max_smem_bytes) {
-  cudaError_t e = cudaFuncSetAttribute(flow_level_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem_bytes);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(flow_level_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem_bytes);
+  const auto set = [&](const void* k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem_bytes); };
+  cudaError_t e = set(reinterpret_cast<const void*>(flow_level_kernel<false, false>));
+  if (e == cudaSuccess) e = set(reinterpret_cast<const void*>(flow_level_kernel<true, false>));
+  if (e == cudaSuccess) e = set(reinterpret_cast<const void*>(flow_level_kernel<false, true>));
+  if (e == cudaSuccess) e = set(reinterpret_cast<const void*>(flow_level_kernel<true, true>));
+  return e;
 }
 
 }  // namespace iodf

@@ -16,10 +16,16 @@ constexpr int kFlowMaxRing = 12;                     // slots of the weight ring
 constexpr int kFlowMaxTiles = 32;                    // of a CTA
 constexpr int kFlowMaxSteps = 18;                    // K steps of the first conv
 
+constexpr int kFlowMaxBlocks = 8;                    // CTAs that share an image (portable cluster size)
+
 // Everything about a level that the kernel needs and that is the same for all its couplings; passed
 // by value (constant bank), so that no index computation waits for a global load.
 struct FlowPlan {
-  int32_t c, h, w, px, ca, cb;
+  int32_t c, h, w, px, ca, cb;   // (h, w, px: of the CTA's block where an image is split)
+  int32_t nbx, nby;              // blocks of an image; more than one: a cluster of CTAs, group = 1
+  int32_t fh, fw, fpx;           // the whole image
+  int32_t halo_bytes[3];         // bytes that a position takes from a neighbour: above / below, beside, at a corner
+  int32_t reds[kFlowMaxBlocks];  // products per channel that block r's neighbours add to its accumulator
   int32_t n_couplings, has_prior, is_first, is_last, keep_c;
   int32_t group;                 // images per CTA
   int32_t pg;                    // pixels of the CTA (group * px): plane stride of the flow variable
@@ -67,6 +73,9 @@ struct FlowMeta {
 static_assert(sizeof(FlowMeta) == 128, "meta header is 128 bytes");
 
 cudaError_t configure_flow_kernels(uint32_t max_smem_bytes);
+// clusters of `ctas` CTAs that can be resident at once (0 if that cannot be determined); smem_limit: what the
+// device allows a block
+int max_flow_clusters(int ctas, uint32_t smem_bytes, uint32_t smem_limit);
 cudaError_t launch_flow_level(const LevelArgs& args, const FlowPlan& plan, bool inverse, int grid, cudaStream_t stream);
 
 }  // namespace iodf

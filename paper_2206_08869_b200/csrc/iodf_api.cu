@@ -1215,6 +1215,9 @@ int pack_residual_level(const iodf_level_desc& lv, const Blobs& B, LevelPlan& P,
   return IODF_OK;
 }
 
+// n / d = umulhi(n, magic(d)) for n * d < 2^32 (0: d = 1)
+uint32_t magic(uint64_t d) { return d <= 1 ? 0u : (uint32_t)(((1ull << 32) + d - 1) / d); }
+
 // Packs a level for the compact kernel, if that can run it.
 bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, const std::vector<std::vector<int>>& cols,
                      const std::vector<std::array<HiddenOrder, 2>>& orders, uint32_t smem_limit, uint32_t max_batch,
@@ -1222,7 +1225,8 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   LevelPlan& P = hl.plan;
   FlowPlan& F = hl.flow;
   std::memset(&F, 0, sizeof(F));
-  F.c = P.c; F.h = P.h; F.w = P.w; F.px = P.px; F.ca = P.ca; F.cb = P.cb;
+  F.c = P.c; F.h = F.fh = P.h; F.w = F.fw = P.w; F.px = F.fpx = P.px; F.ca = P.ca; F.cb = P.cb;
+  F.nbx = F.nby = 1;
   F.n_couplings = P.n_couplings; F.has_prior = P.has_prior; F.is_first = P.is_first; F.is_last = P.is_last; F.keep_c = P.keep_c;
   F.mul_per_img = P.mul_per_img; F.mul_4px = P.mul_4px; F.mul_w2 = P.mul_w2; F.mul_px = P.mul_px; F.mul_w = P.mul_w;
   F.z_off = (int64_t)P.z_off; F.prior_off = (int64_t)P.prior_off; F.z_final_off = (int64_t)P.z_final_off;
@@ -1260,8 +1264,53 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   if (lv.has_prior) add(prior, &P.prior);
   // resident weights where they and the accumulators of two tiles fit; streaming them costs a copy of 16 - 64 KB per GEMM
   // and tile, which one tile's chain of GEMMs does not hide
-  return (nd.n_hidden <= 256 && plan_flow(F, nd, smem_limit, max_batch, num_sms, throughput, false)) ||
-         plan_flow(F, nd, smem_limit, max_batch, num_sms, throughput, true);
+  auto plan = [&](FlowPlan& f) {
+    return (nd.n_hidden <= 256 && plan_flow(f, nd, smem_limit, max_batch, num_sms, throughput, false)) ||
+           plan_flow(f, nd, smem_limit, max_batch, num_sms, throughput, true);
+  };
+  const FlowPlan whole = F;
+  if (!plan(F)) return false;
+  if (throughput || F.im2col || F.tiles_img < 2) return true;
+  // The latency plan splits images over clusters of CTAs where that shortens a full batch. A coupling takes about
+  // `chain` for its serial part, `tile` for each tile of the CTA and `edges` for the exchange with neighbours, in
+  // thousands of clocks: a 32 x 32 level at widths around 90 measured 161, 108, 71 and 56 us in 1, 2, 4 and 8 blocks, one
+  // with streamed weights at width 512 712, 380, 204 and 113 us.
+  auto cost = [&](const FlowPlan& f, int slots) {
+    const double chain = f.ring ? 1.8 : 4.7, tile = f.ring ? 20 : 3.9, edges = f.nbx * f.nby > 1 ? 3.5 : 0;
+    return (double)(((int)max_batch + slots - 1) / slots) * (chain + tile * f.tiles + edges);
+  };
+  double best = cost(F, num_sms);
+  const int th = whole.h % 16 == 0 ? 16 : 8;
+  for (int nbx = 1; nbx <= whole.w / 8; ++nbx)
+    for (int nby = 1; nby <= whole.h / th && nbx * nby <= kFlowMaxBlocks; ++nby) {
+      if (nbx * nby == 1 || whole.w % (8 * nbx) || whole.h % (th * nby)) continue;
+      FlowPlan f = whole;
+      f.nbx = nbx; f.nby = nby;
+      f.w = whole.w / nbx; f.h = whole.h / nby; f.px = f.w * f.h;
+      f.mul_per_img = magic((uint64_t)f.c * f.px); f.mul_4px = magic(4ull * f.px); f.mul_w2 = magic(2ull * f.w);
+      f.mul_px = magic((uint64_t)f.px); f.mul_w = magic((uint64_t)f.w);
+      std::vector<KByte> k2;
+      if (!flow_geometry(f, k2) || f.m != F.m || !plan(f) || f.group != 1) continue;
+      const int slots = max_flow_clusters(nbx * nby, f.s_total, smem_limit);
+      if (slots < 1 || cost(f, slots) >= best) continue;
+      const int words = (f.ca + 3) / 4;
+      f.halo_bytes[0] = words * (f.paired ? 8 : 4);
+      f.halo_bytes[1] = f.halo_bytes[2] = words * 4;
+      // products that cross a block's border: those of a lane quarter's rows (and the one above and below) in the
+      // three columns around each of the tile's eight
+      const int rows = f.m / 32;
+      for (int y0 = 0; y0 < whole.h; y0 += rows)
+        for (int x = 0; x < whole.w; ++x)
+          for (int y = y0 - 1; y <= y0 + rows; ++y)
+            for (int dx = -1; dx <= 1; ++dx) {
+              if (y < 0 || y >= whole.h || x + dx < 0 || x + dx >= whole.w) continue;
+              const int from = y0 / f.h * nbx + x / f.w, to = y / f.h * nbx + (x + dx) / f.w;
+              if (from != to) ++f.reds[to];
+            }
+      best = cost(f, slots);
+      F = f;
+    }
+  return true;
 }
 
 int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_model* m) {
@@ -1387,7 +1436,6 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
     P.d = lay.d; P.d_fact = lay.d_fact;
 
     P.cpad = (int)up(ca, 8); P.cbp = (int)up(cb, 8);
-    auto magic = [](uint64_t d) -> uint32_t { return d <= 1 ? 0u : (uint32_t)(((1ull << 32) + d - 1) / d); };
     P.mul_per_img = magic((uint64_t)c * h * w); P.mul_4px = magic(4ull * h * w); P.mul_w2 = magic(2ull * w);
     P.mul_px = magic((uint64_t)h * w); P.mul_w = magic(w);
     P.recip_gpa = 65536u / (uint32_t)(P.cpad / 8) + 1u;
@@ -1550,7 +1598,7 @@ void set_patch_grid(LevelArgs& a, const PatchGrid& g) {
 cudaError_t launch_any_level(const HostLevel& hl, const LevelArgs& a, bool inverse, int B, cudaStream_t st) {
   const LevelPlan& P = hl.plan;
   const int grid = (B + P.group - 1) / P.group;
-  if (hl.use_flow) return launch_flow_level(a, hl.flow, inverse, grid, st);
+  if (hl.use_flow) return launch_flow_level(a, hl.flow, inverse, grid * hl.flow.nbx * hl.flow.nby, st);
   if (hl.use_rf) return launch_res_flow(a, hl.rf, inverse, grid * hl.rf.nbx * hl.rf.nby, st);
   if (P.residual) return launch_res_level(a, inverse, grid, P.res_bands, P.s_total, st);
   return launch_level(a, inverse, P.lean != 0, grid, P.s_total, st);

@@ -19,6 +19,10 @@ pytestmark = pytest.mark.gpu
     (48, [True], 16, 2),                 # 24 x 24: nine 64-row tiles
     (32, [False, True], 256, 2),         # the widest that can be resident
     (64, [True], 200, 1),                # eight tiles whose accumulators do not fit side by side: streamed
+    (64, [True, True], 48, 1),           # 32 x 32 in eight blocks of one tile, then 16 x 16
+    (64, [True], 48, 20),                # ... in four of two tiles
+    (64, [False], 40, 40),               # ... in two of four
+    (48, [True], 300, 2),                # 24 x 24 in blocks of 64-row tiles, streamed weights
     (64, [True, True], 257, 1),          # the narrowest streamed weights, eight tiles
     (16, [True, True], 512, 6),          # the widest; 4 x 4 level with two ragged groups
 ])
