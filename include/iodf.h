@@ -427,7 +427,7 @@ int iodf_int8_mma_peak(iodf_model* m, uint32_t mma_groups, void* cuda_stream, un
 const char* iodf_level_kernel_name(const iodf_model* m, int level);
 
 /* Images that one CTA of level `level`'s launch holds under the model's plan (1 where an image takes a
- * CTA, or a band of a cluster, of its own); a launch of B images has ceil(B / that) CTAs per band.
+ * CTA, or a band of a cluster, of its own); a launch of max_batch images has ceil(max_batch / that) CTAs per band.
  * IODF_EINVAL for a bad argument. */
 int iodf_level_images_per_cta(const iodf_model* m, int level);
 

@@ -31,8 +31,10 @@ inline uint32_t up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 
 struct HostLevel {
   LevelPlan plan;
-  FlowPlan flow;                     // levels that run in the compact kernel (use_flow)
-  bool use_flow = false;
+  // levels that run in the compact kernel: the launch shapes it has been laid out for, all on the same packed weights. A
+  // launch takes the one that is best for its batch.
+  struct FlowShape { FlowPlan plan; int ctas; double cost; };     // CTAs (clusters) at once; time of one wave
+  std::vector<FlowShape> flow;
   RfPlan rf;                         // residual levels that run in the overlapped kernel (use_rf)
   bool use_rf = false;
   std::vector<uint8_t> blob;
@@ -934,86 +936,79 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
 // Group, tensor-memory columns and shared-memory layout of a level in the compact kernel. false: it does not fit.
 struct FlowNeeds { uint32_t n_hidden = 32, n_taps = 16, kb = 1, meta = 16, w[3] = {16, 16, 16}; };
 // wide: weights streamed for every tile, one tile in flight.
-bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, uint32_t max_batch, int num_sms, bool throughput, bool wide) {
-  int group = F.px >= kTileM ? 1 : kTileM / F.px;
-  if (F.im2col) group = std::min(group, 4);            // an image per lane quarter
-  group = std::max(1, std::min<int>(group, (int)max_batch));
-  // the latency plan keeps groups small while the CTAs of a full batch would not fill the SMs
-  while (!throughput && group > 1 && ((int)max_batch + group - 1) / group < num_sms) group /= 2;
-  for (; group >= 1; group /= 2) {
-    F.group = group;
-    F.pg = group * F.px;
-    F.tiles = F.im2col ? (group + 3) / 4 : group * F.tiles_img;
-    const uint32_t nh = up(nd.n_hidden, 16), nh32 = up(nd.n_hidden, 32);
-    if (nd.n_hidden > 512 || nd.n_taps > 512 || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
-      continue;
-    F.d_col = 0; F.d3_col = 0; F.d3_step = 0;
-    if (wide) {
-      F.tmem_cols = 512;
-    } else if (F.tiles == 1) {
-      F.tmem_cols = (int)pow2_cols(std::max(std::max(nh32, nd.n_taps), (uint32_t)F.n_prior));
+bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool wide) {
+  F.group = group;
+  F.pg = group * F.px;
+  F.tiles = F.im2col ? (group + 3) / 4 : group * F.tiles_img;
+  const uint32_t nh = up(nd.n_hidden, 16), nh32 = up(nd.n_hidden, 32);
+  if (nd.n_hidden > 512 || nd.n_taps > 512 || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
+    return false;
+  F.d_col = 0; F.d3_col = 0; F.d3_step = 0;
+  if (wide) {
+    F.tmem_cols = 512;
+  } else if (F.tiles == 1) {
+    F.tmem_cols = (int)pow2_cols(std::max(std::max(nh32, nd.n_taps), (uint32_t)F.n_prior));
+  } else {
+    // several tiles: two slots; with more than two tiles the per-tap partials need columns of their own, because
+    // a slot's next tile starts before its shifted sum
+    const bool apart = 2 * nh + 2 * nd.n_taps <= 512u && nh + nh32 <= 512u;
+    if (!apart && (F.tiles > 2 || std::max(nh32, nd.n_taps) > 256u)) return false;
+    F.d_col = apart ? (int)nh : 256;
+    F.d3_col = apart ? 2 * (int)nh : 0;
+    F.d3_step = apart ? (int)nd.n_taps : 256;
+    F.tmem_cols = 512;
+  }
+  F.pitch = F.m * 16 + 64;
+  F.acc_stride = F.pg + 4;
+  for (int alias = 0; alias < 2; ++alias) {
+    if (alias && (F.tiles > 2 || wide)) continue;
+    uint32_t off = 0;
+    auto take = [&](uint32_t bytes) { const uint32_t o = off; off = up(off + bytes, kAlign); return o; };
+    F.alias = alias;
+    F.s_v = take((uint32_t)F.c * F.pg * 4);
+    if (F.im2col) {
+      F.plane16 = 16 * group;
+      F.s_xa = take((uint32_t)(F.rec / 16) * F.plane16 * 16 + 64 * 16);       // a tile's 64 rows read past a short last plane
     } else {
-      // several tiles: two slots; with more than two tiles the per-tap partials need columns of their own, because
-      // a slot's next tile starts before its shifted sum
-      const bool apart = 2 * nh + 2 * nd.n_taps <= 512u && nh + nh32 <= 512u;
-      if (!apart && (F.tiles > 2 || std::max(nh32, nd.n_taps) > 256u)) continue;
-      F.d_col = apart ? (int)nh : 256;
-      F.d3_col = apart ? 2 * (int)nh : 0;
-      F.d3_step = apart ? (int)nd.n_taps : 256;
-      F.tmem_cols = 512;
+      F.plane16 = group * F.frame;
+      F.s_xa = take((uint32_t)(F.rec / 16) * F.plane16 * 16);
     }
-    F.pitch = F.m * 16 + 64;
-    F.acc_stride = F.pg + 4;
-    for (int alias = 0; alias < 2; ++alias) {
-      if (alias && (F.tiles > 2 || wide)) continue;
-      uint32_t off = 0;
-      auto take = [&](uint32_t bytes) { const uint32_t o = off; off = up(off + bytes, kAlign); return o; };
-      F.alias = alias;
-      F.s_v = take((uint32_t)F.c * F.pg * 4);
-      if (F.im2col) {
-        F.plane16 = 16 * group;
-        F.s_xa = take((uint32_t)(F.rec / 16) * F.plane16 * 16 + 64 * 16);       // a tile's 64 rows read past a short last plane
-      } else {
-        F.plane16 = group * F.frame;
-        F.s_xa = take((uint32_t)(F.rec / 16) * F.plane16 * 16);
-      }
-      F.s_xa_end = off;
-      F.s_acc = F.im2col ? 0 : take((uint32_t)F.cb * F.acc_stride * 4);
-      const uint32_t a_bytes = 2u * nd.kb * F.pitch;
-      F.s_a[0] = take(a_bytes);
-      F.s_a[1] = F.tiles > 1 && !wide ? take(a_bytes) : F.s_a[0];
-      F.s_meta[0] = take(nd.meta);
-      F.s_meta[1] = take(nd.meta);
-      if (wide) {          // a ring of K steps in what is left: at least three, so that copies and MMAs overlap
-        F.ring_slot_bytes = up(32u * std::max(nd.n_hidden, std::max(nd.n_taps, (uint32_t)F.n_prior)), kAlign);
-        F.s_w[0] = F.s_w[1] = F.s_w[2] = off;
-        if (off + 3 * F.ring_slot_bytes > limit) continue;
-        F.ring = std::min<int>(kFlowMaxRing, (int)((limit - off) / F.ring_slot_bytes));
-        off += (uint32_t)F.ring * F.ring_slot_bytes;
-      } else {
-        F.s_w[0] = take(alias ? std::max(nd.w[0], nd.w[2]) : nd.w[0]);
-        F.s_w[1] = take(nd.w[1]);
-        F.s_w[2] = alias ? F.s_w[0] : take(nd.w[2]);
-      }
-      F.s_total = off;
-      if (off > limit) continue;
-      // operand chunks of the first conv's K steps, now that the planes' distance is known
-      for (int st = 0; st < F.ks1; ++st) {
-        auto chunk = [&](int ck) -> int {
-          if (F.im2col) return ck * F.plane16;
-          const int tap = ck % 9;
-          return (tap / 3 - 1) * F.wp + (tap % 3 - 1) + (ck / 9) * F.plane16;
-        };
-        if (F.paired) {
-          F.step[st] = (uint32_t)((st - 1) * F.wp - 1) + (2u << 16);
-          continue;
-        }
-        const int chunks = F.im2col ? F.rec / 16 : 9 * (F.rec / 16);
-        const int lbo = 2 * st + 1 < chunks ? chunk(2 * st + 1) - chunk(2 * st) : 1;       // (the last may be half used)
-        F.step[st] = (uint32_t)chunk(2 * st) + ((uint32_t)lbo << 16);
-      }
-      return true;
+    F.s_xa_end = off;
+    F.s_acc = F.im2col ? 0 : take((uint32_t)F.cb * F.acc_stride * 4);
+    const uint32_t a_bytes = 2u * nd.kb * F.pitch;
+    F.s_a[0] = take(a_bytes);
+    F.s_a[1] = F.tiles > 1 && !wide ? take(a_bytes) : F.s_a[0];
+    F.s_meta[0] = take(nd.meta);
+    F.s_meta[1] = take(nd.meta);
+    if (wide) {          // a ring of K steps in what is left: at least three, so that copies and MMAs overlap
+      F.ring_slot_bytes = up(32u * std::max(nd.n_hidden, std::max(nd.n_taps, (uint32_t)F.n_prior)), kAlign);
+      F.s_w[0] = F.s_w[1] = F.s_w[2] = off;
+      if (off + 3 * F.ring_slot_bytes > limit) continue;
+      F.ring = std::min<int>(kFlowMaxRing, (int)((limit - off) / F.ring_slot_bytes));
+      off += (uint32_t)F.ring * F.ring_slot_bytes;
+    } else {
+      F.s_w[0] = take(alias ? std::max(nd.w[0], nd.w[2]) : nd.w[0]);
+      F.s_w[1] = take(nd.w[1]);
+      F.s_w[2] = alias ? F.s_w[0] : take(nd.w[2]);
     }
+    F.s_total = off;
+    if (off > limit) continue;
+    // operand chunks of the first conv's K steps, now that the planes' distance is known
+    for (int st = 0; st < F.ks1; ++st) {
+      auto chunk = [&](int ck) -> int {
+        if (F.im2col) return ck * F.plane16;
+        const int tap = ck % 9;
+        return (tap / 3 - 1) * F.wp + (tap % 3 - 1) + (ck / 9) * F.plane16;
+      };
+      if (F.paired) {
+        F.step[st] = (uint32_t)((st - 1) * F.wp - 1) + (2u << 16);
+        continue;
+      }
+      const int chunks = F.im2col ? F.rec / 16 : 9 * (F.rec / 16);
+      const int lbo = 2 * st + 1 < chunks ? chunk(2 * st + 1) - chunk(2 * st) : 1;       // (the last may be half used)
+      F.step[st] = (uint32_t)chunk(2 * st) + ((uint32_t)lbo << 16);
+    }
+    return true;
   }
   return false;
 }
@@ -1223,7 +1218,8 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
                      const std::vector<std::array<HiddenOrder, 2>>& orders, uint32_t smem_limit, uint32_t max_batch,
                      int num_sms, bool throughput) {
   LevelPlan& P = hl.plan;
-  FlowPlan& F = hl.flow;
+  FlowPlan F0;
+  FlowPlan& F = F0;
   std::memset(&F, 0, sizeof(F));
   F.c = P.c; F.h = F.fh = P.h; F.w = F.fw = P.w; F.px = F.fpx = P.px; F.ca = P.ca; F.cb = P.cb;
   F.nbx = F.nby = 1;
@@ -1264,24 +1260,40 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   if (lv.has_prior) add(prior, &P.prior);
   // resident weights where they and the accumulators of two tiles fit; streaming them costs a copy of 16 - 64 KB per GEMM
   // and tile, which one tile's chain of GEMMs does not hide
-  auto plan = [&](FlowPlan& f) {
-    return (nd.n_hidden <= 256 && plan_flow(f, nd, smem_limit, max_batch, num_sms, throughput, false)) ||
-           plan_flow(f, nd, smem_limit, max_batch, num_sms, throughput, true);
+  auto plan = [&](FlowPlan& f, int group) {
+    if ((uint64_t)group * f.c * f.fpx * ((uint64_t)f.c * f.fpx) >= (1ull << 32)) return false;      // (the index maps' divisions)
+    return (nd.n_hidden <= 256 && plan_flow(f, nd, smem_limit, group, false)) || plan_flow(f, nd, smem_limit, group, true);
   };
-  const FlowPlan whole = F;
-  if (!plan(F)) return false;
-  if (throughput || F.im2col || F.tiles_img < 2) return true;
-  // The latency plan splits images over clusters of CTAs where that shortens a full batch. A coupling takes about
-  // `chain` for its serial part, `tile` for each tile of the CTA and `edges` for the exchange with neighbours, in
-  // thousands of clocks: a 32 x 32 level at widths around 90 measured 161, 108, 71 and 56 us in 1, 2, 4 and 8 blocks, one
-  // with streamed weights at width 512 712, 380, 204 and 113 us.
-  auto cost = [&](const FlowPlan& f, int slots) {
-    const double chain = f.ring ? 1.8 : 4.7, tile = f.ring ? 20 : 3.9, edges = f.nbx * f.nby > 1 ? 3.5 : 0;
-    return (double)(((int)max_batch + slots - 1) / slots) * (chain + tile * f.tiles + edges);
+  const FlowPlan whole = F0;
+  hl.flow.clear();
+  if (throughput) {
+    // as many images as fill a tile: a little more time for a launch, but a half to a quarter of the CTAs
+    const int full = whole.im2col ? 4 : std::max(1, kTileM / whole.px);
+    for (int group = std::min<int>(full, (int)max_batch); group >= 1; group /= 2) {
+      FlowPlan f = whole;
+      if (!plan(f, group)) continue;
+      hl.flow.push_back({f, num_sms, 1.0});
+      return true;
+    }
+    return false;
+  }
+  // The latency plan keeps every shape that fits and a launch picks the fastest for its batch: whole images, one or several
+  // per CTA (fewer waves when images outnumber SMs), or images split over clusters of CTAs (idle SMs
+  // otherwise). A coupling takes about `chain` for its serial part, `tile` for each tile of the CTA, `image` for what an
+  // image more costs at 4 x 4 and `edges` for the exchange with neighbours, in thousands of clocks: a 32 x 32 level at widths
+  // around 90 measured 161, 108, 71 and 56 us in 1, 2, 4 and 8 blocks, the 16 x 16 and 8 x 8 ones (two tiles
+  // and one) 63 and 48; one with streamed weights at width 512 712, 380, 204 and 113 us.
+  auto add_shape = [&](const FlowPlan& f, int ctas) {
+    const double chain = f.ring ? 1.8 : 8, tile = f.ring ? 20 : 3.7, edges = f.nbx * f.nby > 1 ? (f.ring ? 3.5 : 1.5) : 0;
+    hl.flow.push_back({f, ctas, chain + tile * f.tiles + edges + (f.im2col ? 0.5 * f.group : 0)});
   };
-  double best = cost(F, num_sms);
+  for (int group = 1; group <= std::min<int>(8, (int)max_batch); group *= 2) {
+    FlowPlan f = whole;
+    if (plan(f, group)) add_shape(f, num_sms);
+  }
+  if (hl.flow.empty()) return false;
   const int th = whole.h % 16 == 0 ? 16 : 8;
-  for (int nbx = 1; nbx <= whole.w / 8; ++nbx)
+  for (int nbx = 1; !whole.im2col && nbx <= whole.w / 8; ++nbx)
     for (int nby = 1; nby <= whole.h / th && nbx * nby <= kFlowMaxBlocks; ++nby) {
       if (nbx * nby == 1 || whole.w % (8 * nbx) || whole.h % (th * nby)) continue;
       FlowPlan f = whole;
@@ -1290,9 +1302,9 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
       f.mul_per_img = magic((uint64_t)f.c * f.px); f.mul_4px = magic(4ull * f.px); f.mul_w2 = magic(2ull * f.w);
       f.mul_px = magic((uint64_t)f.px); f.mul_w = magic((uint64_t)f.w);
       std::vector<KByte> k2;
-      if (!flow_geometry(f, k2) || f.m != F.m || !plan(f) || f.group != 1) continue;
-      const int slots = max_flow_clusters(nbx * nby, f.s_total, smem_limit);
-      if (slots < 1 || cost(f, slots) >= best) continue;
+      if (!flow_geometry(f, k2) || f.m != whole.m || !plan(f, 1)) continue;
+      const int clusters = max_flow_clusters(nbx * nby, f.s_total, smem_limit);
+      if (clusters < 1) continue;
       const int words = (f.ca + 3) / 4;
       f.halo_bytes[0] = words * (f.paired ? 8 : 4);
       f.halo_bytes[1] = f.halo_bytes[2] = words * 4;
@@ -1307,10 +1319,21 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
               const int from = y0 / f.h * nbx + x / f.w, to = y / f.h * nbx + (x + dx) / f.w;
               if (from != to) ++f.reds[to];
             }
-      best = cost(f, slots);
-      F = f;
+      add_shape(f, clusters);
     }
   return true;
+}
+
+// the launch shape of the compact kernel that is fastest for a batch (the first of equals: fewer CTAs)
+const FlowPlan& flow_shape(const HostLevel& hl, int batch) {
+  const HostLevel::FlowShape* best = nullptr;
+  double least = 0;
+  for (const HostLevel::FlowShape& f : hl.flow) {
+    const int ctas = (batch + f.plan.group - 1) / f.plan.group;
+    const double t = (double)((ctas + f.ctas - 1) / f.ctas) * f.cost;
+    if (!best || t < least) { best = &f; least = t; }
+  }
+  return best->plan;
 }
 
 int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_model* m) {
@@ -1486,10 +1509,9 @@ int build_model(const iodf_model_desc* desc, const Blobs& B, int device, iodf_mo
     // the index maps divide numbers below group * c * px by at most c * px with a 32-bit magic multiplier
     auto index_maps_fit = [&](int group) { return (uint64_t)group * c * h * w * ((uint64_t)c * h * w) < (1ull << 32); };
     if (all_folded && plan_flow_level(lv, B, hl, cols, orders, (uint32_t)smem_limit, desc->max_batch, num_sms,
-                                     desc->plan == IODF_PLAN_THROUGHPUT) &&
-        index_maps_fit(hl.flow.group)) {
-      hl.use_flow = true;
-      P.group = hl.flow.group; P.s_total = hl.flow.s_total;
+                                     desc->plan == IODF_PLAN_THROUGHPUT)) {
+      const FlowPlan& f = flow_shape(hl, (int)desc->max_batch);
+      P.group = f.group; P.s_total = f.s_total;
       if (lv.split) c = (uint32_t)ca;
       continue;
     }
@@ -1598,7 +1620,10 @@ void set_patch_grid(LevelArgs& a, const PatchGrid& g) {
 cudaError_t launch_any_level(const HostLevel& hl, const LevelArgs& a, bool inverse, int B, cudaStream_t st) {
   const LevelPlan& P = hl.plan;
   const int grid = (B + P.group - 1) / P.group;
-  if (hl.use_flow) return launch_flow_level(a, hl.flow, inverse, grid * hl.flow.nbx * hl.flow.nby, st);
+  if (!hl.flow.empty()) {
+    const FlowPlan& f = flow_shape(hl, B);
+    return launch_flow_level(a, f, inverse, (B + f.group - 1) / f.group * f.nbx * f.nby, st);
+  }
   if (hl.use_rf) return launch_res_flow(a, hl.rf, inverse, grid * hl.rf.nbx * hl.rf.nby, st);
   if (P.residual) return launch_res_level(a, inverse, grid, P.res_bands, P.s_total, st);
   return launch_level(a, inverse, P.lean != 0, grid, P.s_total, st);
@@ -2234,7 +2259,7 @@ int iodf_int8_mma_peak(iodf_model* m, uint32_t mma_groups, void* cuda_stream, un
 const char* iodf_level_kernel_name(const iodf_model* m, int level) {
   if (!m || level < 0 || level >= (int)m->levels.size()) return "";
   const LevelPlan& P = m->levels[level].plan;
-  if (m->levels[level].use_flow) return "flow_level_kernel";
+  if (!m->levels[level].flow.empty()) return "flow_level_kernel";
   if (m->levels[level].use_rf) return "res_flow_kernel";
   return P.residual ? "res_level_kernel" : "level_kernel";
 }

@@ -24,13 +24,17 @@ pytestmark = pytest.mark.gpu
     (64, [False], 40, 40),               # ... in two of four
     (48, [True], 300, 2),                # 24 x 24 in blocks of 64-row tiles, streamed weights
     (64, [True, True], 257, 1),          # the narrowest streamed weights, eight tiles
+    (32, [True, True, True], 24, 300),   # more images than SMs: two images of two tiles, two and four of one
+    (16, [True, True], 24, 1190),        # eight images per CTA, the last with six
     (16, [True, True], 512, 6),          # the widest; 4 x 4 level with two ragged groups
 ])
 @pytest.mark.parametrize("plan", [0, 1])
 def test_three_conv_levels(G, hw, splits, hidden, batch, plan):
     model = S.make_model(0xF100 + hw + hidden, 3, hw, hw, splits, 3, hidden)
     x = S.smooth_field_images(0xF200 + hw, batch, hw, hw, 2.0)
-    m, _ = _check_both_ways(G, model, x, plan=plan)
+    m, z = _check_both_ways(G, model, x, plan=plan)
+    few, _ = G.iodf_forward(m, _t(x[-3:]))            # (the launch shape depends on the batch of the call)
+    np.testing.assert_array_equal(few.cpu().numpy(), z[-3:])
     assert {G.iodf_level_kernel_name(m, k) for k in range(len(splits))} == {"flow_level_kernel"}
 
 
