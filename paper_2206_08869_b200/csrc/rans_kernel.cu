@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_encode_kernel(const Ran
 //   * the prior parameters: the (mu, scale index) of the next 32 elements are loaded by the 32 lanes
 //     in one go and handed out by shuffle, so no global-memory latency sits between two symbols;
 //   * the coded words: the lanes hold a window of the stream's next 32 words (the decoder reads the
-//     stream backwards), refilled when used up; a renormalisation is a shuffle.
+//     stream backwards); the three words that a symbol can take are handed out before its search.
 // A stream's latency bounds the decompressor (a block's streams are few and long).
 __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const RansArgs a, int q,
                                                                        const uint16_t* __restrict__ words,
@@ -174,37 +174,34 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const Ran
   if (wid >= (long)a.batch * blk.n_streams) return;
   const int b = (int)(wid / blk.n_streams), j = (int)(wid - (long)b * blk.n_streams), ns = blk.n_streams;
   const long sid = (long)b * a.n_streams + blk.first_stream + j;
-  const long n_el = (blk.n - j + ns - 1) / ns;
+  const int n_el = (int)((blk.n - j + ns - 1) / ns);
   const uint16_t* in = words + sid * a.cap;
-  long pos = min((long)counts[sid], (long)a.cap);      // words not yet consumed: in[0 .. pos)
+  int top = (int)min((long)counts[sid], (long)a.cap);  // words not yet consumed when the window was filled: in[0 .. top)
+  int used = 0;                                        // words taken from the window since
   uint32_t bad = 0;
-  // window of the next 32 words: lane L holds in[top - 1 - L] (0 before the stream's first word)
-  long top = pos;
-  uint32_t win = (top - 1 - lane >= 0) ? in[top - 1 - lane] : 0u;
-  auto next = [&]() -> uint32_t {               // never reads before the stream's first word
-    if (pos <= 0) { bad = 1u; return 0u; }
-    int used = (int)(top - pos);
-    if (used == 32) {
-      top = pos;
-      win = (top - 1 - lane >= 0) ? in[top - 1 - lane] : 0u;
-      used = 0;
-    }
-    --pos;
-    return __shfl_sync(0xFFFFFFFFu, win, used);
-  };
-  uint32_t x = next() << 16;
-  x |= next();
-  int32_t* zb = z + (long)b * a.d + blk.z_off;
+  // window of the next 32 words: lane L holds in[top - 1 - L], 0 before the stream's first word
+  auto fill = [&]() { return top > lane ? (uint32_t)in[top - 1 - lane] : 0u; };
+  uint32_t win = fill();
+  uint32_t x = __shfl_sync(0xFFFFFFFFu, win, 0) << 16 | __shfl_sync(0xFFFFFFFFu, win, 1);
+  used = 2;
+  int32_t* zb = z + (long)b * a.d + blk.z_off + j;
   const int32_t* pb = prior + (long)b * 2 * a.d_fact;
-  for (long i0 = 0; i0 < n_el; i0 += 32) {
+  for (int i0 = 0; i0 < n_el; i0 += 32) {
     // this lane's element of the next 32: its prior parameters now, its decoded value at the end
     int32_t mu_l = 0, zv_l = 0;
     int ls_l = a.final_ls;
-    if (i0 + lane < n_el) prior_of(a, blk, pb, j + (i0 + lane) * ns, &mu_l, &ls_l, &bad);
+    if (i0 + lane < n_el) prior_of(a, blk, pb, j + (long)(i0 + lane) * ns, &mu_l, &ls_l, &bad);
     const uint32_t R_l = t.R[ls_l];
-    const int n_here = (int)min(32l, n_el - i0);
+    const int n_here = min(32, n_el - i0);
     for (int ii = 0; ii < n_here; ++ii) {
-      const int32_t mu = __shfl_sync(0xFFFFFFFFu, mu_l, ii);
+      if (used > 29) {                             // (a symbol takes up to three words)
+        top -= used;
+        used = 0;
+        win = fill();
+      }
+      // what does not depend on the state is on its way during the search
+      const uint32_t w0 = __shfl_sync(0xFFFFFFFFu, win, used), w1 = __shfl_sync(0xFFFFFFFFu, win, used + 1);
+      const uint32_t w2 = __shfl_sync(0xFFFFFFFFu, win, used + 2);
       const int ls = __shfl_sync(0xFFFFFFFFu, ls_l, ii);
       const uint32_t R = __shfl_sync(0xFFFFFFFFu, R_l, ii);
       const uint32_t slot = x & 0xFFFFu;
@@ -212,36 +209,33 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const Ran
       const uint32_t range = __ldg(a.ranges + (ls << 8) + (slot >> 8));
       int k = (int)(range & 0xFFFFu);
       const int count = (int)(range >> 16);
-      if (count > 32) {
+      if (count > 31) {                            // (at most nine are left then)
         const int step = (count + 31) >> 5;
         const unsigned ok = __ballot_sync(0xFFFFFFFFu, cum_of(t, R, k + lane * step) <= slot);   // a prefix of the lanes (Cum is monotone)
         k += (31 - __clz((int)ok)) * step;
       }
       const uint32_t cl = cum_of(t, R, k + lane);
-      const int sel = 31 - __clz((int)__ballot_sync(0xFFFFFFFFu, cl <= slot));
+      const int sel = 31 - __clz((int)__ballot_sync(0xFFFFFFFFu, cl <= slot));       // at most 30
+      const uint32_t C = __shfl_sync(0xFFFFFFFFu, cl, sel), Cn = __shfl_sync(0xFFFFFFFFu, cl, sel + 1);
       k += sel;
-      const uint32_t C = __shfl_sync(0xFFFFFFFFu, cl, sel);
-      const uint32_t Cn = sel < 31 ? __shfl_sync(0xFFFFFFFFu, cl, sel + 1) : cum_of(t, R, k + 1);
-      const uint32_t F = Cn - C;
-      x = F * (x >> 16) + slot - C;
-      if (x < (1u << 16)) x = (x << 16) | next();
-      int32_t zv;
+      x = (Cn - C) * (x >> 16) + slot - C;
+      const bool more = x < (1u << 16);
+      if (more) x = (x << 16) | w0;
+      used += more ? 1 : 0;
+      int32_t zv = (int32_t)((uint32_t)mu_l + (uint32_t)(k - kWin));              // (lane ii's is the one that counts)
       if (k == 0 || k == 2 * kWin) {
-        const uint32_t h = x & 0xFFFFu;
-        x >>= 16;                                  // F = 1, C = slot: x = x / M
-        if (x < (1u << 16)) x = (x << 16) | next();
-        const uint32_t l = x & 0xFFFFu;
-        x >>= 16;
-        if (x < (1u << 16)) x = (x << 16) | next();
-        zv = (int32_t)((h << 16) | l);
-      } else {
-        zv = (int32_t)((long long)mu + (k - kWin));
+        // an escape: two symbols of frequency 1, the value's upper and lower half; each takes the state's lower 16 bits and
+        // a word in their place (x >> 16 is always below 2^16)
+        const uint32_t wa = more ? w1 : w0, wb = more ? w2 : w1;
+        zv = (int32_t)((x << 16) | wa);
+        x = (x & 0xFFFF0000u) | wb;
+        used += 2;
       }
       if (lane == ii) zv_l = zv;
     }
-    if (i0 + lane < n_el) zb[j + (i0 + lane) * ns] = zv_l;
+    if (i0 + lane < n_el) zb[(long)(i0 + lane) * ns] = zv_l;
   }
-  if (pos != 0 || x != (1u << 16)) bad = 1u;     // every word used and the state back at its start
+  if (top != used || x != (1u << 16)) bad = 1u;    // every word used, none missing, and the state back at its start
   bad = __any_sync(0xFFFFFFFFu, bad != 0) ? 1u : 0u;
   if (bad && lane == 0 && a.errors) atomicAdd(a.errors, 1u);
 }
@@ -367,6 +361,8 @@ cudaError_t launch_rans_unpack(const RansArgs& a, const uint8_t* packed, unsigne
 
 static size_t table_smem(const RansArgs& a) { return 4 * (size_t)a.n_scales + 2 * (size_t)(2 * a.umax + 1) + 16; }
 
+// (No programmatic launch of the coder: started under a level's kernel, whose CTAs fill their SMs, the coder's CTAs all land
+// on the few SMs that kernel leaves idle, +110 us on a decompression of 128 images.)
 cudaError_t launch_rans_encode(const RansArgs& a, const int32_t* z, const int32_t* prior, uint16_t* words,
                                uint32_t* counts, cudaStream_t stream) {
   const long total = (long)a.batch * a.n_streams;
