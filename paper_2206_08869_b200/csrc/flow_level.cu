@@ -21,6 +21,19 @@
 //   * CTAs of several tiles have two in flight (slots), each with eight of the sixteen workers and an MMA
 //     warp of its own, so that one slot's hand-overs and MMAs run under the other's requantisation; CTAs of
 //     one tile put all sixteen workers on it. One lane of another warp streams weights and meta blocks.
+//   * Weights that do not fit beside two tiles (hidden widths above 256) go through a ring of K steps, one tile in
+//     flight (P.ring).
+//   * An image may be split over a cluster of CTAs (kSplit): edge pixels of the network input are stored into the
+//     neighbours' frames and products across a border added to their accumulators, both asynchronously; the
+//     receiver's barriers count the bytes, so that no CTA waits for more than it needs. A neighbour's products of
+//     the next coupling cannot come before an edge pixel's sum has been read and cleared: they need the edge
+//     byte that the same thread sends afterwards.
+//
+// What bounds it: the chain of a coupling (about 8 000 clocks) and 3 700 clocks per tile of 128 pixels: requantisation,
+// shifted sum and their hand-overs (52 % of all issue slots at 32 x 32, 39 % at 8 x 8, 24 % at 4 x 4). Measured for eight
+// couplings of widths around 90, 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 161 us,
+// 16 x 16 85 -> 63, 8 x 8 63 -> 48, 4 x 4 70 -> 48; one image, 32 x 32 split in eight: 56. Width 512, 64 images of
+// 32 x 32, split in two: 2 357 -> 380 us.
 #include "flow_level.h"
 #include "level_device.cuh"
 
