@@ -43,11 +43,11 @@ __device__ __forceinline__ uint32_t cum_of(const Tables& t, uint32_t R, int k) {
   return (uint32_t)k + t.G[u + t.umax];
 }
 
-// x / F and x mod F for 0 < F <= 2^16 and x < F 2^16: the quotient is below 2^16, so that x times the float reciprocal of F
+// x / F and x mod F for 0 < F <= 2^16 and x < F 2^16, inv = 1 / F rounded: the quotient is below 2^16, so that x * inv
 // is off by less than one before truncation (three roundings of 2^-24 on a value below 2^16), and two
 // conditional corrections make it exact. A 32-bit division is several times as long, and it sits on the chain.
-__device__ __forceinline__ uint32_t divide(uint32_t x, uint32_t F, uint32_t* rem) {
-  uint32_t q = __float2uint_rz(__uint2float_rz(x) * __frcp_rn(__uint2float_rn(F)));
+__device__ __forceinline__ uint32_t divide(uint32_t x, uint32_t F, float inv, uint32_t* rem) {
+  uint32_t q = __float2uint_rz(__uint2float_rz(x) * inv);
   uint32_t r = x - q * F;
   if ((int32_t)r < 0) { --q; r += F; }
   if (r >= F) { ++q; r -= F; }
@@ -55,9 +55,13 @@ __device__ __forceinline__ uint32_t divide(uint32_t x, uint32_t F, uint32_t* rem
   return q;
 }
 
+// (four bytes at a time and eight loads in flight: one entry after the other the tables took a tenth of a short kernel)
 __device__ __forceinline__ void load_tables(const RansArgs& a, uint16_t* sG, uint32_t* sR) {
-  for (int i = threadIdx.x; i < 2 * a.umax + 1; i += blockDim.x) sG[i] = a.G[i];
-  for (int i = threadIdx.x; i < a.n_scales; i += blockDim.x) sR[i] = a.R[i];
+  const uint32_t* g = reinterpret_cast<const uint32_t*>(a.G);
+#pragma unroll 8
+  for (int i = threadIdx.x; i < a.umax; i += kThreadsPerBlock) reinterpret_cast<uint32_t*>(sG)[i] = g[i];
+  if (threadIdx.x == 0) sG[2 * a.umax] = a.G[2 * a.umax];
+  for (int i = threadIdx.x; i < a.n_scales; i += kThreadsPerBlock) sR[i] = a.R[i];
   __syncthreads();
 }
 
@@ -87,56 +91,70 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_encode_kernel(const Ran
   while (q + 1 < a.n_blocks && s >= a.blocks[q + 1].first_stream) ++q;
   const RansBlock blk = a.blocks[q];
   const int j = s - blk.first_stream, ns = blk.n_streams;
-  const long n_el = (blk.n - j + ns - 1) / ns;
-  const int32_t* zb = z + (long)b * a.d + blk.z_off;
-  const int32_t* pb = prior + (long)b * 2 * a.d_fact;
+  const int n_el = (int)((blk.n - j + ns - 1) / ns);
+  const bool has_prior = blk.prior_off >= 0;
+  const int32_t* zb = z + (long)b * a.d + blk.z_off + j;
+  const int32_t* mub = prior + (has_prior ? (long)b * 2 * a.d_fact + blk.prior_off + j : 0);
+  const int32_t* lsb = mub + a.d_fact;
   uint16_t* out = words + gid * a.cap;
   uint32_t pos = 0, x = 1u << 16, bad = 0;
-  auto push = [&](uint32_t F, uint32_t C) {
-    if ((unsigned long long)x >= ((unsigned long long)F << 16)) {
-      out[pos++] = (uint16_t)(x & 0xFFFFu);
-      x >>= 16;
-    }
-    uint32_t r;
-    const uint32_t q = divide(x, F, &r);
-    x = (q << 16) + r + C;
-  };
   // Elements and prior parameters of the next kAhead symbols are on their way while the current ones are coded:
   // their addresses do not depend on the state, and a trip to memory is longer than several symbols.
-  constexpr int kAhead = 4;
+  constexpr int kAhead = 8;
   int32_t zn[kAhead], mun[kAhead];
   int lsn[kAhead];
-  auto fetch = [&](int s, long i) {
+  auto fetch = [&](int s, int i) {
     zn[s] = 0; mun[s] = 0; lsn[s] = a.final_ls;
     if (i < 0) return;
-    const long e = j + i * ns;
+    const long e = (long)i * ns;
     zn[s] = zb[e];
-    if (blk.prior_off >= 0) {
-      mun[s] = pb[blk.prior_off + e];
-      lsn[s] = pb[a.d_fact + blk.prior_off + e];
+    if (has_prior) {
+      mun[s] = mub[e];
+      lsn[s] = lsb[e];
     }
   };
 #pragma unroll
   for (int s = 0; s < kAhead; ++s) fetch(s, n_el - 1 - s);
-  for (long i0 = n_el - 1; i0 >= 0; i0 -= kAhead) {
+  for (int i0 = n_el - 1; i0 >= 0; i0 -= kAhead) {
+    // counts of the next kAhead symbols, all at once: only the loop below is a chain through the state
+    int32_t zv[kAhead];
+    uint32_t C[kAhead], F[kAhead];
+    float inv[kAhead];
+    bool esc[kAhead];
 #pragma unroll
     for (int s = 0; s < kAhead; ++s) {
-      const long i = i0 - s;
-      if (i < 0) break;
-      const int32_t zv = zn[s], mu = mun[s];
+      const int32_t mu = mun[s];
+      zv[s] = zn[s];
       int ls = lsn[s];
-      fetch(s, i - kAhead);
+      fetch(s, i0 - s - kAhead);
       if (ls < 0 || ls >= a.n_scales) { bad = 1u; ls = ls < 0 ? 0 : a.n_scales - 1; }
-      long long r = (long long)zv - (long long)mu;
-      r = r < -kWin ? -kWin : (r > kWin ? kWin : r);
-      const int k = (int)r + kWin;
-      if (k == 0 || k == 2 * kWin) {
-        push(1u, (uint32_t)zv & 0xFFFFu);
-        push(1u, ((uint32_t)zv >> 16) & 0xFFFFu);
-      }
+      int r;
+      asm("sub.sat.s32 %0, %1, %2;" : "=r"(r) : "r"(zv[s]), "r"(mu));
+      const int k = max(-kWin, min(kWin, r)) + kWin;
       const uint32_t R = t.R[ls];
-      const uint32_t C = cum_of(t, R, k), F = cum_of(t, R, k + 1) - C;
-      push(F, C);
+      C[s] = cum_of(t, R, k);
+      F[s] = cum_of(t, R, k + 1) - C[s];
+      inv[s] = __frcp_rn(__uint2float_rn(F[s]));
+      esc[s] = k == 0 || k == 2 * kWin;
+    }
+#pragma unroll
+    for (int s = 0; s < kAhead; ++s) {
+      if (i0 - s < 0) break;
+      if (esc[s]) {
+        // two symbols of frequency 1, the value's lower and upper half: each moves the state's lower 16 bits out (the state
+        // is never below 2^16) and takes their place
+        out[pos] = (uint16_t)(x & 0xFFFFu);
+        out[pos + 1] = (uint16_t)((uint32_t)zv[s] & 0xFFFFu);
+        x = (x & 0xFFFF0000u) | ((uint32_t)zv[s] >> 16);
+        pos += 2;
+      }
+      if ((x >> 16) >= F[s]) {
+        out[pos++] = (uint16_t)(x & 0xFFFFu);
+        x >>= 16;
+      }
+      uint32_t r;
+      const uint32_t q = divide(x, F[s], inv[s], &r);
+      x = (q << 16) + r + C[s];
     }
   }
   out[pos++] = (uint16_t)(x & 0xFFFFu);
@@ -157,7 +175,7 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_encode_kernel(const Ran
 //     in one go and handed out by shuffle, so no global-memory latency sits between two symbols;
 //   * the coded words: the lanes hold a window of the stream's next 32 words (the decoder reads the
 //     stream backwards); the three words that a symbol can take are handed out before its search.
-// A stream's latency bounds the decompressor (a block's streams are few and long): about 600 clocks per symbol, 41 - 120 us
+// A stream's latency bounds the decompressor (a block's streams are few and long): about 500 clocks per symbol, 36 - 116 us
 // for the blocks of 128 images of 64 x 64 at 128 elements per stream (60 - 170 us with three search rounds).
 __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const RansArgs a, int q,
                                                                        const uint16_t* __restrict__ words,
