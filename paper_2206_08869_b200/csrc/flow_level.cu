@@ -26,8 +26,11 @@
 //   * An image may be split over a cluster of CTAs (kSplit): edge pixels of the network input are stored into the
 //     neighbours' frames and products across a border added to their accumulators, both asynchronously; the
 //     receiver's barriers count the bytes, so that no CTA waits for more than it needs. A neighbour's products of
-//     the next coupling cannot come before an edge pixel's sum has been read and cleared: they need the edge
-//     byte that the same thread sends afterwards.
+//     the next coupling must not come before this CTA's sums have been read and cleared. Nothing in an
+//     asynchronous store orders the stores that its thread made earlier, so one lane per neighbour releases them at
+//     cluster scope: an arrival on the neighbour's network-input barrier after the barrier that ends the
+//     translation, acquired by the neighbour's MMA warp, without whose MMAs there are no products. (Overwriting a
+//     frame needs no release: the MMAs that read it have completed before anything is sent that lets a neighbour go on.)
 //
 // What bounds it: the chain of a coupling (about 8 000 clocks) and 3 700 clocks per tile of 128 pixels: requantisation,
 // shifted sum and their hand-overs (52 % of all issue slots at 32 x 32, 39 % at 8 x 8, 24 % at 4 x 4). Measured for eight
@@ -43,7 +46,7 @@ namespace {
 
 struct __align__(16) FlowCtl {
   uint64_t xa_ready[2];   // workers (and the neighbours' edge bytes) -> MMA warp, loader: network input of an even / odd
-                          // step written (count kFlowWarps; a neighbour may be one step ahead)
+                          // step written (count kFlowWarps and the neighbours' releases; a neighbour may be one step ahead)
   uint64_t acc_full;      // split images: the neighbours' products of a coupling have been added
   uint64_t peers_done;    // split images: the neighbours have read the prior head's input
   uint64_t a_ready[2];    // slot's workers -> its MMA warp: the next hidden operand is written
@@ -85,6 +88,16 @@ __device__ __forceinline__ void flow_wait(const Flow& f, uint64_t* bar, uint32_t
   if (ptx::mbar_test_wait(b, parity) || ptx::mbar_try_wait(b, parity)) return;
   flow_wait_at(b, parity, f.ctl, f.status);
 }
+// for phases that neighbours take part in (split images)
+__device__ __forceinline__ void flow_wait_cluster(const Flow& f, uint64_t* bar, uint32_t parity) {
+  const uint32_t b = ptx::smem_u32(bar);
+  for (uint32_t it = 0; it < kSpinLimit; ++it) {
+    if (ptx::mbar_try_wait_cluster(b, parity)) return;
+    if (*reinterpret_cast<volatile uint32_t*>(&f.ctl->abort)) return;
+  }
+  *reinterpret_cast<volatile uint32_t*>(&f.ctl->abort) = 1;
+  atomicExch(f.status, 1u);
+}
 __device__ __forceinline__ void flow_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(ptx::smem_u32(bar)) : "memory");
 }
@@ -101,8 +114,13 @@ __device__ __forceinline__ void flow_hand_over(const Flow& f, uint64_t* bar, uin
 }
 // the MMA warp's wait for the network input of step i; a neighbour's bytes came through the generic proxy
 __device__ __forceinline__ void flow_wait_input(const Flow& f, int i) {
-  flow_wait(f, &f.ctl->xa_ready[i & 1], (uint32_t)(i >> 1) & 1u);
-  if (f.halo) asm volatile("fence.proxy.async;" ::: "memory");
+  uint64_t* bar = &f.ctl->xa_ready[i & 1];
+  if (!f.halo) {
+    flow_wait(f, bar, (uint32_t)(i >> 1) & 1u);
+  } else {
+    flow_wait_cluster(f, bar, (uint32_t)(i >> 1) & 1u);
+    asm volatile("fence.proxy.async;" ::: "memory");
+  }
 }
 // ---- between the CTAs of a split image ----
 __device__ __forceinline__ uint32_t flow_peer(uint32_t addr, uint32_t rank) {
@@ -123,6 +141,16 @@ __device__ __forceinline__ void flow_cluster_sync() {
 }
 __device__ __forceinline__ bool flow_block_exists(const FlowPlan& P, const Flow& f, int dy, int dx) {
   return (uint32_t)(f.by + dy) < (uint32_t)P.nby && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx;
+}
+
+// Lane L < 9 of the calling warp arrives on barrier `bar` of the neighbour in direction (L / 3 - 1, L % 3 - 1), releasing at
+// cluster scope what this CTA's workers wrote before their last barrier.
+__device__ __forceinline__ void flow_release_to_neighbours(const FlowPlan& P, const Flow& f, uint64_t* bar) {
+  const int dy = f.lane / 3 - 1, dx = f.lane % 3 - 1;
+  if (f.lane < 9 && (dy || dx) && flow_block_exists(P, f, dy, dx))
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                     flow_peer(ptx::smem_u32(bar), (uint32_t)(f.rank + dy * P.nbx + dx))) : "memory");
+  __syncwarp();
 }
 
 __device__ __forceinline__ void worker_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kFlowWorkers) : "memory"); }
@@ -745,7 +773,8 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
   for (int i = 0; i <= st.nsteps; ++i) {
     if (prev && !P.im2col) {
       flow_translate<kInv>(P, pm, prev);
-      if (pm.parts > 1) worker_barrier();       // the network input may read channels that were just updated
+      // the network input may read channels that were just updated; what was cleared is released as a whole
+      if (kSplit || pm.parts > 1) worker_barrier();
     }
     if (i == st.nsteps) break;
     flow_wait(f, &ctl->meta_full[i & 1], (uint32_t)(i >> 1) & 1u);
@@ -754,6 +783,7 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
     const FlowMeta* M = reinterpret_cast<const FlowMeta*>(mb);
     // (the first two words of both kinds of meta block)
     uint64_t* input = &ctl->xa_ready[i & 1];
+    if (kSplit && f.warp == kFlowWarps - 1) flow_release_to_neighbours(P, f, input);
     flow_requant<kSplit>(f, P, pm, input, prior ? a.plan->col_out : reinterpret_cast<const int32_t*>(mb + M->off_colA), M->in_m0, M->in_s);
     flow_hand_over(f, input, kSplit && f.warp == 0 ? f.halo : 0u);
     prev = prior ? nullptr : mb;
@@ -791,17 +821,13 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
     worker_barrier();                           // every product has been added
     if constexpr (kSplit) {
       if (!prior) {
-        flow_wait(f, &ctl->acc_full, npar);
+        flow_wait_cluster(f, &ctl->acc_full, npar);
         npar ^= 1u;
       } else if (i + 1 < st.nsteps) {
         // The next step's edge pixels overwrite what the neighbours' prior heads read. (After a coupling their products
         // say that they are past it.)
-        const int dy = f.lane / 3 - 1, dx = f.lane % 3 - 1;
-        if (f.warp == 0 && f.lane < 9 && (dy || dx) && flow_block_exists(P, f, dy, dx))
-          asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
-                           flow_peer(ptx::smem_u32(&ctl->peers_done), (uint32_t)(f.rank + dy * P.nbx + dx))) : "memory");
-        __syncwarp();
-        flow_wait(f, &ctl->peers_done, 0u);
+        if (f.warp == 0) flow_release_to_neighbours(P, f, &ctl->peers_done);
+        flow_wait_cluster(f, &ctl->peers_done, 0u);
       }
     }
   }
@@ -936,7 +962,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
     ptx::mbar_init(ptx::smem_u32(&ctl.acc_full), 1);
     ptx::mbar_init(ptx::smem_u32(&ctl.peers_done), (uint32_t)max(neighbours, 1));
     for (int s = 0; s < 2; ++s) {
-      ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready[s]), (uint32_t)kFlowWarps);
+      ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready[s]), (uint32_t)(kFlowWarps + neighbours));
       ptx::mbar_init(ptx::smem_u32(&ctl.a_ready[s]), (uint32_t)(kFlowWarps / slots));
       ptx::mbar_init(ptx::smem_u32(&ctl.dm_ready[s]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl.d3_ready[s]), 1);

@@ -38,6 +38,26 @@ def test_three_conv_levels(G, hw, splits, hidden, batch, plan):
     assert {G.iodf_level_kernel_name(m, k) for k in range(len(splits))} == {"flow_level_kernel"}
 
 
+@pytest.mark.parametrize("hw,hidden,batch", [
+    (64, 16, 1),         # 32 x 32 in eight blocks, every one with corners
+    (64, 16, 20),        # ... in four
+    (64, 272, 3),        # ... in eight, streamed weights
+    (32, 16, 9),         # 16 x 16 in two blocks; fewer input words than threads per pixel pair
+])
+def test_split_images_through_long_chains(G, hw, hidden, batch):
+    """Blocks of an image exchange edges and add to one another's accumulators at every coupling; short couplings, as
+    many as a level can have, and the same call again and again: a sum that is added to before it has been cleared, or
+    an edge that comes early, changes the latents."""
+    import torch
+    model = S.make_model(0xF600 + hw + hidden, 3, hw, hw, [True], 32 if hidden < 100 else 4, hidden)
+    x = S.smooth_field_images(0xF700 + hw, batch, hw, hw, 2.0)
+    m, z = _check_both_ways(G, model, x)
+    xt, zt = _t(x), _t(z)
+    for _ in range(20):
+        assert torch.equal(G.iodf_forward(m, xt)[0], zt) and torch.equal(G.iodf_inverse(m, zt), xt)
+    G.iodf_check(m)
+
+
 @pytest.mark.parametrize("hw,splits,couplings,hidden,blocks,prune,batch,plan", [
     (64, [True], 1, 128, 1, None, 1, 0),           # 32 x 32 in eight 8 x 16 blocks
     (64, [True], 1, 128, 1, None, 1, 1),           # ... in four 16 x 16 ones
