@@ -47,6 +47,15 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
   return ok != 0;
 }
 
+// A phase that is known to be complete, read again at cluster scope: acquires what other CTAs released into it.
+__device__ __forceinline__ void mbar_acquire_cluster(uint32_t bar, uint32_t parity) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%0], %1;\n\t}" ::"r"(bar),
+      "r"(parity)
+      : "memory");
+}
+
 // Non-blocking probe of a phase (for a thread that polls several barriers in turn).
 __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;

@@ -72,6 +72,19 @@ def test_residual_levels(G, hw, splits, couplings, hidden, blocks, prune, batch,
     assert {G.iodf_level_kernel_name(m, k) for k in range(len(splits))} == {"res_flow_kernel"}
 
 
+@pytest.mark.parametrize("hidden,batch,plan", [(16, 1, 0), (16, 3, 1), (128, 2, 0)])
+def test_residual_blocks_through_long_chains(G, hidden, batch, plan):
+    """Blocks of an image send their edges after every conv, one conv ahead at most: the same call again and again."""
+    import torch
+    model = S.make_residual_model(0xF800 + hidden, 3, 64, 64, [True], 6 if hidden < 100 else 1, hidden, 4)
+    x = S.smooth_field_images(0xF900, batch, 64, 64, 2.0)
+    m, z, _ = _both_ways(G, model, x, plan=plan)
+    xt, zt = _t(x), _t(z)
+    for _ in range(20):
+        assert torch.equal(G.iodf_forward(m, xt)[0], zt) and torch.equal(G.iodf_inverse(m, zt), xt)
+    G.iodf_check(m)
+
+
 @pytest.mark.parametrize("ls", [0, 20, 40, 63])
 def test_symbol_look_up_at_every_kind_of_scale(G, ls):
     """Residuals over the whole window at one scale: slots that mean one symbol and slots that mean hundreds."""
