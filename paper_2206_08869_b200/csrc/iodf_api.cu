@@ -1239,6 +1239,7 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
     if (lv.couplings[ki].in_s < 1 || !shifts_ok(lv.couplings[ki].layers[2])) return false;
   if (lv.has_prior && (lv.prior_in_s < 1 || !shifts_ok(lv.prior_layer))) return false;
   FlowNeeds nd;
+  double widths = 0;                              // of the hidden layers, padded
   std::vector<PackedBlock> blocks;
   for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) {
     FlowDims d;
@@ -1247,6 +1248,7 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
     nd.n_hidden = std::max<uint32_t>(nd.n_hidden, (uint32_t)std::max(d.n1, d.n2));
     nd.n_taps = std::max<uint32_t>(nd.n_taps, (uint32_t)d.n3);
     nd.kb = std::max<uint32_t>(nd.kb, (uint32_t)std::max(d.ks2, d.ks3));
+    widths += d.n1 + d.n2;
   }
   PackedBlock prior;
   if (lv.has_prior) prior = pack_flow_prior(lv, B, F, kmap);
@@ -1278,14 +1280,18 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
     return false;
   }
   // The latency plan keeps every shape that fits and a launch picks the fastest for its batch: whole images, one or several
-  // per CTA (fewer waves when images outnumber SMs), or images split over clusters of CTAs (idle SMs
-  // otherwise). A coupling takes about `chain` for its serial part, `tile` for each tile of the CTA, `image` for what an
-  // image more costs at 4 x 4 and `edges` for the exchange with neighbours, in thousands of clocks: a 32 x 32 level at widths
-  // around 90 measured 161, 108, 71 and 56 us in 1, 2, 4 and 8 blocks, the 16 x 16 and 8 x 8 ones (two tiles
-  // and one) 63 and 48; one with streamed weights at width 512 712, 380, 204 and 113 us.
+  // per CTA (fewer waves when images outnumber SMs), or images split over clusters of CTAs (idle SMs otherwise). Time of a
+  // wave per coupling, in thousands of clocks: a serial part, a part for each tile of the CTA that grows with the mean
+  // hidden width and the channels that are translated, the exchange of edges, what an image more costs at 4 x 4, and a
+  // share of the level's load and store. Fitted to 399 shapes of 31 flows (widths 16 - 512, 4 - 96 channels, 4 x 4 - 32 x
+  // 32, resident and streamed); over batches of 1 - 1 023 the shape it picks takes 0.1 % longer than the best one on
+  // average and 6 % at most, on 14 other flows 0.4 % and 8 % (constants that did not know the width: 0.6 % and 20 %).
   auto add_shape = [&](const FlowPlan& f, int ctas) {
-    const double chain = f.ring ? 1.8 : 8, tile = f.ring ? 20 : 3.7, edges = f.nbx * f.nby > 1 ? (f.ring ? 3.5 : 1.5) : 0;
-    hl.flow.push_back({f, ctas, chain + tile * f.tiles + edges + (f.im2col ? 0.5 * f.group : 0)});
+    const double width = widths / (200.0 * F.n_couplings), cb = f.cb / 10.0;
+    double cost = 11.0 / F.n_couplings + (f.im2col ? 0.7 * f.group : 0);
+    if (f.ring) cost += 4 + f.tiles * (5.7 + 2.9 * width + 2.9 * cb) + (f.nbx * f.nby > 1 ? 3 : 0);
+    else cost += 5 + 0.5 * width + f.tiles * (2.2 + 1.5 * width + 0.8 * cb) + (f.nbx * f.nby > 1 ? 4.7 : 0);
+    hl.flow.push_back({f, ctas, cost});
   };
   for (int group = 1; group <= std::min<int>(8, (int)max_batch); group *= 2) {
     FlowPlan f = whole;

@@ -58,6 +58,18 @@ def test_split_images_through_long_chains(G, hw, hidden, batch):
     G.iodf_check(m)
 
 
+@pytest.mark.parametrize("hidden,batch,images", [
+    (96, 300, 1),        # three waves of one image 92 us, two of two images 102
+    (96, 512, 2),        # four 121, two 107
+    (256, 256, 2),       # two images, streamed weights 143 us; one image in two blocks, resident 156
+])
+def test_images_per_cta_follow_the_hidden_width(G, hidden, batch, images):
+    """A 16 x 16 level of 24 channels: what a tile costs beside a coupling's serial part decides between more waves
+    and more images per CTA."""
+    m = G.iodf_create(S.make_model(0xFA00, 3, 64, 64, [True, True], 4, hidden), batch)
+    assert G.iodf_level_images_per_cta(m, 1) == images
+
+
 @pytest.mark.parametrize("hw,splits,couplings,hidden,blocks,prune,batch,plan", [
     (64, [True], 1, 128, 1, None, 1, 0),           # 32 x 32 in eight 8 x 16 blocks
     (64, [True], 1, 128, 1, None, 1, 1),           # ... in four 16 x 16 ones
