@@ -1282,15 +1282,15 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   // The latency plan keeps every shape that fits and a launch picks the fastest for its batch: whole images, one or several
   // per CTA (fewer waves when images outnumber SMs), or images split over clusters of CTAs (idle SMs otherwise). Time of a
   // wave per coupling, in thousands of clocks: a serial part, a part for each tile of the CTA that grows with the mean
-  // hidden width and the channels that are translated, the exchange of edges, what an image more costs at 4 x 4, and a
+  // hidden width and the channels that are translated, the exchange of their edges, what an image more costs at 4 x 4, and a
   // share of the level's load and store. Fitted to 399 shapes of 31 flows (widths 16 - 512, 4 - 96 channels, 4 x 4 - 32 x
   // 32, resident and streamed); over batches of 1 - 1 023 the shape it picks takes 0.1 % longer than the best one on
-  // average and 6 % at most, on 14 other flows 0.4 % and 8 % (constants that did not know the width: 0.6 % and 20 %).
+  // average and 7 % at most, on 14 other flows 0.4 % and 10 % (constants that did not know the width: 0.6 % and 20 %).
   auto add_shape = [&](const FlowPlan& f, int ctas) {
     const double width = widths / (200.0 * F.n_couplings), cb = f.cb / 10.0;
     double cost = 11.0 / F.n_couplings + (f.im2col ? 0.7 * f.group : 0);
     if (f.ring) cost += 4 + f.tiles * (5.7 + 2.9 * width + 2.9 * cb) + (f.nbx * f.nby > 1 ? 3 : 0);
-    else cost += 5 + 0.5 * width + f.tiles * (2.2 + 1.5 * width + 0.8 * cb) + (f.nbx * f.nby > 1 ? 4.7 : 0);
+    else cost += 5 + 0.5 * width + f.tiles * (2.2 + 1.5 * width + 0.8 * cb) + (f.nbx * f.nby > 1 ? 2.6 + 1.5 * cb : 0);
     hl.flow.push_back({f, ctas, cost});
   };
   for (int group = 1; group <= std::min<int>(8, (int)max_batch); group *= 2) {
