@@ -123,16 +123,17 @@ typedef struct {
   int32_t ls_lo, ls_hi;
 } iodf_level_desc;
 
-/* How the levels whose images are smaller than a 128-pixel tile are shared out over CTAs (the
- * results are the same bit for bit; only the launch shapes differ):
- *   IODF_PLAN_LATENCY     as few images per CTA as keeps the SMs busy with one batch of max_batch
- *                         images: the shortest step
- *   IODF_PLAN_THROUGHPUT  as many images per CTA as a tile holds with the level's weights still
- *                         resident in shared memory (levels with residual-block couplings: as many
- *                         padded frames (h+2)(w+2) as a tile holds): fewer CTAs per launch, a step a
- *                         few percent longer; for callers that keep several batches in flight, each on
- *                         a stream and a model handle of its own, so that one batch's idle SMs run
- *                         another's CTAs
+/* How a level's images are shared out over CTAs (the results are the same bit for bit; only the launch
+ * shapes differ):
+ *   IODF_PLAN_LATENCY     levels of three-conv couplings: the shape that is fastest for the batch of each
+ *                         call alone on the device; other levels: as few images per CTA as keeps the
+ *                         SMs busy with one batch of max_batch images
+ *   IODF_PLAN_THROUGHPUT  the shape that takes the least SM time per image (levels of three-conv
+ *                         couplings; other levels: as many images per CTA as a tile holds, with
+ *                         residual-block couplings as many padded frames (h+2)(w+2)): mostly fewer CTAs
+ *                         per launch, a step a few percent longer; for callers that keep several
+ *                         batches in flight, each on a stream and a model handle of its own, so that
+ *                         one batch's idle SMs run another's CTAs
  */
 #define IODF_PLAN_LATENCY 0u
 #define IODF_PLAN_THROUGHPUT 1u
@@ -427,7 +428,7 @@ int iodf_int8_mma_peak(iodf_model* m, uint32_t mma_groups, void* cuda_stream, un
 const char* iodf_level_kernel_name(const iodf_model* m, int level);
 
 /* Images that one CTA of level `level`'s launch holds under the model's plan (1 where an image takes a
- * CTA, or a band of a cluster, of its own); a launch of max_batch images has ceil(max_batch / that) CTAs per band.
+ * CTA, or several of a cluster, of its own); a launch of max_batch images has ceil(max_batch / that) CTAs per block or band.
  * IODF_EINVAL for a bad argument. */
 int iodf_level_images_per_cta(const iodf_model* m, int level);
 

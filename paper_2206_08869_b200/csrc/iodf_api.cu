@@ -1268,19 +1268,9 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   };
   const FlowPlan whole = F0;
   hl.flow.clear();
-  if (throughput) {
-    // as many images as fill a tile: a little more time for a launch, but a half to a quarter of the CTAs
-    const int full = whole.im2col ? 4 : std::max(1, kTileM / whole.px);
-    for (int group = std::min<int>(full, (int)max_batch); group >= 1; group /= 2) {
-      FlowPlan f = whole;
-      if (!plan(f, group)) continue;
-      hl.flow.push_back({f, num_sms, 1.0});
-      return true;
-    }
-    return false;
-  }
   // The latency plan keeps every shape that fits and a launch picks the fastest for its batch: whole images, one or several
-  // per CTA (fewer waves when images outnumber SMs), or images split over clusters of CTAs (idle SMs otherwise). Time of a
+  // per CTA (fewer waves when images outnumber SMs), or images split over clusters of CTAs (idle SMs otherwise). The
+  // throughput plan keeps the one that takes the least SM time per image, with no more images than fill a tile. Time of a
   // wave per coupling, in thousands of clocks: a serial part, a part for each tile of the CTA that grows with the mean
   // hidden width and the channels that are translated, the exchange of their edges, what an image more costs at 4 x 4, and a
   // share of the level's load and store. Fitted to 399 shapes of 31 flows (widths 16 - 512, 4 - 96 channels, 4 x 4 - 32 x
@@ -1293,11 +1283,13 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
     else cost += 5 + 0.5 * width + f.tiles * (2.2 + 1.5 * width + 0.8 * cb) + (f.nbx * f.nby > 1 ? 2.6 + 1.5 * cb : 0);
     hl.flow.push_back({f, ctas, cost});
   };
-  for (int group = 1; group <= std::min<int>(8, (int)max_batch); group *= 2) {
+  const int full = whole.im2col ? 4 : std::max(1, kTileM / whole.px);
+  const int most = std::min<int>(throughput ? full : 8, (int)max_batch);
+  for (int group = 1; group <= most; group = throughput && group < most ? std::min(2 * group, most) : 2 * group) {
     FlowPlan f = whole;
     if (plan(f, group)) add_shape(f, num_sms);
   }
-  if (hl.flow.empty()) return false;
+  if (hl.flow.empty()) return false;              // (levels that would fit only when split stay with the general kernel)
   const int th = whole.h % 16 == 0 ? 16 : 8;
   for (int nbx = 1; !whole.im2col && nbx <= whole.w / 8; ++nbx)
     for (int nby = 1; nby <= whole.h / th && nbx * nby <= kFlowMaxBlocks; ++nby) {
@@ -1327,6 +1319,15 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
             }
       add_shape(f, clusters);
     }
+  if (throughput) {
+    // Streamed weights cost a tile two to three times what resident ones cost it: one 8 x 8 image of 48 channels at width 256,
+    // resident, is 35 us of an SM, one of two, streamed, 41; a 32 x 32 image at width 192 in four blocks, resident, 175,
+    // whole, streamed, 201. But four 4 x 4 images share a tile: at width 256, streamed, 15 each, one, resident, 37.
+    auto sm_time = [](const HostLevel::FlowShape& f) { return f.cost * f.plan.nbx * f.plan.nby / f.plan.group; };
+    const HostLevel::FlowShape best = *std::min_element(hl.flow.begin(), hl.flow.end(),
+                                                        [&](const auto& a, const auto& b) { return sm_time(a) < sm_time(b); });
+    hl.flow.assign(1, best);
+  }
   return true;
 }
 

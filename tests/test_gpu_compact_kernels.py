@@ -70,6 +70,18 @@ def test_images_per_cta_follow_the_hidden_width(G, hidden, batch, images):
     assert G.iodf_level_images_per_cta(m, 1) == images
 
 
+@pytest.mark.parametrize("hidden,images", [
+    (256, [1, 1, 1, 4]),     # 8 x 8: two images' weights would be streamed, 41 us of an SM each against 35 for one
+    (144, [1, 1, 2, 4]),     # everything resident: as many as a tile holds
+    (512, [1, 1, 2, 4]),     # everything streamed: the same
+])
+def test_throughput_plan_takes_the_least_sm_time_per_image(G, hidden, images):
+    model = S.make_model(0xFB00 + hidden, 3, 64, 64, [True] * 4, 4, hidden)
+    x = S.smooth_field_images(0xFB01, 5, 64, 64, 2.0)
+    m, _ = _check_both_ways(G, model, x, plan=G.IODF_PLAN_THROUGHPUT)
+    assert [G.iodf_level_images_per_cta(m, k) for k in range(4)] == images
+
+
 @pytest.mark.parametrize("hw,splits,couplings,hidden,blocks,prune,batch,plan", [
     (64, [True], 1, 128, 1, None, 1, 0),           # 32 x 32 in eight 8 x 16 blocks
     (64, [True], 1, 128, 1, None, 1, 1),           # ... in four 16 x 16 ones
