@@ -39,7 +39,7 @@ extern "C" {
 typedef enum {
   IODF_OK = 0,
   IODF_EINVAL = -1,       /* null/misaligned pointer, batch out of range, malformed descriptor      */
-  IODF_ENOMEM = -2,       /* host or device allocation failed in iodf_create                         */
+  IODF_ENOMEM = -2,       /* host or device allocation failed (creation of a handle, first host call)  */
   IODF_ECUDA = -3,        /* a CUDA call failed; see iodf_last_cuda_error                            */
   IODF_EVERSION = -4,     /* abi_version mismatch                                                    */
   IODF_ETIMEOUT = -5,     /* a bounded device-side wait gave up (reported by iodf_check)             */

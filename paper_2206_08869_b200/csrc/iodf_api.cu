@@ -1913,6 +1913,32 @@ int iodf_inverse_patches(iodf_model* m, const int32_t* z, int H, int W, uint8_t*
     }                                                                  \
   } while (0)
 
+namespace {
+// Decoder's first look-up: the symbols k whose range [Cum(k), Cum(k + 1)) meets slots 256 b .. 256 b + 255, as {first,
+// count << 16}, for every scale index: at most 257 of the 4 097 (a symbol has at least one slot).
+std::vector<uint32_t> decoder_ranges(const iodf_codec_desc& desc) {
+  std::vector<uint32_t> ranges((size_t)desc.n_scales * 256);
+  std::vector<uint32_t> cum(2 * 2048 + 2);
+  for (uint32_t ls = 0; ls < desc.n_scales; ++ls) {
+    cum[0] = 0;
+    for (int k = 1; k <= 2 * 2048; ++k) {
+      int64_t u = ((int64_t)(2 * (k - 2048) - 1) * (int64_t)desc.inv_scale[ls]) >> 16;       // floor
+      u = std::max<int64_t>(-(int64_t)desc.umax, std::min<int64_t>((int64_t)desc.umax, u));
+      cum[k] = (uint32_t)k + desc.sigmoid_table[u + desc.umax];
+    }
+    cum[2 * 2048 + 1] = 1u << 16;
+    int k = 0;
+    for (uint32_t b = 0; b < 256; ++b) {
+      while (k < 2 * 2048 && cum[k + 1] <= 256 * b) ++k;
+      int e = k;
+      while (e < 2 * 2048 && cum[e + 1] <= 256 * b + 255) ++e;
+      ranges[(size_t)ls * 256 + b] = (uint32_t)k | ((uint32_t)(e - k + 1) << 16);
+    }
+  }
+  return ranges;
+}
+}  // namespace
+
 int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_codec** out) {
   if (!m || !desc || !out) return IODF_EINVAL;
   *out = nullptr;
@@ -1928,6 +1954,12 @@ int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_cod
   }
   for (uint32_t i = 0; i < desc->n_scales; ++i)   // 2^21 / s with s >= 2^-9: the kernels multiply in 32 bits
     if (desc->inv_scale[i] < 1 || desc->inv_scale[i] >= (1u << 30)) return IODF_EINVAL;
+  std::vector<uint32_t> ranges;
+  try {
+    ranges = decoder_ranges(*desc);
+  } catch (const std::bad_alloc&) {
+    return IODF_ENOMEM;
+  }
   iodf_codec* c = new (std::nothrow) iodf_codec();
   if (!c) return IODF_ENOMEM;
   c->device = m->device;
@@ -1978,6 +2010,9 @@ int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_cod
   if (e == cudaSuccess) e = cudaMalloc(&c->d_errors, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_sizes, sizeof(uint32_t) * (size_t)c->max_batch);
   if (e == cudaSuccess) e = cudaMemset(c->d_errors, 0, sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&c->d_ranges, 4 * ranges.size());
+  if (e == cudaSuccess) e = cudaMemcpy(c->d_ranges, ranges.data(), 4 * ranges.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaHostAlloc(&c->h_payload, sizeof(uint32_t), cudaHostAllocDefault);
   cudaSetDevice(prev);
   if (e != cudaSuccess) {
     const int rc = e == cudaErrorMemoryAllocation ? IODF_ENOMEM : IODF_ECUDA;
@@ -1987,40 +2022,7 @@ int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_cod
   a.R = reinterpret_cast<const uint32_t*>(c->d_tables);
   a.G = reinterpret_cast<const uint16_t*>(c->d_tables + rbytes);
   a.errors = c->d_errors;
-  // Decoder's first look-up: the symbols k whose range [Cum(k), Cum(k + 1)) meets slots 256 b .. 256 b + 255, as {first,
-  // count << 16}, for every scale index: at most 257 of the 4 097 (a symbol has at least one slot).
-  {
-    std::vector<uint32_t> ranges((size_t)desc->n_scales * 256);
-    std::vector<uint32_t> cum(2 * 2048 + 2);
-    for (uint32_t ls = 0; ls < desc->n_scales; ++ls) {
-      cum[0] = 0;
-      for (int k = 1; k <= 2 * 2048; ++k) {
-        int64_t u = ((int64_t)(2 * (k - 2048) - 1) * (int64_t)desc->inv_scale[ls]) >> 16;       // floor
-        u = std::max<int64_t>(-(int64_t)desc->umax, std::min<int64_t>((int64_t)desc->umax, u));
-        cum[k] = (uint32_t)k + desc->sigmoid_table[u + desc->umax];
-      }
-      cum[2 * 2048 + 1] = 1u << 16;
-      int k = 0;
-      for (uint32_t b = 0; b < 256; ++b) {
-        while (k < 2 * 2048 && cum[k + 1] <= 256 * b) ++k;
-        int e = k;
-        while (e < 2 * 2048 && cum[e + 1] <= 256 * b + 255) ++e;
-        ranges[(size_t)ls * 256 + b] = (uint32_t)k | ((uint32_t)(e - k + 1) << 16);
-      }
-    }
-    e = cudaGetDevice(&prev);
-    if (e == cudaSuccess) e = cudaSetDevice(c->device);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_ranges, 4 * ranges.size());
-    if (e == cudaSuccess) e = cudaMemcpy(c->d_ranges, ranges.data(), 4 * ranges.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaHostAlloc(&c->h_payload, sizeof(uint32_t), cudaHostAllocDefault);
-    cudaSetDevice(prev);
-    if (e != cudaSuccess) {
-      const int rc = e == cudaErrorMemoryAllocation ? IODF_ENOMEM : IODF_ECUDA;
-      iodf_codec_destroy(c);
-      return rc;
-    }
-    a.ranges = c->d_ranges;
-  }
+  a.ranges = c->d_ranges;
   *out = c;
   return IODF_OK;
 }

@@ -207,3 +207,40 @@ def test_compact_stream_and_host_round_trip(G, hw, splits, batch, eps):
         G.iodf_codec_check(cd)
     with pytest.raises(G.IodfError):                          # too small an output buffer
         G.iodf_compress_host(m, cd, xh, out_host=torch.empty(64, dtype=torch.uint8).pin_memory())
+
+
+_OUT_OF_HOST_MEMORY = """
+import resource, sys
+import numpy as np
+sys.path.insert(0, sys.argv[1])
+import iodf_synth as S
+import paper_2206_08869_b200 as G
+m = G.iodf_create(S.make_model(0xA900, 3, 8, 8, [True], 1, 8), 2)
+codec = S.logistic_codec()
+codec["R"] = np.resize(codec["R"], 1024)
+G.iodf_codec_create(m, codec)                        # everything that is allocated only once
+data = next(int(l.split()[1]) for l in open("/proc/self/status") if l.startswith("VmData")) << 10
+soft, hard = resource.getrlimit(resource.RLIMIT_DATA)
+resource.setrlimit(resource.RLIMIT_DATA, (data + (512 << 10), hard))      # the decoder's table takes 1 MB
+try:
+    G.iodf_codec_create(m, codec)
+    status = 0
+except G.IodfError as e:
+    status = e.status
+resource.setrlimit(resource.RLIMIT_DATA, (soft, hard))
+G.iodf_codec_create(m, codec)
+print("status", status)
+"""
+
+
+def test_a_codec_that_finds_no_host_memory_is_an_error_code():
+    """No exception may leave a C entry point: with too little memory for the decoder's table the call returns
+    IODF_ENOMEM, and the next one, with memory, works."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _OUT_OF_HOST_MEMORY, root], capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, MALLOC_MMAP_THRESHOLD_="65536"))      # large blocks are mapped and given back
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split()[-2:] == ["status", "-2"], r.stdout
