@@ -50,14 +50,14 @@ def _check_both_ways(G, model, x, max_batch=None, sample=None, plan=0):
 
 # ---- small shapes: several tiles, ragged tails, odd widths ---------------------------------------
 @pytest.mark.parametrize("hw,splits,hidden,prune,batch", [
-    (8, [False], 16, None, 3),                   # 16 px per image: several images share one tile
-    (8, [True, True], 24, (0.4, 0.7), 5),        # ragged last group (5 images, 8 and 32 per CTA)
-    (16, [True, True, True], 40, (0.4, 0.7), 9), # three levels, odd kept widths
-    (12, [True, False], 20, (0.4, 0.7), 7),      # 36-px and 9-px levels: tiles straddle images
-    (4, [True], 8, None, 70),                    # 4-px level: 32 images per CTA, three CTAs
+    (8, [False], 16, None, 3),                   # 4 x 4 of six input channels: the general kernel
+    (8, [True, True], 24, (0.4, 0.7), 5),        # 4 x 4 and 2 x 2 levels, odd kept widths
+    (16, [True, True, True], 40, (0.4, 0.7), 9), # 8 x 8 compact, 4 x 4, 2 x 2
+    (12, [True, False], 20, (0.4, 0.7), 7),      # 36-px and 9-px levels: rows that divide nothing
+    (4, [True], 8, None, 70),                    # 4-px level, one image per CTA
     (32, [True, True], 64, (0.4, 0.7), 3),       # 256-px level: two tiles per image
-    (16, [True, True], 320, None, 5),            # hidden width above 256: weights streamed in K-slices
-    (8, [True], 500, (0.6, 1.0), 3),             # odd widths between 300 and 500
+    (16, [True, True], 320, None, 5),            # hidden width above 256: weights streamed (compact kernel)
+    (8, [True], 500, (0.6, 1.0), 3),             # odd widths between 300 and 500, streamed in the general kernel
 ])
 def test_small_models_bit_exact(G, hw, splits, hidden, prune, batch):
     model = S.make_model(100 + hw, 3, hw, hw, splits, 3, hidden, prune=prune)
@@ -218,7 +218,7 @@ def test_host_buffer_entry_points(G):
     (8, [True, True], 24, (0.4, 0.7), 21),       # 16- and 4-px levels: 8 and 32 images per CTA, ragged last CTAs
     (16, [True, True, True], 40, (0.4, 0.7), 37),# 64-, 16- and 4-px levels
     (12, [True, False], 20, (0.4, 0.7), 50),     # 36- and 9-px levels: images that do not divide the tile
-    (16, [True, True], 320, None, 9),            # hidden width above 256: streamed weights only at one image per CTA
+    (16, [True, True], 320, None, 9),            # hidden width above 256: streamed weights
 ])
 def test_throughput_plan_small_models_bit_exact(G, hw, splits, hidden, prune, batch):
     model = S.make_model(300 + hw, 3, hw, hw, splits, 3, hidden, prune=prune)
@@ -228,8 +228,7 @@ def test_throughput_plan_small_models_bit_exact(G, hw, splits, hidden, prune, ba
 
 def test_plans_differ_in_images_per_cta_as_documented(G):
     """Config 2 at batch 128: one image per CTA at every level under the default plan; under the
-    throughput plan two at the 64-pixel level and four at the 16-pixel level (a full tile there would
-    need streamed weights). Config R32: three 4 x 4 images' padded frames per tile."""
+    throughput plan two at the 64-pixel level and four at the 16-pixel level, which fills their tiles. Config R32: three 4 x 4 images' padded frames per tile."""
     model = S.config_model(2)
     m0, m1 = G.iodf_create(model, 128), G.iodf_create(model, 128, plan=G.IODF_PLAN_THROUGHPUT)
     assert [G.iodf_level_images_per_cta(m0, lv) for lv in range(4)] == [1, 1, 1, 1]
@@ -339,14 +338,29 @@ def test_config4_batch_sweep_stress_width_512(G, batch):
 
 @pytest.mark.parametrize("hw,hidden,prune,batch", [
     (64, 40, (0.4, 0.7), 3),     # 1024-pixel first level: eight tiles, per-tap partials in columns of their own
-    (48, 24, None, 2),           # 576 pixels: five tiles, a ragged last one, image rows that straddle warps
-    (64, 200, None, 2),          # wide hidden layers: the per-tap partials share the slot's columns
+    (48, 24, None, 2),           # 576 pixels: nine tiles of 64 rows, then 12 x 12 in the general kernel
+    (64, 200, None, 2),          # wide hidden layers: accumulators that do not fit side by side
 ])
-def test_levels_of_many_tiles_in_the_role_split_kernel(G, hw, hidden, prune, batch):
-    """First levels of four tiles and more run in the kernel that gives the im2col / shifted sum,
-    the requantisation and the MMA issue to different warps; the deeper levels of the same models
-    run in the general kernel. Encode, prior parameters, decode and the out-of-range count against
-    the oracle, for every image."""
+def test_levels_of_many_tiles(G, hw, hidden, prune, batch):
+    """First levels of four tiles and more, whole or in blocks as the batch has it. Encode, prior parameters, decode
+    and the out-of-range count against the oracle, for every image."""
     model = S.make_model(0xB100 + hw + hidden, 3, hw, hw, [True, True], 3, hidden, prune=prune)
     x = S.smooth_field_images(0xB200 + hw, batch, hw, hw, 3.0)
     _check_both_ways(G, model, x)
+
+
+@pytest.mark.parametrize("hw,splits,hidden,batch,act_hi", [
+    (24, [True, True], 320, 3, 127),     # 12 x 12 and 6 x 6: the first and third matrix share a slot
+    (40, [True], 320, 2, 255),           # ... four tiles, unsigned activations
+    (20, [True], 320, 3, 127),           # 10 x 10: all three matrices resident beside one tile
+    (40, [True], 512, 2, 127),           # 20 x 20: weights streamed in slices, four tiles
+    (20, [True], 500, 3, 255),           # ... unsigned activations, a ragged width
+    (4, [True], 512, 300, 127),          # ... two images per CTA
+])
+def test_wide_hidden_layers_in_the_general_kernel(G, hw, splits, hidden, batch, act_hi):
+    """Sides that the compact kernel does not take, with hidden layers whose weights do not all fit: every way in
+    which the general kernel keeps, shares or streams them."""
+    model = S.make_model(0xB300 + hw + hidden, 3, hw, hw, splits, 2, hidden, act_hi=act_hi)
+    x = S.smooth_field_images(0xB400 + hw, batch, hw, hw, 2.0)
+    m, _ = _check_both_ways(G, model, x)
+    assert {G.iodf_level_kernel_name(m, k) for k in range(len(splits))} == {"level_kernel"}

@@ -47,7 +47,7 @@ def _both_ways(G, model, x, plan=0):
     (16, [True, True], 2, 24, 2, (0.4, 0.8), 5),          # 64- and 16-pixel levels, odd kept widths
     (32, [True, True, True], 2, 40, 2, (0.4, 0.7), 3),    # 256 pixels: two tiles per image
     (16, [True, False], 1, 128, 8, (0.4, 0.7), 2),        # the paper's width and depth: 128 channels, 8 blocks
-    (64, [True, True], 1, 24, 2, (0.4, 0.7), 3),          # 1024 pixels: four row bands per image (a cluster), then 256
+    (64, [True, True], 1, 24, 2, (0.4, 0.7), 3),          # 1024 pixels: eight blocks per image (a cluster), then 256
     (48, [True], 2, 16, 1, None, 2),                      # 576 pixels: four bands of six rows, image rows of 24 pixels
 ])
 def test_residual_models_bit_exact(G, hw, splits, couplings, hidden, blocks, prune, batch):
@@ -60,7 +60,7 @@ def test_residual_models_bit_exact(G, hw, splits, couplings, hidden, blocks, pru
     (8, [True, True], 2, 24, 2, (0.4, 0.8), 11),          # 16- and 4-pixel levels: 3 and 8 images per CTA, ragged last CTAs
     (16, [True, True, False], 1, 40, 2, (0.4, 0.7), 7),   # 64 pixels (one image per CTA), then 16 and 4 pixels
     (8, [True], 1, 128, 8, (0.4, 0.7), 4),                # the paper's width and depth at 16 pixels: 3 + 1 images
-    (64, [True, True, True, True], 1, 16, 1, None, 5),    # row bands first (one band per CTA), grouped images at the end
+    (64, [True, True, True, True], 1, 16, 1, None, 5),    # blocks first (one per CTA), grouped images at the end
 ])
 def test_residual_models_throughput_plan(G, hw, splits, couplings, hidden, blocks, prune, batch):
     """The throughput plan puts as many images' padded frames into a CTA's tile as it holds: same
@@ -72,7 +72,7 @@ def test_residual_models_throughput_plan(G, hw, splits, couplings, hidden, block
 
 def test_first_level_of_the_imagenet64_geometry_at_the_papers_width(G):
     """App. B.1 on 64 x 64 images: the first level has 32 x 32 pixels, which one CTA cannot hold; it
-    runs as four row bands per image whose edge rows are exchanged after every conv. Width 128, eight
+    runs in eight blocks per image whose edges are exchanged after every conv. Width 128, eight residual
     blocks, one coupling per level to keep the oracle's time down; batch position must not matter."""
     import torch
     model = S.make_residual_model(0xEA00, 3, 64, 64, [True, True], 1, 128, 8, prune=(0.4, 0.7))
