@@ -240,8 +240,6 @@ struct RfPos {             // a thread's two positions of a tile half (rows of t
   int p0, p1;              // pixels of the CTA
 };
 
-__device__ __forceinline__ uint32_t rf_pack_u8(int y0, int y1, int y2, int y3) { return pack4_sat_u8(y0, y1, y2, y3); }
-
 // 8 (4) bytes of an activation in this CTA's frame and, where the pixel (i, j) of the block lies on an edge, in
 // the neighbours' frames
 template <typename V>
@@ -325,8 +323,8 @@ __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMe
     }
   }
   // ReLU and clip to 0..255 are the pack's saturation
-  const uint2 v0 = make_uint2(rf_pack_u8((int)r[0], (int)r[1], (int)r[4], (int)r[5]), rf_pack_u8((int)r[8], (int)r[9], (int)r[12], (int)r[13]));
-  const uint2 v1 = make_uint2(rf_pack_u8((int)r[2], (int)r[3], (int)r[6], (int)r[7]), rf_pack_u8((int)r[10], (int)r[11], (int)r[14], (int)r[15]));
+  const uint2 v0 = make_uint2(pack4_sat_u8((int)r[0], (int)r[1], (int)r[4], (int)r[5]), pack4_sat_u8((int)r[8], (int)r[9], (int)r[12], (int)r[13]));
+  const uint2 v1 = make_uint2(pack4_sat_u8((int)r[2], (int)r[3], (int)r[6], (int)r[7]), pack4_sat_u8((int)r[10], (int)r[11], (int)r[14], (int)r[15]));
   if (ok0) rf_store(f, P, o, v0, g, j, chunk);
   if (ok1) rf_store(f, P, o + row, v1, g + 1, j, chunk);
 }

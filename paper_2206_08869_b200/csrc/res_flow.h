@@ -57,7 +57,6 @@ struct RfPlan {
   int32_t n_slots;
   uint32_t slot_bytes, conv_off; // conv_off: RfConv[] in the blob (prior head last)
   uint32_t s_v, s_buf[3], s_buf_end, s_const, s_meta[3], s_ring, s_total;
-  uint32_t mul_4px;
   int64_t z_off, prior_off, z_final_off, d, d_fact;
 };
 static_assert(sizeof(RfPlan) < 1024, "travels as a kernel parameter");
