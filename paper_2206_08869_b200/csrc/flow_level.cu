@@ -34,8 +34,8 @@
 //
 // What bounds it: the chain of a coupling (about 8 000 clocks) and 3 700 clocks per tile of 128 pixels: requantisation,
 // shifted sum and their hand-overs (52 % of all issue slots at 32 x 32, 39 % at 8 x 8, 24 % at 4 x 4). Measured for eight
-// couplings of widths around 90, 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 161 us,
-// 16 x 16 85 -> 63, 8 x 8 63 -> 48, 4 x 4 70 -> 48; one image, 32 x 32 split in eight: 56. Width 512, 64 images of
+// couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 161 us,
+// 16 x 16 85 -> 63, 8 x 8 63 -> 48, 4 x 4 70 -> 48; one image, 32 x 32 split in eight: 52. Width 512, 64 images of
 // 32 x 32, split in two: 2 357 -> 380 us.
 #include "flow_level.h"
 #include "level_device.cuh"

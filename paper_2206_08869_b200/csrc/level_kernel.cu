@@ -312,9 +312,9 @@ __device__ void run_control_streamed(const Ctx& cx, const LevelPlan& P, const Le
 }
 
 // ---- workers ----------------------------------------------------------------------------------
-// kLean: every hidden layer of the level is in the folded requantisation flavour with the 0..127
-// clip (what the model packer produces for the usual layers), so that the epilogues need one code
-// path instead of seven. The deep levels run every phase's code once per coupling, and what they
+// kLean: every hidden layer of the level is in the floating-point requantisation flavour (0..127 clip,
+// foldable biases, constants for every channel) and its weights are resident, so that the epilogues need one
+// code path instead of seven. The deep levels run every phase's code once per coupling, and what they
 // wait for most, beside memory, is instruction fetch: the smaller the loop body, the better.
 template <bool kInv, bool kLean>
 __device__ __forceinline__ void run_workers(Ctx& cx, const LevelPlan& P, const LevelArgs& a, const Steps& st, int img0, int pvalid,

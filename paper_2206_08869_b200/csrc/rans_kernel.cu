@@ -44,8 +44,8 @@ __device__ __forceinline__ uint32_t cum_of(const Tables& t, uint32_t R, int k) {
 }
 
 // x / F and x mod F for 0 < F <= 2^16 and x < F 2^16, inv = 1 / F rounded: the quotient is below 2^16, so that x * inv
-// is off by less than one before truncation (three roundings of 2^-24 on a value below 2^16), and two
-// conditional corrections make it exact. A 32-bit division is several times as long, and it sits on the chain.
+// is off by less than one before truncation (one rounding of 2^-23, x truncated to 24 bits, and two of 2^-24, on a value
+// below 2^16), and two conditional corrections make it exact. A 32-bit division is several times as long, and it sits on the chain.
 __device__ __forceinline__ uint32_t divide(uint32_t x, uint32_t F, float inv, uint32_t* rem) {
   uint32_t q = __float2uint_rz(__uint2float_rz(x) * inv);
   uint32_t r = x - q * F;
@@ -175,8 +175,10 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_encode_kernel(const Ran
 //     in one go and handed out by shuffle, so no global-memory latency sits between two symbols;
 //   * the coded words: the lanes hold a window of the stream's next 32 words (the decoder reads the
 //     stream backwards); the three words that a symbol can take are handed out before its search.
-// A stream's latency bounds the decompressor (a block's streams are few and long): about 500 clocks per symbol, 36 - 116 us
-// for the blocks of 128 images of 64 x 64 at 128 elements per stream (60 - 170 us with three search rounds).
+// What bounds it depends on the block (128 images of 64 x 64, 128 elements per stream). The small ones are a stream's chain:
+// 35 us for the final block, 540 clocks per symbol, 50 us for those with prior parameters (60 - 70 with three search
+// rounds). The largest, 6 144 streams, ten warps per scheduler, is bound by issue slots, 0.72 per cycle:
+// 111 us (170), 1 700 clocks per symbol of a warp.
 __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const RansArgs a, int q,
                                                                        const uint16_t* __restrict__ words,
                                                                        const uint32_t* __restrict__ counts,
