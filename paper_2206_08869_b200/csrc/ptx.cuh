@@ -96,19 +96,6 @@ __device__ __forceinline__ void red_add_s32(uint32_t saddr, int val, bool pred) 
       : "memory");
 }
 
-// Two predicated fire-and-forget adds (channels `stride` bytes apart).
-__device__ __forceinline__ void red_add2_s32(uint32_t saddr, uint32_t stride, int v0, int v1, bool pred) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .u32 a;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "add.u32 a, %0, %1;\n\t"
-      "@p red.shared.add.s32 [%0], %2;\n\t"
-      "@p red.shared.add.s32 [a], %3;\n\t}" ::"r"(saddr),
-      "r"(stride), "r"(v0), "r"(v1), "r"((uint32_t)pred)
-      : "memory");
-}
-
-
 __device__ __forceinline__ void red_add_s32_always(uint32_t saddr, int val) {
   asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(saddr), "r"(val) : "memory");
 }
