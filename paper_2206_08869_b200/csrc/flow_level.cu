@@ -17,7 +17,10 @@
 //     eight columns in two rows, which halves the loads of constants; the order of the channels within the
 //     next GEMM's K is free, so a thread's eight results are eight adjacent operand bytes.
 //   * The per-tap partial products of the last conv are added to a pixel-major accumulator (odd
-//     stride) with one shared-memory reduction each.
+//     stride) with one shared-memory reduction each. 8 x 8 images, one tile each, need none of that (P.direct): their hidden
+//     operand is a zero-bordered frame too, the last conv is nine taps of it with as few columns as it has channels (an MMA of 64
+//     rows takes 23 clocks up to 24 columns), its accumulators are the translation, and its K steps start as the blocks of
+//     32 channels are written. 128 images of 24 channels: 48 -> 43 us, two to a CTA 65 -> 54.
 //   * CTAs of several tiles have two in flight (slots), each with eight of the sixteen workers and an MMA
 //     warp of its own, so that one slot's hand-overs and MMAs run under the other's requantisation; CTAs of
 //     one tile put all sixteen workers on it. One lane of another warp streams weights and meta blocks.
@@ -44,12 +47,16 @@ namespace iodf {
 
 namespace {
 
+// Shape of a level's tiles: rows of a tile of images whose sides are multiples of eight, or images of 4 x 4.
+enum FlowShapeKind : int { kRows128, kRows64, kImages4x4 };
+
 struct __align__(16) FlowCtl {
   uint64_t xa_ready[2];   // workers (and the neighbours' edge bytes) -> MMA warp, loader: network input of an even / odd
                           // step written (count kFlowWarps and the neighbours' releases; a neighbour may be one step ahead)
   uint64_t acc_full;      // split images: the neighbours' products of a coupling have been added
   uint64_t peers_done;    // split images: the neighbours have read the prior head's input
-  uint64_t a_ready[2];    // slot's workers -> its MMA warp: the next hidden operand is written
+  uint64_t a_ready[2][kFlowMaxRounds];  // slot's workers -> its MMA warp: a round of blocks of the next hidden operand is
+                          // written (all of them: in the first barrier, unless P.chunk2 / chunk3)
   uint64_t dm_ready[2];   // tensor core -> workers: first / second GEMM of the slot's tile complete
   uint64_t d3_ready[2];   // tensor core -> workers: per-tap partials of the slot's tile complete
   uint64_t w_full[kFlowMaxRing], w_empty[kFlowMaxRing];   // weight slots: copy landed / last MMAs (of each tile slot) that read it complete
@@ -59,6 +66,8 @@ struct __align__(16) FlowCtl {
   int32_t sink[32];                 // sums of products that no pixel of the CTA takes, one word a lane
   int4 tile[kFlowMaxTiles];         // {image, first row, first column, 16-byte units from the frame's start to that position}
 };
+
+static_assert(sizeof(FlowCtl) <= 1024, "the host leaves this much for static shared memory");
 
 struct Flow {
   uint8_t* smem;
@@ -86,7 +95,7 @@ __device__ __noinline__ void flow_wait_at(uint32_t bar, uint32_t parity, FlowCtl
 }
 __device__ __forceinline__ void flow_wait(const Flow& f, uint64_t* bar, uint32_t parity) {
   const uint32_t b = ptx::smem_u32(bar);
-  if (ptx::mbar_test_wait(b, parity) || ptx::mbar_try_wait(b, parity)) return;
+  if (ptx::mbar_try_wait(b, parity)) return;
   flow_wait_at(b, parity, f.ctl, f.status);
 }
 // for phases that neighbours take part in (split images)
@@ -172,9 +181,9 @@ __device__ void flow_loader(const Flow& f, const FlowPlan& P, const LevelArgs& a
   };
   auto load = [&](int step, int g) {
     if (step >= st.nsteps || (g > 0 && st.is_prior(step))) return;
-    const int s = (P.alias && g == 2) ? 0 : g;
+    const int s = (P.alias && g == 2) ? 0 : g, part = P.direct && g == 2 ? 3 : g;
     const BlockRef& br = step_ref(*a.plan, st, step);
-    const uint32_t off = br.w_off[g], bytes = br.w_bytes[g];
+    const uint32_t off = br.w_off[part], bytes = br.w_bytes[part];
     if (nl[s] > 0) flow_wait(f, &ctl->w_empty[s], (nl[s] - 1u) & 1u);
     ++nl[s];
     copy(off, bytes, P.s_w[s], &ctl->w_full[s]);
@@ -238,14 +247,16 @@ __device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelAr
 
 // ---- MMA warp --------------------------------------------------------------------------------------------
 // D (+)= A B^T over ks steps of 32 K bytes; n above 256 in two parts. The whole warp runs the loop on uniform
-// values, `lead` issues.
+// values, `lead` issues. `ahead(k)`: waits for what step k needs.
+template <typename Ahead>
 __device__ __forceinline__ void flow_gemm(bool lead, uint32_t d, uint32_t al, uint32_t a_step, uint32_t bl, int n, int ks,
-                                          uint32_t idesc_m) {
+                                          uint32_t idesc_m, Ahead ahead) {
   const uint32_t hi = ptx::kUmmaDescHi, b_step = 2u * (uint32_t)n;
   const int na = n > 256 ? 256 : n;
   const uint32_t idesc = idesc_m | ((uint32_t)(na >> 3) << 17), idesc2 = idesc_m | ((uint32_t)((n - na) >> 3) << 17);
 #pragma unroll 1
   for (int k = 0; k < ks; ++k) {
+    ahead(k);
     if (lead) ptx::umma_i8_hl(d, al, hi, bl, hi, idesc, k > 0 ? 1u : 0u);
     if (n > 256 && lead) ptx::umma_i8_hl(d + 256u, al, hi, bl + 256u, hi, idesc2, k > 0 ? 1u : 0u);
     al += a_step;
@@ -253,7 +264,20 @@ __device__ __forceinline__ void flow_gemm(bool lead, uint32_t d, uint32_t al, ui
   }
 }
 
+// The nine taps of a 32-channel chunk of the last conv in its direct form (`lead` only): a tap is a start address
+__device__ __forceinline__ void flow_taps(const FlowPlan& P, uint32_t d, uint32_t al, uint32_t a_hi, uint32_t bl, uint32_t b_step,
+                                          uint32_t idesc, bool accumulate) {
+#pragma unroll
+  for (int u = 0; u < 3; ++u)
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      ptx::umma_i8_hl(d, al + (uint32_t)(u * P.wp + v), a_hi, bl, ptx::kUmmaDescHi, idesc, accumulate || u + v > 0 ? 1u : 0u);
+      bl += b_step;
+    }
+}
+
 // MMA warp of tile slot `sl`: tiles sl, sl + 2, ...
+template <int kShape>
 __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int sl) {
   if (sl >= f.slots) return;
   FlowCtl* ctl = f.ctl;
@@ -265,14 +289,19 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
   const uint32_t a1_hi = (uint32_t)P.sbo16 | (1u << 14);
   const uint32_t pitch16 = (uint32_t)P.pitch >> 4;
   const uint32_t a_lo = ((ptx::smem_u32(smem + P.s_a[sl]) >> 4) & 0x3FFFu) | (pitch16 << 16);
-  const uint32_t dm = f.tmem + (uint32_t)(sl * P.d_col), d3 = f.tmem + (uint32_t)(P.d3_col + sl * P.d3_step);
+  const uint32_t dm = f.tmem + (uint32_t)(sl * P.d_col), d2 = dm + (uint32_t)P.d2_col, d3 = f.tmem + (uint32_t)(P.d3_col + sl * P.d3_step);
+  const uint32_t h_lo = ((ptx::smem_u32(smem + P.s_h[sl]) >> 4) & 0x3FFFu) | ((uint32_t)P.frame << 16), h_hi = (uint32_t)P.wp | (1u << 14);
   const int s3 = P.alias ? 0 : 2;
   auto commit = [&](uint64_t* bar) { if (lead) ptx::umma_commit(ptx::smem_u32(bar)); };
   uint32_t used[3] = {0u, 0u, 0u}, apar = 0u;
   auto wait_w = [&](int s) { flow_wait(f, &ctl->w_full[s], used[s] & 1u); };
-  auto wait_a = [&]() {
-    flow_wait(f, &ctl->a_ready[sl], apar);
-    apar ^= 1u;
+  // K step k of a hidden operand: written a round of ncs blocks at a time, or all at once
+  auto wait_a = [&](int k, bool chunked) {
+    const bool c = kShape != kRows128 && chunked;
+    const int r = c ? (f.ncs == 4 ? k >> 2 : k >> 1) : 0;
+    if (c ? (k & (f.ncs - 1)) != 0 : k > 0) return;
+    flow_wait(f, &ctl->a_ready[sl][r], (apar >> r) & 1u);
+    apar ^= 1u << r;
     ptx::tc_fence_after();
   };
 #pragma unroll 1
@@ -283,7 +312,7 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
     // (through a shuffle: tells the compiler that the values are the same in all lanes, so that the operands of
     // the MMAs are computed in uniform registers)
     auto uniform = [](int x) { return __shfl_sync(0xFFFFFFFFu, x, 0); };
-    const int n1 = prior ? P.n_prior : uniform(M->n1), n2 = uniform(M->n2), n3 = uniform(M->n3);
+    const int n1 = prior ? P.n_prior : uniform(M->n1), n2 = uniform(M->n2), n3 = uniform(kShape == kRows64 && P.direct ? M->n3d : M->n3);
     const int ks2 = uniform(M->ks2), ks3 = uniform(M->ks3);
     wait_w(0);
     ++used[0];
@@ -319,13 +348,24 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
       commit(&ctl->dm_ready[sl]);
       if (last) commit(&ctl->w_empty[0]);
       if (t == sl) wait_w(1);
-      wait_a();
-      flow_gemm(lead, dm, a_lo, 2u * pitch16, b2, n2, ks2, idesc_m);
+      if (kShape == kRows128) wait_a(0, false);
+      flow_gemm(lead, d2, a_lo, 2u * pitch16, b2, n2, ks2, idesc_m, [&](int k) { if (kShape != kRows128) wait_a(k, P.chunk2); });
       commit(&ctl->dm_ready[sl]);
       if (last) commit(&ctl->w_empty[1]);
       if (t == sl) wait_w(s3);
-      wait_a();
-      flow_gemm(lead, d3, a_lo, 2u * pitch16, b3, n3, ks3, idesc_m);
+      if (kShape == kRows64 && P.direct) {
+        uint32_t al = h_lo, bl = b3;
+#pragma unroll 1
+        for (int k = 0; k < ks3; ++k) {
+          wait_a(k, P.chunk3);
+          if (lead) flow_taps(P, d3, al, h_hi, bl, 2u * (uint32_t)n3, idesc_m | ((uint32_t)(n3 >> 3) << 17), k > 0);
+          al += 2u * (uint32_t)P.frame;
+          bl += 18u * (uint32_t)n3;
+        }
+      } else {
+        wait_a(0, false);
+        flow_gemm(lead, d3, a_lo, 2u * pitch16, b3, n3, ks3, idesc_m, [](int) {});
+      }
       commit(&ctl->d3_ready[sl]);
       if (last) commit(&ctl->w_empty[s3]);
     }
@@ -365,7 +405,7 @@ __device__ void flow_mma_ring(const Flow& f, const FlowPlan& P, const Steps& st)
     }
   };
   auto wait_a = [&]() {
-    flow_wait(f, &ctl->a_ready[0], apar);
+    flow_wait(f, &ctl->a_ready[0][0], apar);
     apar ^= 1u;
     ptx::tc_fence_after();
   };
@@ -404,76 +444,84 @@ __device__ __forceinline__ uint32_t flow_integer_one(uint32_t acc, float m, int 
   return (uint32_t)max(0, (int)(p >> 32) >> (us - 1));
 }
 
-// Hidden epilogue of one tile: n accumulator columns at `taddr` (this warp's lane quarter) -> bytes of
-// the next GEMM's operand, ks 32-column blocks, dealt to the quarter's warps; rows in halves of 16. A
-// thread meets the same eight columns in all its rows, so their constants are loaded once per block. From
-// block n / 32 on the operand holds constants (cw) beyond the columns.
-template <int kHalves>
-__device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, uint32_t taddr, const FlowMeta* __restrict__ M, int layer,
-                                            uint8_t* __restrict__ sA, uint64_t* ready, uint32_t parity) {
+// Where a hidden epilogue writes: this thread's first row, block 0; bytes to the next block and to the row eight further on
+struct HiddenOut {
+  uint8_t* at;
+  int block, row;
+};
+
+// Hidden epilogue of one tile: accumulator columns at `taddr` (this warp's lane quarter) -> bytes of the next GEMM's
+// operand, 32-column blocks, dealt to the quarter's warps; rows in halves of 16. A thread meets the same eight columns in all
+// its rows, so their constants are loaded once per block: the four bytes per channel that a broadcast load returns to every
+// lane bound the epilogue (addends loaded for all channels: 161 -> 178 us for a 32 x 32 level). Beyond the columns the operand
+// holds constants.
+template <int kShape>
+__device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, uint32_t taddr, const uint8_t* __restrict__ mb, int layer,
+                                            const HiddenOut ho, bool chunked, uint64_t* ready, uint32_t parity) {
+  constexpr int kHalves = kShape == kRows128 ? 2 : 1;
   // everything that does not depend on the accumulator comes before the wait for it
-  const int n = layer ? M->n2 : M->n1, ks = layer ? M->ks3 : M->ks2, nfi = layer ? M->nfi2 : M->nfi1;
-  const int nfb = layer ? M->nfb2 : M->nfb1;
-  const int q = f.lane & 3, nfull = n >> 5, last = (n - 1) >> 5, plain = min(min(nfb, nfi), nfull);
-  const uint8_t* mb = reinterpret_cast<const uint8_t*>(M);
-  const float4* ft = reinterpret_cast<const float4*>(mb + (layer ? M->off_f2 : M->off_f1)) + q * 2;
-  const float4* ct = reinterpret_cast<const float4*>(mb + (layer ? M->off_c2 : M->off_c1)) + q * 2 - nfb * 8;
-  const uint32_t cw = layer ? 0u : kBiasColumnsLo;
-  uint8_t* out = sA + (q >> 1) * P.pitch + ((f.warp & 3) * (16 * kHalves) + (f.lane >> 2)) * 16 + (q & 1) * 8;
+  const FlowLayer L = reinterpret_cast<const FlowMeta*>(mb)->layer[layer];
+  const uint8_t* t = mb + L.off + (f.lane & 3) * 32;
+  const int row = kShape == kRows64 ? ho.row : 128;
+  uint64_t* done = f.ctl->a_ready[f.sl];
   flow_wait(f, ready, parity);
   ptx::tc_fence_after();
 #pragma unroll 1
-  for (int b = f.cs; b < ks; b += f.ncs) {
-    uint32_t r[kHalves][16];
+  for (int b0 = 0; b0 < L.ks; b0 += f.ncs) {
+    const int b = b0 + f.cs;
+    if (b < L.ks) {
+      uint32_t r[kHalves][16];
+      const uint32_t ta = taddr + (uint32_t)(min(b, (int)L.last) << 5);
 #pragma unroll
-    for (int h = 0; h < kHalves; ++h) ptx::tmem_ld_16x32(taddr + ((uint32_t)h << 20) + (uint32_t)(min(b, last) << 5), r[h]);
-    const float4 m0 = ft[b * 8], m1 = ft[b * 8 + 1];
-    float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
-    const float m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-    const bool tail = b >= nfull, none = tail && !(n & 16);
-    uint8_t* o = out + (size_t)(2 * b) * P.pitch;
-    ptx::tmem_ld_wait16(r[0]);
+      for (int h = 0; h < kHalves; ++h) ptx::tmem_ld_16x32(ta + ((uint32_t)h << 20), r[h]);
+      const float4* tb = reinterpret_cast<const float4*>(t + b * 256);
+      const float4 m0 = tb[0], m1 = tb[1];
+      const float m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+      uint8_t* o = ho.at + b * ho.block;
+      // the eight bytes of a thread's row (e = 0: the upper one, 1: eight further on) of a half
+      auto pack = [&](int h, int e) {
+        return make_uint2(pack4_sat((int)r[h][2 * e], (int)r[h][2 * e + 1], (int)r[h][2 * e + 4], (int)r[h][2 * e + 5]),
+                          pack4_sat((int)r[h][2 * e + 8], (int)r[h][2 * e + 9], (int)r[h][2 * e + 12], (int)r[h][2 * e + 13]));
+      };
+      ptx::tmem_ld_wait16(r[0]);
 #pragma unroll
-    for (int h = 1; h < kHalves; ++h) ptx::tmem_ld_wait16_nosync(r[h]);
-    if (b < plain) {
+      for (int h = 1; h < kHalves; ++h) ptx::tmem_ld_wait16_nosync(r[h]);
+      if (b < L.plain) {                           // (in one piece: nothing between the multiplications and the stores)
 #pragma unroll
-      for (int h = 0; h < kHalves; ++h) {
+        for (int h = 0; h < kHalves; ++h) {
 #pragma unroll
-        for (int k = 0; k < 16; ++k) r[h][k] = (uint32_t)FloatRq::one(r[h][k], m[2 * (k >> 2) + (k & 1)], 0.f);
+          for (int k = 0; k < 16; ++k) r[h][k] = (uint32_t)FloatRq::one(r[h][k], m[2 * (k >> 2) + (k & 1)], 0.f);
 #pragma unroll
-        for (int e = 0; e < 4; e += 2)
-          *reinterpret_cast<uint2*>(o + h * 256 + e * 64) =
-              make_uint2(pack4_sat((int)r[h][e], (int)r[h][e + 1], (int)r[h][e + 4], (int)r[h][e + 5]),
-                         pack4_sat((int)r[h][e + 8], (int)r[h][e + 9], (int)r[h][e + 12], (int)r[h][e + 13]));
+          for (int e = 0; e < 2; ++e) *reinterpret_cast<uint2*>(o + (2 * h + e) * row) = pack(h, e);
+        }
+      } else {
+        if (b < L.nfi) {
+          const float4 c0 = tb[8], c1 = tb[9];
+          const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+          for (int h = 0; h < kHalves; ++h)
+#pragma unroll
+            for (int k = 0; k < 16; ++k) r[h][k] = (uint32_t)FloatRq::one(r[h][k], m[2 * (k >> 2) + (k & 1)], c[2 * (k >> 2) + (k & 1)]);
+        } else {
+#pragma unroll
+          for (int h = 0; h < kHalves; ++h)
+#pragma unroll
+            for (int k = 0; k < 16; ++k) r[h][k] = flow_integer_one(r[h][k], m[2 * (k >> 2) + (k & 1)], L.us);
+        }
+        const bool tail = b >= L.nfull, none = b > L.nfull || !L.half;
+#pragma unroll
+        for (int h = 0; h < kHalves; ++h)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            uint2 w = pack(h, e);
+            if (tail) w = make_uint2(none ? L.beyond : w.x, L.beyond);
+            *reinterpret_cast<uint2*>(o + (2 * h + e) * row) = w;
+          }
       }
-      continue;
     }
-    if (b >= nfb) {
-      c0 = ct[b * 8];
-      c1 = ct[b * 8 + 1];
-    }
-    const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-    if (b >= nfi) {
-      const int us = layer ? M->us2 : M->us1;
-#pragma unroll
-      for (int h = 0; h < kHalves; ++h)
-#pragma unroll
-        for (int k = 0; k < 16; ++k) r[h][k] = flow_integer_one(r[h][k], m[2 * (k >> 2) + (k & 1)], us);
-    } else {
-#pragma unroll
-      for (int h = 0; h < kHalves; ++h)
-#pragma unroll
-        for (int k = 0; k < 16; ++k) r[h][k] = (uint32_t)FloatRq::one(r[h][k], m[2 * (k >> 2) + (k & 1)], c[2 * (k >> 2) + (k & 1)]);
-    }
-#pragma unroll
-    for (int h = 0; h < kHalves; ++h)
-#pragma unroll
-      for (int e = 0; e < 4; e += 2) {
-        const uint32_t w0 = pack4_sat((int)r[h][e], (int)r[h][e + 1], (int)r[h][e + 4], (int)r[h][e + 5]);
-        const uint32_t w1 = pack4_sat((int)r[h][e + 8], (int)r[h][e + 9], (int)r[h][e + 12], (int)r[h][e + 13]);
-        *reinterpret_cast<uint2*>(o + h * 256 + e * 64) = make_uint2(none ? cw : w0, tail ? cw : w1);
-      }
+    if (kShape != kRows128 && chunked) flow_hand_over(f, done++);
   }
+  if (kShape == kRows128 || !chunked) flow_hand_over(f, done);
 }
 
 // rq with the shift folded to the high word; the host admits only shifts s >= 1 to this kernel
@@ -614,10 +662,45 @@ __device__ __forceinline__ void flow_sum_4x4(const Flow& f, const FlowPlan& P, i
   }
 }
 
+// Last conv in its direct form: the accumulators of tile t (a lane quarter: 16 pixels) are the translation. Unit = 8 channels.
+template <bool kInv>
+__device__ __forceinline__ void flow_out(const Flow& f, const FlowPlan& P, int t, uint32_t taddr, const uint8_t* mb, int32_t* __restrict__ v,
+                                         uint64_t* ready, uint32_t parity) {
+  const FlowMeta* M = reinterpret_cast<const FlowMeta*>(mb);
+  const int32_t* colB = reinterpret_cast<const int32_t*>(mb + M->off_colB);
+  const OutRq* orq = reinterpret_cast<const OutRq*>(mb + M->off_out);
+  int32_t* vq = v + (4 * t + (f.warp & 3)) * 16 + (f.lane >> 2);
+  flow_wait(f, ready, parity);
+  ptx::tc_fence_after();
+#pragma unroll 1
+  for (int g = f.cs; 8 * g < P.cb; g += f.ncs) {
+    uint32_t r[4];
+    ptx::tmem_ld_16x8(taddr + (uint32_t)(8 * g), r);
+    const int ch = 8 * g + 2 * (f.lane & 3);
+    const bool ok = ch < P.cb;                   // (cb is even)
+    OutRq o[2];
+    int32_t* vp[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      o[e] = orq[ok ? ch + e : 0];
+      vp[e] = vq + colB[ok ? ch + e : 0] * P.pg;
+    }
+    ptx::tmem_ld_wait4(r);
+    if (!ok) continue;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const uint32_t y0 = (uint32_t)rq_hi((int32_t)r[e], o[e]), y8 = (uint32_t)rq_hi((int32_t)r[e + 2], o[e]);
+      const uint32_t x0 = (uint32_t)vp[e][0], x8 = (uint32_t)vp[e][8];
+      vp[e][0] = (int32_t)(kInv ? x0 - y0 : x0 + y0);
+      vp[e][8] = (int32_t)(kInv ? x8 - y8 : x8 + y8);
+    }
+  }
+}
+
 // Prior head: accumulators of all tiles -> mu and clipped log-scale index in global memory. Unit = (tile, 8 columns).
-template <bool kSplit>
+template <bool kSplit, int kShape>
 __device__ void flow_prior(const Flow& f, const FlowPlan& P, const LevelArgs& a, const PriorMeta* M, int img0) {
-  const int wq = f.warp & 3, hs = P.m >> 7;
+  const int wq = f.warp & 3, hs = kShape == kRows128 ? 1 : 0;
   const OutRq* orq = reinterpret_cast<const OutRq*>(reinterpret_cast<const uint8_t*>(M) + M->off_out);
   const int ng = (2 * P.cb + 7) >> 3;
   const int lane_row = (wq << (4 + hs)) + (f.lane & (hs ? 31 : 15));
@@ -632,7 +715,7 @@ __device__ void flow_prior(const Flow& f, const FlowPlan& P, const LevelArgs& a,
     int img = tp.x, at = (tp.y + (lane_row >> 3)) * P.w + tp.z + (lane_row & 7);
     if constexpr (kSplit) at = (f.by * P.h + tp.y + (lane_row >> 3)) * P.fw + f.bx * P.w + tp.z + (lane_row & 7);
     const int plane = kSplit ? P.fpx : P.px;
-    if (P.im2col) { img += lane_row >> 4; at = lane_row & 15; }
+    if (kShape == kImages4x4) { img += lane_row >> 4; at = lane_row & 15; }
     int32_t* mu = a.prior + (size_t)(img0 + img) * (size_t)(2 * P.d_fact) + P.prior_off + at;
     ptx::tmem_ld_wait8(r);
     if (!(hs || f.lane < 16) || img >= f.nimg) continue;
@@ -681,7 +764,7 @@ __device__ __forceinline__ void flow_translate(const FlowPlan& P, const PixelMap
 }
 
 // network input: words of four requantised channels (then the constants 1, 127, 127, ...) into the frame
-template <bool kSplit>
+template <bool kSplit, int kShape>
 __device__ __forceinline__ void flow_requant(const Flow& f, const FlowPlan& P, const PixelMap& pm, uint64_t* input, const int32_t* cols, int32_t m0, int32_t s) {
   const int nw = (P.ca + 3) >> 2;
   const long long rnd = 1ll << (30 + s);
@@ -703,7 +786,7 @@ __device__ __forceinline__ void flow_requant(const Flow& f, const FlowPlan& P, c
       w0 = (w0 & 0xFFFFu) | 0x7F010000u;
       w1 = (w1 & 0xFFFFu) | 0x7F010000u;
     }
-    if (!P.im2col) {
+    if constexpr (kShape != kImages4x4) {
       uint32_t* rec = reinterpret_cast<uint32_t*>(pm.rec + (wd >> 2) * P.plane16 * 16 + (wd & 3) * 4);
       rec[0] = w0;
       rec[4] = w1;
@@ -743,7 +826,7 @@ __device__ __forceinline__ void flow_requant(const Flow& f, const FlowPlan& P, c
   }
 }
 
-template <bool kInv, bool kSplit>
+template <bool kInv, bool kSplit, int kShape>
 __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st, int img0) {
   FlowCtl* ctl = f.ctl;
   uint8_t* smem = f.smem;
@@ -772,12 +855,11 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
     }
   }
   const uint32_t dm = f.tmem + (uint32_t)(f.sl * P.d_col) + lane_field, d3 = f.tmem + (uint32_t)(P.d3_col + f.sl * P.d3_step) + lane_field;
-  uint8_t* sA = smem + P.s_a[f.sl];
   uint32_t dpar = 0u, tpar = 0u, npar = 0u;
   const uint8_t* prev = nullptr;                // coupling whose translation is still to be applied
 #pragma unroll 1
   for (int i = 0; i <= st.nsteps; ++i) {
-    if (prev && !P.im2col) {
+    if (kShape != kImages4x4 && prev && !(kShape == kRows64 && P.direct)) {
       flow_translate<kInv>(P, pm, prev);
       // the network input may read channels that were just updated; what was cleared is released as a whole
       if (kSplit || pm.parts > 1) worker_barrier();
@@ -790,36 +872,52 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
     // (the first two words of both kinds of meta block)
     uint64_t* input = &ctl->xa_ready[i & 1];
     if (kSplit && f.warp == kFlowWarps - 1) flow_release_to_neighbours(P, f, input);
-    flow_requant<kSplit>(f, P, pm, input, prior ? a.plan->col_out : reinterpret_cast<const int32_t*>(mb + M->off_colA), M->in_m0, M->in_s);
+    flow_requant<kSplit, kShape>(f, P, pm, input, prior ? a.plan->col_out : reinterpret_cast<const int32_t*>(mb + M->off_colA), M->in_m0, M->in_s);
     flow_hand_over(f, input, kSplit && f.warp == 0 ? f.halo : 0u);
     prev = prior ? nullptr : mb;
     if (prior) {
       flow_wait(f, &ctl->dm_ready[f.sl], dpar);
       dpar ^= 1u;
       ptx::tc_fence_after();
-      flow_prior<kSplit>(f, P, a, reinterpret_cast<const PriorMeta*>(mb), img0);
+      flow_prior<kSplit, kShape>(f, P, a, reinterpret_cast<const PriorMeta*>(mb), img0);
     } else {
 #pragma unroll 1
       for (int t = f.sl; t < f.tiles; t += f.slots) {
-        const bool quarter = !P.im2col || 4 * t + (f.warp & 3) < f.nimg;
+        const bool quarter = kShape != kImages4x4 || 4 * t + (f.warp & 3) < f.nimg;
 #pragma unroll 1
         for (int layer = 0; layer < 2; ++layer) {
-          if (P.m == 128) flow_hidden<2>(f, P, dm, M, layer, sA, &ctl->dm_ready[f.sl], dpar);
-          else if (quarter) flow_hidden<1>(f, P, dm, M, layer, sA, &ctl->dm_ready[f.sl], dpar);
-          else flow_wait(f, &ctl->dm_ready[f.sl], dpar);      // (never a phase ahead in its arrivals)
+          const bool chunked = kShape != kRows128 && (layer ? P.chunk3 : P.chunk2);
+          const uint32_t d = kShape != kRows128 && layer ? dm + (uint32_t)P.d2_col : dm;
+          const int q = f.lane & 3, row = f.lane >> 2;
+          HiddenOut ho;
+          if (kShape == kRows64 && layer && P.direct) {
+            ho.at = smem + P.s_h[f.sl] + ((q >> 1) * P.frame + ((f.warp & 3) * 2 + 1) * P.wp + 1 + row) * 16 + (q & 1) * 8;
+            ho.block = 32 * P.frame;
+            ho.row = 16 * P.wp;
+          } else {
+            ho.at = smem + P.s_a[f.sl] + (q >> 1) * P.pitch + ((f.warp & 3) * (kShape == kRows128 ? 32 : 16) + row) * 16 + (q & 1) * 8;
+            ho.block = 2 * P.pitch;
+            ho.row = 128;
+          }
+          if (quarter) {
+            flow_hidden<kShape>(f, P, d, mb, layer, ho, chunked, &ctl->dm_ready[f.sl], dpar);
+          } else {
+            flow_wait(f, &ctl->dm_ready[f.sl], dpar);      // (never a phase ahead in its arrivals)
+            const int ks = layer ? M->ks3 : M->ks2;
+            for (int b0 = 0, r = 0; b0 < (chunked ? ks : 1); b0 += f.ncs, ++r) flow_hand_over(f, &ctl->a_ready[f.sl][r]);
+          }
           dpar ^= 1u;
-          flow_hand_over(f, &ctl->a_ready[f.sl]);
         }
-        if (P.im2col) {
+        if (kShape == kRows64 && P.direct) {
+          flow_out<kInv>(f, P, t, d3, mb, v, &ctl->d3_ready[f.sl], tpar);
+        } else if constexpr (kShape == kImages4x4) {
           if (quarter) flow_sum_4x4<kInv>(f, P, t, d3, mb, v, &ctl->d3_ready[f.sl], tpar);
-        } else if (P.m == 128) {
-          flow_sum<4, kSplit>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
         } else {
-          flow_sum<2, kSplit>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
+          flow_sum<kShape == kRows128 ? 4 : 2, kSplit>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
         }
         tpar ^= 1u;
         // (streamed weights: the next tile's first GEMM writes where the partials were)
-        if (P.ring && t + 1 < f.tiles) flow_hand_over(f, &ctl->a_ready[0]);
+        if (P.ring && t + 1 < f.tiles) flow_hand_over(f, &ctl->a_ready[0][0]);
       }
     }
     ptx::tc_fence_before();
@@ -941,7 +1039,7 @@ __device__ __forceinline__ void flow_store(const Flow& f, const FlowPlan& P, con
   }
 }
 
-template <bool kInv, bool kSplit>
+template <bool kInv, bool kSplit, int kShape>
 __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const LevelArgs a, const __grid_constant__ FlowPlan P) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ FlowCtl ctl;
@@ -969,7 +1067,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
     ptx::mbar_init(ptx::smem_u32(&ctl.peers_done), (uint32_t)max(neighbours, 1));
     for (int s = 0; s < 2; ++s) {
       ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready[s]), (uint32_t)(kFlowWarps + neighbours));
-      ptx::mbar_init(ptx::smem_u32(&ctl.a_ready[s]), (uint32_t)(kFlowWarps / slots));
+      for (int r = 0; r < kFlowMaxRounds; ++r) ptx::mbar_init(ptx::smem_u32(&ctl.a_ready[s][r]), (uint32_t)(kFlowWarps / slots));
       ptx::mbar_init(ptx::smem_u32(&ctl.dm_ready[s]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl.d3_ready[s]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl.meta_full[s]), 1);
@@ -1006,7 +1104,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
       else flow_loader(f, P, a, st);
     }
   } else if (warp >= kFlowWarps) {
-    if (!P.ring) flow_mma(f, P, st, warp - kFlowWarps);
+    if (!P.ring) flow_mma<kShape>(f, P, st, warp - kFlowWarps);
     else if (warp == kFlowWarps) flow_mma_ring(f, P, st);
   } else {
     // frame of the network input: zero channels, and the constants that multiply the bias rows in the
@@ -1036,13 +1134,15 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
       }
       ctl.tile[tid] = tp;
     }
-    for (int o = tid; o < (P.im2col ? 0 : P.cb * P.acc_stride); o += kFlowWorkers) reinterpret_cast<int32_t*>(smem + P.s_acc)[o] = 0;
+    if (P.direct)                        // zero border of the last conv's operand
+      for (uint32_t o = P.s_h[0] + 16 * tid; o < P.s_h_end; o += 16 * kFlowWorkers) *reinterpret_cast<uint4*>(smem + o) = make_uint4(0u, 0u, 0u, 0u);
+    for (int o = tid; o < (P.im2col || P.direct ? 0 : P.cb * P.acc_stride); o += kFlowWorkers) reinterpret_cast<int32_t*>(smem + P.s_acc)[o] = 0;
     int32_t* v = reinterpret_cast<int32_t*>(smem + P.s_v);
     if constexpr (kSplit) flow_cluster_sync();     // frame, accumulator and barriers are ready for the neighbours
     ptx::grid_dependency_wait();         // from here on: what the previous kernel in the stream wrote
     flow_load<kInv, kSplit>(f, P, a, img0, v);
     worker_barrier();
-    flow_workers<kInv, kSplit>(f, P, a, st, img0);
+    flow_workers<kInv, kSplit, kShape>(f, P, a, st, img0);
     worker_barrier();
     flow_store<kInv, kSplit>(f, P, a, img0, v);
   }
@@ -1055,7 +1155,7 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
 }  // namespace
 
 namespace {
-template <bool kInv, bool kSplit>
+template <bool kInv, bool kSplit, int kShape>
 cudaError_t launch(const LevelArgs& args, const FlowPlan& plan, int grid, cudaStream_t stream) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
@@ -1071,14 +1171,22 @@ cudaError_t launch(const LevelArgs& args, const FlowPlan& plan, int grid, cudaSt
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = kSplit ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, flow_level_kernel<kInv, kSplit>, args, plan);
+  return cudaLaunchKernelEx(&cfg, flow_level_kernel<kInv, kSplit, kShape>, args, plan);
+}
+}  // namespace
+
+namespace {
+template <bool kInv>
+cudaError_t launch_shape(const LevelArgs& args, const FlowPlan& plan, int grid, cudaStream_t stream) {
+  const bool split = plan.nbx * plan.nby > 1;
+  if (plan.im2col) return launch<kInv, false, kImages4x4>(args, plan, grid, stream);
+  if (plan.m == 128) return split ? launch<kInv, true, kRows128>(args, plan, grid, stream) : launch<kInv, false, kRows128>(args, plan, grid, stream);
+  return split ? launch<kInv, true, kRows64>(args, plan, grid, stream) : launch<kInv, false, kRows64>(args, plan, grid, stream);
 }
 }  // namespace
 
 cudaError_t launch_flow_level(const LevelArgs& args, const FlowPlan& plan, bool inverse, int grid, cudaStream_t stream) {
-  if (plan.nbx * plan.nby > 1)
-    return inverse ? launch<true, true>(args, plan, grid, stream) : launch<false, true>(args, plan, grid, stream);
-  return inverse ? launch<true, false>(args, plan, grid, stream) : launch<false, false>(args, plan, grid, stream);
+  return inverse ? launch_shape<true>(args, plan, grid, stream) : launch_shape<false>(args, plan, grid, stream);
 }
 
 int max_flow_clusters(int ctas, uint32_t smem_bytes, uint32_t smem_limit) {
@@ -1095,7 +1203,7 @@ int max_flow_clusters(int ctas, uint32_t smem_bytes, uint32_t smem_limit) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, flow_level_kernel<false, true>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, flow_level_kernel<false, true, kRows128>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -1104,11 +1212,15 @@ int max_flow_clusters(int ctas, uint32_t smem_bytes, uint32_t smem_limit) {
 
 cudaError_t configure_flow_kernels(uint32_t max_smem_bytes) {
   const auto set = [&](const void* k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem_bytes); };
-  cudaError_t e = set(reinterpret_cast<const void*>(flow_level_kernel<false, false>));
-  if (e == cudaSuccess) e = set(reinterpret_cast<const void*>(flow_level_kernel<true, false>));
-  if (e == cudaSuccess) e = set(reinterpret_cast<const void*>(flow_level_kernel<false, true>));
-  if (e == cudaSuccess) e = set(reinterpret_cast<const void*>(flow_level_kernel<true, true>));
-  return e;
+  const void* kernels[] = {
+      reinterpret_cast<const void*>(flow_level_kernel<false, false, kRows128>), reinterpret_cast<const void*>(flow_level_kernel<true, false, kRows128>),
+      reinterpret_cast<const void*>(flow_level_kernel<false, true, kRows128>), reinterpret_cast<const void*>(flow_level_kernel<true, true, kRows128>),
+      reinterpret_cast<const void*>(flow_level_kernel<false, false, kRows64>), reinterpret_cast<const void*>(flow_level_kernel<true, false, kRows64>),
+      reinterpret_cast<const void*>(flow_level_kernel<false, true, kRows64>), reinterpret_cast<const void*>(flow_level_kernel<true, true, kRows64>),
+      reinterpret_cast<const void*>(flow_level_kernel<false, false, kImages4x4>), reinterpret_cast<const void*>(flow_level_kernel<true, false, kImages4x4>)};
+  for (const void* k : kernels)
+    if (const cudaError_t e = set(k); e != cudaSuccess) return e;
+  return cudaSuccess;
 }
 
 }  // namespace iodf

@@ -15,6 +15,7 @@ constexpr int kFlowThreads = kFlowWorkers + 3 * 32;  // + an MMA-issuing warp pe
 constexpr int kFlowMaxRing = 12;                     // slots of the weight ring
 constexpr int kFlowMaxTiles = 32;                    // of a CTA
 constexpr int kFlowMaxSteps = 18;                    // K steps of the first conv
+constexpr int kFlowMaxRounds = 5;                    // blocks of 32 columns that a warp requantises of a layer
 
 constexpr int kFlowMaxBlocks = 8;                    // CTAs that share an image (portable cluster size)
 
@@ -43,32 +44,43 @@ struct FlowPlan {
   uint32_t step[kFlowMaxSteps];  // (mod 2^32) + distance of the second chunk << 16, in 16-byte units
   int32_t pitch;                 // bytes between 16-byte K chunks of the hidden operands
   int32_t acc_stride;            // words per channel plane of the translation accumulator (pg + 4: no bank conflicts)
+  // 8 x 8 images, one tile each: the last conv as nine taps on the hidden operand itself, in a zero-bordered frame (planes of
+  // 16 channels, s_h), rather than per-tap partials and their shifted sum
+  int32_t direct;
+  // 1: the second (third) GEMM's K steps start as the blocks of its operand are written, a round of blocks at a time
+  int32_t chunk2, chunk3;
   int32_t alias;                 // 1: the third matrix travels through the first one's slot
   int32_t ring;                  // > 0: hidden widths above 256: one tile in flight, weights streamed for every tile in K
   uint32_t ring_slot_bytes;      // steps of 32 bytes through a ring of that many slots at s_w[0]
-  int32_t d_col, d3_col, d3_step;// TMEM columns: slot s has its accumulators at s * d_col, its per-tap partials at
-                                 // d3_col + s * d3_step
+  int32_t d_col, d3_col, d3_step;// TMEM columns: slot s has its accumulators at s * d_col (the second GEMM's d2_col further
+  int32_t d2_col;                // on), those of the last one at d3_col + s * d3_step
   int32_t n_prior;               // columns of the prior head (padded to 16)
   int32_t tmem_cols;
-  uint32_t s_v, s_xa, s_xa_end, s_acc, s_a[2], s_meta[2], s_w[3], s_total;
+  uint32_t s_v, s_xa, s_xa_end, s_acc, s_a[2], s_h[2], s_h_end, s_meta[2], s_w[3], s_total;
   uint32_t mul_per_img, mul_4px, mul_w2, mul_px, mul_w;
   int64_t z_off, prior_off, z_final_off, d, d_fact;
 };
 static_assert(sizeof(FlowPlan) < 1024, "travels as a kernel parameter");
 
 // Meta part of a coupling's packed block. Followed by colA[ca], colB[cb] (physical columns of the flow
-// variable), OutRq[cb], and per hidden layer the FloatRq multipliers of its 32-column blocks, thread
-// order (block, lane & 3, 8 columns), and addends of the blocks from nfb on, in the same order.
+// variable), OutRq[cb], and per hidden layer the FloatRq constants of its 32-column blocks: 32 multipliers, 32 addends, each
+// in thread order (lane & 3, eight columns; so that the four addresses of a 16-byte load lie in different banks).
+struct __align__(16) FlowLayer { // what a hidden epilogue needs, in one load
+  uint8_t ks, nfull, last, plain;// 32-column blocks written, blocks that are full of columns, last block with any, blocks
+                                 // that are full and without an addend
+  int32_t off;                   // its table
+  uint32_t beyond;               // what its output holds where the last blocks have no columns
+  uint8_t half, nfi, us, pad;    // half 1: block nfull has 16 columns; blocks from nfi on have a channel without
+                                 // floating-point constants: integer form with shift us, multipliers M0
+};
 struct FlowMeta {
   int32_t in_m0, in_s;
   int32_t n1, n2, n3;            // MMA N of the three GEMMs
+  int32_t n3d;                   // N of the last conv in its direct form
   int32_t ks2, ks3;              // K steps of the second and third GEMM = 32-column blocks of their operands
-  int32_t nfb1, nfb2;            // blocks below need no addend
-  int32_t nfi1, nfi2;            // blocks from here on hold a channel that has no floating-point constants: integer
-                                 // form, the multiplier table holds M0
-  int32_t us1, us2;              // the layers' shifts (integer form)
-  int32_t off_colA, off_colB, off_out, off_f1, off_f2, off_c1, off_c2;
-  int32_t pad[12];
+  FlowLayer layer[2];
+  int32_t off_colA, off_colB, off_out;
+  int32_t pad[13];
 };
 static_assert(sizeof(FlowMeta) == 128, "meta header is 128 bytes");
 

@@ -319,7 +319,7 @@ void put_out_rq(OutRq* dst, const iodf_layer_desc& L, const Blobs& B) {
 inline size_t wpos(int n_pad, int n, int k) { return (size_t)(k >> 4) * n_pad * 16 + (size_t)n * 16 + (k & 15); }
 
 struct PackedBlock {
-  std::vector<uint8_t> meta, w[3];
+  std::vector<uint8_t> meta, w[4];
   uint32_t k_slices[3] = {0, 0, 0};
 };
 
@@ -331,10 +331,8 @@ void append_block(std::vector<uint8_t>& blob, const PackedBlock& pb, BlockRef* r
     blob.insert(blob.end(), part.begin(), part.end());
   };
   add(pb.meta, &ref->meta_off, &ref->meta_bytes);
-  for (int i = 0; i < 3; ++i) {
-    add(pb.w[i], &ref->w_off[i], &ref->w_bytes[i]);
-    ref->k_slices[i] = pb.k_slices[i];
-  }
+  for (int i = 0; i < 4; ++i) add(pb.w[i], &ref->w_off[i], &ref->w_bytes[i]);
+  for (int i = 0; i < 3; ++i) ref->k_slices[i] = pb.k_slices[i];
   blob.resize(up((uint32_t)blob.size(), kAlign), 0);
 }
 
@@ -539,7 +537,10 @@ void flow_first_matrix(std::vector<uint8_t>& out, int n_pad, const std::vector<K
   }
 }
 
-struct FlowDims { int n1, n2, n3, ks2, ks3; };
+// images of one tile of 64 rows: the last conv can run on the hidden operand directly
+bool flow_direct(const FlowPlan& F) { return F.nbx * F.nby == 1 && F.h == 8 && F.w == 8; }
+
+struct FlowDims { int n1, n2, n3, n3d, ks2, ks3; };
 
 PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, const FlowPlan& F, const std::vector<KByte>& kmap,
                                const HiddenOrder& o1, const HiddenOrder& o2, const int* colA, const int* colB, FlowDims* dims) {
@@ -550,50 +551,54 @@ PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, con
   FlowMeta M{};
   M.in_m0 = cp.in_m0; M.in_s = cp.in_s;
   M.n1 = (int)up(k1, 16); M.n2 = (int)up(k2, 16); M.n3 = (int)up(9 * cbp, 16);
+  M.n3d = (int)(cb <= 32 ? up((uint32_t)cb, 8) : up((uint32_t)cb, 16));        // (M = 64: N a multiple of eight up to 32)
   M.ks2 = (int)up((uint32_t)M.n1 + kBiasRows, 32) / 32; M.ks3 = (int)up((uint32_t)M.n2, 32) / 32;
-  *dims = FlowDims{M.n1, M.n2, M.n3, M.ks2, M.ks3};
+  *dims = FlowDims{M.n1, M.n2, M.n3, M.n3d, M.ks2, M.ks3};
   PackedBlock pb;
   uint32_t off = sizeof(FlowMeta);
   auto take = [&](uint32_t bytes) { const uint32_t o = off; off += up(bytes, 16); return (int)o; };
   M.off_colA = take(16 * ((ca + 3) / 4));
   M.off_colB = take(4 * cb);
   M.off_out = take((uint32_t)sizeof(OutRq) * cb);
-  M.off_f1 = take(128 * M.ks2); M.off_f2 = take(128 * M.ks3);
-  auto first_block = [](const HiddenOrder& o, int blocks, bool integer) {
-    int b = blocks;
-    for (int i = (int)o.ch.size() - 1; i >= 0 && (o.fc[o.ch[i]].none || (!integer && o.fc[o.ch[i]].C)); --i) b = i / 32;
-    return b;
+  auto layer = [&](FlowLayer& l, const HiddenOrder& o, int n, int blocks, uint32_t beyond) {
+    l.ks = (uint8_t)blocks; l.nfull = (uint8_t)(n >> 5); l.last = (uint8_t)((n - 1) >> 5); l.plain = l.nfull; l.nfi = (uint8_t)blocks;
+    for (int i = (int)o.ch.size() - 1; i >= 0 && o.fc[o.ch[i]].none; --i) l.nfi = (uint8_t)(i / 32);
+    for (int i = (int)o.ch.size() - 1; i >= 0 && (o.fc[o.ch[i]].none || o.fc[o.ch[i]].C); --i) l.plain = std::min(l.plain, (uint8_t)(i / 32));
+    l.us = (uint8_t)o.shift;
+    l.off = take(256 * blocks);
+    l.beyond = beyond;
+    l.half = (n >> 4) & 1;
   };
-  M.nfb1 = first_block(o1, M.ks2, false); M.nfb2 = first_block(o2, M.ks3, false);
-  M.nfi1 = first_block(o1, M.ks2, true); M.nfi2 = first_block(o2, M.ks3, true);
-  M.us1 = o1.shift; M.us2 = o2.shift;
-  M.off_c1 = take(128 * (M.ks2 - M.nfb1)); M.off_c2 = take(128 * (M.ks3 - M.nfb2));
+  layer(M.layer[0], o1, M.n1, M.ks2, kBiasColumnsLo);
+  layer(M.layer[1], o2, M.n2, M.ks3, 0u);
   pb.meta.assign(off, 0);
   std::memcpy(pb.meta.data() + M.off_colA, colA, 4 * ca);
   std::memcpy(pb.meta.data() + M.off_colB, colB, 4 * cb);
   put_out_rq(reinterpret_cast<OutRq*>(pb.meta.data() + M.off_out), L3, B);
-  auto tables = [&](const HiddenOrder& o, const iodf_layer_desc& L, int off_f, int off_c, int nfb, int nfi) {
-    float* ft = reinterpret_cast<float*>(pb.meta.data() + off_f);
-    int32_t* ct = reinterpret_cast<int32_t*>(pb.meta.data() + off_c);
+  auto tables = [&](const HiddenOrder& o, const iodf_layer_desc& L, const FlowLayer& l) {
+    uint8_t* t = pb.meta.data() + l.off;
     for (int i = 0; i < (int)o.ch.size(); ++i) {
       const FloatChannel& fc = o.fc[o.ch[i]];
-      if (i >= 32 * nfi) {           // integer blocks: M0 itself
-        std::memcpy(&ft[flow_kpos(i)], B.r + L.requant_off + L.c_out + o.ch[i], 4);
+      const int p = flow_kpos(i);
+      uint8_t* at = t + (p >> 5) * 256 + (p & 31) * 4;
+      const uint32_t addend = 0x80000000u | (uint32_t)fc.C;                     // -C * 2^-149
+      if (i >= 32 * l.nfi) {                       // integer blocks: M0 itself
+        std::memcpy(at, B.r + L.requant_off + L.c_out + o.ch[i], 4);
         continue;
       }
-      ft[flow_kpos(i)] = fc.m;
-      if (fc.C) ct[flow_kpos(i) - 32 * nfb] = (int32_t)(0x80000000u | (uint32_t)fc.C);     // -C * 2^-149
+      std::memcpy(at, &fc.m, 4);
+      if (fc.C) std::memcpy(at + 128, &addend, 4);
     }
   };
-  tables(o1, L1, M.off_f1, M.off_c1, M.nfb1, M.nfi1);
-  tables(o2, L2, M.off_f2, M.off_c2, M.nfb2, M.nfi2);
+  tables(o1, L1, M.layer[0]);
+  tables(o2, L2, M.layer[1]);
   std::memcpy(pb.meta.data(), &M, sizeof(M));
 
   const int32_t* b1 = B.r + L1.requant_off;
   const int32_t* b2 = B.r + L2.requant_off;
   std::vector<int32_t> bias1(k1), bias2(k2);
-  for (int n = 0; n < k1; ++n) bias1[n] = b1[o1.ch[n]] + (n < 32 * M.nfi1 ? o1.fc[o1.ch[n]].beta : 0);
-  for (int n = 0; n < k2; ++n) bias2[n] = b2[o2.ch[n]] + (n < 32 * M.nfi2 ? o2.fc[o2.ch[n]].beta : 0);
+  for (int n = 0; n < k1; ++n) bias1[n] = b1[o1.ch[n]] + (n < 32 * M.layer[0].nfi ? o1.fc[o1.ch[n]].beta : 0);
+  for (int n = 0; n < k2; ++n) bias2[n] = b2[o2.ch[n]] + (n < 32 * M.layer[1].nfi ? o2.fc[o2.ch[n]].beta : 0);
   flow_first_matrix(pb.w[0], M.n1, kmap, B.w + L1.weight_off, ca, k1, o1.ch.data(), bias1.data());
   // 1x1 conv: hidden channels at their operand positions, the bias rows where the epilogue writes the constants
   // (1, 127, 127, 127), the last four bytes of every group of eight in the block behind the columns
@@ -620,6 +625,15 @@ PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, con
     for (int tap = 0; tap < 9; ++tap)
       for (int k = 0; k < k2; ++k)
         pb.w[2][wpos(M.n3, tap * cbp + c, flow_kpos(k))] = (uint8_t)w3[((size_t)c * 9 + tap) * k2 + o2.ch[k]];
+  // the same for the direct form: K chunk by chunk of 32 channels, nine taps each
+  if (flow_direct(F)) {
+    pb.w[3].assign((size_t)M.n3d * 9 * 32 * M.ks3, 0);
+    for (int c = 0; c < cb; ++c)
+      for (int tap = 0; tap < 9; ++tap)
+        for (int k = 0; k < k2; ++k)
+          pb.w[3][wpos(M.n3d, c, (flow_kpos(k) >> 5) * 288 + tap * 32 + (flow_kpos(k) & 31))] =
+              (uint8_t)w3[((size_t)c * 9 + tap) * k2 + o2.ch[k]];
+  }
   pb.k_slices[0] = (uint32_t)kmap.size() / 32; pb.k_slices[1] = (uint32_t)M.ks2; pb.k_slices[2] = (uint32_t)M.ks3;
   return pb;
 }
@@ -934,34 +948,42 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
 }
 
 // Group, tensor-memory columns and shared-memory layout of a level in the compact kernel. false: it does not fit.
-struct FlowNeeds { uint32_t n_hidden = 32, n_taps = 16, kb = 1, meta = 16, w[3] = {16, 16, 16}; };
-// wide: weights streamed for every tile, one tile in flight.
-bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool wide) {
+struct FlowNeeds { uint32_t n_hidden = 32, n_taps = 16, n_direct = 16, kb = 1, meta = 16, w[4] = {16, 16, 16, 16}; };
+// wide: weights streamed for every tile, one tile in flight. direct: the last conv in its direct form.
+bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool wide, bool direct) {
   F.group = group;
+  F.direct = direct;
   F.pg = group * F.px;
   F.tiles = F.im2col ? (group + 3) / 4 : group * F.tiles_img;
-  const uint32_t nh = up(nd.n_hidden, 16), nh32 = up(nd.n_hidden, 32);
-  if (nd.n_hidden > 512 || nd.n_taps > 512 || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
+  const uint32_t nh = up(nd.n_hidden, 16), nh32 = up(nd.n_hidden, 32), n_last = direct ? nd.n_direct : nd.n_taps;
+  if (nd.n_hidden > 512 || n_last > (direct ? 128u : 512u) || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
     return false;
-  F.d_col = 0; F.d3_col = 0; F.d3_step = 0;
+  F.d_col = 0; F.d3_col = 0; F.d3_step = 0; F.d2_col = 0; F.chunk2 = 0;
+  // K steps of the last GEMM run ahead of the epilogue that writes their operand: its accumulators must not lie on columns
+  // that the epilogue's later rounds read
+  F.chunk3 = direct;
   if (wide) {
     F.tmem_cols = 512;
   } else if (F.tiles == 1) {
-    F.tmem_cols = (int)pow2_cols(std::max(std::max(nh32, nd.n_taps), (uint32_t)F.n_prior));
+    F.chunk2 = F.m == 64 && 2 * nh32 <= 512u;
+    F.d2_col = F.chunk2 ? (int)nh32 : 0;
+    F.tmem_cols = (int)pow2_cols(std::max(std::max((uint32_t)F.d2_col + nh32, n_last), (uint32_t)F.n_prior));
   } else {
     // several tiles: two slots; with more than two tiles the per-tap partials need columns of their own, because
     // a slot's next tile starts before its shifted sum
-    const bool apart = 2 * nh + 2 * nd.n_taps <= 512u && nh + nh32 <= 512u;
-    if (!apart && (F.tiles > 2 || std::max(nh32, nd.n_taps) > 256u)) return false;
+    const bool apart = 2 * nh + 2 * n_last <= 512u && nh + nh32 <= 512u;
+    if (!apart && (F.tiles > 2 || std::max(nh32, n_last) > 256u)) return false;
     F.d_col = apart ? (int)nh : 256;
     F.d3_col = apart ? 2 * (int)nh : 0;
-    F.d3_step = apart ? (int)nd.n_taps : 256;
+    F.d3_step = apart ? (int)n_last : 256;
+    F.chunk3 = direct && (apart || n_last <= 64u);
     F.tmem_cols = 512;
   }
   F.pitch = F.m * 16 + 64;
   F.acc_stride = F.pg + 4;
   for (int alias = 0; alias < 2; ++alias) {
     if (alias && (F.tiles > 2 || wide)) continue;
+    const uint32_t w_last = nd.w[direct ? 3 : 2];
     uint32_t off = 0;
     auto take = [&](uint32_t bytes) { const uint32_t o = off; off = up(off + bytes, kAlign); return o; };
     F.alias = alias;
@@ -974,10 +996,16 @@ bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool
       F.s_xa = take((uint32_t)(F.rec / 16) * F.plane16 * 16);
     }
     F.s_xa_end = off;
-    F.s_acc = F.im2col ? 0 : take((uint32_t)F.cb * F.acc_stride * 4);
+    F.s_acc = F.im2col || direct ? 0 : take((uint32_t)F.cb * F.acc_stride * 4);
     const uint32_t a_bytes = 2u * nd.kb * F.pitch;
     F.s_a[0] = take(a_bytes);
     F.s_a[1] = F.tiles > 1 && !wide ? take(a_bytes) : F.s_a[0];
+    if (direct) {
+      const uint32_t h_bytes = 32u * nd.kb * (uint32_t)F.frame;
+      F.s_h[0] = take(h_bytes);
+      F.s_h[1] = F.tiles > 1 ? take(h_bytes) : F.s_h[0];
+      F.s_h_end = off;
+    }
     F.s_meta[0] = take(nd.meta);
     F.s_meta[1] = take(nd.meta);
     if (wide) {          // a ring of K steps in what is left: at least three, so that copies and MMAs overlap
@@ -987,9 +1015,9 @@ bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool
       F.ring = std::min<int>(kFlowMaxRing, (int)((limit - off) / F.ring_slot_bytes));
       off += (uint32_t)F.ring * F.ring_slot_bytes;
     } else {
-      F.s_w[0] = take(alias ? std::max(nd.w[0], nd.w[2]) : nd.w[0]);
+      F.s_w[0] = take(alias ? std::max(nd.w[0], w_last) : nd.w[0]);
       F.s_w[1] = take(nd.w[1]);
-      F.s_w[2] = alias ? F.s_w[0] : take(nd.w[2]);
+      F.s_w[2] = alias ? F.s_w[0] : take(w_last);
     }
     F.s_total = off;
     if (off > limit) continue;
@@ -1247,6 +1275,7 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
                                         cols[ki].data() + F.ca, &d));
     nd.n_hidden = std::max<uint32_t>(nd.n_hidden, (uint32_t)std::max(d.n1, d.n2));
     nd.n_taps = std::max<uint32_t>(nd.n_taps, (uint32_t)d.n3);
+    nd.n_direct = std::max<uint32_t>(nd.n_direct, (uint32_t)d.n3d);
     nd.kb = std::max<uint32_t>(nd.kb, (uint32_t)std::max(d.ks2, d.ks3));
     widths += d.n1 + d.n2;
   }
@@ -1256,7 +1285,7 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   auto add = [&](const PackedBlock& pb, BlockRef* ref) {
     append_block(hl.blob, pb, ref);
     nd.meta = std::max(nd.meta, ref->meta_bytes);
-    for (int g = 0; g < 3; ++g) nd.w[g] = std::max(nd.w[g], ref->w_bytes[g]);
+    for (int g = 0; g < 4; ++g) nd.w[g] = std::max(nd.w[g], ref->w_bytes[g]);
   };
   for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) add(blocks[ki], &P.coupling[ki]);
   if (lv.has_prior) add(prior, &P.prior);
@@ -1264,7 +1293,10 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   // and tile, which one tile's chain of GEMMs does not hide
   auto plan = [&](FlowPlan& f, int group) {
     if ((uint64_t)group * f.c * f.fpx * ((uint64_t)f.c * f.fpx) >= (1ull << 32)) return false;      // (the index maps' divisions)
-    return (nd.n_hidden <= 256 && plan_flow(f, nd, smem_limit, group, false)) || plan_flow(f, nd, smem_limit, group, true);
+    for (int wide = nd.n_hidden > 256; wide < 2; ++wide)
+      for (int direct = flow_direct(f) && !wide; direct >= 0; --direct)
+        if (plan_flow(f, nd, smem_limit, group, wide != 0, direct != 0)) return true;
+    return false;
   };
   const FlowPlan whole = F0;
   hl.flow.clear();
@@ -1279,7 +1311,8 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   auto add_shape = [&](const FlowPlan& f, int ctas) {
     const double width = widths / (200.0 * F.n_couplings), cb = f.cb / 10.0;
     double cost = 11.0 / F.n_couplings + (f.im2col ? 0.7 * f.group : 0);
-    if (f.ring) cost += 4 + f.tiles * (5.7 + 2.9 * width + 2.9 * cb) + (f.nbx * f.nby > 1 ? 3 : 0);
+    if (f.direct) cost += 4.9 + f.tiles * (0.75 + 3 * width + 0.85 * cb) + (f.tiles == 1 ? 1.9 : 0);      // (one tile: all in series)
+    else if (f.ring) cost += 4 + f.tiles * (5.7 + 2.9 * width + 2.9 * cb) + (f.nbx * f.nby > 1 ? 3 : 0);
     else cost += 5 + 0.5 * width + f.tiles * (2.2 + 1.5 * width + 0.8 * cb) + (f.nbx * f.nby > 1 ? 2.6 + 1.5 * cb : 0);
     hl.flow.push_back({f, ctas, cost});
   };

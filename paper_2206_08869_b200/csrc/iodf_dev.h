@@ -91,7 +91,7 @@ static_assert(sizeof(PriorMeta) == 128, "meta header is 128 bytes");
 
 struct BlockRef {                // where a block's parts sit in the level blob (byte offsets)
   uint32_t meta_off, meta_bytes;
-  uint32_t w_off[3], w_bytes[3];
+  uint32_t w_off[4], w_bytes[4]; // (the fourth: the last conv in the compact kernel's direct form)
   uint32_t k_slices[3];          // K / 32 of each matrix (a K-slice of 32 bytes is w_bytes / k_slices contiguous bytes)
 };
 

@@ -12,6 +12,21 @@ from test_gpu_residual import _both_ways
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("splits,hidden,batch,sample", [
+    ([False], 16, 3, None),               # six channels in eight columns; the narrowest layers
+    ([True], 33, 150, [0, 147, 149]),     # more images than SMs: two to a CTA, one alone
+    ([True], 256, 2, None),               # nine blocks: the second GEMM's operand has one more than the third's
+    ([True, True, True], 129, 1, None),   # 24 channels, as many columns as there are
+    ([True, True, True], 160, 700, [0, 1, 349, 698, 699]),      # several to a CTA, the last with fewer
+])
+@pytest.mark.parametrize("plan", [0, 1])
+def test_last_conv_on_8x8_frames(G, splits, hidden, batch, sample, plan):
+    hw = 8 << len(splits)
+    model = S.make_model(0xF800 + hw + hidden, 3, hw, hw, splits, 3, hidden)
+    x = S.smooth_field_images(0xF900 + hw, batch, hw, hw, 2.0)
+    _check_both_ways(G, model, x, sample=sample, plan=plan)
+
+
 @pytest.mark.parametrize("hw,splits,hidden,batch", [
     (16, [True, True], 16, 5),           # the last level 4 x 4: four images and one
     (16, [True, True], 31, 3),           # 8 x 8 tiles of 64 rows, six and twelve channels in
