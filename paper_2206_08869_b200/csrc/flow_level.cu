@@ -39,7 +39,9 @@
 // shifted sum and their hand-overs (52 % of all issue slots at 32 x 32, 39 % at 8 x 8, 24 % at 4 x 4). Measured for eight
 // couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 161 us,
 // 16 x 16 85 -> 63, 8 x 8 63 -> 48, 4 x 4 70 -> 48; one image, 32 x 32 split in eight: 52. Width 512, 64 images of
-// 32 x 32, split in two: 2 357 -> 380 us.
+// 32 x 32, split in two: 2 357 -> 288 us, of which the tensor core works 95.
+#include <stddef.h>
+
 #include "flow_level.h"
 #include "level_device.cuh"
 
@@ -212,16 +214,21 @@ __device__ void flow_loader(const Flow& f, const FlowPlan& P, const LevelArgs& a
   }
 }
 
-// Streamed weights (P.ring): for every tile the K steps of its GEMMs, in order, through the ring
-__device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st) {
+// Streamed weights (P.ring): for every tile the K steps of its GEMMs, in order, through the ring, as many to a slot as it
+// holds. What bounds the stream is the 300 - 600 clocks that a warp spends on a copy, whatever its size (the copies themselves run
+// at over 100 bytes per clock and SM), so two warps take the slots in turn.
+__device__ __forceinline__ int flow_slot_steps(const FlowPlan& P, int n) { return max(1, (int)(P.ring_slot_bytes >> 5) / n); }
+
+__device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st, uint32_t which) {
   FlowCtl* ctl = f.ctl;
-  uint32_t slot = 0, round = 0;
+  const bool lead = ptx::elect_one();
+  uint32_t slot = 0, round = 0, turn = which;          // slot of a GEMM's first step; 0 if that is this warp's, else 1
 #pragma unroll 1
   for (int i = 0; i < st.nsteps; ++i) {
     const BlockRef& br = step_ref(*a.plan, st, i);
     // meta slot of step i: its last reader was the pixel pass of step i - 1
     if (i >= 2) flow_wait(f, &ctl->xa_ready[(i - 1) & 1], (uint32_t)((i - 1) >> 1) & 1u);
-    {
+    if (which == 0 && lead) {
       const uint32_t b = ptx::smem_u32(&ctl->meta_full[i & 1]);
       ptx::mbar_expect_tx(b, br.meta_bytes);
       ptx::bulk_g2s(ptx::smem_u32(f.smem + P.s_meta[i & 1]), a.blob + br.meta_off, br.meta_bytes, b);
@@ -231,16 +238,25 @@ __device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelAr
     for (int t = 0; t < f.tiles; ++t)
 #pragma unroll 1
       for (int g = 0; g < gemms; ++g) {
-        const uint32_t ks = br.k_slices[g], bytes = br.w_bytes[g] / ks;
-        const uint8_t* src = a.blob + br.w_off[g];
+        const uint32_t step = br.w_bytes[g] / br.k_slices[g], all = br.w_bytes[g], bytes = (uint32_t)flow_slot_steps(P, (int)(step >> 5)) * step;
+        uint32_t off = turn * bytes, count = (all + bytes - 1) / bytes;
+        auto advance = [&](uint32_t& sl, uint32_t& ro, uint32_t by) {
+          for (sl += by; sl >= (uint32_t)P.ring; sl -= (uint32_t)P.ring) ++ro;
+        };
+        uint32_t sl = slot, ro = round;
+        advance(sl, ro, turn);
 #pragma unroll 1
-        for (uint32_t k = 0; k < ks; ++k, src += bytes) {
-          if (round > 0) flow_wait(f, &ctl->w_empty[slot], (round - 1u) & 1u);
-          const uint32_t b = ptx::smem_u32(&ctl->w_full[slot]);
-          ptx::mbar_expect_tx(b, bytes);
-          ptx::bulk_g2s(ptx::smem_u32(f.smem + P.s_w[0] + slot * P.ring_slot_bytes), src, bytes, b);
-          if (++slot == (uint32_t)P.ring) { slot = 0; ++round; }
+        for (; off < all; off += 2 * bytes) {
+          if (ro > 0) flow_wait(f, &ctl->w_empty[sl], (ro - 1u) & 1u);
+          if (lead) {
+            const uint32_t b = ptx::smem_u32(&ctl->w_full[sl]), now = min(bytes, all - off);
+            ptx::mbar_expect_tx(b, now);
+            ptx::bulk_g2s(ptx::smem_u32(f.smem + P.s_w[0] + sl * P.ring_slot_bytes), a.blob + br.w_off[g] + off, now, b);
+          }
+          advance(sl, ro, 2);
         }
+        advance(slot, round, count);
+        turn ^= count & 1u;
       }
   }
 }
@@ -374,7 +390,9 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
   }
 }
 
-// MMA warp of levels with streamed weights: one tile at a time, all accumulators from column 0 on
+// MMA warp of levels with streamed weights: one tile at a time, all accumulators from column 0 on. A step of 32 K bytes keeps
+// the tensor core 256 clocks at width 512, and a wait, a commit and the bookkeeping of a slot took this warp 450 (with a copy
+// per step for every GEMM and a wait for each): 64 images of 32 x 32 360 -> 288 us, of 4 x 4 112 -> 98.
 __device__ void flow_mma_ring(const Flow& f, const FlowPlan& P, const Steps& st) {
   FlowCtl* ctl = f.ctl;
   uint8_t* smem = f.smem;
@@ -383,33 +401,45 @@ __device__ void flow_mma_ring(const Flow& f, const FlowPlan& P, const Steps& st)
   const uint32_t xa16 = (ptx::smem_u32(smem + P.s_xa) >> 4) & 0x3FFFu, hi = ptx::kUmmaDescHi;
   const uint32_t a1_hi = (uint32_t)P.sbo16 | (1u << 14), pitch16 = (uint32_t)P.pitch >> 4;
   const uint32_t a_lo = ((ptx::smem_u32(smem + P.s_a[0]) >> 4) & 0x3FFFu) | (pitch16 << 16);
-  uint32_t slot = 0, round = 0, apar = 0;
-  // one GEMM: K step s reads A at al(s); N above 256 in two parts
-  auto gemm = [&](uint32_t d, int n, int ks, auto al, uint32_t ahi, uint64_t* done) {
-    const int na = min(n, 256);
-    const uint32_t idesc = idesc_m | ((uint32_t)(na >> 3) << 17), idesc2 = idesc_m | ((uint32_t)((n - na) >> 3) << 17);
+  const uint32_t w16 = (ptx::smem_u32(smem + P.s_w[0]) >> 4) & 0x3FFFu, slot16 = P.ring_slot_bytes >> 4;
+  const uint32_t full0 = ptx::smem_u32(&ctl->w_full[0]), last = full0 + 8u * (uint32_t)(P.ring - 1);
+  constexpr uint32_t kToEmpty = (uint32_t)(offsetof(FlowCtl, w_empty) - offsetof(FlowCtl, w_full));
+  const bool lead = ptx::elect_one();
+  uint32_t bar = full0, bw = w16, wpar = 0, apar = 0;          // next slot: its barrier, its address, the phase's parity
+  bool full = false;                           // its copy has landed (asked ahead: a wait takes a hundred clocks)
+  // one GEMM: K step s reads A at `al`, then step(s, al) is the next one; N above 256 in two parts
+  auto gemm = [&](uint32_t d, int n, int ks, uint32_t al, auto step, uint32_t ahi, uint64_t* done) {
+    const int na = min(n, 256), sp = flow_slot_steps(P, n);
+    const uint32_t idesc = idesc_m | ((uint32_t)(na >> 3) << 17), idesc2 = idesc_m | ((uint32_t)((n - na) >> 3) << 17), lbo = (uint32_t)n << 16;
+    uint32_t acc = 0;
+    int left = sp;
 #pragma unroll 1
-    for (int s = 0; s < ks; ++s) {
-      flow_wait(f, &ctl->w_full[slot], round & 1u);
+    for (int s = 0; s < ks;) {
+      if (!full) flow_wait_at(bar, wpar, ctl, f.status);
       ptx::tc_fence_after();
-      const uint32_t bl = ((ptx::smem_u32(smem + P.s_w[0] + slot * P.ring_slot_bytes) >> 4) & 0x3FFFu) | ((uint32_t)n << 16);
-      const uint32_t a = al(s);
-      if (ptx::elect_one()) {
-        ptx::umma_i8_hl(d, a, ahi, bl, hi, idesc, s > 0 ? 1u : 0u);
-        if (n > 256) ptx::umma_i8_hl(d + 256u, a, ahi, bl + 256u, hi, idesc2, s > 0 ? 1u : 0u);
-        ptx::umma_commit(ptx::smem_u32(&ctl->w_empty[slot]));
-        if (s + 1 == ks && done) ptx::umma_commit(ptx::smem_u32(done));
+      const uint32_t empty = bar + kToEmpty;
+      uint32_t bl = bw | lbo;
+      if (bar == last) { bar = full0; bw = w16; wpar ^= 1u; }
+      else { bar += 8u; bw += slot16; }
+      full = ptx::mbar_test_wait(bar, wpar);
+      for (left = sp; ; bl += 2u * (uint32_t)n) {
+        if (lead) ptx::umma_i8_hl(d, al, ahi, bl, hi, idesc, acc);
+        if (n > 256 && lead) ptx::umma_i8_hl(d + 256u, al, ahi, bl + 256u, hi, idesc2, acc);
+        acc = 1u;
+        ++s;
+        al = step(s, al);
+        if (--left == 0 || s == ks) break;
       }
-      __syncwarp();
-      if (++slot == (uint32_t)P.ring) { slot = 0; ++round; }
+      if (lead) ptx::umma_commit(empty);
     }
+    if (done && lead) ptx::umma_commit(ptx::smem_u32(done));
   };
   auto wait_a = [&]() {
     flow_wait(f, &ctl->a_ready[0][0], apar);
     apar ^= 1u;
     ptx::tc_fence_after();
   };
-  auto hidden = [&](int s) { return a_lo + (uint32_t)s * 2u * pitch16; };
+  auto hidden = [&](int, uint32_t al) { return al + 2u * pitch16; };
 #pragma unroll 1
   for (int i = 0; i < st.nsteps; ++i) {
     const bool prior = st.is_prior(i);
@@ -422,17 +452,17 @@ __device__ void flow_mma_ring(const Flow& f, const FlowPlan& P, const Steps& st)
 #pragma unroll 1
     for (int t = 0; t < f.tiles; ++t) {
       const uint32_t base = xa16 + (uint32_t)uniform(ctl->tile[t].w);
-      auto first = [&](int s) { return base + P.step[s]; };
+      auto first = [&](int s, uint32_t) { return base + P.step[min(s, kFlowMaxSteps - 1)]; };
       if (prior) {
-        gemm(f.tmem + (uint32_t)(t * P.n_prior), n1, P.ks1, first, a1_hi, t + 1 == f.tiles ? &ctl->dm_ready[0] : nullptr);
+        gemm(f.tmem + (uint32_t)(t * P.n_prior), n1, P.ks1, first(0, 0u), first, a1_hi, t + 1 == f.tiles ? &ctl->dm_ready[0] : nullptr);
         continue;
       }
       if (t > 0) wait_a();                     // the last tile's partials have been summed
-      gemm(f.tmem, n1, P.ks1, first, a1_hi, &ctl->dm_ready[0]);
+      gemm(f.tmem, n1, P.ks1, first(0, 0u), first, a1_hi, &ctl->dm_ready[0]);
       wait_a();
-      gemm(f.tmem, n2, ks2, hidden, hi, &ctl->dm_ready[0]);
+      gemm(f.tmem, n2, ks2, a_lo, hidden, hi, &ctl->dm_ready[0]);
       wait_a();
-      gemm(f.tmem, n3, ks3, hidden, hi, &ctl->d3_ready[0]);
+      gemm(f.tmem, n3, ks3, a_lo, hidden, hi, &ctl->d3_ready[0]);
     }
   }
 }
@@ -1097,15 +1127,13 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
   st.inverse = kInv;
 
   if (warp >= kFlowWarps && kSplit) flow_cluster_sync();        // (the workers below, after the frame)
-  if (warp == kFlowWarps + 2) {
-    // packed blocks: written once, at model creation
-    if (lane == 0) {
-      if (P.ring) flow_loader_ring(f, P, a, st);
-      else flow_loader(f, P, a, st);
-    }
+  // (packed blocks were written once, at model creation)
+  if (warp == kFlowWarps + 2 && !P.ring) {
+    if (lane == 0) flow_loader(f, P, a, st);
   } else if (warp >= kFlowWarps) {
     if (!P.ring) flow_mma<kShape>(f, P, st, warp - kFlowWarps);
     else if (warp == kFlowWarps) flow_mma_ring(f, P, st);
+    else flow_loader_ring(f, P, a, st, (uint32_t)(warp - kFlowWarps - 1));
   } else {
     // frame of the network input: zero channels, and the constants that multiply the bias rows in the
     // bytes that no channel uses (at 4 x 4 levels: after the nine taps)
