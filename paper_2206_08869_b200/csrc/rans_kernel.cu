@@ -25,6 +25,9 @@ namespace {
 constexpr int kWin = 2048;
 constexpr uint32_t kM = 1u << 16;
 constexpr int kThreadsPerBlock = 128;
+// More streams than this (24 per SM): half a warp each. Whole warps and halves measured: 3 072 streams 69 and 73 us, 3 600 75 and 75 (55
+// and 44 without prior parameters), 6 144 111 and 88, 7 200 122 and 103.
+constexpr long kHalfWarpStreams = 3584;
 
 struct Tables {
   const uint16_t* G;       // shared memory
@@ -177,8 +180,7 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_encode_kernel(const Ran
 //     stream backwards); the three words that a symbol can take are handed out before its search.
 // What bounds it depends on the block (128 images of 64 x 64, 128 elements per stream). The small ones are a stream's chain:
 // 35 us for the final block, 540 clocks per symbol, 50 us for those with prior parameters (60 - 70 with three search
-// rounds). The largest, 6 144 streams, ten warps per scheduler, is bound by issue slots, 0.72 per cycle:
-// 111 us (170), 1 700 clocks per symbol of a warp.
+// rounds). Blocks of more streams than kHalfWarpStreams go to the kernel below.
 __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const RansArgs a, int q,
                                                                        const uint16_t* __restrict__ words,
                                                                        const uint32_t* __restrict__ counts,
@@ -259,6 +261,100 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const Ran
   if (top != used || x != (1u << 16)) bad = 1u;    // every word used, none missing, and the state back at its start
   bad = __any_sync(0xFFFFFFFFu, bad != 0) ? 1u : 0u;
   if (bad && lane == 0 && a.errors) atomicAdd(a.errors, 1u);
+}
+
+// The same with HALF a warp per stream, for blocks of so many streams that issue slots bound the time (6 144 streams: ten warps
+// per scheduler, 0.72 of the slots used) and not a stream's chain, which is longer with fewer lanes: more symbols need a
+// first round. A warp's two streams go side by side, so steps that only some symbols take (escapes, a word more)
+// are selections, not branches. Words: the lanes hold the next 16, replaced lane by lane every four symbols from the ones after
+// them, which were asked for four symbols earlier; prior parameters are loaded 16 symbols ahead.
+// 128 elements per stream: 6 144 streams 111 -> 88 us, 28 800 412 -> 305. (No gain in either kernel: the first look-up in shared
+// memory, 34 clocks instead of 106 but 33 KB to load per CTA; warp reductions instead of ballot and shuffles.)
+__global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_half_kernel(const RansArgs a, int q,
+                                                                       const uint16_t* __restrict__ words,
+                                                                       const uint32_t* __restrict__ counts,
+                                                                       const int32_t* __restrict__ prior,
+                                                                       int32_t* __restrict__ z) {
+  constexpr unsigned kAll = 0xFFFFFFFFu;
+  constexpr int kLanes = 16;
+  extern __shared__ __align__(16) uint8_t smem[];
+  uint32_t* sR = reinterpret_cast<uint32_t*>(smem);
+  uint16_t* sG = reinterpret_cast<uint16_t*>(smem + 4 * a.n_scales);
+  load_tables(a, sG, sR);
+  const Tables t{sG, sR, a.umax, a.n_scales};
+  const RansBlock blk = a.blocks[q];
+  const int lane = threadIdx.x & (kLanes - 1), shift = threadIdx.x & 31 & ~(kLanes - 1);      // in the stream's lanes; the first of them
+  const long wid = ((long)blockIdx.x * blockDim.x + threadIdx.x) / kLanes, total = (long)a.batch * blk.n_streams;
+  if (((long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) / kLanes >= total) return;       // (no stream in the whole warp)
+  const long me = min(wid, total - 1);                 // (a warp's second half may have none: it decodes nothing)
+  const int b = (int)(me / blk.n_streams), j = (int)(me - (long)b * blk.n_streams), ns = blk.n_streams;
+  const long sid = (long)b * a.n_streams + blk.first_stream + j;
+  const int n_el = wid < total ? (int)((blk.n - j + ns - 1) / ns) : 0;
+  const int top = (int)min((long)counts[sid], (long)a.cap);
+  const uint16_t* in = words + sid * a.cap + top - 1;
+  // word i from the stream's end, 0 before its first word
+  auto word = [&](int i) { return i < top ? (uint32_t)in[-i] : 0u; };
+  int used = 2, mine = lane;                           // words taken; the one that this lane holds (of used .. used + kLanes - 1)
+  uint32_t win = word(lane), next = word(lane + kLanes), bad = 0;
+  uint32_t x = __shfl_sync(kAll, win, 0, kLanes) << 16 | __shfl_sync(kAll, win, 1, kLanes);
+  int32_t* zb = z + (long)b * a.d + blk.z_off + j;
+  const int32_t* pb = prior + (long)b * 2 * a.d_fact;
+  // this lane's element of the next kLanes: its prior parameters, a round ahead
+  int32_t mu_n = 0;
+  int ls_n = a.final_ls;
+  if (lane < n_el) prior_of(a, blk, pb, j + (long)lane * ns, &mu_n, &ls_n, &bad);
+  const int n_most = (int)__reduce_max_sync(kAll, (unsigned)n_el);      // (a warp's streams differ by one element at most)
+  for (int i0 = 0; i0 < n_most; i0 += kLanes) {
+    const int32_t mu_l = mu_n;
+    const uint32_t R_l = t.R[ls_n], row_l = (uint32_t)ls_n << 8;
+    if (i0 + kLanes + lane < n_el) prior_of(a, blk, pb, j + (long)(i0 + kLanes + lane) * ns, &mu_n, &ls_n, &bad);
+    int32_t zv_l = 0;
+    const int n_here = min(kLanes, n_most - i0);
+    for (int ii = 0; ii < n_here; ++ii) {
+      if ((ii & (kLanes / 4 - 1)) == 0 && mine < used) {          // (kLanes / 4 symbols take three quarters of the words at most)
+        win = next;
+        mine += kLanes;
+        next = word(mine + kLanes);
+      }
+      // what does not depend on the state is on its way during the search
+      const uint32_t R = __shfl_sync(kAll, R_l, ii, kLanes), row = __shfl_sync(kAll, row_l, ii, kLanes);
+      const uint32_t w0 = __shfl_sync(kAll, win, used, kLanes), w1 = __shfl_sync(kAll, win, used + 1, kLanes);
+      const uint32_t w2 = __shfl_sync(kAll, win, used + 2, kLanes);
+      const uint32_t slot = x & 0xFFFFu;
+      // largest k with Cum(k) <= slot, among the symbols that the slot can mean
+      const uint32_t range = __ldg(a.ranges + row + (slot >> 8));
+      int k = (int)(range & 0xFFFFu), d = (int)(range >> 16) - 1;            // k .. k + d
+      auto last_below = [&](uint32_t c) {              // lane of the stream's last value that is not above the slot (Cum is monotone)
+        return 31 - __clz((int)((__ballot_sync(kAll, c <= slot) >> shift) & (kAll >> (32 - kLanes))));
+      };
+      while (__any_sync(kAll, d > kLanes - 2)) {       // (at most twice)
+        const int step = d > kLanes - 2 ? (d + kLanes) / kLanes : 1;
+        k += last_below(cum_of(t, R, k + lane * step)) * step;
+        d = step - 1;
+      }
+      const uint32_t cl = cum_of(t, R, k + lane);
+      const int sel = last_below(cl);                  // at most kLanes - 2
+      const uint32_t C = __shfl_sync(kAll, cl, sel, kLanes), Cn = __shfl_sync(kAll, cl, sel + 1, kLanes);
+      k += sel;
+      uint32_t y = (Cn - C) * (x >> 16) + slot - C;
+      const bool more = y < (1u << 16), escape = k == 0 || k == 2 * kWin;
+      if (more) y = (y << 16) | w0;
+      // an escape: two symbols of frequency 1, the value's upper and lower half; each takes the state's lower 16 bits and
+      // a word in their place (x >> 16 is always below 2^16)
+      const uint32_t wa = more ? w1 : w0, wb = more ? w2 : w1;
+      const int32_t zv = escape ? (int32_t)((y << 16) | wa) : (int32_t)((uint32_t)mu_l + (uint32_t)(k - kWin));      // (lane ii's counts)
+      if (escape) y = (y & 0xFFFF0000u) | wb;
+      if (lane == ii) zv_l = zv;
+      if (i0 + ii < n_el) {
+        x = y;
+        used += (more ? 1 : 0) + (escape ? 2 : 0);
+      }
+    }
+    if (i0 + lane < n_el) zb[(long)(i0 + lane) * ns] = zv_l;
+  }
+  if (n_el > 0 && (top != used || x != (1u << 16))) bad = 1u;    // every word used, none missing, and the state back at its start
+  const unsigned any = __ballot_sync(kAll, bad != 0) >> shift & (kAll >> (32 - kLanes));
+  if (any && lane == 0 && wid < total && a.errors) atomicAdd(a.errors, 1u);
 }
 
 // ---- compact byte stream -----------------------------------------------------------------------------
@@ -394,9 +490,12 @@ cudaError_t launch_rans_encode(const RansArgs& a, const int32_t* z, const int32_
 
 cudaError_t launch_rans_decode(const RansArgs& a, int block, const uint16_t* words, const uint32_t* counts,
                                const int32_t* prior, int32_t* z, cudaStream_t stream) {
-  const long total = (long)a.batch * a.blocks[block].n_streams * 32;        // a warp per stream
+  const long streams = (long)a.batch * a.blocks[block].n_streams;
+  const bool half = streams > kHalfWarpStreams;
+  const long total = streams * (half ? 16 : 32);
   const unsigned grid = (unsigned)((total + kThreadsPerBlock - 1) / kThreadsPerBlock);
-  rans_decode_kernel<<<grid, kThreadsPerBlock, table_smem(a), stream>>>(a, block, words, counts, prior, z);
+  if (half) rans_decode_half_kernel<<<grid, kThreadsPerBlock, table_smem(a), stream>>>(a, block, words, counts, prior, z);
+  else rans_decode_kernel<<<grid, kThreadsPerBlock, table_smem(a), stream>>>(a, block, words, counts, prior, z);
   return cudaGetLastError();
 }
 

@@ -124,13 +124,14 @@ def test_residual_blocks_through_long_chains(G, hidden, batch, plan):
     G.iodf_check(m)
 
 
+@pytest.mark.parametrize("B,elems", [(3, 97), (241, 103)])          # 45 and 3 615 streams to a block: a warp each, half of one
 @pytest.mark.parametrize("ls", [0, 20, 40, 63])
-def test_symbol_look_up_at_every_kind_of_scale(G, ls):
+def test_symbol_look_up_at_every_kind_of_scale(G, ls, B, elems):
     """Residuals over the whole window at one scale: slots that mean one symbol and slots that mean hundreds."""
     import torch
     model = S.make_model(0xF500, 3, 32, 32, [True, False], 1, 16)
-    codec = S.logistic_codec(elems_per_stream=97)
-    B, d, d_fact = 3, 3 * 32 * 32, 6 * 256
+    codec = S.logistic_codec(elems_per_stream=elems)
+    d, d_fact = 3 * 32 * 32, 6 * 256
     rng = np.random.default_rng(ls)
     prior = np.stack([rng.integers(-50, 50, (B, d_fact)), np.full((B, d_fact), ls)], axis=1).astype(np.int32)
     z = rng.integers(-2200, 2201, (B, d)).astype(np.int32)
@@ -149,3 +150,9 @@ def test_symbol_look_up_at_every_kind_of_scale(G, ls):
         G.iodf_rans_decode_block(cd, q, words, counts, _t(prior), out)
     G.iodf_codec_check(cd)
     np.testing.assert_array_equal(out.cpu().numpy(), z)
+    counts[B - 1, 0] -= 1                             # a stream that lacks its last word is noticed, the others are not touched
+    out.zero_()
+    G.iodf_rans_decode_block(cd, 0, words, counts, _t(prior), out)
+    with pytest.raises(G.IodfError):
+        G.iodf_codec_check(cd)
+    np.testing.assert_array_equal(out.cpu().numpy()[:B - 1, :d_fact], z[:B - 1, :d_fact])
