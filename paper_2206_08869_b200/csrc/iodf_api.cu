@@ -1304,16 +1304,18 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   // per CTA (fewer waves when images outnumber SMs), or images split over clusters of CTAs (idle SMs otherwise). The
   // throughput plan keeps the one that takes the least SM time per image, with no more images than fill a tile. Time of a
   // wave per coupling, in thousands of clocks: a serial part, a part for each tile of the CTA that grows with the mean
-  // hidden width and the channels that are translated, the exchange of their edges, what an image more costs at 4 x 4, and a
-  // share of the level's load and store. Fitted to 399 shapes of 31 flows (widths 16 - 512, 4 - 96 channels, 4 x 4 - 32 x
-  // 32, resident and streamed); over batches of 1 - 1 023 the shape it picks takes 0.1 % longer than the best one on
-  // average and 7 % at most, on 14 other flows 0.4 % and 10 % (constants that did not know the width: 0.6 % and 20 %).
+  // hidden width and the channels that are translated, the exchange of their edges, what an image more costs at 4 x 4, a
+  // weight ring too short to run ahead of wide layers, and a share of the level's load and store. Fitted to 87 shapes of five flows
+  // (mean widths 64 - 512, 6 - 48 channels, 4 x 4 - 32 x 32, resident, streamed and direct: 3 % off on average); over batches
+  // of 1 - 1 184 the shape it picks takes 0.1 % longer than the best one on average and 2 % at most, 13 % at eight 4 x 4 images of
+  // width 512 (constants of before those kernels changed: 0.7 % and 19 %).
   auto add_shape = [&](const FlowPlan& f, int ctas) {
     const double width = widths / (200.0 * F.n_couplings), cb = f.cb / 10.0;
-    double cost = 11.0 / F.n_couplings + (f.im2col ? 0.7 * f.group : 0);
-    if (f.direct) cost += 4.9 + f.tiles * (0.75 + 3 * width + 0.85 * cb) + (f.tiles == 1 ? 1.9 : 0);      // (one tile: all in series)
-    else if (f.ring) cost += 4 + f.tiles * (5.7 + 2.9 * width + 2.9 * cb) + (f.nbx * f.nby > 1 ? 3 : 0);
-    else cost += 5 + 0.5 * width + f.tiles * (2.2 + 1.5 * width + 0.8 * cb) + (f.nbx * f.nby > 1 ? 2.6 + 1.5 * cb : 0);
+    const bool split = f.nbx * f.nby > 1;
+    double cost = 11.0 / F.n_couplings;
+    if (f.direct) cost += 2.3 + f.tiles * (0.3 + 4.5 * width + 0.7 * cb) + (f.tiles == 1 ? 1.7 : 0);      // (one tile: all in series)
+    else if (f.ring) cost += 1.2 + f.tiles * (4.6 + (f.ring <= 3 ? 5.6 : 4.4) * width + 1.6 * cb) + (split ? 2.8 : 0) + (f.im2col ? 0.9 * f.group - 1.2 : 0);
+    else cost += 2.5 + 1.5 * width + f.tiles * (1.2 + 2.6 * width + 1.3 * cb) + (split ? 2.3 + 1.3 * cb : 0) + (f.im2col ? 1.2 * f.group - 3.9 : 0);
     hl.flow.push_back({f, ctas, cost});
   };
   const int full = whole.im2col ? 4 : std::max(1, kTileM / whole.px);
@@ -1353,9 +1355,9 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
       add_shape(f, clusters);
     }
   if (throughput) {
-    // Streamed weights cost a tile two to three times what resident ones cost it: one 8 x 8 image of 48 channels at width 256,
-    // resident, is 35 us of an SM, one of two, streamed, 41; a 32 x 32 image at width 192 in four blocks, resident, 175,
-    // whole, streamed, 201. But four 4 x 4 images share a tile: at width 256, streamed, 15 each, one, resident, 37.
+    // Streamed weights cost a tile about twice what resident ones cost it (eight couplings): one 8 x 8 image of 48 channels at width
+    // 256, resident, is 55 us of an SM, one of two, streamed, 62; a 32 x 32 image at width 200 in four blocks, resident, 285,
+    // whole, streamed, 323. But four 4 x 4 images share a tile: at width 256, streamed, 22 each.
     auto sm_time = [](const HostLevel::FlowShape& f) { return f.cost * f.plan.nbx * f.plan.nby / f.plan.group; };
     const HostLevel::FlowShape best = *std::min_element(hl.flow.begin(), hl.flow.end(),
                                                         [&](const auto& a, const auto& b) { return sm_time(a) < sm_time(b); });
