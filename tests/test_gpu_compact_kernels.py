@@ -156,3 +156,33 @@ def test_symbol_look_up_at_every_kind_of_scale(G, ls, B, elems):
     with pytest.raises(G.IodfError):
         G.iodf_codec_check(cd)
     np.testing.assert_array_equal(out.cpu().numpy()[:B - 1, :d_fact], z[:B - 1, :d_fact])
+
+
+@pytest.mark.parametrize("elems", [1, 7, 8, 9, 300])
+def test_coder_with_the_largest_table(G, elems):
+    """The widest sigmoid table (its kernels ask for more than 48 KB of shared memory) and streams on either side of the
+    encoder's batches of eight symbols, the last of a block shorter."""
+    import torch
+    model = S.make_model(0xF510, 3, 16, 16, [True], 1, 16)
+    codec = S.logistic_codec(elems_per_stream=elems)
+    umax = 8192
+    u = np.arange(-umax, umax + 1) / (umax / 16.0)
+    codec.update(G=np.floor((65536 - 4097) / (1 + np.exp(-u)) + 0.5).astype(np.uint16), umax=umax)
+    B, d, d_fact = 2, 3 * 16 * 16, 6 * 64
+    rng = np.random.default_rng(elems)
+    prior = np.stack([rng.integers(-50, 50, (B, d_fact)), rng.integers(0, 64, (B, d_fact))], axis=1).astype(np.int32)
+    z = rng.integers(-2200, 2201, (B, d)).astype(np.int32)
+    w_ref, c_ref = O.rans_encode(codec, model, z, prior)
+    m = G.iodf_create(model, B)
+    cd = G.iodf_codec_create(m, codec)
+    words, counts = G.iodf_rans_encode(cd, _t(z), _t(prior))
+    cc = counts.cpu().numpy().view(np.uint32)
+    np.testing.assert_array_equal(cc, c_ref)
+    w = words.cpu().numpy().view(np.uint16)
+    valid = np.arange(w.shape[2])[None, None, :] < cc[:, :, None]
+    np.testing.assert_array_equal(np.where(valid, w, 0), np.where(valid, w_ref, 0))
+    out = torch.zeros((B, d), dtype=torch.int32, device="cuda")
+    for q in range(cd.n_blocks):
+        G.iodf_rans_decode_block(cd, q, words, counts, _t(prior), out)
+    G.iodf_codec_check(cd)
+    np.testing.assert_array_equal(out.cpu().numpy(), z)
