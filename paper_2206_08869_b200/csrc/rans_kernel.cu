@@ -446,8 +446,9 @@ __global__ void pack_offsets_kernel(const uint32_t* __restrict__ sizes, int B, u
 }
 
 // kPack: container -> records; !kPack: records -> container. One CTA per image.
+constexpr int kCopyThreads = 1024;
 template <bool kPack>
-__global__ void __launch_bounds__(256) pack_copy_kernel(uint16_t* __restrict__ words, uint32_t* __restrict__ counts,
+__global__ void __launch_bounds__(kCopyThreads) pack_copy_kernel(uint16_t* __restrict__ words, uint32_t* __restrict__ counts,
                                                         int n_streams, int cap, uint8_t* __restrict__ packed,
                                                         int B, unsigned long long payload_bytes, uint32_t* errors) {
   extern __shared__ uint32_t start[];       // word offset of every stream inside the record, after the counts
@@ -503,14 +504,14 @@ cudaError_t launch_rans_pack(const RansArgs& a, const uint16_t* words, const uin
                              uint8_t* packed, cudaStream_t stream) {
   pack_sizes_kernel<<<a.batch, 256, 0, stream>>>(counts, a.n_streams, a.cap, sizes);
   pack_offsets_kernel<<<1, 32, 0, stream>>>(sizes, a.batch, reinterpret_cast<uint32_t*>(packed));
-  pack_copy_kernel<true><<<a.batch, 256, 4 * (a.n_streams + 1), stream>>>(
+  pack_copy_kernel<true><<<a.batch, kCopyThreads, 4 * (a.n_streams + 1), stream>>>(
       const_cast<uint16_t*>(words), const_cast<uint32_t*>(counts), a.n_streams, a.cap, packed, a.batch, 0ull, a.errors);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rans_unpack(const RansArgs& a, const uint8_t* packed, unsigned long long payload_bytes,
                                uint16_t* words, uint32_t* counts, cudaStream_t stream) {
-  pack_copy_kernel<false><<<a.batch, 256, 4 * (a.n_streams + 1), stream>>>(
+  pack_copy_kernel<false><<<a.batch, kCopyThreads, 4 * (a.n_streams + 1), stream>>>(
       words, counts, a.n_streams, a.cap, const_cast<uint8_t*>(packed), a.batch, payload_bytes, a.errors);
   return cudaGetLastError();
 }
