@@ -12,6 +12,16 @@ from test_gpu_residual import _both_ways
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("in_c", [1, 2, 3])
+def test_whole_images_of_few_channels(G, in_c):
+    """32 x 32 images whole in a CTA: two, four and six input channels in a record's eight bytes."""
+    model = S.make_model(0xFA00 + in_c, in_c, 64, 64, [True], 2, 24)
+    rng = np.random.default_rng(in_c)
+    x = rng.integers(0, 256, (2, in_c, 64, 64), dtype=np.uint8)
+    m, _ = _check_both_ways(G, model, x, plan=1)
+    assert G.iodf_level_kernel_name(m, 0) == "flow_level_kernel" and G.iodf_level_images_per_cta(m, 0) == 1
+
+
 @pytest.mark.parametrize("splits,hidden,batch,sample", [
     ([False], 16, 3, None),               # six channels in eight columns; the narrowest layers
     ([True], 33, 150, [0, 147, 149]),     # more images than SMs: two to a CTA, one alone
