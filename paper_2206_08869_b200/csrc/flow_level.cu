@@ -35,11 +35,12 @@
 //     translation, acquired by the neighbour's MMA warp, without whose MMAs there are no products. (Overwriting a
 //     frame needs no release: the MMAs that read it have completed before anything is sent that lets a neighbour go on.)
 //
-// What bounds it: the chain of a coupling (about 8 000 clocks) and 3 700 clocks per tile of 128 pixels: requantisation,
-// shifted sum and their hand-overs (52 % of all issue slots at 32 x 32, 39 % at 8 x 8, 24 % at 4 x 4). Measured for eight
-// couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 161 us,
-// 16 x 16 85 -> 63, 8 x 8 63 -> 48, 4 x 4 70 -> 48; one image, 32 x 32 split in eight: 52. Width 512, 64 images of
-// 32 x 32, split in two: 2 357 -> 288 us, of which the tensor core works 95.
+// What bounds it: the chain of a coupling (7 000 - 9 000 clocks where a CTA has one tile) and 3 300 clocks per tile of 128 pixels:
+// requantisation, shifted sum and their hand-overs, at five to nine clocks an instruction and warp (50 % of all issue slots at
+// 32 x 32, 33 % at 8 x 8, 23 % at 4 x 4; of 32 x 32's 143 us the phases' skeleton of waits, hand-overs and MMAs takes half). Measured for eight
+// couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 143 us,
+// 16 x 16 85 -> 57, 8 x 8 63 -> 43, 4 x 4 70 -> 47; one image, 32 x 32 split in eight: 51. Width 512, 64 images of
+// 32 x 32, split in two: 2 357 -> 288 us, the tensor core busy a third of it.
 #include <stddef.h>
 
 #include "flow_level.h"
@@ -491,7 +492,7 @@ __device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, ui
   constexpr int kHalves = kShape == kRows128 ? 2 : 1;
   // everything that does not depend on the accumulator comes before the wait for it
   const FlowLayer L = reinterpret_cast<const FlowMeta*>(mb)->layer[layer];
-  const uint8_t* t = mb + L.off + (f.lane & 3) * 32;
+  const uint8_t* t = mb + 16 * L.off + (f.lane & 3) * 32;
   const int row = kShape == kRows64 ? ho.row : 128;
   uint64_t* done = f.ctl->a_ready[f.sl];
   flow_wait(f, ready, parity);
@@ -504,7 +505,7 @@ __device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, ui
       const uint32_t ta = taddr + (uint32_t)(min(b, (int)L.last) << 5);
 #pragma unroll
       for (int h = 0; h < kHalves; ++h) ptx::tmem_ld_16x32(ta + ((uint32_t)h << 20), r[h]);
-      const float4* tb = reinterpret_cast<const float4*>(t + b * 256);
+      const float4* tb = reinterpret_cast<const float4*>(t + b * 128);
       const float4 m0 = tb[0], m1 = tb[1];
       const float m[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
       uint8_t* o = ho.at + b * ho.block;
@@ -526,7 +527,12 @@ __device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, ui
         }
       } else {
         if (b < L.nfi) {
-          const float4 c0 = tb[8], c1 = tb[9];
+          float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
+          if (b >= L.nfb) {
+            const float4* tc = reinterpret_cast<const float4*>(mb + 16 * L.off_c + (f.lane & 3) * 32 + (b - L.nfb) * 128);
+            c0 = tc[0];
+            c1 = tc[1];
+          }
           const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
           for (int h = 0; h < kHalves; ++h)

@@ -63,15 +63,16 @@ struct FlowPlan {
 static_assert(sizeof(FlowPlan) < 1024, "travels as a kernel parameter");
 
 // Meta part of a coupling's packed block. Followed by colA[ca], colB[cb] (physical columns of the flow
-// variable), OutRq[cb], and per hidden layer the FloatRq constants of its 32-column blocks: 32 multipliers, 32 addends, each
-// in thread order (lane & 3, eight columns; so that the four addresses of a 16-byte load lie in different banks).
+// variable), OutRq[cb], and per hidden layer the FloatRq constants of its 32-column blocks in thread order (lane & 3, eight
+// columns; so that the four addresses of a 16-byte load lie in different banks): 32 multipliers a block, then 32 addends a
+// block from the first that has any.
 struct __align__(16) FlowLayer { // what a hidden epilogue needs, in one load
   uint8_t ks, nfull, last, plain;// 32-column blocks written, blocks that are full of columns, last block with any, blocks
                                  // that are full and without an addend
-  int32_t off;                   // its table
+  uint16_t off, off_c;           // multipliers of block 0, addends of block nfb, in 16-byte units
   uint32_t beyond;               // what its output holds where the last blocks have no columns
-  uint8_t half, nfi, us, pad;    // half 1: block nfull has 16 columns; blocks from nfi on have a channel without
-                                 // floating-point constants: integer form with shift us, multipliers M0
+  uint8_t half, nfb, nfi, us;    // half 1: block nfull has 16 columns; blocks from nfb on may have addends, from nfi on a channel
+                                 // without floating-point constants: integer form with shift us, multipliers M0
 };
 struct FlowMeta {
   int32_t in_m0, in_s;

@@ -561,11 +561,13 @@ PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, con
   M.off_colB = take(4 * cb);
   M.off_out = take((uint32_t)sizeof(OutRq) * cb);
   auto layer = [&](FlowLayer& l, const HiddenOrder& o, int n, int blocks, uint32_t beyond) {
-    l.ks = (uint8_t)blocks; l.nfull = (uint8_t)(n >> 5); l.last = (uint8_t)((n - 1) >> 5); l.plain = l.nfull; l.nfi = (uint8_t)blocks;
+    l.ks = (uint8_t)blocks; l.nfull = (uint8_t)(n >> 5); l.last = (uint8_t)((n - 1) >> 5); l.nfb = l.nfi = (uint8_t)blocks;
     for (int i = (int)o.ch.size() - 1; i >= 0 && o.fc[o.ch[i]].none; --i) l.nfi = (uint8_t)(i / 32);
-    for (int i = (int)o.ch.size() - 1; i >= 0 && (o.fc[o.ch[i]].none || o.fc[o.ch[i]].C); --i) l.plain = std::min(l.plain, (uint8_t)(i / 32));
+    for (int i = (int)o.ch.size() - 1; i >= 0 && (o.fc[o.ch[i]].none || o.fc[o.ch[i]].C); --i) l.nfb = (uint8_t)(i / 32);
+    l.plain = std::min(l.nfull, l.nfb);
     l.us = (uint8_t)o.shift;
-    l.off = take(256 * blocks);
+    l.off = (uint16_t)(take(128 * blocks) / 16);
+    l.off_c = (uint16_t)(take(128 * (blocks - l.nfb)) / 16);
     l.beyond = beyond;
     l.half = (n >> 4) & 1;
   };
@@ -576,18 +578,18 @@ PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, con
   std::memcpy(pb.meta.data() + M.off_colB, colB, 4 * cb);
   put_out_rq(reinterpret_cast<OutRq*>(pb.meta.data() + M.off_out), L3, B);
   auto tables = [&](const HiddenOrder& o, const iodf_layer_desc& L, const FlowLayer& l) {
-    uint8_t* t = pb.meta.data() + l.off;
+    uint8_t* t = pb.meta.data() + 16 * l.off;
+    uint8_t* addends = pb.meta.data() + 16 * l.off_c;
     for (int i = 0; i < (int)o.ch.size(); ++i) {
       const FloatChannel& fc = o.fc[o.ch[i]];
       const int p = flow_kpos(i);
-      uint8_t* at = t + (p >> 5) * 256 + (p & 31) * 4;
       const uint32_t addend = 0x80000000u | (uint32_t)fc.C;                     // -C * 2^-149
       if (i >= 32 * l.nfi) {                       // integer blocks: M0 itself
-        std::memcpy(at, B.r + L.requant_off + L.c_out + o.ch[i], 4);
+        std::memcpy(t + 4 * p, B.r + L.requant_off + L.c_out + o.ch[i], 4);
         continue;
       }
-      std::memcpy(at, &fc.m, 4);
-      if (fc.C) std::memcpy(at + 128, &addend, 4);
+      std::memcpy(t + 4 * p, &fc.m, 4);
+      if (fc.C) std::memcpy(addends + 4 * (p - 32 * l.nfb), &addend, 4);
     }
   };
   tables(o1, L1, M.layer[0]);
