@@ -1980,8 +1980,8 @@ int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_cod
   if (!m || !desc || !out) return IODF_EINVAL;
   *out = nullptr;
   if (desc->abi_version != IODF_ABI_VERSION) return IODF_EVERSION;
-  if (!desc->sigmoid_table || !desc->inv_scale || desc->umax < 1 || desc->umax > 8192 || desc->n_scales < 1 ||
-      desc->n_scales > 1024 || desc->elems_per_stream < 1 || desc->elems_per_stream > 65536)
+  if (!desc->sigmoid_table || !desc->inv_scale || desc->umax < 1 || desc->umax > (uint32_t)kMaxRansUmax ||
+      desc->n_scales < 1 || desc->n_scales > (uint32_t)kMaxRansScales || desc->elems_per_stream < 1 || desc->elems_per_stream > 65536)
     return IODF_EINVAL;
   if (desc->final_ls < 0 || desc->final_ls >= (int32_t)desc->n_scales) return IODF_EINVAL;
   const uint32_t top = (1u << 16) - (2u * 2048u + 1u);
@@ -2041,7 +2041,8 @@ int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_cod
     delete c;
     return IODF_ECUDA;
   }
-  e = cudaMalloc(&c->d_tables, rbytes + gbytes);
+  e = configure_rans_kernels();
+  if (e == cudaSuccess) e = cudaMalloc(&c->d_tables, rbytes + gbytes);
   if (e == cudaSuccess) e = cudaMemcpy(c->d_tables, desc->inv_scale, rbytes, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(c->d_tables + rbytes, desc->sigmoid_table, gbytes, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_errors, sizeof(uint32_t));

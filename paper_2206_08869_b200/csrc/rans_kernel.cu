@@ -516,6 +516,18 @@ cudaError_t launch_rans_unpack(const RansArgs& a, const uint8_t* packed, unsigne
   return cudaGetLastError();
 }
 
+static size_t encode_smem(const RansArgs& a) { return encode_buffers_at(a) + 2 * kBatch * kEncodeStreams * (sizeof(EncodeSymbol) + 4); }
+
+// The encoder's dynamic shared memory may exceed what a kernel has without asking: 48 KB, its static part included (tables of
+// more than 5 947 entries a side with 64 scales). The limit belongs to the kernel, not to a codec or a launch: it is always
+// the largest codec's, so that one codec cannot lower it under another's launch from a second thread.
+cudaError_t configure_rans_kernels() {
+  RansArgs largest{};
+  largest.umax = kMaxRansUmax;
+  largest.n_scales = kMaxRansScales;
+  return cudaFuncSetAttribute(rans_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)encode_smem(largest));
+}
+
 static size_t table_smem(const RansArgs& a) { return 4 * (size_t)a.n_scales + 2 * (size_t)(2 * a.umax + 1) + 16; }
 
 // (No programmatic launch of the coder: started under a level's kernel, whose CTAs fill their SMs, the coder's CTAs all land
@@ -524,10 +536,7 @@ cudaError_t launch_rans_encode(const RansArgs& a, const int32_t* z, const int32_
                                uint32_t* counts, cudaStream_t stream) {
   const long total = (long)a.batch * a.n_streams;
   const unsigned grid = (unsigned)((total + kEncodeStreams - 1) / kEncodeStreams);
-  const size_t smem = encode_buffers_at(a) + 2 * kBatch * kEncodeStreams * (sizeof(EncodeSymbol) + 4);
-  if (smem > 48 * 1024)                                  // (beyond this a kernel has to ask; tables of more than 6 000 entries)
-    if (const cudaError_t e = cudaFuncSetAttribute(rans_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); e != cudaSuccess) return e;
-  rans_encode_kernel<<<grid, kEncodeThreads, smem, stream>>>(a, z, prior, words, counts);
+  rans_encode_kernel<<<grid, kEncodeThreads, encode_smem(a), stream>>>(a, z, prior, words, counts);
   return cudaGetLastError();
 }
 

@@ -6,6 +6,7 @@
 namespace iodf {
 
 constexpr int kMaxRansBlocks = 9;      // one per flow level plus the final block
+constexpr int kMaxRansUmax = 8192, kMaxRansScales = 1024;      // largest tables of a codec
 
 struct RansBlock {
   long long z_off;         // offset of the block in an image's z
@@ -29,6 +30,8 @@ struct RansArgs {
   RansBlock blocks[kMaxRansBlocks];
 };
 
+// Once per codec, on its device, before any of the launches below.
+cudaError_t configure_rans_kernels();
 cudaError_t launch_rans_encode(const RansArgs& a, const int32_t* z, const int32_t* prior, uint16_t* words,
                                uint32_t* counts, cudaStream_t stream);
 cudaError_t launch_rans_decode(const RansArgs& a, int block, const uint16_t* words, const uint32_t* counts,

@@ -168,14 +168,18 @@ def test_symbol_look_up_at_every_kind_of_scale(G, ls, B, elems):
     np.testing.assert_array_equal(out.cpu().numpy()[:B - 1, :d_fact], z[:B - 1, :d_fact])
 
 
-@pytest.mark.parametrize("elems", [1, 7, 8, 9, 300])
-def test_coder_with_the_largest_table(G, elems):
-    """The widest sigmoid table (its kernels ask for more than 48 KB of shared memory) and streams on either side of the
-    encoder's batches of eight symbols, the last of a block shorter."""
+@pytest.mark.parametrize("umax,scales,elems", [
+    (8192, 64, 1), (8192, 64, 7), (8192, 64, 8), (8192, 64, 9), (8192, 64, 300),
+    (8192, 1024, 9),                      # the largest tables that a codec may have
+    (5947, 64, 9), (5948, 64, 9), (6079, 64, 9), (6080, 64, 9),      # about 48 KB of shared memory
+])
+def test_coder_with_large_tables(G, umax, scales, elems):
+    """The widest sigmoid tables, on either side of the shared memory that a kernel has without asking for it, and streams
+    on either side of the encoder's batches of eight symbols, the last of a block shorter."""
     import torch
     model = S.make_model(0xF510, 3, 16, 16, [True], 1, 16)
     codec = S.logistic_codec(elems_per_stream=elems)
-    umax = 8192
+    codec["R"] = np.resize(codec["R"], scales)
     u = np.arange(-umax, umax + 1) / (umax / 16.0)
     codec.update(G=np.floor((65536 - 4097) / (1 + np.exp(-u)) + 0.5).astype(np.uint16), umax=umax)
     B, d, d_fact = 2, 3 * 16 * 16, 6 * 64
@@ -196,3 +200,41 @@ def test_coder_with_the_largest_table(G, elems):
         G.iodf_rans_decode_block(cd, q, words, counts, _t(prior), out)
     G.iodf_codec_check(cd)
     np.testing.assert_array_equal(out.cpu().numpy(), z)
+
+
+_FIRST_CODEC = """
+import sys
+import numpy as np
+import torch
+sys.path.insert(0, sys.argv[1])
+import iodf_synth as S
+import paper_2206_08869_b200 as G
+umax = int(sys.argv[2])
+m = G.iodf_create(S.make_model(0xF520, 3, 16, 16, [True], 1, 16), 2)
+codec = S.logistic_codec(umax=umax)
+cd = G.iodf_codec_create(m, codec)
+z, prior = G.iodf_forward(m, torch.from_numpy(S.smooth_field_images(0xF521, 2, 16, 16, 2.0)).cuda())
+words, counts = G.iodf_rans_encode(cd, z, prior)
+out = torch.zeros_like(z)
+for q in range(cd.n_blocks):
+    G.iodf_rans_decode_block(cd, q, words, counts, prior, out)
+G.iodf_codec_check(cd)
+print("equal", torch.equal(out, z))
+"""
+
+
+@pytest.mark.parametrize("umax", [
+    5947,      # the encoder's dynamic and static shared memory together: 48 KB
+    5948,      # ... 16 bytes more
+    6079,      # its dynamic shared memory alone: 48 KB
+    6080,      # ... 16 bytes more
+])
+def test_first_codec_of_a_process_about_48_kb(umax):
+    """What shared memory a kernel may use is a state of the process, so each size is the first one of its own process."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FIRST_CODEC, root, str(umax)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split()[-2:] == ["equal", "True"], r.stdout
