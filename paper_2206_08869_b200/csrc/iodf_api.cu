@@ -537,13 +537,17 @@ void flow_first_matrix(std::vector<uint8_t>& out, int n_pad, const std::vector<K
   }
 }
 
-// images of one tile of 64 rows: the last conv can run on the hidden operand directly
-bool flow_direct(const FlowPlan& F) { return F.nbx * F.nby == 1 && F.h == 8 && F.w == 8; }
+// images of one tile of 64 rows and resident weights (`widest` of the level's hidden layers): the last conv can run on the
+// hidden operand directly
+constexpr uint32_t kFlowMaxResident = 256;
+bool flow_direct(const FlowPlan& F, uint32_t widest) {
+  return F.nbx * F.nby == 1 && F.h == 8 && F.w == 8 && widest <= kFlowMaxResident;
+}
 
 struct FlowDims { int n1, n2, n3, n3d, ks2, ks3; };
 
 PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, const FlowPlan& F, const std::vector<KByte>& kmap,
-                               const HiddenOrder& o1, const HiddenOrder& o2, const int* colA, const int* colB, FlowDims* dims) {
+                               const HiddenOrder& o1, const HiddenOrder& o2, const int* colA, const int* colB, bool direct, FlowDims* dims) {
   const iodf_layer_desc& L1 = cp.layers[0];
   const iodf_layer_desc& L2 = cp.layers[1];
   const iodf_layer_desc& L3 = cp.layers[2];
@@ -628,7 +632,7 @@ PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, con
       for (int k = 0; k < k2; ++k)
         pb.w[2][wpos(M.n3, tap * cbp + c, flow_kpos(k))] = (uint8_t)w3[((size_t)c * 9 + tap) * k2 + o2.ch[k]];
   // the same for the direct form: K chunk by chunk of 32 channels, nine taps each
-  if (flow_direct(F)) {
+  if (direct) {
     pb.w[3].assign((size_t)M.n3d * 9 * 32 * M.ks3, 0);
     for (int c = 0; c < cb; ++c)
       for (int tap = 0; tap < 9; ++tap)
@@ -1270,33 +1274,35 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   if (lv.has_prior && (lv.prior_in_s < 1 || !shifts_ok(lv.prior_layer))) return false;
   FlowNeeds nd;
   double widths = 0;                              // of the hidden layers, padded
+  for (uint32_t ki = 0; ki < lv.n_couplings; ++ki)
+    for (int q = 0; q < 2; ++q) {
+      const uint32_t n = up(lv.couplings[ki].layers[q].c_out, 16);
+      nd.n_hidden = std::max(nd.n_hidden, n);
+      widths += n;
+    }
   std::vector<PackedBlock> blocks;
   for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) {
     FlowDims d;
     blocks.push_back(pack_flow_coupling(lv.couplings[ki], B, F, kmap, orders[ki][0], orders[ki][1], cols[ki].data(),
-                                        cols[ki].data() + F.ca, &d));
-    nd.n_hidden = std::max<uint32_t>(nd.n_hidden, (uint32_t)std::max(d.n1, d.n2));
+                                        cols[ki].data() + F.ca, flow_direct(F, nd.n_hidden), &d));
     nd.n_taps = std::max<uint32_t>(nd.n_taps, (uint32_t)d.n3);
     nd.n_direct = std::max<uint32_t>(nd.n_direct, (uint32_t)d.n3d);
     nd.kb = std::max<uint32_t>(nd.kb, (uint32_t)std::max(d.ks2, d.ks3));
-    widths += d.n1 + d.n2;
   }
   PackedBlock prior;
   if (lv.has_prior) prior = pack_flow_prior(lv, B, F, kmap);
-  hl.blob.clear();
-  auto add = [&](const PackedBlock& pb, BlockRef* ref) {
-    append_block(hl.blob, pb, ref);
-    nd.meta = std::max(nd.meta, ref->meta_bytes);
-    for (int g = 0; g < 4; ++g) nd.w[g] = std::max(nd.w[g], ref->w_bytes[g]);
+  auto need = [&](const PackedBlock& pb) {
+    nd.meta = std::max(nd.meta, (uint32_t)pb.meta.size());
+    for (int g = 0; g < 4; ++g) nd.w[g] = std::max(nd.w[g], (uint32_t)pb.w[g].size());
   };
-  for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) add(blocks[ki], &P.coupling[ki]);
-  if (lv.has_prior) add(prior, &P.prior);
+  for (const PackedBlock& pb : blocks) need(pb);
+  if (lv.has_prior) need(prior);
   // resident weights where they and the accumulators of two tiles fit; streaming them costs a copy of 16 - 64 KB per GEMM
   // and tile, which one tile's chain of GEMMs does not hide
   auto plan = [&](FlowPlan& f, int group) {
     if ((uint64_t)group * f.c * f.fpx * ((uint64_t)f.c * f.fpx) >= (1ull << 32)) return false;      // (the index maps' divisions)
-    for (int wide = nd.n_hidden > 256; wide < 2; ++wide)
-      for (int direct = flow_direct(f) && !wide; direct >= 0; --direct)
+    for (int wide = nd.n_hidden > kFlowMaxResident; wide < 2; ++wide)
+      for (int direct = flow_direct(f, nd.n_hidden) && !wide; direct >= 0; --direct)
         if (plan_flow(f, nd, smem_limit, group, wide != 0, direct != 0)) return true;
     return false;
   };
@@ -1365,6 +1371,16 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
                                                         [&](const auto& a, const auto& b) { return sm_time(a) < sm_time(b); });
     hl.flow.assign(1, best);
   }
+  // of the last conv's two forms, those that a launch shape reads
+  bool direct = false, taps = false;
+  for (const HostLevel::FlowShape& f : hl.flow) (f.plan.direct ? direct : taps) = true;
+  hl.blob.clear();
+  for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) {
+    if (!taps) blocks[ki].w[2].clear();
+    if (!direct) blocks[ki].w[3].clear();
+    append_block(hl.blob, blocks[ki], &P.coupling[ki]);
+  }
+  if (lv.has_prior) append_block(hl.blob, prior, &P.prior);
   return true;
 }
 

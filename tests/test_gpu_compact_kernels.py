@@ -238,3 +238,19 @@ def test_first_codec_of_a_process_about_48_kb(umax):
     r = subprocess.run([sys.executable, "-c", _FIRST_CODEC, root, str(umax)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
     assert r.stdout.split()[-2:] == ["equal", "True"], r.stdout
+
+
+def test_matrices_that_no_launch_shape_reads_are_not_kept(G):
+    """Weights of an 8 x 8 level at width 512 are streamed, so that its last conv never runs in its direct form. 48 channels
+    translated: that form's matrices would be 7 MB of 32 couplings' 32; the rest is the allocator's granularity."""
+    import torch
+    G.iodf_create(S.make_model(0xFC00, 3, 16, 16, [True], 1, 16), 1)          # (whatever is allocated only once)
+    model = S.make_model(0xFC01, 24, 16, 16, [True], 32, 512)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    m = G.iodf_create(model, 1)
+    taken = before - torch.cuda.mem_get_info()[0]
+    assert G.iodf_level_kernel_name(m, 0) == "flow_level_kernel"
+    first, second, last, meta = 512 * 36 * 16, 512 * 17 * 32, 432 * 16 * 32, 8192        # bytes of a coupling's parts
+    prior = 96 * 36 * 16 + 8192
+    assert taken <= 32 * (first + second + last + meta) + prior + (4 << 20)
