@@ -2057,7 +2057,8 @@ int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_cod
     delete c;
     return IODF_ECUDA;
   }
-  e = configure_rans_kernels();
+  e = cudaDeviceGetAttribute(&a.n_sms, cudaDevAttrMultiProcessorCount, c->device);
+  if (e == cudaSuccess) e = configure_rans_kernels();
   if (e == cudaSuccess) e = cudaMalloc(&c->d_tables, rbytes + gbytes);
   if (e == cudaSuccess) e = cudaMemcpy(c->d_tables, desc->inv_scale, rbytes, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(c->d_tables + rbytes, desc->sigmoid_table, gbytes, cudaMemcpyHostToDevice);

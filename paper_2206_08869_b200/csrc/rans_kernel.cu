@@ -29,9 +29,10 @@ constexpr int kEncodeStreams = 128, kEncodeThreads = 3 * kEncodeStreams, kBatch 
 __host__ __device__ inline size_t encode_buffers_at(const RansArgs& a) {       // offset in the encoder's shared memory, after the tables
   return (4 * (size_t)a.n_scales + 2 * (size_t)(2 * a.umax + 1) + 15) / 16 * 16;
 }
-// More streams than this (24 per SM): half a warp each. Whole warps and halves measured: 3 072 streams 69 and 73 us, 3 600 75 and 75 (55
-// and 44 without prior parameters), 6 144 111 and 88, 7 200 122 and 103.
-constexpr long kHalfWarpStreams = 3584;
+// More streams of a block than this per SM: half a warp each. A warp per stream is then six warps and more per scheduler, and issue slots
+// bound it. Whole warps and halves measured at 148 SMs: 3 072 streams 69 and 73 us, 3 600 75 and 75 (55 and 44 without prior
+// parameters), 6 144 111 and 88, 7 200 122 and 103.
+constexpr long kHalfWarpStreamsPerSm = 24;
 
 struct Tables {
   const uint16_t* G;       // shared memory
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(kEncodeThreads) rans_encode_kernel(const RansA
 //     stream backwards); the three words that a symbol can take are handed out before its search.
 // What bounds it depends on the block (128 images of 64 x 64, 128 elements per stream). The small ones are a stream's chain:
 // 35 us for the final block, 540 clocks per symbol, 50 us for those with prior parameters (60 - 70 with three search
-// rounds). Blocks of more streams than kHalfWarpStreams go to the kernel below.
+// rounds). Blocks of more than kHalfWarpStreamsPerSm streams per SM go to the kernel below.
 __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const RansArgs a, int q,
                                                                        const uint16_t* __restrict__ words,
                                                                        const uint32_t* __restrict__ counts,
@@ -543,7 +544,7 @@ cudaError_t launch_rans_encode(const RansArgs& a, const int32_t* z, const int32_
 cudaError_t launch_rans_decode(const RansArgs& a, int block, const uint16_t* words, const uint32_t* counts,
                                const int32_t* prior, int32_t* z, cudaStream_t stream) {
   const long streams = (long)a.batch * a.blocks[block].n_streams;
-  const bool half = streams > kHalfWarpStreams;
+  const bool half = streams > kHalfWarpStreamsPerSm * a.n_sms;
   const long total = streams * (half ? 16 : 32);
   const unsigned grid = (unsigned)((total + kThreadsPerBlock - 1) / kThreadsPerBlock);
   if (half) rans_decode_half_kernel<<<grid, kThreadsPerBlock, table_smem(a), stream>>>(a, block, words, counts, prior, z);

@@ -24,6 +24,7 @@ struct RansArgs {
   int n_blocks, n_streams; // per image
   int cap;                 // words per stream in the container (3 * elems_per_stream + 2)
   int batch;
+  int n_sms;               // of the codec's device
   long long d, d_fact;
   uint32_t* errors;        // device counter or null: streams with an out-of-range scale index or a
                            // malformed word sequence

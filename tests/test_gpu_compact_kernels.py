@@ -134,11 +134,13 @@ def test_residual_blocks_through_long_chains(G, hidden, batch, plan):
     G.iodf_check(m)
 
 
-@pytest.mark.parametrize("B,elems", [(3, 97), (241, 103)])          # 45 and 3 615 streams to a block: a warp each, half of one
-@pytest.mark.parametrize("ls", [0, 20, 40, 63])
-def test_symbol_look_up_at_every_kind_of_scale(G, ls, B, elems):
+@pytest.mark.parametrize("per_sm,elems", [(0, 97), (24, 103), (25, 103)])      # most streams per SM: a warp each, the last of
+@pytest.mark.parametrize("ls", [0, 20, 40, 63])                                # those, half of one
+def test_symbol_look_up_at_every_kind_of_scale(G, ls, per_sm, elems):
     """Residuals over the whole window at one scale: slots that mean one symbol and slots that mean hundreds."""
     import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B = max(3, per_sm * sms // 15)                                             # 15 streams of an image to a block
     model = S.make_model(0xF500, 3, 32, 32, [True, False], 1, 16)
     codec = S.logistic_codec(elems_per_stream=elems)
     d, d_fact = 3 * 32 * 32, 6 * 256
