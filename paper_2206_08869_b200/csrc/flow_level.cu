@@ -39,7 +39,7 @@
 // requantisation, shifted sum and their hand-overs, at five to nine clocks an instruction and warp (50 % of all issue slots at
 // 32 x 32, 33 % at 8 x 8, 23 % at 4 x 4; of 32 x 32's 143 us the phases' skeleton of waits, hand-overs and MMAs takes half). Measured for eight
 // couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 143 us,
-// 16 x 16 85 -> 57, 8 x 8 63 -> 43, 4 x 4 70 -> 47; one image, 32 x 32 split in eight: 51. Width 512, 64 images of
+// 16 x 16 85 -> 58, 8 x 8 63 -> 43, 4 x 4 70 -> 47; one image, 32 x 32 split in eight: 51. Width 512, 64 images of
 // 32 x 32, split in two: 2 357 -> 288 us, the tensor core busy a third of it.
 #include <stddef.h>
 
@@ -216,8 +216,9 @@ __device__ void flow_loader(const Flow& f, const FlowPlan& P, const LevelArgs& a
 }
 
 // Streamed weights (P.ring): for every tile the K steps of its GEMMs, in order, through the ring, as many to a slot as it
-// holds. What bounds the stream is the 300 - 600 clocks that a warp spends on a copy, whatever its size (the copies themselves run
-// at over 100 bytes per clock and SM), so two warps take the slots in turn.
+// holds. A copy takes its warp 290 clocks whatever its size, 135 with two warps that take the slots in turn, and runs at over 100 bytes per
+// clock and SM. Neither bounds the stream while a slot carries several steps (one warp for all slots: the same within 4 % at each
+// of 352 levels and batches of widths 176 - 512, 0.1 % on average); that is the GEMMs and epilogues of the one tile in series.
 __device__ __forceinline__ int flow_slot_steps(const FlowPlan& P, int n) { return max(1, (int)(P.ring_slot_bytes >> 5) / n); }
 
 __device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st, uint32_t which) {

@@ -1,7 +1,7 @@
 // Entropy coding of the flow's latents on the GPU: the discrete logistic prior of Sec. 3 in integer
 // table form and range-ANS (App. A) with a 32-bit state renormalised in 16-bit words, one chain
 // per stream. The streams are independent (an image's coded blocks are cut into streams of about
-// `elems_per_stream` interleaved elements), so a batch of 128 ImageNet64-sized latents is 6 144
+// `elems_per_stream` interleaved elements), so a batch of 128 ImageNet64-sized latents in streams of 128 is 12 288
 // streams: the GPU coder that Sec. 5.3 names as future work (the paper codes on the CPU).
 //
 //   symbol of an element   k = clamp(z - mu, -2048, 2048) + 2048          (0 and 4096: escapes, then
