@@ -217,8 +217,8 @@ __device__ void flow_loader(const Flow& f, const FlowPlan& P, const LevelArgs& a
 
 // Streamed weights (P.ring): for every tile the K steps of its GEMMs, in order, through the ring, as many to a slot as it
 // holds. A copy takes its warp 290 clocks whatever its size, 135 with two warps that take the slots in turn, and runs at over 100 bytes per
-// clock and SM. Neither bounds the stream while a slot carries several steps (one warp for all slots: the same within 4 % at each
-// of 352 levels and batches of widths 176 - 512, 0.1 % on average); that is the GEMMs and epilogues of the one tile in series.
+// clock and SM. Neither bounds the stream while a slot carries several steps (one warp for all slots: 0.1 % faster on average over
+// 192 levels and batches of widths 264 - 512, 3 % either way above 100 us); what does is one tile's GEMMs and epilogues in series.
 __device__ __forceinline__ int flow_slot_steps(const FlowPlan& P, int n) { return max(1, (int)(P.ring_slot_bytes >> 5) / n); }
 
 __device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st, uint32_t which) {

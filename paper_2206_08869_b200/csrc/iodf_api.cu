@@ -1313,17 +1313,19 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   // throughput plan keeps the one that takes the least SM time per image, with no more images than fill a tile. Time of a
   // wave per coupling, in thousands of clocks: a share of the level's load and store, a serial part, a part for each tile of the
   // CTA that grows with the mean hidden width and the channels that are translated, the exchange of edges, what an image more costs
-  // at 4 x 4, a weight ring too short to run ahead of wide layers. Fitted to 564 shapes of 53 flows (widths 16 - 512, 2 - 56
-  // translated channels, 4 x 4 - 32 x 32, 2 - 12 couplings) at batches of 1 - 1 184: 5 % off on average. The shape it picks takes 0.12 %
-  // longer than the best one on average and 13 % at most (eight 4 x 4 images of width 512 rather than four); for 223
-  // shapes of 26 other flows 0.25 % and 18 % (a 4 x 4 level of a single coupling, 13 us). Constants fitted to five flows and used
-  // with twice the width that they were fitted with: 0.38 % and 25 %, 0.35 % and 18 %.
+  // at 4 x 4, a weight ring too short to run ahead of wide layers (without that term shapes of three slots take 17 % longer than
+  // the rule says, of four 11 %, of five and more 1 %). Fitted to 564 shapes of 53 flows (widths 16 - 512, 2 - 56 translated
+  // channels, 4 x 4 - 32 x 32, 2 - 12 couplings) at batches of 1 - 1 184: 5 % off on average. The shape it picks takes 0.09 % longer than
+  // the best one on average and 12 % at most (a 4 x 4 level of two couplings, 20 us); for 253 shapes of 27 flows that had no
+  // part in it 0.12 % and 11 %. Constants fitted to five flows and used with twice the width that they were fitted with: 0.38 %
+  // and 25 %, 0.34 % and 12 %.
   auto add_shape = [&](const FlowPlan& f, int ctas) {
     const double width = widths / (400.0 * F.n_couplings), cb = f.cb / 10.0;        // mean of both layers, in 200 channels
     const bool split = f.nbx * f.nby > 1;
+    const int missing = std::max(0, 5 - f.ring);                                      // slots of the weight ring
     double cost = 13.0 / F.n_couplings;
     if (f.direct) cost += 0.2 + f.tiles * (0.9 + 2.9 * width + 0.8 * cb) + (f.tiles == 1 ? 1 + 1.35 * width : 0);      // (one tile: all in series)
-    else if (f.ring) cost += f.tiles * (4.7 + (f.ring <= 3 ? 5.6 : 3.75) * width + 1.8 * cb) + (split ? 4 : 0) + (f.im2col ? 0.1 * f.group - 1.4 : 0);
+    else if (f.ring) cost += f.tiles * (4.7 + (3.75 + 0.45 * missing * missing) * width + 1.8 * cb) + (split ? 4 : 0) + (f.im2col ? 0.1 * f.group - 1.4 : 0);
     else if (f.im2col) cost += 0.65 + 2.7 * width + 1.2 * cb + 0.55 * f.group;
     else cost += 2.5 * width + f.tiles * (1.5 + 1.6 * width + 1.55 * cb) + (split ? 3.2 + 0.65 * cb : 0);
     hl.flow.push_back({f, ctas, cost});
