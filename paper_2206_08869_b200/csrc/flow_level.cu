@@ -264,34 +264,57 @@ __device__ void flow_loader_ring(const Flow& f, const FlowPlan& P, const LevelAr
 }
 
 // ---- MMA warp --------------------------------------------------------------------------------------------
-// D (+)= A B^T over ks steps of 32 K bytes; n above 256 in two parts. The whole warp runs the loop on uniform
-// values, `lead` issues. `ahead(k)`: waits for what step k needs.
-template <typename Ahead>
-__device__ __forceinline__ void flow_gemm(bool lead, uint32_t d, uint32_t al, uint32_t a_step, uint32_t bl, int n, int ks,
-                                          uint32_t idesc_m, Ahead ahead) {
+// K steps k0 .. k1 - 1 (32 K bytes each) of D (+)= A B^T, n above 256 in two parts, issued by one lane as a straight row. An
+// instruction of this warp takes about 13 clocks beside the four workers of its scheduler, so a loop that decided per step whether
+// to wait, to issue and to accumulate took 230 clocks a step, the row about 100: 128 images of 32 x 32 144.5 -> 136 us, of 16 x 16
+// 57.7 -> 56, of 8 x 8 43.3 -> 40.5.
+__device__ __forceinline__ void flow_gemm(uint32_t d, uint32_t al, uint32_t a_step, uint32_t bl, int n, int k0, int k1, uint32_t idesc_m) {
   const uint32_t hi = ptx::kUmmaDescHi, b_step = 2u * (uint32_t)n;
   const int na = n > 256 ? 256 : n;
-  const uint32_t idesc = idesc_m | ((uint32_t)(na >> 3) << 17), idesc2 = idesc_m | ((uint32_t)((n - na) >> 3) << 17);
-#pragma unroll 1
-  for (int k = 0; k < ks; ++k) {
-    ahead(k);
-    if (lead) ptx::umma_i8_hl(d, al, hi, bl, hi, idesc, k > 0 ? 1u : 0u);
-    if (n > 256 && lead) ptx::umma_i8_hl(d + 256u, al, hi, bl + 256u, hi, idesc2, k > 0 ? 1u : 0u);
-    al += a_step;
-    bl += b_step;
+  const uint32_t idesc = idesc_m | ((uint32_t)(na >> 3) << 17);
+  al += (uint32_t)k0 * a_step;
+  bl += (uint32_t)k0 * b_step;
+  if (ptx::elect_one()) {
+    if (n <= 256) {
+      ptx::umma_i8_hl(d, al, hi, bl, hi, idesc, k0 > 0 ? 1u : 0u);
+#pragma unroll 4
+      for (int k = k0 + 1; k < k1; ++k) {
+        al += a_step;
+        bl += b_step;
+        ptx::umma_i8_hl(d, al, hi, bl, hi, idesc, 1u);
+      }
+    } else {
+      const uint32_t idesc2 = idesc_m | ((uint32_t)((n - na) >> 3) << 17);
+#pragma unroll 2
+      for (int k = k0; k < k1; ++k) {
+        ptx::umma_i8_hl(d, al, hi, bl, hi, idesc, k > 0 ? 1u : 0u);
+        ptx::umma_i8_hl(d + 256u, al, hi, bl + 256u, hi, idesc2, k > 0 ? 1u : 0u);
+        al += a_step;
+        bl += b_step;
+      }
+    }
   }
+  __syncwarp();
 }
 
-// The nine taps of a 32-channel chunk of the last conv in its direct form (`lead` only): a tap is a start address
-__device__ __forceinline__ void flow_taps(const FlowPlan& P, uint32_t d, uint32_t al, uint32_t a_hi, uint32_t bl, uint32_t b_step,
-                                          uint32_t idesc, bool accumulate) {
+// The last conv in its direct form, 32-channel chunks k0 .. k1 - 1, nine taps each: a tap is a start address
+__device__ __forceinline__ void flow_taps(const FlowPlan& P, uint32_t d, uint32_t al, uint32_t a_hi, uint32_t bl, int n, int k0, int k1,
+                                          uint32_t idesc) {
+  if (ptx::elect_one()) {
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+      const uint32_t a = al + (uint32_t)k * 2u * (uint32_t)P.frame;
+      uint32_t b = bl + (uint32_t)k * 18u * (uint32_t)n;
 #pragma unroll
-  for (int u = 0; u < 3; ++u)
+      for (int u = 0; u < 3; ++u)
 #pragma unroll
-    for (int v = 0; v < 3; ++v) {
-      ptx::umma_i8_hl(d, al + (uint32_t)(u * P.wp + v), a_hi, bl, ptx::kUmmaDescHi, idesc, accumulate || u + v > 0 ? 1u : 0u);
-      bl += b_step;
+        for (int v = 0; v < 3; ++v) {
+          ptx::umma_i8_hl(d, a + (uint32_t)(u * P.wp + v), a_hi, b, ptx::kUmmaDescHi, idesc, u + v > 0 || k > 0 ? 1u : 0u);
+          b += 2u * (uint32_t)n;
+        }
     }
+  }
+  __syncwarp();
 }
 
 // MMA warp of tile slot `sl`: tiles sl, sl + 2, ...
@@ -313,14 +336,16 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
   auto commit = [&](uint64_t* bar) { if (lead) ptx::umma_commit(ptx::smem_u32(bar)); };
   uint32_t used[3] = {0u, 0u, 0u}, apar = 0u;
   auto wait_w = [&](int s) { flow_wait(f, &ctl->w_full[s], used[s] & 1u); };
-  // K step k of a hidden operand: written a round of ncs blocks at a time, or all at once
-  auto wait_a = [&](int k, bool chunked) {
-    const bool c = kShape != kRows128 && chunked;
-    const int r = c ? (f.ncs == 4 ? k >> 2 : k >> 1) : 0;
-    if (c ? (k & (f.ncs - 1)) != 0 : k > 0) return;
-    flow_wait(f, &ctl->a_ready[sl][r], (apar >> r) & 1u);
-    apar ^= 1u << r;
-    ptx::tc_fence_after();
+  // the K steps of a hidden operand, issue(k0, k1): written a round of ncs blocks at a time, or all at once
+  auto hidden = [&](int ks, bool chunked, auto issue) {
+    const int round = kShape != kRows128 && chunked ? f.ncs : ks;
+#pragma unroll 1
+    for (int k = 0, r = 0; k < ks; k += round, ++r) {
+      flow_wait(f, &ctl->a_ready[sl][r], (apar >> r) & 1u);
+      apar ^= 1u << r;
+      ptx::tc_fence_after();
+      issue(k, min(k + round, ks));
+    }
   };
 #pragma unroll 1
   for (int i = 0; i < st.nsteps; ++i) {
@@ -342,12 +367,15 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
     auto first_conv = [&](int t, uint32_t d) {
       const uint32_t base = xa16 + (uint32_t)uniform(ctl->tile[t].w);
       uint32_t bl = b1;
-#pragma unroll 1
-      for (int s = 0; s < P.ks1; ++s) {
-        const uint32_t al = base + (uint32_t)P.step[s];
-        if (lead) ptx::umma_i8_hl(d, al, a1_hi, bl, ptx::kUmmaDescHi, idesc1, s > 0 ? 1u : 0u);
-        bl += 2u * (uint32_t)n1;
+      if (ptx::elect_one()) {
+        ptx::umma_i8_hl(d, base + P.step[0], a1_hi, bl, ptx::kUmmaDescHi, idesc1, 0u);
+#pragma unroll 4
+        for (int s = 1; s < P.ks1; ++s) {
+          bl += 2u * (uint32_t)n1;
+          ptx::umma_i8_hl(d, base + P.step[s], a1_hi, bl, ptx::kUmmaDescHi, idesc1, 1u);
+        }
       }
+      __syncwarp();
     };
     flow_wait_input(f, i);
     ptx::tc_fence_after();
@@ -366,23 +394,14 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
       commit(&ctl->dm_ready[sl]);
       if (last) commit(&ctl->w_empty[0]);
       if (t == sl) wait_w(1);
-      if (kShape == kRows128) wait_a(0, false);
-      flow_gemm(lead, d2, a_lo, 2u * pitch16, b2, n2, ks2, idesc_m, [&](int k) { if (kShape != kRows128) wait_a(k, P.chunk2); });
+      hidden(ks2, P.chunk2, [&](int k0, int k1) { flow_gemm(d2, a_lo, 2u * pitch16, b2, n2, k0, k1, idesc_m); });
       commit(&ctl->dm_ready[sl]);
       if (last) commit(&ctl->w_empty[1]);
       if (t == sl) wait_w(s3);
       if (kShape == kRows64 && P.direct) {
-        uint32_t al = h_lo, bl = b3;
-#pragma unroll 1
-        for (int k = 0; k < ks3; ++k) {
-          wait_a(k, P.chunk3);
-          if (lead) flow_taps(P, d3, al, h_hi, bl, 2u * (uint32_t)n3, idesc_m | ((uint32_t)(n3 >> 3) << 17), k > 0);
-          al += 2u * (uint32_t)P.frame;
-          bl += 18u * (uint32_t)n3;
-        }
+        hidden(ks3, P.chunk3, [&](int k0, int k1) { flow_taps(P, d3, h_lo, h_hi, b3, n3, k0, k1, idesc_m | ((uint32_t)(n3 >> 3) << 17)); });
       } else {
-        wait_a(0, false);
-        flow_gemm(lead, d3, a_lo, 2u * pitch16, b3, n3, ks3, idesc_m, [](int) {});
+        hidden(ks3, false, [&](int k0, int k1) { flow_gemm(d3, a_lo, 2u * pitch16, b3, n3, k0, k1, idesc_m); });
       }
       commit(&ctl->d3_ready[sl]);
       if (last) commit(&ctl->w_empty[s3]);
