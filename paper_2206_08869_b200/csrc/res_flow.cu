@@ -19,8 +19,9 @@
 //   * Larger images are cut into 16 x 16 blocks, one CTA of a cluster each. Edge positions are also stored
 //     into the neighbours' frames, asynchronously: the neighbours' chunk barriers count the bytes, and there is no
 //     cluster barrier between convs.
-//   * One warp issues the MMAs (a chunk's nine taps per wait: waits and commits cost its lane 150 clocks
-//     each, an MMA 40), one lane of another streams weights and the convs' meta blocks.
+//   * Two warps issue the MMAs (a chunk's nine taps per wait: waits and commits cost a lane 150 clocks
+//     each, an MMA 40): a tile each, or, where there is one tile, its chunks in turn, with an accumulator each that the
+//     epilogue adds. One lane of another streams weights and the convs' meta blocks.
 //
 // What bounds it: a conv's chain of first chunk -> 36 MMAs (1 500 - 2 400 clocks) -> last chunk's epilogue -> hand-over,
 // 3 800 clocks at 8 x 8 and 4 x 4 images, 6 200 at 16 x 16, 145 convs one after another. Measured at width 128 with
@@ -37,7 +38,7 @@ struct __align__(16) RfCtl {
   uint64_t chunk_ready[2][kRfChunks];  // workers (and the neighbours' edge bytes) -> MMA warp: 32 channels of the output of
                                        // an even / odd conv (a neighbour may be one conv ahead)
   uint64_t xa_ready;                // the same for the network input
-  uint64_t d_ready[2];              // tensor core -> workers: conv's accumulators complete
+  uint64_t d_ready[2][2];           // tensor core -> workers: accumulators of an even / odd conv complete, by tile (one tile: both)
   uint64_t w_full[kRfMaxSlots], w_empty[kRfMaxSlots];
   uint64_t meta_full[3];
   uint32_t tmem_base, abort;
@@ -140,7 +141,7 @@ __device__ void rf_loader(const Rf& f, const RfPlan& P, const LevelArgs& a, cons
     const RfConv c = convs[sq.index(q)];
     // meta slot: its last readers were the workers at the epilogue of conv q - 3, over when conv q - 2 is
     // complete (whose barrier cannot complete again before conv q, so the wait cannot miss its phase)
-    if (q >= 3) rf_wait(f, &ctl->d_ready[q & 1], (uint32_t)((q - 2) >> 1) & 1u);
+    if (q >= 3) rf_wait(f, &ctl->d_ready[q & 1][0], (uint32_t)((q - 2) >> 1) & 1u);
     {
       const uint32_t b = ptx::smem_u32(&ctl->meta_full[ms]);
       ptx::mbar_expect_tx(b, c.meta_bytes);
@@ -161,14 +162,19 @@ __device__ void rf_loader(const Rf& f, const RfPlan& P, const LevelArgs& a, cons
   }
 }
 
-// ---- MMA warp ------------------------------------------------------------------------------------------------
-__device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq) {
+// ---- MMA warps -----------------------------------------------------------------------------------------------
+// Two tiles: a warp each. One tile: the warps take its chunks in turn, each into an accumulator of its own (the epilogue adds
+// them), so that one warp's waits and commit, 250 - 450 clocks a chunk, pass under the other's MMAs (360 - 570): 64 images of 8 x 8
+// 285 -> 248 us, of 4 x 4 289 -> 260, three of 32 x 32 in 8 x 16 blocks 539 -> 438; with two tiles a chunk's MMAs hid them already
+// (16 x 16 466 -> 465).
+__device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq, int which) {
   RfCtl* ctl = f.ctl;
   uint8_t* smem = f.smem;
   auto uniform = [](int x) { return __shfl_sync(0xFFFFFFFFu, x, 0); };
   // (in a cluster a shared-memory address also carries the CTA's rank above the descriptor's 14 bits)
   auto addr16 = [&](uint32_t s) { return (ptx::smem_u32(smem + s) >> 4) & 0x3FFFu; };
   const uint32_t a_hi = (uint32_t)P.wp | (1u << 14), plane = (uint32_t)P.plane16;
+  const bool one = P.tiles == 1;
   uint32_t slot = 0, round = 0, ready = 0, xa_par = 0;     // ready: bit 4 s + c: parity of chunk barrier [s][c]
   int ms = 0;
   uint32_t mpar = 0;
@@ -179,58 +185,53 @@ __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq) {
     const int n = uniform(M->n_pad), nk = uniform(M->nk), src = uniform(M->src), uns = uniform(M->a_unsigned), input = uniform(M->input);
     if (++ms == 3) { ms = 0; mpar ^= 1u; }
     const uint32_t idesc = (2u << 4) | ((uns ? 0u : 1u) << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(P.m >> 4) << 24);
-    const uint32_t d0 = f.tmem + (uint32_t)((q & 1) * P.tiles * 128);
+    const uint32_t d0 = f.tmem + (uint32_t)((q & 1) * 256 + which * 128);
     const uint32_t b_lbo = (uint32_t)n << 16, tap_step = 2u * (uint32_t)n;
-    // first interior position of tile 0 in the source, chunk 0
-    uint32_t a_chunk = addr16(P.s_buf[src]) + (uint32_t)P.wp + 1u + (plane << 16);
+    // first position of the tile's first tap in the source, chunk 0
+    uint32_t a_chunk = addr16(P.s_buf[src]) + (plane << 16) + (one ? 0u : 8u * (uint32_t)which);
+    uint32_t acc = 0u;
+    const int set = (q - 1) & 1;
+    auto wait_chunk = [&](int kc) {
+      if (!input) rf_wait_operand(f, &ctl->chunk_ready[set][kc], (ready >> (4 * set + kc)) & 1u);
+      else if (kc < 2) rf_wait_operand(f, &ctl->xa_ready, xa_par);
+    };
+    // (a warp without a chunk of this conv commits no sooner than the other one: never a phase ahead)
+    if (one && which >= nk) wait_chunk(0);
 #pragma unroll 1
     for (int kc = 0; kc < nk; ++kc) {
-      rf_wait(f, &ctl->w_full[slot], round & 1u);
-      if (input) {
-        if (kc == 0) { rf_wait_operand(f, &ctl->xa_ready, xa_par); xa_par ^= 1u; }
-      } else {
-        const int set = (q - 1) & 1;
-        rf_wait_operand(f, &ctl->chunk_ready[set][kc], (ready >> (4 * set + kc)) & 1u);
-        ready ^= 1u << (4 * set + kc);
-      }
-      uint32_t bl = addr16(P.s_ring + slot * P.slot_bytes) | b_lbo;
-      const uint32_t a_bias = addr16(P.s_const + (uns ? 0u : 2304u)) | (8u << 16);
-      if (ptx::elect_one()) {
-        if (kc == 0) {                    // bias rows: the operand is the same constant row everywhere
-          ptx::umma_i8_hl(d0, a_bias, ptx::kUmmaDescHi, bl, ptx::kUmmaDescHi, idesc, 0u);
-          if (P.tiles == 2) ptx::umma_i8_hl(d0 + 128u, a_bias, ptx::kUmmaDescHi, bl, ptx::kUmmaDescHi, idesc, 0u);
-          bl += tap_step;
-        }
-        uint32_t al = a_chunk - (uint32_t)P.wp - 1u;
-        if (P.tiles == 2) {
+      if (!one || (kc & 1) == which) {
+        rf_wait(f, &ctl->w_full[slot], round & 1u);
+        wait_chunk(kc);
+        uint32_t bl = addr16(P.s_ring + slot * P.slot_bytes) | b_lbo;
+        const uint32_t a_bias = addr16(P.s_const + (uns ? 0u : 2304u)) | (8u << 16);
+        if (ptx::elect_one()) {
+          if (kc == 0) {                    // bias rows: the operand is the same constant row everywhere
+            ptx::umma_i8_hl(d0, a_bias, ptx::kUmmaDescHi, bl, ptx::kUmmaDescHi, idesc, 0u);
+            bl += tap_step;
+            acc = 1u;
+          }
+          uint32_t al = a_chunk;
 #pragma unroll
           for (int u = 0; u < 3; ++u) {
 #pragma unroll
             for (int v = 0; v < 3; ++v) {
-              ptx::umma_i8_hl(d0, al + (uint32_t)v, a_hi, bl, ptx::kUmmaDescHi, idesc, 1u);
-              ptx::umma_i8_hl(d0 + 128u, al + (uint32_t)(v + 8), a_hi, bl, ptx::kUmmaDescHi, idesc, 1u);
+              ptx::umma_i8_hl(d0, al + (uint32_t)v, a_hi, bl, ptx::kUmmaDescHi, idesc, u + v > 0 ? 1u : acc);
               bl += tap_step;
             }
             al += (uint32_t)P.wp;
           }
-        } else {
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-#pragma unroll
-            for (int v = 0; v < 3; ++v) {
-              ptx::umma_i8_hl(d0, al + (uint32_t)v, a_hi, bl, ptx::kUmmaDescHi, idesc, 1u);
-              bl += tap_step;
-            }
-            al += (uint32_t)P.wp;
-          }
+          ptx::umma_commit(ptx::smem_u32(&ctl->w_empty[slot]));
         }
-        ptx::umma_commit(ptx::smem_u32(&ctl->w_empty[slot]));
-        if (kc + 1 == nk) ptx::umma_commit(ptx::smem_u32(&ctl->d_ready[q & 1]));
+        acc = 1u;
+        __syncwarp();
       }
-      __syncwarp();
       if (++slot == (uint32_t)P.n_slots) { slot = 0; ++round; }
       a_chunk += 2u * plane;
     }
+    if (input) xa_par ^= 1u;
+    else ready ^= ((1u << nk) - 1u) << (4 * set);
+    if (ptx::elect_one()) ptx::umma_commit(ptx::smem_u32(&ctl->d_ready[q & 1][one ? 0 : which]));
+    __syncwarp();
   }
 }
 
@@ -263,6 +264,7 @@ __device__ __forceinline__ void rf_store(const Rf& f, const RfPlan& P, uint8_t* 
 // One unit: 16 rows (half `h` of this warp's lane quarter of tile `t`) x 32 columns (chunk b) of a hidden or branch conv.
 __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMeta* __restrict__ M, uint32_t d, int t, int h, int b,
                                         uint64_t* ready, uint32_t parity, uint64_t* chunk) {
+  const bool both = P.tiles == 1 && M->nk > 1;           // two accumulators
   const int q = f.lane & 3, x = f.lane >> 2, hs = P.m >> 7;
   // (what does not depend on the accumulator comes before the wait for it)
   uint32_t r[16];
@@ -282,8 +284,18 @@ __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMe
   auto accumulator = [&]() {
     rf_wait(f, ready, parity);
     ptx::tc_fence_after();
-    ptx::tmem_ld_16x32(d + (uint32_t)(t * 128 + b * 32) + ((uint32_t)h << 20) + ((uint32_t)((f.warp & 3) * 32) << 16), r);
-    ptx::tmem_ld_wait16(r);
+    const uint32_t at = d + (uint32_t)(t * 128 + b * 32) + ((uint32_t)h << 20) + ((uint32_t)((f.warp & 3) * 32) << 16);
+    ptx::tmem_ld_16x32(at, r);
+    if (both) {
+      uint32_t r2[16];
+      ptx::tmem_ld_16x32(at + 128u, r2);
+      ptx::tmem_ld_wait16(r);
+      ptx::tmem_ld_wait16_nosync(r2);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) r[k] += r2[k];
+    } else {
+      ptx::tmem_ld_wait16(r);
+    }
   };
   if (M->kind == kRfHidden) {
     float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
@@ -353,11 +365,16 @@ __device__ void rf_out(const Rf& f, const RfPlan& P, const LevelArgs& a, const R
 #pragma unroll 1
   for (int un = f.warp >> 2; un < units; un += 4) {
     const int gr = un / (P.tiles << hs), th = un - gr * (P.tiles << hs), h = th & hs, t = th >> hs;
-    uint32_t r[4];
-    ptx::tmem_ld_16x8(d + (uint32_t)(t * 128 + gr * 8) + ((uint32_t)h << 20) + ((uint32_t)((f.warp & 3) * 32) << 16), r);
+    uint32_t r[4], r2[4] = {0u, 0u, 0u, 0u};
+    const uint32_t at = d + (uint32_t)(t * 128 + gr * 8) + ((uint32_t)h << 20) + ((uint32_t)((f.warp & 3) * 32) << 16);
+    ptx::tmem_ld_16x8(at, r);
+    if (P.tiles == 1 && M->nk > 1) ptx::tmem_ld_16x8(at + 128u, r2);
     int p[2];
     rf_pixels(f, P, t, ((f.warp & 3) << (1 + hs)) + 2 * h, &p[0], &p[1]);
     ptx::tmem_ld_wait4(r);
+    ptx::tmem_ld_wait4_nosync(r2);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[k] += r2[k];
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const int ch = gr * 8 + 2 * (f.lane & 3) + e;
@@ -423,9 +440,9 @@ __device__ void rf_workers(const Rf& f, const RfPlan& P, const LevelArgs& a, con
       rf_requant(f, P, M, v);
       rf_hand_over(f, &ctl->xa_ready, f.warp == 0 ? f.halo * 4u * (uint32_t)((P.ca + 3) >> 2) : 0u);
     }
-    const uint32_t d = f.tmem + (uint32_t)((q & 1) * P.tiles * 128);
+    const uint32_t d = f.tmem + (uint32_t)((q & 1) * 256);
     const int nb = M->nb, kind = M->kind;
-    uint64_t* dr = &ctl->d_ready[q & 1];
+    uint64_t* dr = &ctl->d_ready[q & 1][t];
     const uint32_t dp = (uint32_t)(q >> 1) & 1u;
     if (kind == kRfHidden || kind == kRfBranch) {
       if (c0 != 0) {                       // every warp arrives once per conv: nobody can miss a phase
@@ -440,7 +457,8 @@ __device__ void rf_workers(const Rf& f, const RfPlan& P, const LevelArgs& a, con
         rf_hand_over(f, cr, me == 0 && (f.warp & 3) == 0 ? f.halo * 32u : 0u);
       }
     } else {
-      rf_wait(f, dr, dp);
+      rf_wait(f, &ctl->d_ready[q & 1][0], dp);
+      if (P.tiles == 2) rf_wait(f, &ctl->d_ready[q & 1][1], dp);
       ptx::tc_fence_after();
       rf_out<kInv>(f, P, a, M, d, v, b0);
       ptx::tc_fence_before();
@@ -537,16 +555,16 @@ __global__ void __launch_bounds__(kRfThreads, 1) res_flow_kernel(const LevelArgs
     for (int c = 0; c < 2 * kRfChunks; ++c)
       ptx::mbar_init(ptx::smem_u32(&ctl.chunk_ready[c >> 2][c & 3]), (c & 3) ? (uint32_t)(4 * (P.tiles * (P.m >> 6))) : (uint32_t)kRfWarps);
     ptx::mbar_init(ptx::smem_u32(&ctl.xa_ready), (uint32_t)kRfWarps);
-    for (int s = 0; s < 2; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.d_ready[s]), 1);
+    for (int s = 0; s < 4; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.d_ready[s >> 1][s & 1]), P.tiles == 1 ? 2u : 1u);
     for (int s = 0; s < 3; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.meta_full[s]), 1);
     for (int s = 0; s < kRfMaxSlots; ++s) {
       ptx::mbar_init(ptx::smem_u32(&ctl.w_full[s]), 1);
-      ptx::mbar_init(ptx::smem_u32(&ctl.w_empty[s]), 1);
+      ptx::mbar_init(ptx::smem_u32(&ctl.w_empty[s]), (uint32_t)P.tiles);
     }
     ptx::mbar_init_fence();
     ctl.abort = 0;
   }
-  if (warp == 0) ptx::tmem_alloc(ptx::smem_u32(&ctl.tmem_base), (uint32_t)(P.tiles * 256));
+  if (warp == 0) ptx::tmem_alloc(ptx::smem_u32(&ctl.tmem_base), kRfTmemCols);
   // activation buffers start at zero (borders, channels beyond a conv's outputs); the constant operand rows
   for (uint32_t o = P.s_buf[0] + 16 * tid; o < P.s_buf_end; o += 16 * kRfThreads) *reinterpret_cast<uint4*>(smem + o) = make_uint4(0u, 0u, 0u, 0u);
   for (uint32_t o = 16 * tid; o < 2u * 2304u; o += 16 * kRfThreads) {
@@ -567,10 +585,10 @@ __global__ void __launch_bounds__(kRfThreads, 1) res_flow_kernel(const LevelArgs
   sq.prior_first = prior && kInv; sq.prior_last = prior && !kInv; sq.inverse = kInv;
   sq.count = sq.n_couplings * sq.cpc + (prior ? 1 : 0);
 
-  if (warp == kRfWarps + 1) {
+  if (warp == kRfWarps + 2) {
     if (lane == 0) rf_loader(f, P, a, sq);
-  } else if (warp == kRfWarps) {
-    rf_mma(f, P, sq);
+  } else if (warp >= kRfWarps) {
+    rf_mma(f, P, sq, warp - kRfWarps);
   } else {
     int32_t* v = reinterpret_cast<int32_t*>(smem + P.s_v);
     ptx::grid_dependency_wait();
@@ -583,7 +601,7 @@ __global__ void __launch_bounds__(kRfThreads, 1) res_flow_kernel(const LevelArgs
   ptx::tc_fence_before();
   // (a neighbour may still be storing edges here: nobody leaves before everybody is done)
   if (nblk > 1) rf_cluster_barrier(); else __syncthreads();
-  if (warp == 0) ptx::tmem_dealloc(ctl.tmem_base, (uint32_t)(P.tiles * 256));
+  if (warp == 0) ptx::tmem_dealloc(ctl.tmem_base, kRfTmemCols);
 }
 
 }  // namespace

@@ -11,7 +11,8 @@ namespace iodf {
 
 constexpr int kRfWarps = 16;                        // requantising warps, four per TMEM lane quarter
 constexpr int kRfWorkers = kRfWarps * 32;
-constexpr int kRfThreads = kRfWorkers + 2 * 32;     // + the MMA-issuing warp and the weight-loading warp
+constexpr int kRfThreads = kRfWorkers + 3 * 32;     // + two MMA-issuing warps and the weight-loading warp
+constexpr int kRfTmemCols = 512;                    // two convs of two accumulators of 128 columns
 constexpr int kRfMaxSlots = 4;                      // weight ring
 constexpr int kRfChunks = 4;                        // 32-channel chunks of the widest activation (128 channels)
 
