@@ -21,6 +21,9 @@
 //     operand is a zero-bordered frame too, the last conv is nine taps of it with as few columns as it has channels (an MMA of 64
 //     rows takes 23 clocks up to 24 columns), its accumulators are the translation, and its K steps start as the blocks of
 //     32 channels are written. 128 images of 24 channels: 48 -> 43 us, two to a CTA 65 -> 54.
+//   * A lane quarter of a 4 x 4 level's tile is an image. A CTA of one image (two) has four (two) copies of it in the operands' rows,
+//     so that all sixteen warps, not four, share its columns (P.copies): 128 images of 96 channels 47 -> 45 us, 64 of width 512
+//     98 -> 92.
 //   * CTAs of several tiles have two in flight (slots), each with eight of the sixteen workers and an MMA
 //     warp of its own, so that one slot's hand-overs and MMAs run under the other's requantisation; CTAs of
 //     one tile put all sixteen workers on it. One lane of another warp streams weights and meta blocks.
@@ -82,7 +85,8 @@ struct Flow {
   int slots;                    // tile slots in use: 1 or 2
   int rank, by, bx;             // split images: this CTA's block
   uint32_t halo;                // ... and the bytes of network input that its neighbours send each step
-  int sl, cs, ncs;              // worker: its slot, its share of a lane quarter's work (cs of ncs warps)
+  int sl, cs, ncs;              // worker: its slot, its share of a lane quarter's work (cs of ncs warps; of an image's, 4 x 4)
+  int image;                    // 4 x 4: image of the tile in this warp's lane quarter
 };
 
 // One test, then suspended (spinning warps take issue slots and shared-memory bandwidth from the others).
@@ -514,6 +518,13 @@ __device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, ui
   const FlowLayer L = reinterpret_cast<const FlowMeta*>(mb)->layer[layer];
   const uint8_t* t = mb + 16 * L.off + (f.lane & 3) * 32;
   const int row = kShape == kRows64 ? ho.row : 128;
+  auto put = [&](uint8_t* to, uint2 w) {
+    *reinterpret_cast<uint2*>(to) = w;
+    if constexpr (kShape == kImages4x4)
+#pragma unroll
+      for (int c = 1; c < 4; ++c)
+        if (c < P.copies) *reinterpret_cast<uint2*>(to + 256 * c) = w;
+  };
   uint64_t* done = f.ctl->a_ready[f.sl];
   flow_wait(f, ready, parity);
   ptx::tc_fence_after();
@@ -543,7 +554,7 @@ __device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, ui
 #pragma unroll
           for (int k = 0; k < 16; ++k) r[h][k] = (uint32_t)FloatRq::one(r[h][k], m[2 * (k >> 2) + (k & 1)], 0.f);
 #pragma unroll
-          for (int e = 0; e < 2; ++e) *reinterpret_cast<uint2*>(o + (2 * h + e) * row) = pack(h, e);
+          for (int e = 0; e < 2; ++e) put(o + (2 * h + e) * row, pack(h, e));
         }
       } else {
         if (b < L.nfi) {
@@ -571,7 +582,7 @@ __device__ __forceinline__ void flow_hidden(const Flow& f, const FlowPlan& P, ui
           for (int e = 0; e < 2; ++e) {
             uint2 w = pack(h, e);
             if (tail) w = make_uint2(none ? L.beyond : w.x, L.beyond);
-            *reinterpret_cast<uint2*>(o + (2 * h + e) * row) = w;
+            put(o + (2 * h + e) * row, w);
           }
       }
     }
@@ -678,7 +689,7 @@ __device__ __forceinline__ void flow_sum_4x4(const Flow& f, const FlowPlan& P, i
   const OutRq* orq = reinterpret_cast<const OutRq*>(mb + M->off_out);
   const bool odd = lane >= 16;
   // a unit's constants and its part of the flow variable, which nobody else writes: the first unit's before the wait
-  int32_t* vq = v + (4 * t + (f.warp & 3)) * 16 + (lane >> 2);
+  int32_t* vq = v + (4 * t + f.image) * 16 + (lane >> 2);
   OutRq o[2];
   int32_t* vp[2];
   uint32_t x[2][2];
@@ -803,7 +814,7 @@ __device__ void flow_prior(const Flow& f, const FlowPlan& P, const LevelArgs& a,
     const int4 tp = f.ctl->tile[t];
     int img = tp.x, at = (tp.y + (lane_row >> 3)) * P.w + tp.z + (lane_row & 7);
     if constexpr (kSplit) at = (f.by * P.h + tp.y + (lane_row >> 3)) * P.fw + f.bx * P.w + tp.z + (lane_row & 7);
-    if (kShape == kImages4x4) { img += lane_row >> 4; at = lane_row & 15; }
+    if (kShape == kImages4x4) { img += f.image; at = lane_row & 15; }
     int32_t* mu = a.prior + (size_t)(img0 + img) * (size_t)(2 * P.d_fact) + P.prior_off + at;
     OutRq o[8];
 #pragma unroll
@@ -957,18 +968,25 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
   int32_t* v = reinterpret_cast<int32_t*>(smem + P.s_v);
   int32_t* acc = reinterpret_cast<int32_t*>(smem + P.s_acc);
   const uint32_t lane_field = (uint32_t)((f.warp & 3) * 32) << 16;
-  // (4 x 4 levels: a lane quarter is an image; quarters without one only take part in the hand-overs)
+  // (4 x 4 levels: a lane quarter is an image, or a copy of one; quarters without one only take part in the hand-overs)
   PixelMap pm;
   const int pairs = P.pg >> 1;
   pm.parts = kFlowWorkers / pairs;
   pm.j = f.tid / pairs;
   pm.p = 2 * (f.tid - pm.j * pairs);
+  int copy = 0;                                 // (4 x 4: threads of their own for each copy of the operand)
+  if (kShape == kImages4x4) {
+    pm.parts /= P.copies;
+    copy = pm.j / pm.parts;
+    pm.j -= copy * pm.parts;
+    if (copy >= P.copies) pm.j = 1 << 20;
+  }
   if (pm.j >= pm.parts || pm.p >= f.pvalid) pm.j = 1 << 20;      // no work
   {
     const int img = fdiv(pm.p, P.mul_px), px = pm.p - img * P.px, r = fdiv(px, P.mul_w), c = px - r * P.w;
     pm.v = v + pm.p;
     pm.acc = acc + pm.p;
-    pm.rec = smem + P.s_xa + 16 * (P.im2col ? img * 16 + px : img * P.frame + (r + 1) * P.wp + c + 1);
+    pm.rec = smem + P.s_xa + 16 * (P.im2col ? (img * P.copies + copy) * 16 + px : img * P.frame + (r + 1) * P.wp + c + 1);
     pm.dy = r == 0 ? -1 : (r == P.h - 1 ? 1 : 0);
     pm.dx = c == 0 ? -1 : (c == P.w - 2 ? 1 : 0);
     pm.taps = 0;
@@ -1007,7 +1025,7 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
     } else {
 #pragma unroll 1
       for (int t = f.sl; t < f.tiles; t += f.slots) {
-        const bool quarter = kShape != kImages4x4 || 4 * t + (f.warp & 3) < f.nimg;
+        const bool quarter = kShape != kImages4x4 || 4 * t + f.image < f.nimg;
 #pragma unroll 1
         for (int layer = 0; layer < 2; ++layer) {
           const bool chunked = kShape != kRows128 && (layer ? P.chunk3 : P.chunk2);
@@ -1019,7 +1037,8 @@ __device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& 
             ho.block = 32 * P.frame;
             ho.row = 16 * P.wp;
           } else {
-            ho.at = smem + P.s_a[f.sl] + (q >> 1) * P.pitch + ((f.warp & 3) * (kShape == kRows128 ? 32 : 16) + row) * 16 + (q & 1) * 8;
+            const int first = kShape == kImages4x4 ? f.image * P.copies * 16 : (f.warp & 3) * (kShape == kRows128 ? 32 : 16);
+            ho.at = smem + P.s_a[f.sl] + (q >> 1) * P.pitch + (first + row) * 16 + (q & 1) * 8;
             ho.block = 2 * P.pitch;
             ho.row = 128;
           }
@@ -1211,9 +1230,11 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
   f.smem = smem; f.ctl = &ctl; f.status = a.status; f.tmem = ctl.tmem_base;
   f.tid = tid; f.warp = warp; f.lane = lane;
   f.nimg = nimg; f.pvalid = nimg * P.px; f.tiles = tiles; f.slots = slots;
-  f.ncs = kFlowWarps / 4 / slots;
+  const int copies = kShape == kImages4x4 ? P.copies : 1;
+  f.ncs = kFlowWarps / 4 / slots * copies;
   f.sl = slots == 2 && warp >= kFlowWarps / 2 ? 1 : 0;
-  f.cs = (warp - f.sl * (kFlowWarps / 2)) >> 2;
+  f.cs = ((warp - f.sl * (kFlowWarps / 2)) >> 2) * copies + (warp & 3) % copies;
+  f.image = (warp & 3) / copies;
   Steps st;
   st.n_couplings = (kInv && a.phase == 1) ? 0 : P.n_couplings;
   st.do_prior = P.has_prior && a.prior != nullptr && !(kInv && a.phase == 2);

@@ -987,15 +987,20 @@ bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool
   }
   F.pitch = F.m * 16 + 64;
   F.acc_stride = F.pg + 4;
-  for (int alias = 0; alias < 2; ++alias) {
+  // (4 x 4: operands with copies of the images where they fit, also where that makes two matrices share a slot)
+  const int most_copies = F.im2col && group <= 2 ? 4 / group : 1;
+  for (int form = 0; form < 4; ++form) {
+    const int alias = form & 1;
+    F.copies = form < 2 ? most_copies : 1;
     if (alias && (F.tiles > 2 || wide)) continue;
+    if (form >= 2 && most_copies == 1) continue;
     const uint32_t w_last = nd.w[direct ? 3 : 2];
     uint32_t off = 0;
     auto take = [&](uint32_t bytes) { const uint32_t o = off; off = up(off + bytes, kAlign); return o; };
     F.alias = alias;
     F.s_v = take((uint32_t)F.c * F.pg * 4);
     if (F.im2col) {
-      F.plane16 = 16 * group;
+      F.plane16 = 16 * group * F.copies;
       F.s_xa = take((uint32_t)(F.rec / 16) * F.plane16 * 16 + 64 * 16);       // a tile's 64 rows read past a short last plane
     } else {
       F.plane16 = group * F.frame;

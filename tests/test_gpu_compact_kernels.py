@@ -37,6 +37,20 @@ def test_last_conv_on_8x8_frames(G, splits, hidden, batch, sample, plan):
     _check_both_ways(G, model, x, sample=sample, plan=plan)
 
 
+@pytest.mark.parametrize("in_c,hidden,batch,plan,sample", [
+    (2, 16, 1, 0, None),                  # one image in four lane quarters, a block for one of sixteen warps
+    (6, 256, 1, 0, None),                 # nine blocks
+    (24, 176, 3, 0, None),                # 96 channels: the first and the last matrix share a slot
+    (12, 512, 2, 0, None),                # streamed weights
+    (4, 33, 3, 1, None),                  # several images to a CTA
+    (12, 130, 299, 0, [0, 1, 297, 298]),  # two to a CTA, the last alone: two copies, and two quarters without an image
+])
+def test_copies_of_4x4_images(G, in_c, hidden, batch, plan, sample):
+    model = S.make_model(0xFD00 + in_c + hidden, in_c, 8, 8, [True], 3, hidden)
+    x = np.random.default_rng(in_c).integers(0, 256, (batch, in_c, 8, 8), dtype=np.uint8)
+    _check_both_ways(G, model, x, sample=sample, plan=plan)
+
+
 @pytest.mark.parametrize("hw,splits,hidden,batch", [
     (16, [True, True], 16, 5),           # the last level 4 x 4: four images and one
     (16, [True, True], 31, 3),           # 8 x 8 tiles of 64 rows, six and twelve channels in
