@@ -18,9 +18,12 @@
 //     next GEMM's K is free, so a thread's eight results are eight adjacent operand bytes.
 //   * The per-tap partial products of the last conv are added to a pixel-major accumulator (odd
 //     stride) with one shared-memory reduction each. 8 x 8 images, one tile each, need none of that (P.direct): their hidden
-//     operand is a zero-bordered frame too, the last conv is nine taps of it with as few columns as it has channels (an MMA of 64
-//     rows takes 23 clocks up to 24 columns), its accumulators are the translation, and its K steps start as the blocks of
-//     32 channels are written. 128 images of 24 channels: 48 -> 43 us, two to a CTA 65 -> 54.
+//     operand is a zero-bordered frame too, and the last conv is taps of it. An MMA of 64 rows takes 23 clocks up to 24 columns and N / 2
+//     beyond, and this warp 28 to issue, so with an MMA per tap (kFlowNine) 45 of them took longer than the epilogues before them. With one
+//     per row of taps (kFlowRows) it is fifteen of three times the columns; the three products of a pixel lie in neighbouring lanes and
+//     meet by shuffles as the translation is applied. K steps start as the blocks of 32 channels are written. 128 images of 48
+//     channels: 48 us with per-tap partials, 40 by taps, 37.5 by rows; 256 of 24, two to a CTA: 65, 49.5, 45. The three products
+//     need columns: where those of both slots do not fit beside the hidden layers' and a slot has more tiles than one, taps stay.
 //   * A lane quarter of a 4 x 4 level's tile is an image. A CTA of one image (two) has four (two) copies of it in the operands' rows,
 //     so that all sixteen warps, not four, share its columns (P.copies): 128 images of 96 channels 47 -> 45 us, 64 of width 512
 //     98 -> 92.
@@ -301,21 +304,33 @@ __device__ __forceinline__ void flow_gemm(uint32_t d, uint32_t al, uint32_t a_st
   __syncwarp();
 }
 
-// The last conv in its direct form, 32-channel chunks k0 .. k1 - 1, nine taps each: a tap is a start address
+// The last conv in its direct forms, 32-channel chunks k0 .. k1 - 1: a tap is a start address of the operand, and the weights of a
+// chunk's tap row are [2][three taps of n rows][16 bytes]. kFlowNine: an MMA of n columns per tap. kFlowRows: one of 3 n columns per
+// row of taps, its three products summed by the epilogue.
 __device__ __forceinline__ void flow_taps(const FlowPlan& P, uint32_t d, uint32_t al, uint32_t a_hi, uint32_t bl, int n, int k0, int k1,
-                                          uint32_t idesc) {
+                                          uint32_t idesc_m) {
   if (ptx::elect_one()) {
+    if (P.direct == kFlowRows) {
+      const uint32_t idesc = idesc_m | ((uint32_t)((3 * n + 15) >> 4) << 18);
 #pragma unroll 1
-    for (int k = k0; k < k1; ++k) {
-      const uint32_t a = al + (uint32_t)k * 2u * (uint32_t)P.frame;
-      uint32_t b = bl + (uint32_t)k * 18u * (uint32_t)n;
+      for (int k = k0; k < k1; ++k) {
+        const uint32_t a = al + (uint32_t)k * 2u * (uint32_t)P.frame + 1u, b = bl + (uint32_t)k * 18u * (uint32_t)n;
 #pragma unroll
-      for (int u = 0; u < 3; ++u)
+        for (int u = 0; u < 3; ++u)
+          ptx::umma_i8_hl(d, a + (uint32_t)(u * P.wp), a_hi, b + (uint32_t)(6 * u * n), ptx::kUmmaDescHi, idesc, u > 0 || k > 0 ? 1u : 0u);
+      }
+    } else {
+      const uint32_t idesc = idesc_m | ((uint32_t)(n >> 3) << 17);
+#pragma unroll 1
+      for (int k = k0; k < k1; ++k) {
+        const uint32_t a = al + (uint32_t)k * 2u * (uint32_t)P.frame, b = bl + (uint32_t)k * 18u * (uint32_t)n;
 #pragma unroll
-        for (int v = 0; v < 3; ++v) {
-          ptx::umma_i8_hl(d, a + (uint32_t)(u * P.wp + v), a_hi, b, ptx::kUmmaDescHi, idesc, u + v > 0 || k > 0 ? 1u : 0u);
-          b += 2u * (uint32_t)n;
-        }
+        for (int u = 0; u < 3; ++u)
+#pragma unroll
+          for (int v = 0; v < 3; ++v)
+            ptx::umma_i8_hl(d, a + (uint32_t)(u * P.wp + v), a_hi, b + (uint32_t)((6 * u + v) * n), ptx::kUmmaDescHi, idesc,
+                            u + v > 0 || k > 0 ? 1u : 0u);
+      }
     }
   }
   __syncwarp();
@@ -365,7 +380,7 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
     ++used[0];
     const uint32_t b1 = ((ptx::smem_u32(smem + P.s_w[0]) >> 4) & 0x3FFFu) | ((uint32_t)n1 << 16);
     const uint32_t b2 = ((ptx::smem_u32(smem + P.s_w[1]) >> 4) & 0x3FFFu) | ((uint32_t)n2 << 16);
-    const uint32_t b3 = ((ptx::smem_u32(smem + P.s_w[s3]) >> 4) & 0x3FFFu) | ((uint32_t)n3 << 16);
+    const uint32_t b3 = ((ptx::smem_u32(smem + P.s_w[s3]) >> 4) & 0x3FFFu) | ((uint32_t)(kShape == kRows64 && P.direct ? 3 * n3 : n3) << 16);
     const uint32_t idesc1 = idesc_m | ((uint32_t)(n1 >> 3) << 17);
     // first conv of a tile: steps from the table {start offset, leading offset}
     auto first_conv = [&](int t, uint32_t d) {
@@ -403,7 +418,7 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
       if (last) commit(&ctl->w_empty[1]);
       if (t == sl) wait_w(s3);
       if (kShape == kRows64 && P.direct) {
-        hidden(ks3, P.chunk3, [&](int k0, int k1) { flow_taps(P, d3, h_lo, h_hi, b3, n3, k0, k1, idesc_m | ((uint32_t)(n3 >> 3) << 17)); });
+        hidden(ks3, P.chunk3, [&](int k0, int k1) { flow_taps(P, d3, h_lo, h_hi, b3, n3, k0, k1, idesc_m); });
       } else {
         hidden(ks3, false, [&](int k0, int k1) { flow_gemm(d3, a_lo, 2u * pitch16, b3, n3, k0, k1, idesc_m); });
       }
@@ -777,8 +792,24 @@ __device__ __forceinline__ void flow_out(const Flow& f, const FlowPlan& P, int t
 #pragma unroll 1
   while (8 * g < P.cb) {
     uint32_t r[4];
-    ptx::tmem_ld_16x8(taddr + (uint32_t)(8 * g), r);
-    ptx::tmem_ld_wait4(r);
+    if (P.direct == kFlowRows) {       // products of the taps left, middle and right: of the columns x - 1, x and x + 1
+      uint32_t r0[4], r2[4];
+      const uint32_t at = taddr + (uint32_t)(8 * g), n = (uint32_t)M->n3d;
+      ptx::tmem_ld_16x8(at, r0);
+      ptx::tmem_ld_16x8(at + n, r);
+      ptx::tmem_ld_16x8(at + 2u * n, r2);
+      ptx::tmem_ld_wait4(r0);
+      ptx::tmem_ld_wait4_nosync(r);
+      ptx::tmem_ld_wait4_nosync(r2);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t left = __shfl_up_sync(0xFFFFFFFFu, r0[k], 4), right = __shfl_down_sync(0xFFFFFFFFu, r2[k], 4);
+        r[k] += (f.lane >= 4 ? left : 0u) + (f.lane < 28 ? right : 0u);
+      }
+    } else {
+      ptx::tmem_ld_16x8(taddr + (uint32_t)(8 * g), r);
+      ptx::tmem_ld_wait4(r);
+    }
     if (ok) {
 #pragma unroll
       for (int e = 0; e < 2; ++e)

@@ -17,6 +17,8 @@ constexpr int kFlowMaxTiles = 32;                    // of a CTA
 constexpr int kFlowMaxSteps = 18;                    // K steps of the first conv
 constexpr int kFlowMaxRounds = 5;                    // blocks of 32 columns that a warp requantises of a layer
 
+enum FlowDirect : int { kFlowNine = 1, kFlowRows = 2 };   // forms of the last conv on the hidden operand: an MMA per tap, per row of taps
+
 constexpr int kFlowMaxBlocks = 8;                    // CTAs that share an image (portable cluster size)
 
 // Everything about a level that the kernel needs and that is the same for all its couplings; passed
@@ -45,8 +47,8 @@ struct FlowPlan {
   uint32_t step[kFlowMaxSteps];  // (mod 2^32) + distance of the second chunk << 16, in 16-byte units
   int32_t pitch;                 // bytes between 16-byte K chunks of the hidden operands
   int32_t acc_stride;            // words per channel plane of the translation accumulator (pg + 4: no bank conflicts)
-  // 8 x 8 images, one tile each: the last conv as nine taps on the hidden operand itself, in a zero-bordered frame (planes of
-  // 16 channels, s_h), rather than per-tap partials and their shifted sum
+  // 8 x 8 images, one tile each: the last conv on the hidden operand itself, in a zero-bordered frame (planes of 16 channels,
+  // s_h), rather than per-tap partials and their shifted sum. kFlowRows where its accumulators fit, else kFlowNine
   int32_t direct;
   // 1: the second (third) GEMM's K steps start as the blocks of its operand are written, a round of blocks at a time
   int32_t chunk2, chunk3;

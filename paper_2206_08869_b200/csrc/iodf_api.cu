@@ -631,13 +631,13 @@ PackedBlock pack_flow_coupling(const iodf_coupling_desc& cp, const Blobs& B, con
     for (int tap = 0; tap < 9; ++tap)
       for (int k = 0; k < k2; ++k)
         pb.w[2][wpos(M.n3, tap * cbp + c, flow_kpos(k))] = (uint8_t)w3[((size_t)c * 9 + tap) * k2 + o2.ch[k]];
-  // the same for the direct form: K chunk by chunk of 32 channels, nine taps each
+  // the same for the direct forms: K chunk by chunk of 32 channels, three rows of taps each, in a row's matrix tap by tap
   if (direct) {
     pb.w[3].assign((size_t)M.n3d * 9 * 32 * M.ks3, 0);
     for (int c = 0; c < cb; ++c)
       for (int tap = 0; tap < 9; ++tap)
         for (int k = 0; k < k2; ++k)
-          pb.w[3][wpos(M.n3d, c, (flow_kpos(k) >> 5) * 288 + tap * 32 + (flow_kpos(k) & 31))] =
+          pb.w[3][wpos(3 * M.n3d, tap % 3 * M.n3d + c, ((flow_kpos(k) >> 5) * 3 + tap / 3) * 32 + (flow_kpos(k) & 31))] =
               (uint8_t)w3[((size_t)c * 9 + tap) * k2 + o2.ch[k]];
   }
   pb.k_slices[0] = (uint32_t)kmap.size() / 32; pb.k_slices[1] = (uint32_t)M.ks2; pb.k_slices[2] = (uint32_t)M.ks3;
@@ -955,29 +955,31 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
 
 // Group, tensor-memory columns and shared-memory layout of a level in the compact kernel. false: it does not fit.
 struct FlowNeeds { uint32_t n_hidden = 32, n_taps = 16, n_direct = 16, kb = 1, meta = 16, w[4] = {16, 16, 16, 16}; };
-// wide: weights streamed for every tile, one tile in flight. direct: the last conv in its direct form.
-bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool wide, bool direct) {
+// wide: weights streamed for every tile, one tile in flight. direct: form of the last conv on the hidden operand (0: taps and sum).
+bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool wide, int direct) {
   F.group = group;
   F.direct = direct;
   F.pg = group * F.px;
   F.tiles = F.im2col ? (group + 3) / 4 : group * F.tiles_img;
-  const uint32_t nh = up(nd.n_hidden, 16), nh32 = up(nd.n_hidden, 32), n_last = direct ? nd.n_direct : nd.n_taps;
-  if (nd.n_hidden > 512 || n_last > (direct ? 128u : 512u) || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
+  const uint32_t nh = up(nd.n_hidden, 16), nh32 = up(nd.n_hidden, 32), n_last = direct == kFlowRows ? up(3 * nd.n_direct, 16) : direct ? nd.n_direct : nd.n_taps;
+  if (nd.n_hidden > 512 || n_last > (direct == kFlowNine ? 128u : direct ? 256u : 512u) || (uint32_t)F.tiles * F.n_prior > 512u || F.tiles > kFlowMaxTiles || F.pg > 2 * kFlowWorkers)
     return false;
   F.d_col = 0; F.d3_col = 0; F.d3_step = 0; F.d2_col = 0; F.chunk2 = 0;
   // K steps of the last GEMM run ahead of the epilogue that writes their operand: its accumulators must not lie on columns
   // that the epilogue's later rounds read
-  F.chunk3 = direct;
+  F.chunk3 = direct != 0;
   if (wide) {
     F.tmem_cols = 512;
   } else if (F.tiles == 1) {
     F.chunk2 = F.m == 64 && 2 * nh32 <= 512u;
     F.d2_col = F.chunk2 ? (int)nh32 : 0;
+    if (nh32 > 128u && n_last > nh32) F.chunk3 = 0;          // (up to four blocks: one round)
     F.tmem_cols = (int)pow2_cols(std::max(std::max((uint32_t)F.d2_col + nh32, n_last), (uint32_t)F.n_prior));
   } else {
     // several tiles: two slots; with more than two tiles the per-tap partials need columns of their own, because
     // a slot's next tile starts before its shifted sum
     const bool apart = 2 * nh + 2 * n_last <= 512u && nh + nh32 <= 512u;
+    if (direct == kFlowRows && !apart && F.tiles > 2) return false;
     if (!apart && (F.tiles > 2 || std::max(nh32, n_last) > 256u)) return false;
     F.d_col = apart ? (int)nh : 256;
     F.d3_col = apart ? 2 * (int)nh : 0;
@@ -994,7 +996,8 @@ bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool
     F.copies = form < 2 ? most_copies : 1;
     if (alias && (F.tiles > 2 || wide)) continue;
     if (form >= 2 && most_copies == 1) continue;
-    const uint32_t w_last = nd.w[direct ? 3 : 2];
+    // (kFlowRows: N is rounded up to sixteen, the last matrix read that far)
+    const uint32_t w_last = nd.w[direct ? 3 : 2] + (direct == kFlowRows ? 128u : 0u);
     uint32_t off = 0;
     auto take = [&](uint32_t bytes) { const uint32_t o = off; off = up(off + bytes, kAlign); return o; };
     F.alias = alias;
@@ -1307,8 +1310,8 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   auto plan = [&](FlowPlan& f, int group) {
     if ((uint64_t)group * f.c * f.fpx * ((uint64_t)f.c * f.fpx) >= (1ull << 32)) return false;      // (the index maps' divisions)
     for (int wide = nd.n_hidden > kFlowMaxResident; wide < 2; ++wide)
-      for (int direct = flow_direct(f, nd.n_hidden) && !wide; direct >= 0; --direct)
-        if (plan_flow(f, nd, smem_limit, group, wide != 0, direct != 0)) return true;
+      for (int direct = flow_direct(f, nd.n_hidden) && !wide ? kFlowRows : 0; direct >= 0; --direct)
+        if (plan_flow(f, nd, smem_limit, group, wide != 0, direct)) return true;
     return false;
   };
   const FlowPlan whole = F0;

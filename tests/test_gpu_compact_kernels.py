@@ -38,6 +38,21 @@ def test_last_conv_on_8x8_frames(G, splits, hidden, batch, sample, plan):
 
 
 @pytest.mark.parametrize("in_c,hidden,batch,plan,sample", [
+    (1, 16, 2, 0, None),                  # two translated channels: three products of eight columns, N rounded up
+    (10, 129, 2, 0, None),                # twenty: 72 columns of 80; five blocks, the last conv starts after four
+    (20, 129, 1, 0, None),                # forty in 48
+    (28, 160, 1, 0, None),                # 56: wider than the hidden layer's columns, the last conv waits for all blocks
+    (12, 192, 2, 1, None),                # two images whose accumulators do not fit side by side
+    (12, 130, 2, 1, None),                # ... that do
+    (12, 192, 600, 0, [0, 3, 596, 599]),  # four and more to a CTA: an MMA per tap
+])
+def test_last_conv_by_rows_of_taps(G, in_c, hidden, batch, plan, sample):
+    model = S.make_model(0xFC00 + in_c + hidden, in_c, 16, 16, [False], 3, hidden)
+    x = np.random.default_rng(in_c).integers(0, 256, (batch, in_c, 16, 16), dtype=np.uint8)
+    _check_both_ways(G, model, x, sample=sample, plan=plan)
+
+
+@pytest.mark.parametrize("in_c,hidden,batch,plan,sample", [
     (2, 16, 1, 0, None),                  # one image in four lane quarters, a block for one of sixteen warps
     (6, 256, 1, 0, None),                 # nine blocks
     (24, 176, 3, 0, None),                # 96 channels: the first and the last matrix share a slot
