@@ -766,7 +766,7 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
     // more to the exchange of edges than it gains: 0.52 against 0.47 ms)
     R.bh = R.bw = 16; R.m = 128;
     const int split = (R.w / 8) * (R.h / 16);
-    if (!throughput && R.w * R.h > 256 && split <= 8 && (int)max_batch <= max_res_flow_clusters(split, smem_limit)) R.bw = 8;
+    if (!throughput && split <= 8 && (int)max_batch <= max_res_flow_clusters(split, smem_limit)) R.bw = 8;
     R.tiles = R.bw / 8;
   } else if (R.w == 8 && R.h == 8) {
     R.bw = R.bh = 8; R.m = 64; R.tiles = 1;
