@@ -1982,7 +1982,8 @@ namespace {
 // Decoder's first look-up: the symbols k whose range [Cum(k), Cum(k + 1)) meets slots 256 b .. 256 b + 255, as {first,
 // count << 16}, for every scale index: at most 257 of the 4 097 (a symbol has at least one slot).
 std::vector<uint32_t> decoder_ranges(const iodf_codec_desc& desc) {
-  std::vector<uint32_t> ranges((size_t)desc.n_scales * 256);
+  std::vector<uint32_t> ranges((size_t)desc.n_scales * (256 + 64));
+  uint32_t* coarse = ranges.data() + (size_t)desc.n_scales * 256;
   std::vector<uint32_t> cum(2 * 2048 + 2);
   for (uint32_t ls = 0; ls < desc.n_scales; ++ls) {
     cum[0] = 0;
@@ -1992,6 +1993,7 @@ std::vector<uint32_t> decoder_ranges(const iodf_codec_desc& desc) {
       cum[k] = (uint32_t)k + desc.sigmoid_table[u + desc.umax];
     }
     cum[2 * 2048 + 1] = 1u << 16;
+    for (uint32_t i = 0; i < 64; ++i) coarse[(size_t)ls * 64 + i] = cum[64 * i + 32] | cum[64 * i + 64] << 16;
     int k = 0;
     for (uint32_t b = 0; b < 256; ++b) {
       while (k < 2 * 2048 && cum[k + 1] <= 256 * b) ++k;
@@ -2090,6 +2092,7 @@ int iodf_codec_create(const iodf_model* m, const iodf_codec_desc* desc, iodf_cod
   a.G = reinterpret_cast<const uint16_t*>(c->d_tables + rbytes);
   a.errors = c->d_errors;
   a.ranges = c->d_ranges;
+  a.coarse = c->d_ranges + (size_t)desc->n_scales * 256;
   *out = c;
   return IODF_OK;
 }

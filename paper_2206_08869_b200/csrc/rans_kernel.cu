@@ -29,10 +29,11 @@ constexpr int kEncodeStreams = 128, kEncodeThreads = 3 * kEncodeStreams, kBatch 
 __host__ __device__ inline size_t encode_buffers_at(const RansArgs& a) {       // offset in the encoder's shared memory, after the tables
   return (4 * (size_t)a.n_scales + 2 * (size_t)(2 * a.umax + 1) + 15) / 16 * 16;
 }
-// More streams of a block than this per SM: half a warp each. A warp per stream is then six warps and more per scheduler, and issue slots
-// bound it. Whole warps and halves measured at 148 SMs: 3 072 streams 69 and 73 us, 3 600 75 and 75 (55 and 44 without prior
-// parameters), 6 144 111 and 88, 7 200 122 and 103.
-constexpr long kHalfWarpStreamsPerSm = 24;
+// More streams of a block with prior parameters than this per SM: half a warp each. A warp per stream is then ten warps and more per
+// scheduler, and issue slots bound it. Whole warps and halves measured at 148 SMs, streams of 128: 1 536 39 and 66 us, 3 072 56 and 70,
+// 4 800 78 and 80, 6 144 93 and 89, 7 200 105 and 103, 28 800 354 and 304. Blocks without prior parameters have one scale, whose look-up
+// table stays in the L1 cache, and always take halves: 192 and 768 streams 35 either way, 2 400 47 and 39, 3 600 64 and 43.
+constexpr long kHalfWarpStreamsPerSm = 40;
 
 struct Tables {
   const uint16_t* G;       // shared memory
@@ -49,6 +50,13 @@ __device__ __forceinline__ uint32_t cum_of(const Tables& t, uint32_t R, int k) {
   int u = edge2 * (int)(R >> 16) + ((edge2 * (int)(R & 0xFFFFu)) >> 16);      // arithmetic shift: floor
   u = max(-t.umax, min(t.umax, u));
   return (uint32_t)k + t.G[u + t.umax];
+}
+
+// The same for 0 < k < 4097 (any value otherwise), one wide multiplication and a shift: fewer instructions in a row, 37 -> 35 us for a
+// chain of 128; but where issue slots count the pieces are cheaper (encoder 29 against 33 us).
+__device__ __forceinline__ uint32_t inner_cum_of(const Tables& t, uint32_t R, int k) {
+  const int u = (int)(((long long)(2 * (k - kWin) - 1) * (long long)(int)R) >> 16);       // (fits: above)
+  return (uint32_t)k + t.G[max(-t.umax, min(t.umax, u)) + t.umax];
 }
 
 // x / F and x mod F for 0 < F <= 2^16 and x < F 2^16, inv = 1 / F rounded: the quotient is below 2^16, so that x * inv
@@ -209,18 +217,17 @@ __global__ void __launch_bounds__(kEncodeThreads) rans_encode_kernel(const RansA
 // Decode: one WARP per stream. The state, the word pointer and every step are the same in all 32
 // lanes; what the lanes share out is everything that would otherwise be a dependent trip to memory
 // or a dependent search step on the stream's serial chain (state -> symbol -> state):
-//   * the symbol search: the slot's upper eight bits select, for the element's scale, the symbols that it can
-//     mean (a table made with the codec: first and count, usually a handful, 257 at most); lane L tests one
-//     candidate and a ballot picks the largest k with Cum(k) <= slot, after a round in steps of up to nine where there
-//     are more than 32. The last round's values also give C = Cum(k) and Cum(k + 1) by shuffle. (Three rounds
-//     over all 4 097 symbols before.)
+//   * the symbol search: the lanes hold Cum(32), Cum(64), .. Cum(4096) of the element's scale, four each, from a table made with the
+//     codec; they do not depend on the state and are asked for a symbol ahead. Four ballots select 32 symbols; lane L tests one
+//     and a ballot picks the largest k with Cum(k) <= slot. The same values give C = Cum(k) and Cum(k + 1) by shuffle;
 //   * the prior parameters: the (mu, scale index) of the next 32 elements are loaded by the 32 lanes
-//     in one go and handed out by shuffle, so no global-memory latency sits between two symbols;
+//     in one go, a round ahead, and handed out by shuffle, so no global-memory latency sits between two symbols;
 //   * the coded words: the lanes hold a window of the stream's next 32 words (the decoder reads the
-//     stream backwards); the three words that a symbol can take are handed out before its search.
-// What bounds it depends on the block (128 images of 64 x 64, 128 elements per stream). The small ones are a stream's chain:
-// 35 us for the final block, 540 clocks per symbol, 50 us for those with prior parameters (60 - 70 with three search
-// rounds). Blocks of more than kHalfWarpStreamsPerSm streams per SM go to the kernel below.
+//     stream backwards).
+// What bounds it is a stream's chain, the instructions of a warp that has its scheduler nearly to itself: 35 - 37 us for 768 - 1 536
+// streams of 128, 530 clocks per symbol. So the symbols that need more code (escapes, the last of a group of 32) take a branch of
+// their own: 47 us with that code in line. With the first look-up in a table of 256 slot ranges per scale, as in the kernel below,
+// it was 50: 64 KB of ranges do not stay in the L1 cache, and the load was on the chain.
 __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const RansArgs a, int q,
                                                                        const uint16_t* __restrict__ words,
                                                                        const uint32_t* __restrict__ counts,
@@ -249,12 +256,18 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const Ran
   used = 2;
   int32_t* zb = z + (long)b * a.d + blk.z_off + j;
   const int32_t* pb = prior + (long)b * 2 * a.d_fact;
+  // this lane's element of the next 32: its prior parameters, a round ahead
+  int32_t mu_n = 0;
+  int ls_n = a.final_ls;
+  if (lane < n_el) prior_of(a, blk, pb, j + (long)lane * ns, &mu_n, &ls_n, &bad);
+  const uint2* coarse = reinterpret_cast<const uint2*>(a.coarse) + lane;
+  uint2 next = __ldg(coarse + (__shfl_sync(0xFFFFFFFFu, ls_n, 0) << 5));
   for (int i0 = 0; i0 < n_el; i0 += 32) {
-    // this lane's element of the next 32: its prior parameters now, its decoded value at the end
-    int32_t mu_l = 0, zv_l = 0;
-    int ls_l = a.final_ls;
-    if (i0 + lane < n_el) prior_of(a, blk, pb, j + (long)(i0 + lane) * ns, &mu_l, &ls_l, &bad);
+    const int32_t mu_l = mu_n;
+    const int ls_l = ls_n;
     const uint32_t R_l = t.R[ls_l];
+    if (i0 + 32 + lane < n_el) prior_of(a, blk, pb, j + (long)(i0 + 32 + lane) * ns, &mu_n, &ls_n, &bad);
+    int32_t zv_l = 0;
     const int n_here = min(32, n_el - i0);
     for (int ii = 0; ii < n_here; ++ii) {
       if (used > 29) {                             // (a symbol takes up to three words)
@@ -263,36 +276,43 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const Ran
         win = fill();
       }
       // what does not depend on the state is on its way during the search
-      const uint32_t w0 = __shfl_sync(0xFFFFFFFFu, win, used), w1 = __shfl_sync(0xFFFFFFFFu, win, used + 1);
-      const uint32_t w2 = __shfl_sync(0xFFFFFFFFu, win, used + 2);
-      const int ls = __shfl_sync(0xFFFFFFFFu, ls_l, ii);
-      const uint32_t R = __shfl_sync(0xFFFFFFFFu, R_l, ii);
-      const uint32_t slot = x & 0xFFFFu;
-      // largest k with Cum(k) <= slot, among the symbols that the slot can mean
-      const uint32_t range = __ldg(a.ranges + (ls << 8) + (slot >> 8));
-      int k = (int)(range & 0xFFFFu);
-      const int count = (int)(range >> 16);
-      if (count > 31) {                            // (at most nine are left then)
-        const int step = (count + 31) >> 5;
-        const unsigned ok = __ballot_sync(0xFFFFFFFFu, cum_of(t, R, k + lane * step) <= slot);   // a prefix of the lanes (Cum is monotone)
-        k += (31 - __clz((int)ok)) * step;
-      }
-      const uint32_t cl = cum_of(t, R, k + lane);
-      const int sel = 31 - __clz((int)__ballot_sync(0xFFFFFFFFu, cl <= slot));       // at most 30
-      const uint32_t C = __shfl_sync(0xFFFFFFFFu, cl, sel), Cn = __shfl_sync(0xFFFFFFFFu, cl, sel + 1);
-      k += sel;
-      x = (Cn - C) * (x >> 16) + slot - C;
-      const bool more = x < (1u << 16);
-      if (more) x = (x << 16) | w0;
-      used += more ? 1 : 0;
-      int32_t zv = (int32_t)((uint32_t)mu_l + (uint32_t)(k - kWin));              // (lane ii's is the one that counts)
-      if (k == 0 || k == 2 * kWin) {
-        // an escape: two symbols of frequency 1, the value's upper and lower half; each takes the state's lower 16 bits and
-        // a word in their place (x >> 16 is always below 2^16)
-        const uint32_t wa = more ? w1 : w0, wb = more ? w2 : w1;
-        zv = (int32_t)((x << 16) | wa);
-        x = (x & 0xFFFF0000u) | wb;
-        used += 2;
+      const uint2 edge = next;
+      next = __ldg(coarse + (__shfl_sync(0xFFFFFFFFu, ii == 31 ? ls_n : ls_l, ii + 1) << 5));
+      const uint32_t w0 = __shfl_sync(0xFFFFFFFFu, win, used), R = __shfl_sync(0xFFFFFFFFu, R_l, ii);
+      const uint32_t slot = x & 0xFFFFu, high = x >> 16;
+      // largest k with Cum(k) <= slot: how many of Cum(32), Cum(64), .. Cum(4096) are not above the slot (a prefix: Cum is monotone),
+      // then the lanes' 32 symbols from there on
+      const int k0 = 32 * (__popc(__ballot_sync(0xFFFFFFFFu, (edge.x & 0xFFFFu) <= slot)) + __popc(__ballot_sync(0xFFFFFFFFu, (edge.x >> 16) <= slot)) +
+                           __popc(__ballot_sync(0xFFFFFFFFu, (edge.y & 0xFFFFu) <= slot)) + __popc(__ballot_sync(0xFFFFFFFFu, (edge.y >> 16) <= slot)));
+      const uint32_t c = inner_cum_of(t, R, k0 + lane);
+      const int sel = 31 - __clz((int)__ballot_sync(0xFFFFFFFFu, c <= slot));
+      const uint32_t C = __shfl_sync(0xFFFFFFFFu, c, sel), Cn = __shfl_sync(0xFFFFFFFFu, c, sel + 1);
+      int32_t zv;
+      if (k0 > 0 && k0 < 2 * kWin && sel < 31) {
+        x = (Cn - C) * high + slot - C;
+        zv = (int32_t)((uint32_t)mu_l + (uint32_t)(k0 + sel - kWin));             // (lane ii's is the one that counts)
+        if (x < (1u << 16)) {
+          x = (x << 16) | w0;
+          ++used;
+        }
+      } else {
+        // the first and the last symbols, and a group's last one, whose upper end is another group's
+        const uint32_t w1 = __shfl_sync(0xFFFFFFFFu, win, used + 1), w2 = __shfl_sync(0xFFFFFFFFu, win, used + 2);
+        const int k = k0 + 31 - __clz((int)__ballot_sync(0xFFFFFFFFu, cum_of(t, R, k0 + lane) <= slot));
+        const uint32_t Ck = cum_of(t, R, k);
+        x = (cum_of(t, R, k + 1) - Ck) * high + slot - Ck;
+        const bool more = x < (1u << 16);
+        if (more) x = (x << 16) | w0;
+        used += more ? 1 : 0;
+        zv = (int32_t)((uint32_t)mu_l + (uint32_t)(k - kWin));
+        if (k == 0 || k == 2 * kWin) {
+          // an escape: two symbols of frequency 1, the value's upper and lower half; each takes the state's lower 16 bits and
+          // a word in their place (x >> 16 is always below 2^16)
+          const uint32_t wa = more ? w1 : w0, wb = more ? w2 : w1;
+          zv = (int32_t)((x << 16) | wa);
+          x = (x & 0xFFFF0000u) | wb;
+          used += 2;
+        }
       }
       if (lane == ii) zv_l = zv;
     }
@@ -303,13 +323,14 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const Ran
   if (bad && lane == 0 && a.errors) atomicAdd(a.errors, 1u);
 }
 
-// The same with HALF a warp per stream, for blocks of so many streams that issue slots bound the time (6 144 streams: ten warps
-// per scheduler, 0.72 of the slots used) and not a stream's chain, which is longer with fewer lanes: more symbols need a
-// first round. A warp's two streams go side by side, so steps that only some symbols take (escapes, a word more)
+// The same with HALF a warp per stream, for blocks of so many streams that issue slots bound the time and not a stream's chain, which
+// is longer here, and for those without prior parameters. The slot's upper eight bits select, for the element's scale, the symbols
+// that it can mean (a table made with the codec: first and count, usually a handful, 257 at most); a lane tests one candidate,
+// after a round in steps where there are more than fifteen. A warp's two streams go side by side, so steps that only some symbols take (escapes, a word more)
 // are selections, not branches. Words: the lanes hold the next 16, replaced lane by lane every four symbols from the ones after
 // them, which were asked for four symbols earlier; prior parameters are loaded 16 symbols ahead.
-// 128 elements per stream: 6 144 streams 111 -> 88 us, 28 800 412 -> 305. (No gain in either kernel: the first look-up in shared
-// memory, 34 clocks instead of 106 but 33 KB to load per CTA; warp reductions instead of ballot and shuffles.)
+// 128 elements per stream: 6 144 streams 88 us, 28 800 305. (No gain: the first look-up in shared memory, 34 clocks instead of 106 but
+// 33 KB to load per CTA; warp reductions instead of ballot and shuffles; the wide multiplication of inner_cum_of.)
 __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_half_kernel(const RansArgs a, int q,
                                                                        const uint16_t* __restrict__ words,
                                                                        const uint32_t* __restrict__ counts,
@@ -544,7 +565,7 @@ cudaError_t launch_rans_encode(const RansArgs& a, const int32_t* z, const int32_
 cudaError_t launch_rans_decode(const RansArgs& a, int block, const uint16_t* words, const uint32_t* counts,
                                const int32_t* prior, int32_t* z, cudaStream_t stream) {
   const long streams = (long)a.batch * a.blocks[block].n_streams;
-  const bool half = streams > kHalfWarpStreamsPerSm * a.n_sms;
+  const bool half = a.blocks[block].prior_off < 0 || streams > kHalfWarpStreamsPerSm * a.n_sms;
   const long total = streams * (half ? 16 : 32);
   const unsigned grid = (unsigned)((total + kThreadsPerBlock - 1) / kThreadsPerBlock);
   if (half) rans_decode_half_kernel<<<grid, kThreadsPerBlock, table_smem(a), stream>>>(a, block, words, counts, prior, z);

@@ -20,6 +20,7 @@ struct RansArgs {
   const uint16_t* G;       // device: sigmoid table, 2 * umax + 1 entries
   const uint32_t* R;       // device: reciprocal scales, n_scales entries
   const uint32_t* ranges;  // device: [n_scales][256] symbols that slots 256 b .. 256 b + 255 can mean: first | count << 16
+  const uint32_t* coarse;  // device: [n_scales][64] Cum(32), Cum(64), .. Cum(4096), two to a word
   int umax, n_scales, final_ls;
   int n_blocks, n_streams; // per image
   int cap;                 // words per stream in the container (3 * elems_per_stream + 2)

@@ -165,8 +165,8 @@ def test_residual_blocks_through_long_chains(G, hidden, batch, plan):
     G.iodf_check(m)
 
 
-@pytest.mark.parametrize("per_sm,elems", [(0, 97), (24, 103), (25, 103)])      # most streams per SM: a warp each, the last of
-@pytest.mark.parametrize("ls", [0, 20, 40, 63])                                # those, half of one
+@pytest.mark.parametrize("per_sm,elems", [(0, 97), (24, 103), (25, 103), (40, 31), (41, 33)])   # streams per SM: up to 40 a warp each,
+@pytest.mark.parametrize("ls", [0, 20, 40, 63])                                                 # then half of one
 def test_symbol_look_up_at_every_kind_of_scale(G, ls, per_sm, elems):
     """Residuals over the whole window at one scale: slots that mean one symbol and slots that mean hundreds."""
     import torch
