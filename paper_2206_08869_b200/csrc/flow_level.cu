@@ -998,125 +998,6 @@ __device__ __forceinline__ void flow_requant(const Flow& f, const FlowPlan& P, c
   }
 }
 
-template <bool kInv, bool kSplit, int kShape>
-__device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st, int img0) {
-  FlowCtl* ctl = f.ctl;
-  uint8_t* smem = f.smem;
-  int32_t* v = reinterpret_cast<int32_t*>(smem + P.s_v);
-  int32_t* acc = reinterpret_cast<int32_t*>(smem + P.s_acc);
-  const uint32_t lane_field = (uint32_t)((f.warp & 3) * 32) << 16;
-  // (4 x 4 levels: a lane quarter is an image, or a copy of one; quarters without one only take part in the hand-overs)
-  PixelMap pm;
-  const int pairs = P.pg >> 1;
-  pm.parts = kFlowWorkers / pairs;
-  pm.j = f.tid / pairs;
-  pm.p = 2 * (f.tid - pm.j * pairs);
-  int copy = 0;                                 // (4 x 4: threads of their own for each copy of the operand)
-  if (kShape == kImages4x4) {
-    pm.parts /= P.copies;
-    copy = pm.j / pm.parts;
-    pm.j -= copy * pm.parts;
-    if (copy >= P.copies) pm.j = 1 << 20;
-  }
-  if (pm.j >= pm.parts || pm.p >= f.pvalid) pm.j = 1 << 20;      // no work
-  {
-    const int img = fdiv(pm.p, P.mul_px), px = pm.p - img * P.px, r = fdiv(px, P.mul_w), c = px - r * P.w;
-    pm.v = v + pm.p;
-    pm.acc = acc + pm.p;
-    pm.rec = smem + P.s_xa + 16 * (P.im2col ? (img * P.copies + copy) * 16 + px : img * P.frame + (r + 1) * P.wp + c + 1);
-    pm.dy = r == 0 ? -1 : (r == P.h - 1 ? 1 : 0);
-    pm.dx = c == 0 ? -1 : (c == P.w - 2 ? 1 : 0);
-    pm.taps = 0;
-    for (int t = 0; t < 9; ++t) {
-      const int oi = r - (t / 3 - 1), oj = c - (t % 3 - 1);
-      if ((uint32_t)oi < (uint32_t)P.h && (uint32_t)oj < (uint32_t)P.w) pm.taps |= 1u << t;
-      if ((uint32_t)oi < (uint32_t)P.h && (uint32_t)(oj + 1) < (uint32_t)P.w) pm.taps |= 1u << (16 + t);
-    }
-  }
-  const uint32_t dm = f.tmem + (uint32_t)(f.sl * P.d_col) + lane_field, d3 = f.tmem + (uint32_t)(P.d3_col + f.sl * P.d3_step) + lane_field;
-  uint32_t dpar = 0u, tpar = 0u, npar = 0u;
-  const uint8_t* prev = nullptr;                // coupling whose translation is still to be applied
-#pragma unroll 1
-  for (int i = 0; i <= st.nsteps; ++i) {
-    if (kShape != kImages4x4 && prev && !(kShape == kRows64 && P.direct)) {
-      flow_translate<kInv>(P, pm, prev);
-      // the network input may read channels that were just updated; what was cleared is released as a whole
-      if (kSplit || pm.parts > 1) worker_barrier();
-    }
-    if (i == st.nsteps) break;
-    flow_wait(f, &ctl->meta_full[i & 1], (uint32_t)(i >> 1) & 1u);
-    const uint8_t* mb = smem + P.s_meta[i & 1];
-    const bool prior = st.is_prior(i);
-    const FlowMeta* M = reinterpret_cast<const FlowMeta*>(mb);
-    // (the first two words of both kinds of meta block)
-    uint64_t* input = &ctl->xa_ready[i & 1];
-    if (kSplit && f.warp == kFlowWarps - 1) flow_release_to_neighbours(P, f, input);
-    flow_requant<kSplit, kShape>(f, P, pm, input, prior ? a.plan->col_out : reinterpret_cast<const int32_t*>(mb + M->off_colA), M->in_m0, M->in_s);
-    flow_hand_over(f, input, kSplit && f.warp == 0 ? f.halo : 0u);
-    prev = prior ? nullptr : mb;
-    if (prior) {
-      flow_wait(f, &ctl->dm_ready[f.sl], dpar);
-      dpar ^= 1u;
-      ptx::tc_fence_after();
-      flow_prior<kSplit, kShape>(f, P, a, reinterpret_cast<const PriorMeta*>(mb), img0);
-    } else {
-#pragma unroll 1
-      for (int t = f.sl; t < f.tiles; t += f.slots) {
-        const bool quarter = kShape != kImages4x4 || 4 * t + f.image < f.nimg;
-#pragma unroll 1
-        for (int layer = 0; layer < 2; ++layer) {
-          const bool chunked = kShape != kRows128 && (layer ? P.chunk3 : P.chunk2);
-          const uint32_t d = kShape != kRows128 && layer ? dm + (uint32_t)P.d2_col : dm;
-          const int q = f.lane & 3, row = f.lane >> 2;
-          HiddenOut ho;
-          if (kShape == kRows64 && layer && P.direct) {
-            ho.at = smem + P.s_h[f.sl] + ((q >> 1) * P.frame + ((f.warp & 3) * 2 + 1) * P.wp + 1 + row) * 16 + (q & 1) * 8;
-            ho.block = 32 * P.frame;
-            ho.row = 16 * P.wp;
-          } else {
-            const int first = kShape == kImages4x4 ? f.image * P.copies * 16 : (f.warp & 3) * (kShape == kRows128 ? 32 : 16);
-            ho.at = smem + P.s_a[f.sl] + (q >> 1) * P.pitch + (first + row) * 16 + (q & 1) * 8;
-            ho.block = 2 * P.pitch;
-            ho.row = 128;
-          }
-          if (quarter) {
-            flow_hidden<kShape>(f, P, d, mb, layer, ho, chunked, &ctl->dm_ready[f.sl], dpar);
-          } else {
-            flow_wait(f, &ctl->dm_ready[f.sl], dpar);      // (never a phase ahead in its arrivals)
-            const int ks = layer ? M->ks3 : M->ks2;
-            for (int b0 = 0, r = 0; b0 < (chunked ? ks : 1); b0 += f.ncs, ++r) flow_hand_over(f, &ctl->a_ready[f.sl][r]);
-          }
-          dpar ^= 1u;
-        }
-        if (kShape == kRows64 && P.direct) {
-          flow_out<kInv>(f, P, t, d3, mb, v, &ctl->d3_ready[f.sl], tpar);
-        } else if constexpr (kShape == kImages4x4) {
-          if (quarter) flow_sum_4x4<kInv>(f, P, t, d3, mb, v, &ctl->d3_ready[f.sl], tpar);
-        } else {
-          flow_sum<kShape == kRows128 ? 4 : 2, kSplit>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
-        }
-        tpar ^= 1u;
-        // (streamed weights: the next tile's first GEMM writes where the partials were)
-        if (P.ring && t + 1 < f.tiles) flow_hand_over(f, &ctl->a_ready[0][0]);
-      }
-    }
-    ptx::tc_fence_before();
-    if (kSplit && !prior && f.tid == 0) ptx::mbar_expect_tx(ptx::smem_u32(&ctl->acc_full), (uint32_t)(P.reds[f.rank] * P.cb * 4));
-    worker_barrier();                           // every product has been added
-    if constexpr (kSplit) {
-      if (!prior) {
-        flow_wait_cluster(f, &ctl->acc_full, npar);
-        npar ^= 1u;
-      } else if (i + 1 < st.nsteps) {
-        // The next step's edge pixels overwrite what the neighbours' prior heads read. (After a coupling their products
-        // say that they are past it.)
-        if (f.warp == 0) flow_release_to_neighbours(P, f, &ctl->peers_done);
-        flow_wait_cluster(f, &ctl->peers_done, 0u);
-      }
-    }
-  }
-}
-
 // ---- a level's input and output index maps (four neighbouring elements per thread and step) ----------------
 __device__ __forceinline__ size_t patch_index(const FlowPlan& P, const LevelArgs& a, int b, int ci, int y, int x) {
   const int by = fdiv(b, a.mul_patches_x), bx = b - by * a.patches_x;
@@ -1215,6 +1096,132 @@ __device__ __forceinline__ void flow_store(const Flow& f, const FlowPlan& P, con
     if (P.is_first && a.oor != nullptr) {
       bad = __reduce_add_sync(0xFFFFFFFFu, bad);
       if (f.lane == 0 && bad) atomicAdd(a.oor, bad);
+    }
+  }
+}
+
+template <bool kInv, bool kSplit, int kShape>
+__device__ void flow_workers(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st, int img0) {
+  FlowCtl* ctl = f.ctl;
+  uint8_t* smem = f.smem;
+  int32_t* v = reinterpret_cast<int32_t*>(smem + P.s_v);
+  int32_t* acc = reinterpret_cast<int32_t*>(smem + P.s_acc);
+  const uint32_t lane_field = (uint32_t)((f.warp & 3) * 32) << 16;
+  // (4 x 4 levels: a lane quarter is an image, or a copy of one; quarters without one only take part in the hand-overs)
+  PixelMap pm;
+  const int pairs = P.pg >> 1;
+  pm.parts = kFlowWorkers / pairs;
+  pm.j = f.tid / pairs;
+  pm.p = 2 * (f.tid - pm.j * pairs);
+  int copy = 0;                                 // (4 x 4: threads of their own for each copy of the operand)
+  if (kShape == kImages4x4) {
+    pm.parts /= P.copies;
+    copy = pm.j / pm.parts;
+    pm.j -= copy * pm.parts;
+    if (copy >= P.copies) pm.j = 1 << 20;
+  }
+  if (pm.j >= pm.parts || pm.p >= f.pvalid) pm.j = 1 << 20;      // no work
+  {
+    const int img = fdiv(pm.p, P.mul_px), px = pm.p - img * P.px, r = fdiv(px, P.mul_w), c = px - r * P.w;
+    pm.v = v + pm.p;
+    pm.acc = acc + pm.p;
+    pm.rec = smem + P.s_xa + 16 * (P.im2col ? (img * P.copies + copy) * 16 + px : img * P.frame + (r + 1) * P.wp + c + 1);
+    pm.dy = r == 0 ? -1 : (r == P.h - 1 ? 1 : 0);
+    pm.dx = c == 0 ? -1 : (c == P.w - 2 ? 1 : 0);
+    pm.taps = 0;
+    for (int t = 0; t < 9; ++t) {
+      const int oi = r - (t / 3 - 1), oj = c - (t % 3 - 1);
+      if ((uint32_t)oi < (uint32_t)P.h && (uint32_t)oj < (uint32_t)P.w) pm.taps |= 1u << t;
+      if ((uint32_t)oi < (uint32_t)P.h && (uint32_t)(oj + 1) < (uint32_t)P.w) pm.taps |= 1u << (16 + t);
+    }
+  }
+  const uint32_t dm = f.tmem + (uint32_t)(f.sl * P.d_col) + lane_field, d3 = f.tmem + (uint32_t)(P.d3_col + f.sl * P.d3_step) + lane_field;
+  uint32_t dpar = 0u, tpar = 0u, npar = 0u;
+  const uint8_t* prev = nullptr;                // coupling whose translation is still to be applied
+#pragma unroll 1
+  for (int i = 0; i <= st.nsteps; ++i) {
+    if (kShape != kImages4x4 && prev && !(kShape == kRows64 && P.direct)) {
+      flow_translate<kInv>(P, pm, prev);
+      // the network input may read channels that were just updated; what was cleared is released as a whole
+      if (kSplit || pm.parts > 1) worker_barrier();
+    }
+    const uint8_t* mb = smem + P.s_meta[i & 1];
+    const FlowMeta* M = reinterpret_cast<const FlowMeta*>(mb);
+    const bool prior = i < st.nsteps && st.is_prior(i);
+    if (i < st.nsteps) {
+    flow_wait(f, &ctl->meta_full[i & 1], (uint32_t)(i >> 1) & 1u);
+    // (the first two words of both kinds of meta block)
+    uint64_t* input = &ctl->xa_ready[i & 1];
+    if (kSplit && f.warp == kFlowWarps - 1) flow_release_to_neighbours(P, f, input);
+    flow_requant<kSplit, kShape>(f, P, pm, input, prior ? a.plan->col_out : reinterpret_cast<const int32_t*>(mb + M->off_colA), M->in_m0, M->in_s);
+    flow_hand_over(f, input, kSplit && f.warp == 0 ? f.halo : 0u);
+    prev = prior ? nullptr : mb;
+    }
+    // the flow variable is complete: it is stored, under the prior head's GEMM where that is the last step
+    if (i == (kInv ? st.nsteps : st.n_couplings)) {
+      worker_barrier();
+      flow_store<kInv, kSplit>(f, P, a, img0, v);
+    }
+    if (i == st.nsteps) break;
+    if (prior) {
+      flow_wait(f, &ctl->dm_ready[f.sl], dpar);
+      dpar ^= 1u;
+      ptx::tc_fence_after();
+      flow_prior<kSplit, kShape>(f, P, a, reinterpret_cast<const PriorMeta*>(mb), img0);
+    } else {
+#pragma unroll 1
+      for (int t = f.sl; t < f.tiles; t += f.slots) {
+        const bool quarter = kShape != kImages4x4 || 4 * t + f.image < f.nimg;
+#pragma unroll 1
+        for (int layer = 0; layer < 2; ++layer) {
+          const bool chunked = kShape != kRows128 && (layer ? P.chunk3 : P.chunk2);
+          const uint32_t d = kShape != kRows128 && layer ? dm + (uint32_t)P.d2_col : dm;
+          const int q = f.lane & 3, row = f.lane >> 2;
+          HiddenOut ho;
+          if (kShape == kRows64 && layer && P.direct) {
+            ho.at = smem + P.s_h[f.sl] + ((q >> 1) * P.frame + ((f.warp & 3) * 2 + 1) * P.wp + 1 + row) * 16 + (q & 1) * 8;
+            ho.block = 32 * P.frame;
+            ho.row = 16 * P.wp;
+          } else {
+            const int first = kShape == kImages4x4 ? f.image * P.copies * 16 : (f.warp & 3) * (kShape == kRows128 ? 32 : 16);
+            ho.at = smem + P.s_a[f.sl] + (q >> 1) * P.pitch + (first + row) * 16 + (q & 1) * 8;
+            ho.block = 2 * P.pitch;
+            ho.row = 128;
+          }
+          if (quarter) {
+            flow_hidden<kShape>(f, P, d, mb, layer, ho, chunked, &ctl->dm_ready[f.sl], dpar);
+          } else {
+            flow_wait(f, &ctl->dm_ready[f.sl], dpar);      // (never a phase ahead in its arrivals)
+            const int ks = layer ? M->ks3 : M->ks2;
+            for (int b0 = 0, r = 0; b0 < (chunked ? ks : 1); b0 += f.ncs, ++r) flow_hand_over(f, &ctl->a_ready[f.sl][r]);
+          }
+          dpar ^= 1u;
+        }
+        if (kShape == kRows64 && P.direct) {
+          flow_out<kInv>(f, P, t, d3, mb, v, &ctl->d3_ready[f.sl], tpar);
+        } else if constexpr (kShape == kImages4x4) {
+          if (quarter) flow_sum_4x4<kInv>(f, P, t, d3, mb, v, &ctl->d3_ready[f.sl], tpar);
+        } else {
+          flow_sum<kShape == kRows128 ? 4 : 2, kSplit>(f, P, t, d3, acc, &ctl->d3_ready[f.sl], tpar);
+        }
+        tpar ^= 1u;
+        // (streamed weights: the next tile's first GEMM writes where the partials were)
+        if (P.ring && t + 1 < f.tiles) flow_hand_over(f, &ctl->a_ready[0][0]);
+      }
+    }
+    ptx::tc_fence_before();
+    if (kSplit && !prior && f.tid == 0) ptx::mbar_expect_tx(ptx::smem_u32(&ctl->acc_full), (uint32_t)(P.reds[f.rank] * P.cb * 4));
+    worker_barrier();                           // every product has been added
+    if constexpr (kSplit) {
+      if (!prior) {
+        flow_wait_cluster(f, &ctl->acc_full, npar);
+        npar ^= 1u;
+      } else if (i + 1 < st.nsteps) {
+        // The next step's edge pixels overwrite what the neighbours' prior heads read. (After a coupling their products
+        // say that they are past it.)
+        if (f.warp == 0) flow_release_to_neighbours(P, f, &ctl->peers_done);
+        flow_wait_cluster(f, &ctl->peers_done, 0u);
+      }
     }
   }
 }
@@ -1323,8 +1330,6 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
     flow_load<kInv, kSplit>(f, P, a, img0, v);
     worker_barrier();
     flow_workers<kInv, kSplit, kShape>(f, P, a, st, img0);
-    worker_barrier();
-    flow_store<kInv, kSplit>(f, P, a, img0, v);
   }
   ptx::tc_fence_before();
   __syncthreads();
