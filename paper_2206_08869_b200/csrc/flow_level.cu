@@ -1299,16 +1299,10 @@ __global__ void __launch_bounds__(kFlowThreads, 1) flow_level_kernel(const Level
     const int lim = P.im2col ? 9 * P.ca : P.ca, unit = P.paired ? 8 : P.plane16 * 16;
     for (uint32_t o = 16 * tid; o < P.s_xa_end - P.s_xa; o += 16 * kFlowWorkers) {
       const int first = P.paired ? 0 : (int)(o / (uint32_t)unit) * 16;       // first byte of the 16-byte plane in a record
-      uint32_t wd[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        wd[k] = 0;
-        for (int e = 0; e < 4; ++e) {
-          const int byte = first + ((P.paired ? k & 1 : k) << 2) + e;
-          wd[k] |= (byte < lim ? 0u : (byte == lim ? 1u : 127u)) << (8 * e);
-        }
-      }
-      *reinterpret_cast<uint4*>(smem + P.s_xa + o) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+      // word of bytes b .. b + 3: zeros up to lim (an even number), then 1, 127, 127, ...
+      auto word = [&](int b) { return b + 4 <= lim ? 0u : (b > lim ? 0x7F7F7F7Fu : (b == lim ? 0x7F7F7F01u : 0x7F010000u)); };
+      const uint32_t w0 = word(first), w1 = word(first + 4), w2 = P.paired ? w0 : word(first + 8), w3 = P.paired ? w1 : word(first + 12);
+      *reinterpret_cast<uint4*>(smem + P.s_xa + o) = make_uint4(w0, w1, w2, w3);
     }
     if (tid < f.tiles) {
       int4 tp = make_int4(4 * tid, 0, 0, 64 * tid);                          // (im2col: first of four images)
