@@ -41,12 +41,12 @@
 //     translation, acquired by the neighbour's MMA warp, without whose MMAs there are no products. (Overwriting a
 //     frame needs no release: the MMAs that read it have completed before anything is sent that lets a neighbour go on.)
 //
-// What bounds it: the chain of a coupling (7 000 - 9 000 clocks where a CTA has one tile) and 3 300 clocks per tile of 128 pixels:
+// What bounds it: the chain of a coupling (7 000 - 9 000 clocks where a CTA has one tile) and 3 000 clocks per tile of 128 pixels:
 // requantisation, shifted sum and their hand-overs, at five to nine clocks an instruction and warp (50 % of all issue slots at
-// 32 x 32, 33 % at 8 x 8, 23 % at 4 x 4; of 32 x 32's 143 us the phases' skeleton of waits, hand-overs and MMAs takes half). Measured for eight
-// couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 143 us,
-// 16 x 16 85 -> 58, 8 x 8 63 -> 43, 4 x 4 70 -> 47; one image, 32 x 32 split in eight: 51. Width 512, 64 images of
-// 32 x 32, split in two: 2 357 -> 288 us, the tensor core busy a third of it.
+// 32 x 32, 33 % at 8 x 8, 23 % at 4 x 4; of 32 x 32's 130 us the phases' skeleton of waits, hand-overs and MMAs takes half). Measured for eight
+// couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 130 us,
+// 16 x 16 85 -> 53, 8 x 8 63 -> 37, 4 x 4 70 -> 45; one image, 32 x 32 split in eight: 48. Width 512, 64 images of
+// 32 x 32, split in two: 2 357 -> 286 us, the tensor core busy a third of it.
 #include <stddef.h>
 
 #include "flow_level.h"

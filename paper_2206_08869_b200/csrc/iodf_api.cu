@@ -761,9 +761,8 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
   R.d = (int64_t)P.d; R.d_fact = (int64_t)P.d_fact;
   R.group = 1;
   if (R.w % 16 == 0 && R.h % 16 == 0) {
-    // 16 x 16 blocks; images of several blocks in 8 x 16 ones while all clusters of a batch run at once (half the
-    // multiply time per conv: 0.53 against 0.68 ms for three 32 x 32 images; a 16 x 16 image cut in two loses
-    // more to the exchange of edges than it gains: 0.52 against 0.47 ms)
+    // 16 x 16 blocks, or 8 x 16 ones while all clusters of a batch run at once (half the multiply time per conv for an exchange of
+    // edges: 0.44 against 0.65 ms for three 32 x 32 images, 432 against 459 us for 64 of 16 x 16)
     R.bh = R.bw = 16; R.m = 128;
     const int split = (R.w / 8) * (R.h / 16);
     if (!throughput && split <= 8 && (int)max_batch <= max_res_flow_clusters(split, smem_limit)) R.bw = 8;
@@ -1325,7 +1324,8 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   // the rule says, of four 11 %, of five and more 1 %). Fitted to 564 shapes of 53 flows (widths 16 - 512, 2 - 56 translated
   // channels, 4 x 4 - 32 x 32, 2 - 12 couplings) at batches of 1 - 1 184: 5 % off on average. The shape it picks takes 0.09 % longer than
   // the best one on average and 12 % at most (a 4 x 4 level of two couplings, 20 us); for 253 shapes of 27 flows that had no
-  // part in it 0.12 % and 11 %. Constants fitted to five flows and used with twice the width that they were fitted with: 0.38 %
+  // part in it 0.12 % and 11 %. (Fitted before a slot's first GEMM went ahead of the other's and 8 x 8 convs went by rows of taps:
+  // shapes of two slots take 2 - 8 % less since, 8 x 8 ones 6 - 10 %.) Constants fitted to five flows and used with twice the width that they were fitted with: 0.38 %
   // and 25 %, 0.34 % and 12 %.
   auto add_shape = [&](const FlowPlan& f, int ctas) {
     const double width = widths / (400.0 * F.n_couplings), cb = f.cb / 10.0;        // mean of both layers, in 200 channels

@@ -24,9 +24,9 @@
 //     epilogue adds. One lane of another streams weights and the convs' meta blocks.
 //
 // What bounds it: a conv's chain of first chunk -> 36 MMAs (1 500 - 2 400 clocks) -> last chunk's epilogue -> hand-over,
-// 3 800 clocks at 8 x 8 and 4 x 4 images, 6 200 at 16 x 16, 145 convs one after another. Measured at width 128 with
-// eight blocks, eight couplings (res_level.cu before): 64 images of 16 x 16 1 610 -> 467 us, 8 x 8 750 -> 289,
-// 4 x 4 740 -> 293; 32 images of 32 x 32 1 750 -> 685.
+// 3 200 clocks at 8 x 8 and 4 x 4 images, 5 600 at 16 x 16 (in two blocks), 145 convs one after another. Measured at width 128 with
+// eight blocks, eight couplings (res_level.cu before): 64 images of 16 x 16 1 610 -> 410 us, 8 x 8 750 -> 233,
+// 4 x 4 740 -> 240; 32 images of 32 x 32 1 750 -> 635.
 #include "res_flow.h"
 #include "level_device.cuh"
 
@@ -200,10 +200,11 @@ __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq, int which)
 #pragma unroll 1
     for (int kc = 0; kc < nk; ++kc) {
       if (!one || (kc & 1) == which) {
-        rf_wait(f, &ctl->w_full[slot], round & 1u);
-        wait_chunk(kc);
+        // (all that the wait need not precede: an instruction of this warp takes about 13 clocks)
         uint32_t bl = addr16(P.s_ring + slot * P.slot_bytes) | b_lbo;
         const uint32_t a_bias = addr16(P.s_const + (uns ? 0u : 2304u)) | (8u << 16);
+        rf_wait(f, &ctl->w_full[slot], round & 1u);
+        wait_chunk(kc);
         if (ptx::elect_one()) {
           if (kc == 0) {                    // bias rows: the operand is the same constant row everywhere
             ptx::umma_i8_hl(d0, a_bias, ptx::kUmmaDescHi, bl, ptx::kUmmaDescHi, idesc, 0u);
@@ -241,24 +242,21 @@ struct RfPos {             // a thread's two positions of a tile half (rows of t
   int p0, p1;              // pixels of the CTA
 };
 
-// 8 (4) bytes of an activation in this CTA's frame and, where the pixel (i, j) of the block lies on an edge, in
-// the neighbours' frames
+// 8 (4) bytes of an activation, stored at `d` in this CTA's frame, into the neighbours' frames if the pixel (i, j) of the block lies on
+// an edge. (Apart from the store itself, so that whole images test once for neighbours: 64 images of 4 x 4 260 -> 254 us.)
 template <typename V>
-__device__ __forceinline__ void rf_store(const Rf& f, const RfPlan& P, uint8_t* d, const V v, int i, int j, uint64_t* bar) {
-  *reinterpret_cast<V*>(d) = v;
-  if (f.halo) {
-    const int dy = i == 0 ? -1 : (i == P.bh - 1 ? 1 : 0), dx = j == 0 ? -1 : (j == P.bw - 1 ? 1 : 0);
-    const bool ny = dy && (uint32_t)(f.by + dy) < (uint32_t)P.nby, nx = dx && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx;
-    const uint32_t s = ptx::smem_u32(d), b = ptx::smem_u32(bar);
-    auto put = [&](int oy, int ox) {
-      const uint32_t rank = (uint32_t)(f.rank + oy * P.nbx + ox), at = rf_peer(s - (uint32_t)((oy * P.bh * P.wp + ox * P.bw) * 16), rank);
-      if constexpr (sizeof(V) == 8) rf_store_async8(at, rf_peer(b, rank), v);
-      else rf_store_async4(at, rf_peer(b, rank), v);
-    };
-    if (ny) put(dy, 0);
-    if (nx) put(0, dx);
-    if (ny && nx) put(dy, dx);
-  }
+__device__ __forceinline__ void rf_send(const Rf& f, const RfPlan& P, uint8_t* d, const V v, int i, int j, uint64_t* bar) {
+  const int dy = i == 0 ? -1 : (i == P.bh - 1 ? 1 : 0), dx = j == 0 ? -1 : (j == P.bw - 1 ? 1 : 0);
+  const bool ny = dy && (uint32_t)(f.by + dy) < (uint32_t)P.nby, nx = dx && (uint32_t)(f.bx + dx) < (uint32_t)P.nbx;
+  const uint32_t s = ptx::smem_u32(d), b = ptx::smem_u32(bar);
+  auto put = [&](int oy, int ox) {
+    const uint32_t rank = (uint32_t)(f.rank + oy * P.nbx + ox), at = rf_peer(s - (uint32_t)((oy * P.bh * P.wp + ox * P.bw) * 16), rank);
+    if constexpr (sizeof(V) == 8) rf_store_async8(at, rf_peer(b, rank), v);
+    else rf_store_async4(at, rf_peer(b, rank), v);
+  };
+  if (ny) put(dy, 0);
+  if (nx) put(0, dx);
+  if (ny && nx) put(dy, dx);
 }
 
 // One unit: 16 rows (half `h` of this warp's lane quarter of tile `t`) x 32 columns (chunk b) of a hidden or branch conv.
@@ -337,8 +335,12 @@ __device__ __forceinline__ void rf_unit(const Rf& f, const RfPlan& P, const RfMe
   // ReLU and clip to 0..255 are the pack's saturation
   const uint2 v0 = make_uint2(pack4_sat_u8((int)r[0], (int)r[1], (int)r[4], (int)r[5]), pack4_sat_u8((int)r[8], (int)r[9], (int)r[12], (int)r[13]));
   const uint2 v1 = make_uint2(pack4_sat_u8((int)r[2], (int)r[3], (int)r[6], (int)r[7]), pack4_sat_u8((int)r[10], (int)r[11], (int)r[14], (int)r[15]));
-  if (ok0) rf_store(f, P, o, v0, g, j, chunk);
-  if (ok1) rf_store(f, P, o + row, v1, g + 1, j, chunk);
+  if (ok0) *reinterpret_cast<uint2*>(o) = v0;
+  if (ok1) *reinterpret_cast<uint2*>(o + row) = v1;
+  if (f.halo) {
+    rf_send(f, P, o, v0, g, j, chunk);
+    rf_send(f, P, o + row, v1, g + 1, j, chunk);
+  }
 }
 
 // thread's two pixels (of the CTA) for operand rows g, g + 1 of tile t; -1: none
@@ -416,7 +418,9 @@ __device__ __forceinline__ void rf_requant(const Rf& f, const RfPlan& P, const R
     }
     const int row = P.small ? (p >> 4) * 5 + ((p >> 2) & 3) : p / P.bw, j = P.small ? p & 3 : p - row * P.bw;
     uint8_t* d = f.smem + P.s_buf[M->src] + ((wd >> 2) * P.plane16 + (row + 1) * P.wp + 1 + j) * 16 + (wd & 3) * 4;
-    rf_store(f, P, d, pack4_sat(y[0], y[1], y[2], y[3]), row, j, &f.ctl->xa_ready);
+    const uint32_t word = pack4_sat(y[0], y[1], y[2], y[3]);
+    *reinterpret_cast<uint32_t*>(d) = word;
+    if (f.halo) rf_send(f, P, d, word, row, j, &f.ctl->xa_ready);
   }
 }
 
@@ -449,6 +453,11 @@ __device__ void rf_workers(const Rf& f, const RfPlan& P, const LevelArgs& a, con
         rf_wait(f, dr, dp);
         __syncwarp();
         if (f.lane == 0) rf_arrive_local(&ctl->chunk_ready[q & 1][0]);
+        // The next conv starts with chunk 0, so that chunk's warps go first: with all at once each takes longer and the MMAs wait
+        // (arrivals ahead of the wait, without the delay that this wait is: 64 images of 32 x 32 927 -> 970 us for the whole call; with
+        // the pauses 895 -> 870).
+        if (per == 2) __nanosleep(120);
+        else if (c0 >= 2) __nanosleep(c0 == 2 ? 200 : 300);
       }
 #pragma unroll 1
       for (int b = c0; b < nb; b += cstep) {
