@@ -1981,6 +1981,7 @@ int iodf_inverse_patches(iodf_model* m, const int32_t* z, int H, int W, uint8_t*
 namespace {
 // Decoder's first look-up: the symbols k whose range [Cum(k), Cum(k + 1)) meets slots 256 b .. 256 b + 255, as {first,
 // count << 16}, for every scale index: at most 257 of the 4 097 (a symbol has at least one slot).
+// Behind them, for every scale index: Cum(32), Cum(64), .. Cum(4096), two to a word (RansArgs::coarse).
 std::vector<uint32_t> decoder_ranges(const iodf_codec_desc& desc) {
   std::vector<uint32_t> ranges((size_t)desc.n_scales * (256 + 64));
   uint32_t* coarse = ranges.data() + (size_t)desc.n_scales * 256;
