@@ -39,7 +39,8 @@ struct __align__(16) RfCtl {
                                        // an even / odd conv (a neighbour may be one conv ahead)
   uint64_t xa_ready;                // the same for the network input
   uint64_t d_ready[2][2];           // tensor core -> workers: accumulators of an even / odd conv complete, by tile (one tile: both)
-  uint64_t w_full[kRfMaxSlots], w_empty[kRfMaxSlots];
+  uint64_t w_full[kRfMaxSlots];     // weight slots: copy landed
+  uint64_t w_empty[kRfMaxSlots];    // ... and both MMA warps are past it (count 2)
   uint64_t meta_full[3];
   uint32_t tmem_base, abort;
 };
@@ -167,6 +168,9 @@ __device__ void rf_loader(const Rf& f, const RfPlan& P, const LevelArgs& a, cons
 // them), so that one warp's waits and commit, 250 - 450 clocks a chunk, pass under the other's MMAs (360 - 570): 64 images of 8 x 8
 // 285 -> 248 us, of 4 x 4 289 -> 260, three of 32 x 32 in 8 x 16 blocks 539 -> 438; with two tiles a chunk's MMAs hid them already
 // (16 x 16 466 -> 465).
+// Every copy is seen by both warps, and a slot is empty when both are past it. A barrier's parity tells a phase only from the one before
+// it: a warp that tested a slot whose last copy had been the other's (rings of three slots, convs of three chunks) could take the
+// phase before that for its own, if that copy was late, and multiply with what was in the slot.
 __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq, int which) {
   RfCtl* ctl = f.ctl;
   uint8_t* smem = f.smem;
@@ -199,7 +203,10 @@ __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq, int which)
     if (one && which >= nk) wait_chunk(0);
 #pragma unroll 1
     for (int kc = 0; kc < nk; ++kc) {
-      if (!one || (kc & 1) == which) {
+      if (one && (kc & 1) != which) {
+        rf_wait(f, &ctl->w_full[slot], round & 1u);
+        if (ptx::elect_one()) rf_arrive_local(&ctl->w_empty[slot]);
+      } else {
         // (all that the wait need not precede: an instruction of this warp takes about 13 clocks)
         uint32_t bl = addr16(P.s_ring + slot * P.slot_bytes) | b_lbo;
         const uint32_t a_bias = addr16(P.s_const + (uns ? 0u : 2304u)) | (8u << 16);
@@ -224,8 +231,8 @@ __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq, int which)
           ptx::umma_commit(ptx::smem_u32(&ctl->w_empty[slot]));
         }
         acc = 1u;
-        __syncwarp();
       }
+      __syncwarp();
       if (++slot == (uint32_t)P.n_slots) { slot = 0; ++round; }
       a_chunk += 2u * plane;
     }
@@ -568,7 +575,7 @@ __global__ void __launch_bounds__(kRfThreads, 1) res_flow_kernel(const LevelArgs
     for (int s = 0; s < 3; ++s) ptx::mbar_init(ptx::smem_u32(&ctl.meta_full[s]), 1);
     for (int s = 0; s < kRfMaxSlots; ++s) {
       ptx::mbar_init(ptx::smem_u32(&ctl.w_full[s]), 1);
-      ptx::mbar_init(ptx::smem_u32(&ctl.w_empty[s]), (uint32_t)P.tiles);
+      ptx::mbar_init(ptx::smem_u32(&ctl.w_empty[s]), 2);
     }
     ptx::mbar_init_fence();
     ctl.abort = 0;

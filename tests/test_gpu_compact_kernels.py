@@ -165,6 +165,25 @@ def test_residual_blocks_through_long_chains(G, hidden, batch, plan):
     G.iodf_check(m)
 
 
+@pytest.mark.parametrize("in_c,hw,hidden,prune,batch", [
+    (6, 32, 128, (0.6, 0.9), 2),     # 16 x 16 in two blocks, 24 channels: three slots, convs of one, three and four chunks
+    (3, 16, 96, None, 3),            # 8 x 8: four slots, three chunks everywhere
+    (12, 8, 128, (0.4, 0.7), 2),     # 4 x 4: two to four chunks
+])
+def test_weight_slots_pass_between_the_warps_that_read_them(G, in_c, hw, hidden, prune, batch):
+    """Levels of one tile have two warps that take a conv's chunks in turn, and with it a slot of the weight ring is now one's, now
+    the other's: the same call again and again."""
+    import torch
+    model = S.make_residual_model(0xFE00 + hw, in_c, hw, hw, [True], 2, hidden, 4, prune=prune)
+    x = np.random.default_rng(hw).integers(0, 256, (batch, in_c, hw, hw), dtype=np.uint8)
+    m, z, _ = _both_ways(G, model, x)
+    assert G.iodf_level_kernel_name(m, 0) == "res_flow_kernel"
+    xt, zt = _t(x), _t(z)
+    for _ in range(50):
+        assert torch.equal(G.iodf_forward(m, xt)[0], zt) and torch.equal(G.iodf_inverse(m, zt), xt)
+    G.iodf_check(m)
+
+
 @pytest.mark.parametrize("per_sm,elems", [(0, 97), (24, 103), (25, 103), (40, 31), (41, 33)])   # streams per SM: up to 40 a warp each,
 @pytest.mark.parametrize("ls", [0, 20, 40, 63])                                                 # then half of one
 def test_symbol_look_up_at_every_kind_of_scale(G, ls, per_sm, elems):
