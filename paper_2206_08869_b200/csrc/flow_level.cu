@@ -174,6 +174,7 @@ __device__ __forceinline__ void flow_release_to_neighbours(const FlowPlan& P, co
 }
 
 __device__ __forceinline__ void worker_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kFlowWorkers) : "memory"); }
+__device__ __forceinline__ void mma_barrier() { asm volatile("bar.sync 2, %0;" ::"n"(2 * 32) : "memory"); }      // both slots' MMA warps
 
 // ---- weight and meta loader (one lane) -----------------------------------------------------------------
 __device__ void flow_loader(const Flow& f, const FlowPlan& P, const LevelArgs& a, const Steps& st) {
@@ -411,12 +412,14 @@ __device__ void flow_mma(const Flow& f, const FlowPlan& P, const Steps& st, int 
       const bool last = t + 2 >= f.tiles;
       // A step starts both slots at once, and MMAs issued in turn complete together: both slots would wait for the sum of their GEMMs, at
       // this one and, in step, at every later one. Slot 0's go first (two images of 8 x 8 with 48 channels 53 -> 49 us, of 24 45 -> 43,
-      // 128 images of 16 x 16 55.2 -> 53.2, of 32 x 32 132 -> 131.5; slot 1 a whole GEMM and epilogue behind: 32 x 32 133).
+      // 128 images of 16 x 16 55.2 -> 53.2, of 32 x 32 132 -> 131.5; slot 1 a whole GEMM and epilogue behind: 32 x 32 133). Both
+      // warps wait, slot 0's for one that is there by then: a warp that only arrived would run ahead once a wait has given up, and two
+      // of its arrivals would stand for one of the other's, which would then wait for good.
       const bool order = f.slots == 2 && t == sl;
-      if (order && sl == 1) asm volatile("bar.sync 2, 64;" ::: "memory");
+      if (order && sl == 1) mma_barrier();
       first_conv(t, dm);
       commit(&ctl->dm_ready[sl]);
-      if (order && sl == 0) asm volatile("bar.arrive 2, 64;" ::: "memory");
+      if (order && sl == 0) mma_barrier();
       if (last) commit(&ctl->w_empty[0]);
       if (t == sl) wait_w(1);
       hidden(ks2, P.chunk2, [&](int k0, int k1) { flow_gemm(d2, a_lo, 2u * pitch16, b2, n2, k0, k1, idesc_m); });
