@@ -29,11 +29,15 @@ constexpr int kEncodeStreams = 128, kEncodeThreads = 3 * kEncodeStreams, kBatch 
 __host__ __device__ inline size_t encode_buffers_at(const RansArgs& a) {       // offset in the encoder's shared memory, after the tables
   return (4 * (size_t)a.n_scales + 2 * (size_t)(2 * a.umax + 1) + 15) / 16 * 16;
 }
-// More streams of a block with prior parameters than this per SM: half a warp each. A warp per stream is then ten warps and more per
-// scheduler, and issue slots bound it. Whole warps and halves measured at 148 SMs, streams of 128: 1 536 39 and 66 us, 3 072 56 and 70,
-// 4 800 78 and 80, 6 144 93 and 89, 7 200 105 and 103, 28 800 354 and 304. Blocks without prior parameters have one scale, whose look-up
-// table stays in the L1 cache, and always take halves: 192 and 768 streams 35 either way, 2 400 47 and 39, 3 600 64 and 43.
-constexpr long kHalfWarpStreamsPerSm = 40;
+// More streams of a block than this per SM: half a warp each. A warp per stream then has six warps and more per scheduler, and issue
+// slots bound it. Where the line lies depends on the residuals, which a launch does not know: us for streams of 128 at 148 SMs, residuals
+// distributed as the prior says (scales 1 - 32) | uniform over +-3 000, a third of them escapes:
+//   streams per SM        5          10          16          21          28          36          49
+//   a warp each     40 | 46     42 | 50     52 | 60     58 | 68     66 | 78     83 | 97   109 | 126
+//   half of one     49 | 70     50 | 70     46 | 72     46 | 75     50 | 79     54 | 87    68 | 110
+// Blocks without prior parameters have one scale, whose look-up table stays in the L1 cache: 36 | 46, 40 | 48, 48 | 58, 56 | 68, 64 | 77
+// a warp each and 40 | 52, 42 | 52, 45 | 56, 46 | 56, 50 | 62 half of one.
+constexpr long kHalfWarpStreamsPerSm = 24, kHalfWarpStreamsPerSmOneScale = 12;
 
 struct Tables {
   const uint16_t* G;       // shared memory
@@ -324,7 +328,7 @@ __global__ void __launch_bounds__(kThreadsPerBlock) rans_decode_kernel(const Ran
 }
 
 // The same with HALF a warp per stream, for blocks of so many streams that issue slots bound the time and not a stream's chain, which
-// is longer here, and for those without prior parameters. The slot's upper eight bits select, for the element's scale, the symbols
+// is longer here. The slot's upper eight bits select, for the element's scale, the symbols
 // that it can mean (a table made with the codec: first and count, usually a handful, 257 at most); a lane tests one candidate,
 // after a round in steps where there are more than fifteen. A warp's two streams go side by side, so steps that only some symbols take (escapes, a word more)
 // are selections, not branches. Words: the lanes hold the next 16, replaced lane by lane every four symbols from the ones after
@@ -565,7 +569,7 @@ cudaError_t launch_rans_encode(const RansArgs& a, const int32_t* z, const int32_
 cudaError_t launch_rans_decode(const RansArgs& a, int block, const uint16_t* words, const uint32_t* counts,
                                const int32_t* prior, int32_t* z, cudaStream_t stream) {
   const long streams = (long)a.batch * a.blocks[block].n_streams;
-  const bool half = a.blocks[block].prior_off < 0 || streams > kHalfWarpStreamsPerSm * a.n_sms;
+  const bool half = streams > (a.blocks[block].prior_off < 0 ? kHalfWarpStreamsPerSmOneScale : kHalfWarpStreamsPerSm) * a.n_sms;
   const long total = streams * (half ? 16 : 32);
   const unsigned grid = (unsigned)((total + kThreadsPerBlock - 1) / kThreadsPerBlock);
   if (half) rans_decode_half_kernel<<<grid, kThreadsPerBlock, table_smem(a), stream>>>(a, block, words, counts, prior, z);

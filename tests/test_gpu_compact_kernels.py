@@ -184,8 +184,8 @@ def test_weight_slots_pass_between_the_warps_that_read_them(G, in_c, hw, hidden,
     G.iodf_check(m)
 
 
-@pytest.mark.parametrize("per_sm,elems", [(0, 97), (24, 103), (25, 103), (40, 31), (41, 33)])   # streams per SM: up to 40 a warp each,
-@pytest.mark.parametrize("ls", [0, 20, 40, 63])                                                 # then half of one
+@pytest.mark.parametrize("per_sm,elems", [(0, 97), (24, 103), (25, 103), (40, 31), (41, 33)])   # streams per SM: up to 24 a warp each
+@pytest.mark.parametrize("ls", [0, 20, 40, 63])                                                 # (one scale: 12), then half of one
 def test_symbol_look_up_at_every_kind_of_scale(G, ls, per_sm, elems):
     """Residuals over the whole window at one scale: slots that mean one symbol and slots that mean hundreds."""
     import torch

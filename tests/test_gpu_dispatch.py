@@ -1,0 +1,51 @@
+"""Which kernel, and how many CTAs of it, a call of a given size is: rules that only change the time, so that no comparison of
+outputs notices when a range of sizes ends up on the slower side."""
+import json
+import re
+
+import numpy as np
+import pytest
+
+import iodf_synth as S
+from test_gpu_parity import G  # noqa: F401  (the fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def _launches(fn, tmp_path):
+    """(kernel name, CTAs) of what fn launches."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        fn()
+        torch.cuda.synchronize()
+    trace = tmp_path / "trace.json"
+    prof.export_chrome_trace(str(trace))
+    events = [e for e in json.loads(trace.read_text())["traceEvents"] if e.get("cat") == "kernel"]
+    if not events:
+        pytest.skip("kernel activity is not recorded here")
+    return [(re.search(r"\w+_kernel", e["name"]).group(), int(np.prod(e["args"]["grid"]))) for e in sorted(events, key=lambda e: e["ts"])]
+
+
+@pytest.mark.parametrize("block,line", [(0, 24), (1, 12)])       # with prior parameters; the final block, of one scale
+@pytest.mark.parametrize("more", [0, 1])
+def test_streams_take_half_a_warp_above_a_line(G, block, line, more, tmp_path):
+    import torch
+    per_image = 16                                               # streams of an image to a block
+    B = line * torch.cuda.get_device_properties(0).multi_processor_count // per_image + more
+    model = S.make_model(0xFF00, 3, 32, 32, [True, False], 1, 16)
+    d, d_fact = 3 * 32 * 32, 6 * 256
+    m = G.iodf_create(model, B)
+    codec = G.iodf_codec_create(m, S.logistic_codec(elems_per_stream=96))
+    rng = np.random.default_rng(block)
+    z = torch.from_numpy(rng.integers(-40, 41, (B, d)).astype(np.int32)).cuda()
+    prior = torch.from_numpy(np.stack([rng.integers(-9, 10, (B, d_fact)), np.full((B, d_fact), 20)], axis=1).astype(np.int32)).cuda()
+    words, counts = G.iodf_rans_encode(codec, z, prior)
+    assert counts.shape == (B, 2 * per_image)
+    out = torch.zeros_like(z)
+    run = _launches(lambda: G.iodf_rans_decode_block(codec, block, words, counts, prior, out), tmp_path)
+    G.iodf_codec_check(codec)
+    part = slice(0, d_fact) if block == 0 else slice(d_fact, d)
+    assert torch.equal(out[:, part], z[:, part])
+    assert [name for name, _ in run] == ["rans_decode_half_kernel" if more else "rans_decode_kernel"]
