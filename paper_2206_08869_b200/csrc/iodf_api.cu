@@ -762,10 +762,14 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
   R.group = 1;
   if (R.w % 16 == 0 && R.h % 16 == 0) {
     // 16 x 16 blocks, or 8 x 16 ones while all clusters of a batch run at once (half the multiply time per conv for an exchange of
-    // edges: 0.44 against 0.65 ms for three 32 x 32 images, 432 against 459 us for 64 of 16 x 16)
+    // edges: 0.44 against 0.65 ms for three 32 x 32 images). An image of 16 x 16, which would need no exchange, is cut only where convs
+    // have more than one chunk of 32 channels. 64 images, two couplings of eight blocks, whole and cut: width 16 52 and 56 us,
+    // 32 54 and 57, 40 80 and 72, 64 82 and 73, 96 104 and 108 (pruned to 40 - 70 % 94 and 93), 128 131 and 125; one image the same.
     R.bh = R.bw = 16; R.m = 128;
     const int split = (R.w / 8) * (R.h / 16);
-    if (!throughput && split <= 8 && (int)max_batch <= max_res_flow_clusters(split, smem_limit)) R.bw = 8;
+    uint32_t width = 0;
+    for (uint32_t ki = 0; ki < lv.n_couplings; ++ki) width = std::max(width, lv.couplings[ki].layers[0].c_out);
+    if (!throughput && split <= 8 && (R.w * R.h > 256 || width > 32) && (int)max_batch <= max_res_flow_clusters(split, smem_limit)) R.bw = 8;
     R.tiles = R.bw / 8;
   } else if (R.w == 8 && R.h == 8) {
     R.bw = R.bh = 8; R.m = 64; R.tiles = 1;

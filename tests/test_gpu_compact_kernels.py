@@ -141,7 +141,7 @@ def test_throughput_plan_takes_the_least_sm_time_per_image(G, hidden, images):
 @pytest.mark.parametrize("hw,splits,couplings,hidden,blocks,prune,batch,plan", [
     (64, [True], 1, 128, 1, None, 1, 0),           # 32 x 32 in eight 8 x 16 blocks
     (64, [True], 1, 128, 1, None, 1, 1),           # ... in four 16 x 16 ones
-    (32, [True], 2, 97, 2, (0.4, 0.7), 2, 0),      # 16 x 16: one block, four chunks with a ragged last one
+    (32, [True], 2, 97, 2, (0.4, 0.7), 2, 0),      # 16 x 16: two blocks, four chunks with a ragged last one
     (16, [True], 1, 32, 1, None, 3, 0),            # 8 x 8: one chunk
     (8, [True], 1, 65, 2, None, 5, 1),             # 4 x 4: three images and two
 ])

@@ -7,7 +7,8 @@ import numpy as np
 import pytest
 
 import iodf_synth as S
-from test_gpu_parity import G  # noqa: F401  (the fixture)
+from test_gpu_parity import G, _t  # noqa: F401  (G: the fixture)
+from test_gpu_residual import _both_ways
 
 pytestmark = pytest.mark.gpu
 
@@ -49,3 +50,18 @@ def test_streams_take_half_a_warp_above_a_line(G, block, line, more, tmp_path):
     part = slice(0, d_fact) if block == 0 else slice(d_fact, d)
     assert torch.equal(out[:, part], z[:, part])
     assert [name for name, _ in run] == ["rans_decode_half_kernel" if more else "rans_decode_kernel"]
+
+
+@pytest.mark.parametrize("hidden,batch,plan,blocks", [
+    (32, 2, 0, 1),           # convs of one chunk: the exchange of edges costs more than the halved multiply time
+    (33, 2, 0, 2),           # two chunks
+    (97, 2, 0, 2),           # four, the last ragged
+    (97, 2, 1, 1),           # ... one block of two tiles, without neighbours
+    (33, 149, 0, 1),         # more images than half the SMs
+])
+def test_blocks_of_a_16x16_residual_image(G, hidden, batch, plan, blocks, tmp_path):
+    model = S.make_residual_model(0xFF20 + hidden, 3, 32, 32, [True], 2, hidden, 2, prune=(0.4, 0.7))
+    x = np.random.default_rng(hidden).integers(0, 256, (batch, 3, 32, 32), dtype=np.uint8)
+    m = _both_ways(G, model, x, plan=plan)[0] if batch < 9 else G.iodf_create(model, batch, plan=plan)
+    assert _launches(lambda: G.iodf_forward(m, _t(x)), tmp_path) == [("res_flow_kernel", batch * blocks)]
+    G.iodf_check(m)
