@@ -24,9 +24,9 @@
 //     meet by shuffles as the translation is applied. K steps start as the blocks of 32 channels are written. 128 images of 48
 //     channels: 48 us with per-tap partials, 40 by taps, 37.5 by rows; 256 of 24, two to a CTA: 65, 49.5, 45. The three products
 //     need columns: where those of both slots do not fit beside the hidden layers' and a slot has more tiles than one, taps stay.
-//   * A lane quarter of a 4 x 4 level's tile is an image. A CTA of one image (two) has four (two) copies of it in the operands' rows,
-//     so that all sixteen warps, not four, share its columns (P.copies): 128 images of 96 channels 47 -> 45 us, 64 of width 512
-//     98 -> 92.
+//   * A lane quarter of a 4 x 4 level's tile is an image. Of a CTA's one image (two) the operands' rows can hold four (two) copies,
+//     so that all sixteen warps, not four, share its columns (P.copies; the host's rule says where there is enough to share): 64 images
+//     of 96 channels, eight couplings of width 128: 40 -> 37 us, of width 512 95 -> 86.
 //   * CTAs of several tiles have two in flight (slots), each with eight of the sixteen workers and an MMA
 //     warp of its own, so that one slot's hand-overs and MMAs run under the other's requantisation; CTAs of
 //     one tile put all sixteen workers on it. One lane of another warp streams weights and meta blocks.

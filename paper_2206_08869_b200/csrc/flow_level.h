@@ -35,7 +35,7 @@ struct FlowPlan {
   // GEMM tiles. A tile is an 8-column block of an image, 16 (m = 128) or 8 (m = 64) rows high, or, at
   // 4 x 4 levels (im2col), up to four whole images of 16 pixels each (m = 64)
   int32_t m, im2col;
-  int32_t copies;                // 4 x 4: operand rows hold every image that often, in a lane quarter each (one tile of one or two images)
+  int32_t copies;                // 4 x 4: operand rows hold every image that often, in a lane quarter each (1, or up to four rows of images)
   int32_t tiles;                 // of the CTA
   int32_t tiles_img, tiles_x;    // of an image; 8-column blocks per row
   int32_t rec;                   // bytes of a position's record in the network-input frame

@@ -992,8 +992,12 @@ bool plan_flow(FlowPlan& F, const FlowNeeds& nd, uint32_t limit, int group, bool
   }
   F.pitch = F.m * 16 + 64;
   F.acc_stride = F.pg + 4;
-  // (4 x 4: operands with copies of the images where they fit, also where that makes two matrices share a slot)
-  const int most_copies = F.im2col && group <= 2 ? 4 / group : 1;
+  // 4 x 4: operands with copies of the images, also where that makes two matrices share a slot. What they share out over more warps is
+  // the last conv's units of eight channels and a streamed level's blocks; where a quarter's four warps have a unit and
+  // a few blocks each, the copies' stores cost more. 64 images, eight couplings, without and with: 8 channels of width 16 23 and 25 us,
+  // of 256 32 and 34; 24 channels 24 and 25, 34 and 36; 48 25 and 26, 39 and 40; 72 30 and 28, 48 and 47; 96 31 and 29, 52 and 52;
+  // streamed at width 512 8 channels 63 and 59, 96 95 and 86. Two images (200 in the call): 72 channels 33 and 32, 51 and 51.
+  const int most_copies = F.im2col && group <= 2 && (wide || F.cb > 32) ? 4 / group : 1;
   for (int form = 0; form < 4; ++form) {
     const int alias = form & 1;
     F.copies = form < 2 ? most_copies : 1;

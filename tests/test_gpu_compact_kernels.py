@@ -53,12 +53,12 @@ def test_last_conv_by_rows_of_taps(G, in_c, hidden, batch, plan, sample):
 
 
 @pytest.mark.parametrize("in_c,hidden,batch,plan,sample", [
-    (2, 16, 1, 0, None),                  # one image in four lane quarters, a block for one of sixteen warps
+    (2, 16, 1, 0, None),                  # one image in one of four lane quarters, a block for one of four warps
     (6, 256, 1, 0, None),                 # nine blocks
-    (24, 176, 3, 0, None),                # 96 channels: the first and the last matrix share a slot
-    (12, 512, 2, 0, None),                # streamed weights
+    (24, 176, 3, 0, None),                # 96 channels, copies: the first and the last matrix share a slot
+    (12, 512, 2, 0, None),                # streamed weights: copies in all lane quarters
     (4, 33, 3, 1, None),                  # several images to a CTA
-    (12, 130, 299, 0, [0, 1, 297, 298]),  # two to a CTA, the last alone: two copies, and two quarters without an image
+    (12, 130, 299, 0, [0, 1, 297, 298]),  # two to a CTA, the last alone, and quarters without an image
 ])
 def test_copies_of_4x4_images(G, in_c, hidden, batch, plan, sample):
     model = S.make_model(0xFD00 + in_c + hidden, in_c, 8, 8, [True], 3, hidden)
