@@ -42,9 +42,9 @@
 //     frame needs no release: the MMAs that read it have completed before anything is sent that lets a neighbour go on.)
 //
 // What bounds it: the chain of a coupling (7 000 - 9 000 clocks where a CTA has one tile) and 3 000 clocks per tile of 128 pixels:
-// requantisation, shifted sum and their hand-overs, at five to nine clocks an instruction and warp (50 % of all issue slots at
-// 32 x 32, 33 % at 8 x 8, 23 % at 4 x 4; of 32 x 32's 130 us the phases' skeleton of waits, hand-overs and MMAs takes half). Measured for eight
-// couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 130 us,
+// requantisation, shifted sum and their hand-overs, at five to nine clocks an instruction and warp (54 % of an SM's issue slots at
+// 32 x 32, 41 % at 8 x 8, 34 % at 4 x 4; of 32 x 32's 133 us the phases' skeleton of waits, hand-overs and MMAs takes half). Measured for eight
+// couplings of hidden widths 103 - 179 (mean 143), 128 images (general kernel before): 32 x 32 x 12 channels 218 -> 133 us,
 // 16 x 16 85 -> 53, 8 x 8 63 -> 37, 4 x 4 70 -> 45; one image, 32 x 32 split in eight: 48. Width 512, 64 images of
 // 32 x 32, split in two: 2 357 -> 286 us, the tensor core busy a third of it.
 #include <stddef.h>

@@ -762,7 +762,7 @@ bool plan_res_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& h
   R.group = 1;
   if (R.w % 16 == 0 && R.h % 16 == 0) {
     // 16 x 16 blocks, or 8 x 16 ones while all clusters of a batch run at once (half the multiply time per conv for an exchange of
-    // edges: 0.44 against 0.65 ms for three 32 x 32 images). An image of 16 x 16, which would need no exchange, is cut only where convs
+    // edges: 0.43 against 0.63 ms for three 32 x 32 images). An image of 16 x 16, which would need no exchange, is cut only where convs
     // have more than one chunk of 32 channels. 64 images, two couplings of eight blocks, whole and cut: width 16 52 and 56 us,
     // 32 54 and 57, 40 80 and 72, 64 82 and 73, 96 104 and 108 (pruned to 40 - 70 % 94 and 93), 128 131 and 125; one image the same.
     R.bh = R.bw = 16; R.m = 128;
@@ -1330,11 +1330,11 @@ bool plan_flow_level(const iodf_level_desc& lv, const Blobs& B, HostLevel& hl, c
   // CTA that grows with the mean hidden width and the channels that are translated, the exchange of edges, what an image more costs
   // at 4 x 4, a weight ring too short to run ahead of wide layers (without that term shapes of three slots take 17 % longer than
   // the rule says, of four 11 %, of five and more 1 %). Fitted to 564 shapes of 53 flows (widths 16 - 512, 2 - 56 translated
-  // channels, 4 x 4 - 32 x 32, 2 - 12 couplings) at batches of 1 - 1 184: 5 % off on average. The shape it picks takes 0.09 % longer than
-  // the best one on average and 12 % at most (a 4 x 4 level of two couplings, 20 us); for 253 shapes of 27 flows that had no
-  // part in it 0.12 % and 11 %. (Fitted before a slot's first GEMM went ahead of the other's and 8 x 8 convs went by rows of taps:
-  // shapes of two slots take 2 - 8 % less since, 8 x 8 ones 6 - 10 %.) Constants fitted to five flows and used with twice the width that they were fitted with: 0.38 %
-  // and 25 %, 0.34 % and 12 %.
+  // channels, 4 x 4 - 32 x 32, 2 - 12 couplings) at batches of 1 - 1 184, when its choice took 0.09 % longer than the best shape on
+  // average. The kernels have changed since: shapes of two slots take 2 - 8 % less, 8 x 8 ones 6 - 10 %, 4 x 4 ones with copies of their
+  // images up to 10 %. For 456 calls of 42 levels (12 - 96 channels, 4 x 4 - 32 x 32, widths 64 - 400, batches of 1 - 1 000) the
+  // choice takes 0.3 % longer than the best shape on average and 9 % at most (16 x 16 images of 24 channels, width 256: 512 of
+  // them two to a CTA 436 us, four 399); width 400 has four calls of 5 - 6 %.
   auto add_shape = [&](const FlowPlan& f, int ctas) {
     const double width = widths / (400.0 * F.n_couplings), cb = f.cb / 10.0;        // mean of both layers, in 200 channels
     const bool split = f.nbx * f.nby > 1;

@@ -16,7 +16,8 @@
 //   * Biases are a tenth operand row group: one more K step against a constant operand (1, c, ..., c).
 //     Hidden outputs are then one fma.rn.sat each (FloatRq), the branch of a block one high multiply-add
 //     and shift, its shortcut one multiply on the byte as a subnormal.
-//   * Larger images are cut into 16 x 16 blocks, one CTA of a cluster each. Edge positions are also stored
+//   * Larger images are cut into blocks of 16 x 16 or 8 x 16, one CTA of a cluster each, and so are 16 x 16 images whose convs
+//     have more than one chunk, while a batch leaves SMs for it. Edge positions are also stored
 //     into the neighbours' frames, asynchronously: the neighbours' chunk barriers count the bytes, and there is no
 //     cluster barrier between convs.
 //   * Two warps issue the MMAs (a chunk's nine taps per wait: waits and commits cost a lane 150 clocks
@@ -24,9 +25,9 @@
 //     epilogue adds. One lane of another streams weights and the convs' meta blocks.
 //
 // What bounds it: a conv's chain of first chunk -> 36 MMAs (1 500 - 2 400 clocks) -> last chunk's epilogue -> hand-over,
-// 3 200 clocks at 8 x 8 and 4 x 4 images, 5 600 at 16 x 16 (in two blocks), 145 convs one after another. Measured at width 128 with
-// eight blocks, eight couplings (res_level.cu before): 64 images of 16 x 16 1 610 -> 410 us, 8 x 8 750 -> 233,
-// 4 x 4 740 -> 240; 32 images of 32 x 32 1 750 -> 635.
+// 3 300 clocks at 8 x 8 and 4 x 4 images, 5 700 at 16 x 16 (in two blocks), 145 convs one after another. Measured at width 128 with
+// eight blocks, eight couplings (res_level.cu before): 64 images of 16 x 16 1 610 -> 420 us, 8 x 8 750 -> 240,
+// 4 x 4 740 -> 245; 32 images of 32 x 32 1 750 -> 627.
 #include "res_flow.h"
 #include "level_device.cuh"
 
@@ -170,7 +171,8 @@ __device__ void rf_loader(const Rf& f, const RfPlan& P, const LevelArgs& a, cons
 // (16 x 16 466 -> 465).
 // Every copy is seen by both warps, and a slot is empty when both are past it. A barrier's parity tells a phase only from the one before
 // it: a warp that tested a slot whose last copy had been the other's (rings of three slots, convs of three chunks) could take the
-// phase before that for its own, if that copy was late, and multiply with what was in the slot.
+// phase before that for its own, if that copy was late, and multiply with what was in the slot. (The other's copies cost it a test and an
+// arrival each: 64 images of 32 x 32 873 -> 890 us for the whole call.)
 __device__ void rf_mma(const Rf& f, const RfPlan& P, const RfSeq& sq, int which) {
   RfCtl* ctl = f.ctl;
   uint8_t* smem = f.smem;
@@ -462,7 +464,8 @@ __device__ void rf_workers(const Rf& f, const RfPlan& P, const LevelArgs& a, con
         if (f.lane == 0) rf_arrive_local(&ctl->chunk_ready[q & 1][0]);
         // The next conv starts with chunk 0, so that chunk's warps go first: with all at once each takes longer and the MMAs wait
         // (arrivals ahead of the wait, without the delay that this wait is: 64 images of 32 x 32 927 -> 970 us for the whole call; with
-        // the pauses 895 -> 870).
+        // the pauses 895 -> 870). A pause is a hint, of nothing to twice its length, and nothing but time depends on it. At width 128
+        // convs take 1 - 3 % longer without, at 16 - 64 the same, with three 4 x 4 images to a CTA 2 - 4 % less.
         if (per == 2) __nanosleep(120);
         else if (c0 >= 2) __nanosleep(c0 == 2 ? 200 : 300);
       }

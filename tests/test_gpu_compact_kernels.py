@@ -113,11 +113,11 @@ def test_split_images_through_long_chains(G, hw, hidden, batch):
 
 
 @pytest.mark.parametrize("hidden,batch,images", [
-    (96, 300, 1),        # three waves of one image 82 us, two of two images 92
-    (96, 512, 2),        # four 109, two 94
-    (256, 256, 2),       # two images, streamed weights 124 us; one image in two blocks, resident 140
-    (288, 160, 2),       # streamed: two waves of one image in two blocks 130 us, one of two images 123
-    (320, 200, 2),       # ... 133 and 127
+    (96, 300, 1),        # three waves of one image 72 us, two of two images 80
+    (96, 512, 2),        # four 96, two 82
+    (256, 256, 2),       # two images, streamed weights 116 us; one image in two blocks, resident 127
+    (288, 160, 2),       # streamed: two waves of one image in two blocks 119 us, one of two images 116
+    (320, 200, 2),       # ... 125 and 120
 ])
 def test_images_per_cta_follow_the_hidden_width(G, hidden, batch, images):
     """A 16 x 16 level of 24 channels: what a tile costs beside a coupling's serial part decides between more waves
